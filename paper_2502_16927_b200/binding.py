@@ -131,15 +131,19 @@ def _check(status: int, where: str) -> None:
         raise BigmacError(status, where)
 
 
+# The marshalling sits in front of every launch, and for one decoded token it took longer than the kernel (14 us of Python
+# around 5 us in the library): addresses are passed as plain integers, and the stream handle comes from the accessor that
+# builds no Stream object (0.1 us against 3.3).
+
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
         return None
     assert t.is_cuda and t.is_contiguous(), "tensors passed to libbigmac must be contiguous CUDA tensors"
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream() -> C.c_void_p:
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 # ---- the C ABI, name for name -------------------------------------------------------------------------
@@ -163,8 +167,9 @@ def bigmac_workspace_bytes(handle, T: int, training: bool):
 
 def _weights(W: Dict[str, torch.Tensor]) -> bigmac_weights_t:
     # w_down / w_up are absent for the projection-free layer (BIGMAC_FLAG_CDAC)
-    return bigmac_weights_t(_ptr(W.get("w_gate")), _ptr(W.get("b_gate")), _ptr(W.get("w_down")), _ptr(W.get("w1")),
-                            _ptr(W.get("w2")), _ptr(W.get("w_up")), _ptr(W.get("b1")), _ptr(W.get("b2")))
+    get = W.get
+    return bigmac_weights_t(_ptr(get("w_gate")), _ptr(get("b_gate")), _ptr(get("w_down")), _ptr(get("w1")),
+                            _ptr(get("w2")), _ptr(get("w_up")), _ptr(get("b1")), _ptr(get("b2")))
 
 
 def _grads(G: Dict[str, torch.Tensor]) -> bigmac_grads_t:
@@ -320,6 +325,7 @@ class Layer:
         self.tdtype = torch.bfloat16 if dtype == BIGMAC_BF16 else torch.float32
         self._scratch = None
         self._saved = None
+        self._need = {}
         self._T = None
 
     def close(self):
@@ -334,19 +340,29 @@ class Layer:
             pass
 
     def _workspaces(self, T, training):
-        s, v = bigmac_workspace_bytes(self.handle, T, training)
+        need = self._need.get((T, training))
+        if need is None:                                # a function of the handle's configuration, T and the direction
+            if len(self._need) >= 4096:
+                self._need.clear()
+            need = self._need[(T, training)] = bigmac_workspace_bytes(self.handle, T, training)
+        s, v = need
         if self._scratch is None or self._scratch.numel() < s:
             self._scratch = torch.empty(max(s, 256), dtype=torch.uint8, device=self.device)
         if training and (self._saved is None or self._saved.numel() < v):
             self._saved = torch.empty(max(v, 256), dtype=torch.uint8, device=self.device)
 
     def empty_routing(self, T):
-        E, k = self.cfg["E"], self.cfg["k"]
-        i32 = dict(dtype=torch.int32, device=self.device)
-        return {"topk_idx": torch.empty(T * k, **i32), "topk_w": torch.empty(T * k, dtype=torch.float32, device=self.device),
-                "counts": torch.empty(E, **i32), "offsets": torch.empty(E + 1, **i32),
-                "row_of_slot": torch.empty(T * k, **i32), "slot_of_row": torch.empty(T * k, **i32),
-                "counts_chosen": torch.empty(E, **i32), "aux_loss": torch.empty(1, dtype=torch.float32, device=self.device)}
+        # one allocation and one split instead of eight allocations (13 us); every table starts on a 16-byte boundary
+        E, n = self.cfg["E"], T * self.cfg["k"]
+        nn, ee = n + -n % 4, E + -E % 4
+        idx, w, row, slot, counts, chosen, aux, _, offsets = torch.empty(4 * nn + 3 * ee + 5, dtype=torch.int32, device=self.device).split_with_sizes(
+            [nn, nn, nn, nn, ee, ee, 1, 3, ee + 1])
+        if nn != n:
+            idx, w, row, slot = idx[:n], w[:n], row[:n], slot[:n]
+        if ee != E:
+            counts, chosen, offsets = counts[:E], chosen[:E], offsets[:E + 1]
+        return {"topk_idx": idx, "topk_w": w.view(torch.float32), "counts": counts, "offsets": offsets, "row_of_slot": row,
+                "slot_of_row": slot, "counts_chosen": chosen, "aux_loss": aux.view(torch.float32)}
 
     def route(self, x, W):
         T = x.shape[0]

@@ -294,7 +294,8 @@ void carve_ep_scratch(Carver& cv, const EpDims& m, EpBuffers& b) {
     b.splitk_ws = (float*)cv.take_bytes(dense_ws > expert_ws ? dense_ws : expert_ws);
     b.colsum_part = cv.take<float>((size_t)kColsumChunks * m.E);
     b.logits = cv.take<float>((size_t)m.T * m.E);
-    b.tb.block_counts = cv.take<int32_t>((size_t)(sort_blocks(m.N) + 1) * m.E);
+    b.tb.block_rows = sort_blocks(m.N) + 1;
+    b.tb.block_counts = cv.take<int32_t>((size_t)b.tb.block_rows * m.E);
     b.dy_lo = cv.take_bytes((size_t)m.T * m.r * es);
     b.dcat = cv.take_bytes((size_t)m.T * m.ldcat * es);
     b.dx_lo = m.cdac ? nullptr : b.dcat;                              // Eq. 3: dx' is dx itself
@@ -399,8 +400,15 @@ int bigmac_ep_route(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_we
         q.M = m.T; q.N = m.r; q.K = m.d;
         BIGMAC_TRY(gemm(L, G_DESCEND, q, st));
     }
-    { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_topk(b.logits, W->b_gate, m.T, m.E, m.k, b.tb.topk_idx, b.tb.topk_w, st)); }
-    { Stage s(L, S_TABLES, st, tables_kernel_count(m.N, m.E)); BIGMAC_CUDA(launch_tables(b.tb, m.T, m.E, m.k, kNoCapacity, st, L->status)); }
+    if (route_fused_supported(m.E, m.k)) {
+        const RouteSource src{b.logits, m.E, 1, 0, nullptr};
+        const int sms = gemm_tc_sm_count();
+        { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_route_fused(src, RouteMove{}, W->b_gate, b.tb, m.T, m.E, m.k, kNoCapacity, nullptr, sms, st, L->status, 0)); }
+        { Stage s(L, S_TABLES, st); BIGMAC_CUDA(launch_route_fused(src, RouteMove{}, W->b_gate, b.tb, m.T, m.E, m.k, kNoCapacity, nullptr, sms, st, L->status, 1)); }
+    } else {
+        { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_topk(b.logits, W->b_gate, m.T, m.E, m.k, b.tb.topk_idx, b.tb.topk_w, st)); }
+        { Stage s(L, S_TABLES, st, tables_kernel_count(m.N, m.E)); BIGMAC_CUDA(launch_tables(b.tb, m.T, m.E, m.k, kNoCapacity, st, L->status)); }
+    }
     BIGMAC_CUDA(cudaMemcpyAsync(my_counts, b.tb.counts, sizeof(int32_t) * m.E, cudaMemcpyDeviceToDevice, st));
     if (routing_out) {
         const cudaMemcpyKind kind = cudaMemcpyDeviceToDevice;

@@ -134,7 +134,8 @@ struct Tables {
     int32_t* slot_of_prow;  // [P]     -1 on padding rows
     int32_t* tile_expert;   // [P/kPad]
     int32_t* n_tiles;       // [1]     number of kPad-row tiles in use
-    int32_t* block_counts;  // [n_blocks, E] scratch of the counting sort
+    int32_t* block_counts;  // [block_rows, E] scratch of the counting sort
+    int block_rows;
     int32_t* counts_chosen; // [E]     slots that chose the expert, before any dropping (nullable)
 };
 
@@ -172,6 +173,27 @@ inline int tables_kernel_count(int64_t N, int E) {
 // is placed nowhere (row -1) and recorded there as 2.
 cudaError_t launch_tables(const Tables& tb, int T, int E, int k, int cap, cudaStream_t stream, int* status = nullptr);
 
+// Top-k, tables and (if mv.grouped is set) the dispatch in two launches, for the (E, k) of route_fused_supported.
+struct RouteSource {                    // gate logits [T, ld]; parts > 1: the sum of `parts` such matrices, part_stride apart
+    const float* logits;
+    int ld, parts;
+    int64_t part_stride;
+    float* logits_out;                  // nullable: the logits as [T, E]
+};
+struct RouteMove {                      // rows of row_bytes bytes to the expert-grouped matrix `grouped` (null: tables only)
+    const void* src;                    // the rows, or
+    const float* partial;               // (non-null) fp32 partial results [parts][T, ld], added and rounded to bf16
+    int ld, parts;
+    int64_t part_stride;
+    void* grouped;
+    int row_bytes;
+    bool zero_padding;                  // padding rows are needed as zeros (what an inference forward finds there is never read)
+};
+bool route_fused_supported(int E, int k);
+// which: 0 = first launch (top-k, gate values, block counts), 1 = second launch (tables, rows).
+cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, const float* b_gate, const Tables& tb, int T, int E,
+                               int k, int cap, float* zero_word, int sm_count, cudaStream_t stream, int* status, int which);
+
 // Row moves.  `width` elements of the dtype per row; all row pointers 16-byte aligned.
 // grouped[prow,:] = src[slot_of_prow[prow]/k,:], zeros on padding rows, for prow < n_tiles*kPad.
 cudaError_t launch_dispatch(const void* src, void* grouped, const Tables& tb, int k, int width, int dtype,
@@ -186,9 +208,9 @@ cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float
                                int width, int dtype, int64_t max_prows, cudaStream_t stream);
 // Softmax-over-k backward: g = sum_i p_i dp_i, dl_j = p_j (dp_j - g); writes the dense [T,E] matrix
 // (zeros off the top-k set, and in the padding columns E..width-1) in the dtype, rows `ld` elements apart, and
-// leaves the fp32 dl_j in dp[slot].
+// leaves the fp32 dl_j in dp[slot].  may_drop: the dp of a slot without a row (prow_of_slot < 0) is taken as 0.
 cudaError_t launch_gate_bwd(float* dp, const Tables& tb, void* dlogits, int T, int E, int width, int ld, int k,
-                            int dtype, cudaStream_t stream);
+                            int dtype, cudaStream_t stream, bool may_drop = false);
 // Load-balancing loss (Table 5; conventional form, the paper prints none):
 //   L_aux = coef * E * sum_e f_e P_e,  f_e = counts_chosen[e] / (T k),  P_e = mean_t softmax_E(logits[t,:] + b_gate)[e].
 // Forward: loss[0] = L_aux; `partial` holds kAuxChunks * E floats of scratch.  Deterministic summation order.
@@ -199,7 +221,7 @@ cudaError_t launch_aux_loss(const float* logits, const float* b_gate, const int3
 // column sums of the second term go to aux_partial [kAuxChunks, E] for launch_gate_colsum.
 cudaError_t launch_gate_bwd_aux(float* dp, const Tables& tb, void* dlogits, const float* logits, const float* b_gate,
                                 float coef, float* aux_partial, int T, int E, int width, int ld, int k, int dtype,
-                                cudaStream_t stream);
+                                cudaStream_t stream, bool may_drop = false);
 // db[e] (+)= sum over the slots routed to e of dl_slot[slot] (the fp32 per-slot gate gradients launch_gate_bwd
 // leaves in dp); `partial` holds kColsumChunks * E floats of scratch.  Deterministic summation order.
 constexpr int kColsumChunks = 296;
@@ -220,6 +242,15 @@ cudaError_t launch_splitk_reduce(const float* ws, int parts, int M, int N, void*
 // [x' (bf16) | logits (fp32)] from the [parts][T][r + E] fp32 partial results of a split descend launch (r, E % 4 == 0).
 cudaError_t launch_descend_reduce(const float* ws, int parts, int T, int r, int E, void* x_lo, float* logits,
                                   cudaStream_t stream);
+
+// A few arrays of 32-bit words copied by one launch.
+struct WordCopies {
+    uint32_t* dst[8];
+    const uint32_t* src[8];
+    int64_t words[8];
+    int n;
+};
+cudaError_t launch_word_copies(const WordCopies& c, cudaStream_t stream);
 
 // Small-batch inference forward in one cooperative kernel (bf16, T <= 16): scratch logits [T,E], x_lo [T,r],
 // a [T*k,h], u [T*k,r] fp32; writes y, topk_idx, topk_w.  `barrier` is one device word owned by the handle.

@@ -100,9 +100,13 @@ void carve_saved(Carver& cv, const Dims& m, Buffers& b, bool with_z) {
     b.logits_saved = (with_z && m.aux > 0) ? cv.take<float>((size_t)m.T * m.E) : nullptr;
 }
 
-void carve_route_scratch(Carver& cv, const Dims& m, Buffers& b) {
+// `spare`: rows of block counts for a block of the routing kernel on every SM (bigmac_route_static, whose scratch has a fixed
+// size, makes do with the fewer blocks of the three-pass sort).
+void carve_route_scratch(Carver& cv, const Dims& m, Buffers& b, bool spare = true) {
     b.logits = cv.take<float>((size_t)m.T * m.E);
-    b.tb.block_counts = cv.take<int32_t>((size_t)(sort_blocks(m.N) + 1) * m.E);
+    b.tb.block_rows = sort_blocks(m.N) + 1;
+    if (spare && b.tb.block_rows < 192) b.tb.block_rows = 192;
+    b.tb.block_counts = cv.take<int32_t>((size_t)b.tb.block_rows * m.E);
     b.aux_part = m.aux > 0 ? cv.take<float>((size_t)kAuxChunks * m.E) : nullptr;
 }
 
@@ -199,24 +203,30 @@ int choose_split_k(int M, int N, int K) {
 }
 
 // Steps F2-F3 from the gate logits: top-k with softmax gate values, dispatch layout (under the capacity limit, if
-// any), load-balancing loss.
-int route_from_logits(const bigmac_layer* L, const Dims& m, const bigmac_weights_t* W, Buffers& b, cudaStream_t st) {
-    { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_topk(b.logits, W->b_gate, m.T, m.E, m.k, b.tb.topk_idx, b.tb.topk_w, st)); }
-    { Stage s(L, S_TABLES, st, tables_kernel_count(m.N, m.E)); BIGMAC_CUDA(launch_tables(b.tb, m.T, m.E, m.k, m.cap, st, L->status)); }
+// any), load-balancing loss; with mv.grouped set also F5, the rows of x' to their places.  zero_word: see launch_route_fused.
+int route_from_logits(const bigmac_layer* L, const Dims& m, const bigmac_weights_t* W, Buffers& b, const RouteSource& src,
+                      const RouteMove& mv, float* zero_word, cudaStream_t st) {
+    if (route_fused_supported(m.E, m.k)) {
+        const int sms = gemm_tc_sm_count();
+        { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_route_fused(src, mv, W->b_gate, b.tb, m.T, m.E, m.k, m.cap, zero_word, sms, st, L->status, 0)); }
+        { Stage s(L, mv.grouped ? S_DISPATCH : S_TABLES, st); BIGMAC_CUDA(launch_route_fused(src, mv, W->b_gate, b.tb, m.T, m.E, m.k, m.cap, zero_word, sms, st, L->status, 1)); }
+    } else {
+        { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_topk(src.logits, W->b_gate, m.T, m.E, m.k, b.tb.topk_idx, b.tb.topk_w, st)); }
+        { Stage s(L, S_TABLES, st, tables_kernel_count(m.N, m.E)); BIGMAC_CUDA(launch_tables(b.tb, m.T, m.E, m.k, m.cap, st, L->status)); }
+        if (zero_word) BIGMAC_CUDA(cudaMemsetAsync(zero_word, 0, sizeof(float), st));
+        if (mv.grouped) { Stage s(L, S_DISPATCH, st); BIGMAC_CUDA(launch_dispatch(mv.src, mv.grouped, b.tb, m.k, m.r, m.dtype, m.P, st)); }
+    }
     if (m.aux > 0) {
         Stage s(L, S_AUX_LOSS, st, 2);
         BIGMAC_CUDA(launch_aux_loss(b.logits, W->b_gate, b.tb.counts_chosen, m.T, m.E, m.k, m.aux, b.aux_part, b.aux_loss, st));
-        if (b.logits_saved)
-            BIGMAC_CUDA(cudaMemcpyAsync(b.logits_saved, b.logits, sizeof(float) * (size_t)m.T * m.E, cudaMemcpyDeviceToDevice, st));
     }
     return BIGMAC_OK;
 }
 
-// Steps F1-F3: gate logits on x, top-k with softmax gate values, dispatch layout.
-int run_routing(const bigmac_layer* L, const Dims& m, const void* x, const bigmac_weights_t* W, Buffers& b,
-                cudaStream_t st) {
+// Step F1 as a launch of its own: gate logits on x (a gate on x': descend first, logits from its stored value).
+int run_logits(const bigmac_layer* L, const Dims& m, const void* x, const bigmac_weights_t* W, Buffers& b, cudaStream_t st) {
     GemmArgs g;
-    if (m.gate_low) {                                // the gate reads x': descend first, logits from its stored value
+    if (m.gate_low) {
         GemmArgs q;
         q.A = x; q.lda = m.d; q.B = W->w_down; q.ldb = m.d; q.C = b.x_lo; q.ldc = m.r;
         q.M = m.T; q.N = m.r; q.K = m.d;
@@ -226,8 +236,17 @@ int run_routing(const bigmac_layer* L, const Dims& m, const void* x, const bigma
         g.A = x; g.lda = m.d; g.B = W->w_gate; g.ldb = m.d; g.K = m.d;
     }
     g.C = b.logits; g.ldc = m.E; g.M = m.T; g.N = m.E; g.out_f32 = true;
-    BIGMAC_TRY(gemm(L, G_LOGITS, g, st));
-    return route_from_logits(L, m, W, b, st);
+    return gemm(L, G_LOGITS, g, st);
+}
+
+// The word of a caller's aux_loss table that has to be set to zero because the layer has no such loss.
+float* aux_word_to_zero(const Dims& m, const bigmac_routing_t* out) { return out && m.aux <= 0 ? out->aux_loss : nullptr; }
+
+// Steps F1-F3 without the rest of the layer.
+int run_routing(const bigmac_layer* L, const Dims& m, const void* x, const bigmac_weights_t* W, Buffers& b,
+                const bigmac_routing_t* out, cudaStream_t st) {
+    BIGMAC_TRY(run_logits(L, m, x, W, b, st));
+    return route_from_logits(L, m, W, b, RouteSource{b.logits, m.E, 1, 0, nullptr}, RouteMove{}, aux_word_to_zero(m, out), st);
 }
 
 // Calls that keep no saved state (bigmac_route, the inference forward): the tables the caller asked for are produced
@@ -244,27 +263,25 @@ void alias_routing(Buffers& b, const bigmac_routing_t* out) {
     if (out->aux_loss) b.aux_loss = out->aux_loss;
 }
 
-// Copies the tables into the caller's arrays (a training forward keeps its own copy in `saved` for the backward);
-// members that alias_routing pointed at the caller's arrays are already in place.
-int export_routing(const Dims& m, const Buffers& b, bigmac_routing_t* out, cudaStream_t st) {
+// Copies the tables into the caller's arrays (a training forward keeps its own copy in `saved` for the backward), all in
+// one launch; members that alias_routing pointed at the caller's arrays are already in place.
+int export_routing(const bigmac_layer* L, const Dims& m, const Buffers& b, bigmac_routing_t* out, cudaStream_t st) {
     if (!out) return BIGMAC_OK;
-    const cudaMemcpyKind kind = cudaMemcpyDeviceToDevice;
-    if (out->topk_idx && out->topk_idx != b.tb.topk_idx)
-        BIGMAC_CUDA(cudaMemcpyAsync(out->topk_idx, b.tb.topk_idx, sizeof(int32_t) * m.N, kind, st));
-    if (out->topk_w && out->topk_w != b.tb.topk_w) BIGMAC_CUDA(cudaMemcpyAsync(out->topk_w, b.tb.topk_w, sizeof(float) * m.N, kind, st));
-    if (out->counts && out->counts != b.tb.counts) BIGMAC_CUDA(cudaMemcpyAsync(out->counts, b.tb.counts, sizeof(int32_t) * m.E, kind, st));
-    if (out->offsets && out->offsets != b.tb.offsets)
-        BIGMAC_CUDA(cudaMemcpyAsync(out->offsets, b.tb.offsets, sizeof(int32_t) * (m.E + 1), kind, st));
-    if (out->row_of_slot && out->row_of_slot != b.tb.row_of_slot)
-        BIGMAC_CUDA(cudaMemcpyAsync(out->row_of_slot, b.tb.row_of_slot, sizeof(int32_t) * m.N, kind, st));
-    if (out->slot_of_row && out->slot_of_row != b.tb.slot_of_row)
-        BIGMAC_CUDA(cudaMemcpyAsync(out->slot_of_row, b.tb.slot_of_row, sizeof(int32_t) * m.N, kind, st));
-    if (out->counts_chosen && out->counts_chosen != b.tb.counts_chosen)
-        BIGMAC_CUDA(cudaMemcpyAsync(out->counts_chosen, b.tb.counts_chosen, sizeof(int32_t) * m.E, kind, st));
-    if (out->aux_loss) {
-        if (m.aux <= 0) BIGMAC_CUDA(cudaMemsetAsync(out->aux_loss, 0, sizeof(float), st));
-        else if (out->aux_loss != b.aux_loss) BIGMAC_CUDA(cudaMemcpyAsync(out->aux_loss, b.aux_loss, sizeof(float), kind, st));
-    }
+    WordCopies c{};
+    auto add = [&](void* dst, const void* src, int64_t words) {
+        if (dst && dst != src) { c.dst[c.n] = (uint32_t*)dst; c.src[c.n] = (const uint32_t*)src; c.words[c.n++] = words; }
+    };
+    add(out->topk_idx, b.tb.topk_idx, m.N);
+    add(out->topk_w, b.tb.topk_w, m.N);
+    add(out->counts, b.tb.counts, m.E);
+    add(out->offsets, b.tb.offsets, m.E + 1);
+    add(out->row_of_slot, b.tb.row_of_slot, m.N);
+    add(out->slot_of_row, b.tb.slot_of_row, m.N);
+    add(out->counts_chosen, b.tb.counts_chosen, m.E);
+    if (m.aux > 0) add(out->aux_loss, b.aux_loss, 1);
+    if (c.n == 0) return BIGMAC_OK;
+    Stage s(L, S_TABLES, st);
+    BIGMAC_CUDA(launch_word_copies(c, st));
     return BIGMAC_OK;
 }
 
@@ -426,8 +443,8 @@ int bigmac_route(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_weigh
     carve_saved(cv, m, b, false);
     alias_routing(b, out);
     cudaStream_t st = (cudaStream_t)stream;
-    BIGMAC_TRY(run_routing(L, m, x, W, b, st));
-    return export_routing(m, b, out, st);
+    BIGMAC_TRY(run_routing(L, m, x, W, b, out, st));
+    return export_routing(L, m, b, out, st);
 }
 
 int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_weights_t* W, void* y,
@@ -448,6 +465,7 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
     if (training) {
         Carver cv(saved);
         carve_saved(cv, m, b, true);
+        if (b.logits_saved) b.logits = b.logits_saved;        // the backward of the load-balancing loss reads them
     } else {
         carve_saved(cs, m, b, false);
         alias_routing(b, routing_out);
@@ -466,47 +484,59 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
         }
         if (routing_out) {
             { Stage s(L, S_TABLES, st, tables_kernel_count(m.N, m.E)); BIGMAC_CUDA(launch_tables(b.tb, m.T, m.E, m.k, m.cap, st, L->status)); }
-            BIGMAC_TRY(export_routing(m, b, routing_out, st));
+            if (float* word = aux_word_to_zero(m, routing_out)) BIGMAC_CUDA(cudaMemsetAsync(word, 0, sizeof(float), st));
+            BIGMAC_TRY(export_routing(L, m, b, routing_out, st));
         }
         return BIGMAC_OK;
     }
     // F1 + F4 in one pass over x when the tile grid allows it: [x' | logits] = x [W'_down ; W_gate]^T, logits in fp32
     const int bn_desc = (m.r + m.E) >= 256 ? 256 : 128;
     const bool fuse_gate = !m.cdac && !m.gate_low && c.dtype == BIGMAC_BF16 && L->use_tc && L->tc_mask == ~0u && m.r % bn_desc == 0;
+    if (m.cdac) b.x_lo = const_cast<void*>(x);                                    // Eq. 3: experts read the token itself
+    const bool gather_dispatch = dispatch_is_fused(L, m, training);
+    RouteSource src{b.logits, m.E, 1, 0, nullptr};
+    RouteMove mv{};
     if (fuse_gate) {
         GemmArgs g;
         g.A = x; g.lda = m.d; g.B = W->w_down; g.ldb = m.d; g.C = b.x_lo; g.ldc = m.r;
         g.B2 = W->w_gate; g.ldb2 = m.d; g.n_split = m.r; g.C2 = b.logits; g.ldc2 = m.E; g.N2 = m.E;
         g.M = m.T; g.N = m.r + m.E; g.K = m.d;
-        if (b.descend_ws) {                                   // few tokens: contraction in parts, then [x' | logits] from them
-            g.split_k = descend_split_parts(m); g.out_f32 = true;
-            g.C = b.descend_ws; g.ldc = m.r + m.E; g.C2 = b.descend_ws + m.r; g.ldc2 = m.r + m.E;
+        if (b.descend_ws) {                                   // few tokens: contraction in parts, added by the routing kernels
+            const int ld = m.r + m.E, parts = descend_split_parts(m);
+            const int64_t part_stride = (int64_t)m.T * ld;
+            g.split_k = parts; g.out_f32 = true;
+            g.C = b.descend_ws; g.ldc = ld; g.C2 = b.descend_ws + m.r; g.ldc2 = ld;
             BIGMAC_TRY(gemm(L, G_DESCEND, g, st));
-            Stage s(L, S_SPLITK_REDUCE, st);
-            BIGMAC_CUDA(launch_descend_reduce(b.descend_ws, g.split_k, m.T, m.r, m.E, b.x_lo, b.logits, st));
+            if (route_fused_supported(m.E, m.k) && !gather_dispatch) {
+                src = RouteSource{b.descend_ws + m.r, ld, parts, part_stride, m.aux > 0 ? b.logits : nullptr};
+                mv.partial = b.descend_ws; mv.ld = ld; mv.parts = parts; mv.part_stride = part_stride;
+            } else {
+                Stage s(L, S_SPLITK_REDUCE, st);
+                BIGMAC_CUDA(launch_descend_reduce(b.descend_ws, parts, m.T, m.r, m.E, b.x_lo, b.logits, st));
+            }
         } else {
             BIGMAC_TRY(gemm(L, G_DESCEND, g, st));
         }
-        BIGMAC_TRY(route_from_logits(L, m, W, b, st));
     } else {
-        BIGMAC_TRY(run_routing(L, m, x, W, b, st));                               // F1-F3
+        BIGMAC_TRY(run_logits(L, m, x, W, b, st));                                // F1
+        if (!m.cdac && !m.gate_low) {                                             // F4 descend: x' = x W'_down
+            GemmArgs g;
+            g.A = x; g.lda = m.d; g.B = W->w_down; g.ldb = m.d; g.C = b.x_lo; g.ldc = m.r;
+            g.M = m.T; g.N = m.r; g.K = m.d;
+            BIGMAC_TRY(gemm(L, G_DESCEND, g, st));
+        }
     }
-    BIGMAC_TRY(export_routing(m, b, routing_out, st));
-    if (m.cdac) b.x_lo = const_cast<void*>(x);                                    // Eq. 3: experts read the token itself
-    if (!fuse_gate && !m.cdac && !m.gate_low) {                                   // F4 descend: x' = x W'_down
-        GemmArgs g;
-        g.A = x; g.lda = m.d; g.B = W->w_down; g.ldb = m.d; g.C = b.x_lo; g.ldc = m.r;
-        g.M = m.T; g.N = m.r; g.K = m.d;
-        BIGMAC_TRY(gemm(L, G_DESCEND, g, st));
+    // F2, F3 and F5 (dispatch at width r) - unless the dispatch is fused into its consumers: expert GEMM1's producer warp
+    // then gathers the rows of x' itself (slot_of_prow names the token of every grouped row, -1 the zero padding rows) and
+    // the grouped copy xg is never written.
+    if (!gather_dispatch) {
+        mv.src = b.x_lo; mv.grouped = b.xg; mv.row_bytes = m.r * (int)esize(m.dtype); mv.zero_padding = training;
     }
-    // F5 dispatch at width r - unless it is fused into its consumers: expert GEMM1's producer warp then gathers the
-    // rows of x' itself (slot_of_prow names the token of every grouped row, -1 the zero padding rows) and the grouped
-    // copy xg is never written.
+    BIGMAC_TRY(route_from_logits(L, m, W, b, src, mv, aux_word_to_zero(m, routing_out), st));
+    BIGMAC_TRY(export_routing(L, m, b, routing_out, st));
     const bool short_list = m.P / kPad <= 2 * (int64_t)gemm_tc_sm_count();
     const bool mlp_fused_ = !training && !m.bias && (switches().fused_mlp == 2 || (switches().fused_mlp == 1 && short_list)) &&
                             sigma_as_bytes(L) && fused_mlp_supported(m.r, m.h, m.dtype);
-    const bool gather_dispatch = dispatch_is_fused(L, m, training);
-    if (!gather_dispatch) { Stage s(L, S_DISPATCH, st); BIGMAC_CUDA(launch_dispatch(b.x_lo, b.xg, b.tb, m.k, m.r, m.dtype, m.P, st)); }
     // Inference, low width r <= 256, up to two row tiles per SM: F6 + F7 in one kernel, the hidden activations stay on
     // the SM.  On long tile lists the two separate GEMMs are faster (the fused kernel is bound by the issue of its many
     // narrow MMA instructions): measured 0.375 vs 0.329 ms forward at the medium workload, 0.099 vs 0.106 ms at 512
@@ -627,7 +657,6 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
     }
     if (overlap) BIGMAC_CUDA(cudaEventRecord(L->fork_join[1], sd));          // dW_up done: the fp32 workspace is free again
     // du = p dy'[t], dp = <dy'[t], u>; then the softmax-over-k backward
-    if (m.cap != kNoCapacity) BIGMAC_CUDA(cudaMemsetAsync(b.dp, 0, sizeof(float) * m.N, st));   // dropped slots: dp = 0
     { Stage s(L, S_COMBINE_BWD, st); BIGMAC_CUDA(launch_combine_bwd(b.dy_lo, b.u, b.du, b.dp, b.tb, m.k, m.r, m.dtype, m.P, st)); }
     // The gate backward (dp -> dl) and the gate-bias column sums feed only dx, dW_gate and db_gate at the end of the pass:
     // with the second stream they run beside the expert contractions instead of in front of them.
@@ -640,10 +669,10 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         aux_part = b.colsum_part + (size_t)kColsumChunks * m.E;
         Stage s(L, S_GATE_BWD, sd);
         BIGMAC_CUDA(launch_gate_bwd_aux(b.dp, b.tb, b.dlogits, b.logits_saved, W->b_gate, m.aux, aux_part, m.T, m.E, m.E64,
-                                        ldcat, m.k, m.dtype, sd));
+                                        ldcat, m.k, m.dtype, sd, m.cap != kNoCapacity));
     } else {
         Stage s(L, S_GATE_BWD, sd);
-        BIGMAC_CUDA(launch_gate_bwd(b.dp, b.tb, b.dlogits, m.T, m.E, m.E64, ldcat, m.k, m.dtype, sd));
+        BIGMAC_CUDA(launch_gate_bwd(b.dp, b.tb, b.dlogits, m.T, m.E, m.E64, ldcat, m.k, m.dtype, sd, m.cap != kNoCapacity));
     }
     bool colsum_done = false;
     if (overlap) {
@@ -932,7 +961,7 @@ int static_scratch_address(int device, void** ptr) {
 
 // Only what routing needs: logits, counting-sort counters and the tables (no float intermediates).
 void carve_route_only(Carver& cv, const Dims& m, Buffers& b) {
-    carve_route_scratch(cv, m, b);
+    carve_route_scratch(cv, m, b, false);
     b.tb.topk_idx = cv.take<int32_t>(m.N);
     b.tb.topk_w = cv.take<float>(m.N);
     b.tb.counts = cv.take<int32_t>(m.E);
@@ -974,8 +1003,8 @@ int bigmac_route_static(bigmac_layer_t* L, const void* x, int32_t T, const bigma
     carve_route_only(cv, m, b);
     alias_routing(b, out);
     cudaStream_t st = (cudaStream_t)stream;
-    BIGMAC_TRY(run_routing(L, m, x, W, b, st));
-    return export_routing(m, b, out, st);
+    BIGMAC_TRY(run_routing(L, m, x, W, b, out, st));
+    return export_routing(L, m, b, out, st);
 }
 
 int bigmac_profile_enable(bigmac_layer_t* L, int on) {

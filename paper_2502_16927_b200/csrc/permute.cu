@@ -152,7 +152,8 @@ __global__ void __launch_bounds__(256) combine_bwd_kernel(const uint4* __restric
 template <typename T>
 __global__ void __launch_bounds__(256) gate_bwd_kernel(float* __restrict__ dp, const float* __restrict__ topk_w,
                                                        const int32_t* __restrict__ topk_idx, T* __restrict__ dlogits,
-                                                       int n_tokens, int E, int width, int ld, int k) {
+                                                       int n_tokens, int E, int width, int ld, int k,
+                                                       const int32_t* __restrict__ prow_of_slot /* nullable */) {
     grid_dependency_wait();
     grid_dependency_launch();
     const int t = warp_global_id();
@@ -161,7 +162,10 @@ __global__ void __launch_bounds__(256) gate_bwd_kernel(float* __restrict__ dp, c
     const float* p = topk_w + (int64_t)t * k;
     float* g = dp + (int64_t)t * k;
     float part = 0.0f;
-    for (int j = lane; j < k; j += 32) part = fmaf(p[j], g[j], part);
+    for (int j = lane; j < k; j += 32) {
+        if (prow_of_slot && prow_of_slot[(int64_t)t * k + j] < 0) g[j] = 0.0f;   // dropped under a capacity limit
+        part = fmaf(p[j], g[j], part);
+    }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(kFull, part, off);
     T* row = dlogits + (int64_t)t * ld;
@@ -337,6 +341,16 @@ __global__ void __launch_bounds__(256) grouped_colsum_final_kernel(const float* 
     out[i] = accumulate ? out[i] + total : total;
 }
 
+// The arrays one after another, each over the whole grid (the routing tables of a training call, handed to the caller:
+// nine copies by the copy engine's path cost 4 us each, 36 us of 411 at 2999 tokens).
+__global__ void __launch_bounds__(256) word_copies_kernel(const WordCopies c) {
+    grid_dependency_wait();
+    grid_dependency_launch();
+    for (int a = 0; a < c.n; ++a)
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < c.words[a]; i += (int64_t)gridDim.x * blockDim.x)
+            c.dst[a][i] = c.src[a][i];
+}
+
 inline int elem_bytes(int dtype) { return dtype == BIGMAC_BF16 ? 2 : 4; }
 inline unsigned warp_blocks(int64_t warps) { return (unsigned)((warps + 7) / 8); }
 
@@ -383,13 +397,14 @@ cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float
 }
 
 cudaError_t launch_gate_bwd(float* dp, const Tables& tb, void* dlogits, int T, int E, int width, int ld, int k,
-                            int dtype, cudaStream_t stream) {
+                            int dtype, cudaStream_t stream, bool may_drop) {
     if (T == 0) return cudaSuccess;
+    const int32_t* prow = may_drop ? tb.prow_of_slot : nullptr;
     if (dtype == BIGMAC_BF16)
         (void)launch_chained(gate_bwd_kernel<__nv_bfloat16>, warp_blocks(T), 256, 0, stream, dp, tb.topk_w, tb.topk_idx,
-                                                                          (__nv_bfloat16*)dlogits, T, E, width, ld, k);
+                                                                          (__nv_bfloat16*)dlogits, T, E, width, ld, k, prow);
     else
-        (void)launch_chained(gate_bwd_kernel<float>, warp_blocks(T), 256, 0, stream, dp, tb.topk_w, tb.topk_idx, (float*)dlogits, T, E, width, ld, k);
+        (void)launch_chained(gate_bwd_kernel<float>, warp_blocks(T), 256, 0, stream, dp, tb.topk_w, tb.topk_idx, (float*)dlogits, T, E, width, ld, k, prow);
     return cudaGetLastError();
 }
 
@@ -412,6 +427,14 @@ cudaError_t launch_grouped_colsum(const void* src, const int32_t* poffsets, floa
     const int64_t n = (int64_t)E * width;
     (void)launch_chained(grouped_colsum_final_kernel, (unsigned)((n + 255) / 256), 256, 0, stream, partial, out, n, width, accumulate ? 1 : 0);
     return cudaGetLastError();
+}
+
+cudaError_t launch_word_copies(const WordCopies& c, cudaStream_t stream) {
+    int64_t most = 0;
+    for (int a = 0; a < c.n; ++a) most = c.words[a] > most ? c.words[a] : most;
+    if (most == 0) return cudaSuccess;
+    const int64_t blocks = (most + 1023) / 1024;
+    return launch_chained(word_copies_kernel, (unsigned)(blocks < 592 ? blocks : 592), 256, 0, stream, c);
 }
 
 cudaError_t launch_descend_reduce(const float* ws, int parts, int T, int r, int E, void* x_lo, float* logits,

@@ -83,65 +83,6 @@ __global__ void __launch_bounds__(256) topk_kernel(const float* __restrict__ log
     for (int j = lane; j < k; j += 32) out_w[j] = (none ? 1.0f : expf(out_w[j] - top)) / part;
 }
 
-// Four tokens per warp, eight lanes per token, for k <= 8 and E a multiple of 32 up to 256: lane l of a group
-// holds the experts 4 (l + 8 i) + c (one float4 per i), the arg-max tree has three levels, and the j-th winner
-// stays in lane j of the group until one store.  Same order (logit descending, expert id ascending).
-template <int Q>   // float4 loads per lane: E = 32 Q
-__global__ void __launch_bounds__(256) topk8_kernel(const float* __restrict__ logits, const float* __restrict__ b_gate,
-                                                    int T, int k, int32_t* __restrict__ topk_idx,
-                                                    float* __restrict__ topk_w) {
-    grid_dependency_wait();
-    grid_dependency_launch();
-    constexpr int E = 32 * Q;
-    const int lane = threadIdx.x & 31, sub = lane & 7;
-    const int t = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 4 + (lane >> 3);
-    const bool live = t < T;
-    const float4* row = reinterpret_cast<const float4*>(logits + (size_t)(live ? t : 0) * E);
-    float v[4 * Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        float4 x = row[sub + 8 * i];
-        if (b_gate) {
-            const float4 b = reinterpret_cast<const float4*>(b_gate)[sub + 8 * i];
-            x.x += b.x; x.y += b.y; x.z += b.z; x.w += b.w;
-        }
-        v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
-    }
-#pragma unroll
-    for (int i = 0; i < 4 * Q; ++i) v[i] = v[i] == v[i] ? v[i] : -INFINITY;     // NaN is ordered as -inf
-    float my_v = -INFINITY;
-    int my_e = 0;
-    uint32_t taken = 0;                            // bit i: this lane's i-th expert already chosen
-    for (int j = 0; j < k; ++j) {
-        float best = -INFINITY;
-        int best_e = kNoExpert;
-#pragma unroll
-        for (int i = 0; i < 4 * Q; ++i) {          // ascending expert id within the lane: strict > keeps the lowest id
-            const int e = 4 * (sub + 8 * (i >> 2)) + (i & 3);
-            if (!((taken >> i) & 1u) && (best_e == kNoExpert || v[i] > best)) { best = v[i]; best_e = e; }
-        }
-#pragma unroll
-        for (int off = 4; off > 0; off >>= 1) {
-            const float ov = __shfl_xor_sync(kFull, best, off);
-            const int oe = __shfl_xor_sync(kFull, best_e, off);
-            if (ov > best || (ov == best && oe < best_e)) { best = ov; best_e = oe; }
-        }
-#pragma unroll
-        for (int i = 0; i < 4 * Q; ++i)
-            if (4 * (sub + 8 * (i >> 2)) + (i & 3) == best_e) taken |= 1u << i;
-        if (sub == j) { my_v = best; my_e = best_e; }
-    }
-    const float top = __shfl_sync(kFull, my_v, lane & 24);
-    const float ex = sub < k ? (top == -INFINITY ? 1.0f : expf(my_v - top)) : 0.0f;
-    float part = ex;
-#pragma unroll
-    for (int off = 4; off > 0; off >>= 1) part += __shfl_xor_sync(kFull, part, off);
-    if (live && sub < k) {
-        topk_idx[(size_t)t * k + sub] = my_e;
-        topk_w[(size_t)t * k + sub] = ex / part;
-    }
-}
-
 // Pass 1 of the counting sort.  Block b owns slots [b*kSortChunk, (b+1)*kSortChunk); it writes, per
 // slot, the number of earlier slots of the same block routed to the same expert, and per expert the
 // block's count.  Warps own consecutive sub-chunks, so the order is the slot order.
@@ -401,26 +342,290 @@ __global__ void __launch_bounds__(1024) tables_small_kernel(const int32_t* __res
     }
 }
 
+// ---- Routing in two launches (k <= 8, E a multiple of 4 up to 256: every configuration of the paper) -------------
+// A forward used to spend six launches between the gate logits and the experts (top-k, fill, three passes of the
+// counting sort, dispatch): about 2.5 us each for work of well under a microsecond, 20 us of 128 at 3001 tokens of the
+// d = 2048 widths.  Here the first kernel does the top-k and sorts inside its block, the second adds up the blocks'
+// counts for itself, places the slots and moves the rows; nothing between them is a fill or a scan launch of its own.
+
+// Where the gate logits (and the rows of x') come from: matrices in memory, or the fp32 partial results
+// [parts][T][ld] of a descend launch whose contraction was cut into parts - then added in part order on the way.
+// Kernel 1: top-k with gate values as topk8_kernel, four tokens per warp, plus pass 1 of the counting sort.  Block b owns
+// tokens [b TB, (b + 1) TB), TB = 4 warps iters.  Lane 8 g + j of a warp holds slot j of the warp's token g, so the lane
+// order is the slot order: ranks inside a warp by match_any, across the warps by a scan over per-warp counts.
+template <int Q>   // float4 loads per lane: E <= 32 Q
+__global__ void __launch_bounds__(1024) topk_count_kernel(const float* __restrict__ logits, int ld, int parts, int64_t part_stride,
+                                                          float* __restrict__ logits_out, const float* __restrict__ b_gate, int T,
+                                                          int E, int k, int iters, int32_t* __restrict__ topk_idx,
+                                                          float* __restrict__ topk_w, int32_t* __restrict__ local_rank,
+                                                          int32_t* __restrict__ block_counts) {
+    grid_dependency_wait();
+    grid_dependency_launch();
+    extern __shared__ int32_t warp_run[];            // [warps][E], then [E] the block's totals so far
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5, sub = lane & 7;
+    int32_t* total = warp_run + warps * E;
+    for (int i = threadIdx.x; i < (warps + 1) * E; i += blockDim.x) warp_run[i] = 0;
+    __syncthreads();
+    for (int it = 0; it < iters; ++it) {
+        const int64_t t = ((int64_t)blockIdx.x * iters + it) * (4 * warps) + 4 * warp + (lane >> 3);
+        const bool live = t < T;
+        const float* row = logits + (live ? t : 0) * ld;
+        float v[4 * Q];
+        uint32_t taken = 0;                          // bit i: this lane's i-th expert already chosen (or past E)
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const int e0 = 4 * (sub + 8 * i);
+            float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (e0 < E) {
+                x = *reinterpret_cast<const float4*>(row + e0);
+                for (int s = 1; s < parts; ++s) {
+                    const float4 y = *reinterpret_cast<const float4*>(row + s * part_stride + e0);
+                    x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+                }
+                if (logits_out && live) *reinterpret_cast<float4*>(logits_out + t * E + e0) = x;
+                if (b_gate) { x.x += b_gate[e0]; x.y += b_gate[e0 + 1]; x.z += b_gate[e0 + 2]; x.w += b_gate[e0 + 3]; }
+            } else {
+                taken |= 15u << (4 * i);
+            }
+            v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 4 * Q; ++i) v[i] = v[i] == v[i] ? v[i] : -INFINITY;     // NaN is ordered as -inf
+        float my_v = -INFINITY;
+        int my_e = 0;
+        for (int j = 0; j < k; ++j) {
+            float best = -INFINITY;
+            int best_e = kNoExpert;
+#pragma unroll
+            for (int i = 0; i < 4 * Q; ++i) {        // ascending expert id within the lane: strict > keeps the lowest id
+                const int e = 4 * (sub + 8 * (i >> 2)) + (i & 3);
+                if (!((taken >> i) & 1u) && (best_e == kNoExpert || v[i] > best)) { best = v[i]; best_e = e; }
+            }
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) {
+                const float ov = __shfl_xor_sync(kFull, best, off);
+                const int oe = __shfl_xor_sync(kFull, best_e, off);
+                if (ov > best || (ov == best && oe < best_e)) { best = ov; best_e = oe; }
+            }
+            if (((best_e >> 2) & 7) == sub) taken |= 1u << (((best_e >> 5) << 2) | (best_e & 3));
+            if (sub == j) { my_v = best; my_e = best_e; }
+        }
+        const float top = __shfl_sync(kFull, my_v, lane & 24);
+        const float ex = sub < k ? (top == -INFINITY ? 1.0f : expf(my_v - top)) : 0.0f;
+        float part = ex;
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) part += __shfl_xor_sync(kFull, part, off);
+        const bool slot = live && sub < k;
+        const int e = slot ? my_e : -1;
+        const unsigned peers = __match_any_sync(kFull, e);
+        if (slot && lane == __ffs(peers) - 1) warp_run[warp * E + e] = __popc(peers);
+        __syncthreads();
+        for (int x = threadIdx.x; x < E; x += blockDim.x) {      // exclusive scan over the warps, on top of the earlier rounds
+            int run = total[x];
+            int w = 0;
+            for (; w + 8 <= warps; w += 8) {
+                int c[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) c[i] = warp_run[(w + i) * E + x];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { warp_run[(w + i) * E + x] = run; run += c[i]; }
+            }
+            for (; w < warps; ++w) { const int c = warp_run[w * E + x]; warp_run[w * E + x] = run; run += c; }
+            total[x] = run;
+        }
+        __syncthreads();
+        if (slot) {
+            const int64_t s = t * k + sub;
+            topk_idx[s] = my_e;
+            topk_w[s] = ex / part;
+            local_rank[s] = warp_run[warp * E + e] + __popc(peers & ((1u << lane) - 1u));
+        }
+        if (it + 1 < iters) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < warps * E; i += blockDim.x) warp_run[i] = 0;
+            __syncthreads();
+        }
+    }
+    for (int x = threadIdx.x; x < E; x += blockDim.x) block_counts[(size_t)blockIdx.x * E + x] = total[x];
+}
+
+struct PlaceArgs {
+    const int32_t *topk_idx, *block_counts;
+    int T, E, k, nb, tokens_per_block, splits, cap;  // nb blocks of kernel 1, each cut into `splits` blocks of this kernel
+    int32_t *counts, *counts_chosen, *offsets, *poffsets, *tile_expert, *n_tiles;
+    int32_t *prow_of_slot /* in: rank inside the block of kernel 1 */, *row_of_slot, *slot_of_row, *slot_of_prow;
+    float* zero_word;                                // nullable: set to 0 (the loss of a layer without one)
+    // the rows to move: [T, 16 vecs bytes] at src, or fp32 partial results [parts][T][ld] rounded to bf16
+    const uint4* src;
+    const float* partial;
+    int parts, ld;
+    int64_t part_stride;
+    uint4* grouped;
+    int vecs;
+    bool zero_padding;                               // write zeros on the padding rows (a training step contracts over them)
+    int* status;
+};
+
+constexpr int kPlaceThreads = 512, kPlaceMaxExperts = 256;
+
+// Kernel 2: the whole placement, and the dispatch as a scatter: a warp reads the row of a token once and writes it to
+// its k grouped rows (the gather form reads it k times).  Every block adds up the counts of all blocks of kernel 1 for
+// itself (a few tens of KB from L2), which takes less than a launch of a scan kernel.
+// MOVE 0: tables only; 1: rows of a matrix; 2: rows from partial results.
+template <int MOVE>
+__global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p) {
+    grid_dependency_wait();
+    grid_dependency_launch();
+    __shared__ int4 s_all[kPlaceThreads], s_below[kPlaceThreads];           // [parts][E / 4]
+    __shared__ int32_t s_base[kPlaceMaxExperts], s_total[kPlaceMaxExperts], s_off[kPlaceMaxExperts + 1], s_poff[kPlaceMaxExperts + 1];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kWarps = kPlaceThreads / 32;
+    const int E = p.E, groups = E >> 2, nparts = min(32, kPlaceThreads / groups);
+    const int b = blockIdx.x / p.splits;             // the block of kernel 1 whose slots these are
+    {
+        const int g = tid % groups, part = tid / groups;
+        int4 all = make_int4(0, 0, 0, 0), below = all;
+        if (part < nparts)
+            for (int row = part; row < p.nb; row += nparts) {
+                const int4 c = *reinterpret_cast<const int4*>(p.block_counts + (size_t)row * E + 4 * g);
+                all.x += c.x; all.y += c.y; all.z += c.z; all.w += c.w;
+                if (row < b) { below.x += c.x; below.y += c.y; below.z += c.z; below.w += c.w; }
+            }
+        s_all[tid] = all;
+        s_below[tid] = below;
+    }
+    __syncthreads();
+    if (tid < E) {
+        int all = 0, below = 0;
+        for (int q = 0; q < nparts; ++q) {
+            all += reinterpret_cast<const int32_t*>(s_all)[q * E + tid];
+            below += reinterpret_cast<const int32_t*>(s_below)[q * E + tid];
+        }
+        s_total[tid] = all;
+        s_base[tid] = below;
+    }
+    __syncthreads();
+    if (warp == 0) {                                 // offsets: lane l scans the experts [l per, (l + 1) per)
+        const int per = (E + 31) / 32, e0 = min(E, lane * per), e1 = min(E, e0 + per);
+        int rows = 0, padded = 0;
+        for (int e = e0; e < e1; ++e) {
+            const int kept = min(s_total[e], p.cap);
+            rows += kept;
+            padded += (kept + kPad - 1) / kPad * kPad;
+        }
+        int r = rows, q = padded;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_up_sync(kFull, r, o), c = __shfl_up_sync(kFull, q, o);
+            if (lane >= o) { r += a; q += c; }
+        }
+        int off = r - rows, poff = q - padded;
+        for (int e = e0; e < e1; ++e) {
+            const int kept = min(s_total[e], p.cap);
+            s_off[e] = off;
+            s_poff[e] = poff;
+            off += kept;
+            poff += (kept + kPad - 1) / kPad * kPad;
+        }
+        if (lane == 31) { s_off[E] = off; s_poff[E] = poff; }
+    }
+    __syncthreads();
+    // ---- this block's tokens
+    const int per_split = (p.tokens_per_block + p.splits - 1) / p.splits;
+    const int64_t first = (int64_t)b * p.tokens_per_block + (int64_t)(blockIdx.x - b * p.splits) * per_split;
+    const int64_t last = min(min(first + per_split, (int64_t)(b + 1) * p.tokens_per_block), (int64_t)p.T);
+    for (int64_t t = first + warp; t < last; t += kWarps) {
+        uint4 v0 = make_uint4(0, 0, 0, 0), v1 = v0;
+        if (MOVE == 1) {                             // the first 64 pieces of the row are on their way before its place is known
+            if (lane < p.vecs) v0 = __ldg(p.src + t * p.vecs + lane);
+            if (lane + 32 < p.vecs) v1 = __ldg(p.src + t * p.vecs + lane + 32);
+        }
+        int prow = -1;
+        if (lane < p.k) {
+            const int64_t s = t * p.k + lane;
+            const int e = p.topk_idx[s];
+            int row = -1;
+            if ((unsigned)e >= (unsigned)E) {        // second line of defence: the slot goes nowhere, the call reports it
+                if (p.status) atomicExch(p.status, 2);
+            } else {
+                const int within = s_base[e] + p.prow_of_slot[s];
+                if (within < p.cap) {                // else dropped under a capacity limit
+                    row = s_off[e] + within;
+                    prow = s_poff[e] + within;
+                    p.slot_of_row[row] = (int32_t)s;
+                    p.slot_of_prow[prow] = (int32_t)s;
+                }
+            }
+            p.row_of_slot[s] = row;
+            p.prow_of_slot[s] = prow;
+        }
+        if (MOVE == 0) continue;
+        for (int c = lane; c - lane < p.vecs; c += 64) {
+            if (MOVE == 1) {
+                if (c >= 64) {
+                    if (c < p.vecs) v0 = __ldg(p.src + t * p.vecs + c);
+                    if (c + 32 < p.vecs) v1 = __ldg(p.src + t * p.vecs + c + 32);
+                }
+            } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int cc = c + 32 * h;
+                    if (cc >= p.vecs) continue;
+                    const float* from = p.partial + t * p.ld + 8 * cc;
+                    float4 a = *reinterpret_cast<const float4*>(from), d = *reinterpret_cast<const float4*>(from + 4);
+#pragma unroll 4
+                    for (int s = 1; s < p.parts; ++s) {
+                        const float4 x = *reinterpret_cast<const float4*>(from + s * p.part_stride), y = *reinterpret_cast<const float4*>(from + s * p.part_stride + 4);
+                        a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+                        d.x += y.x; d.y += y.y; d.z += y.z; d.w += y.w;
+                    }
+                    __nv_bfloat162 o[4] = {__floats2bfloat162_rn(a.x, a.y), __floats2bfloat162_rn(a.z, a.w),
+                                           __floats2bfloat162_rn(d.x, d.y), __floats2bfloat162_rn(d.z, d.w)};
+                    (h ? v1 : v0) = *reinterpret_cast<uint4*>(o);
+                }
+            }
+            for (int j = 0; j < p.k; ++j) {
+                const int to = __shfl_sync(kFull, prow, j);
+                if (to < 0) continue;                // uniform
+                if (c < p.vecs) p.grouped[(int64_t)to * p.vecs + c] = v0;
+                if (c + 32 < p.vecs) p.grouped[(int64_t)to * p.vecs + c + 32] = v1;
+            }
+        }
+    }
+    // ---- padding rows: the gaps behind the experts' rows, dealt out over all blocks
+    const int share = max(1, (int)gridDim.x / E);    // blocks per expert
+    for (int e = blockIdx.x / share; e < E; e += gridDim.x / share) {
+        const int r0 = s_poff[e] + (s_off[e + 1] - s_off[e]), r1 = s_poff[e + 1];
+        for (int r = r0 + (int)(blockIdx.x % share) * kWarps + warp; r < r1; r += share * kWarps) {
+            if (lane == 0) p.slot_of_prow[r] = -1;
+            if (MOVE != 0 && p.zero_padding)
+                for (int c = lane; c < p.vecs; c += 32) p.grouped[(int64_t)r * p.vecs + c] = make_uint4(0, 0, 0, 0);
+        }
+        if (blockIdx.x % share == 0)
+            for (int tile = s_poff[e] / kPad + tid; tile < s_poff[e + 1] / kPad; tile += kPlaceThreads) p.tile_expert[tile] = e;
+    }
+    if (p.cap < kNoCapacity)                         // rows past the kept ones exist only under a capacity limit
+        for (int64_t r = s_off[E] + (int64_t)blockIdx.x * kPlaceThreads + tid; r < (int64_t)p.T * p.k; r += (int64_t)gridDim.x * kPlaceThreads)
+            p.slot_of_row[r] = -1;
+    if (blockIdx.x == 0) {
+        for (int e = tid; e <= E; e += kPlaceThreads) { p.offsets[e] = s_off[e]; p.poffsets[e] = s_poff[e]; }
+        for (int e = tid; e < E; e += kPlaceThreads) {
+            p.counts[e] = min(s_total[e], p.cap);
+            if (p.counts_chosen) p.counts_chosen[e] = s_total[e];
+        }
+        if (tid == 0) {
+            *p.n_tiles = s_poff[E] / kPad;
+            if (p.zero_word) *p.zero_word = 0.0f;
+        }
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_topk(const float* logits, const float* b_gate, int T, int E, int k, int32_t* topk_idx,
                         float* topk_w, cudaStream_t stream) {
     if (T == 0) return cudaSuccess;
     const int warps = 8;
-    if (k <= 8 && E % 32 == 0 && E <= 256 && ((uintptr_t)logits % 16 == 0) && ((uintptr_t)b_gate % 16 == 0)) {
-        const unsigned blocks = (unsigned)((T + 4 * warps - 1) / (4 * warps));
-        switch (E / 32) {
-            case 1: return launch_chained(topk8_kernel<1>, blocks, warps * 32, 0, stream, logits, b_gate, T, k, topk_idx, topk_w);
-            case 2: return launch_chained(topk8_kernel<2>, blocks, warps * 32, 0, stream, logits, b_gate, T, k, topk_idx, topk_w);
-            case 3: return launch_chained(topk8_kernel<3>, blocks, warps * 32, 0, stream, logits, b_gate, T, k, topk_idx, topk_w);
-            case 4: return launch_chained(topk8_kernel<4>, blocks, warps * 32, 0, stream, logits, b_gate, T, k, topk_idx, topk_w);
-            case 5: return launch_chained(topk8_kernel<5>, blocks, warps * 32, 0, stream, logits, b_gate, T, k, topk_idx, topk_w);
-            case 6: return launch_chained(topk8_kernel<6>, blocks, warps * 32, 0, stream, logits, b_gate, T, k, topk_idx, topk_w);
-            case 7: return launch_chained(topk8_kernel<7>, blocks, warps * 32, 0, stream, logits, b_gate, T, k, topk_idx, topk_w);
-            default: return launch_chained(topk8_kernel<8>, blocks, warps * 32, 0, stream, logits, b_gate, T, k, topk_idx, topk_w);
-        }
-        return cudaGetLastError();
-    }
     dim3 grid((T + warps - 1) / warps), block(warps * 32);
     const int vpl = (E + 31) / 32;
 #define BIGMAC_TOPK(V)                                                                                   \
@@ -466,6 +671,48 @@ cudaError_t launch_tables(const Tables& tb, int T, int E, int k, int cap, cudaSt
                              tb.offsets, tb.poffsets, tb.prow_of_slot, tb.row_of_slot, tb.slot_of_row, tb.slot_of_prow, cap,
                              status);
     return err;
+}
+
+// The two-launch form wants a lane per slot of a token, eight lanes per token, and at most 32 logits per lane.
+bool route_fused_supported(int E, int k) { return k <= 8 && E % 4 == 0 && E <= kPlaceMaxExperts; }
+
+cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, const float* b_gate, const Tables& tb, int T, int E,
+                               int k, int cap, float* zero_word, int sm_count, cudaStream_t stream, int* status,
+                               int which) {
+    // As many blocks as there are SMs (and rows in block_counts) at most, 32 tokens in each at least: top-k is bound by
+    // issue and latency inside a block, so few fat blocks are slow (128 tokens a block: 2 us more at 512 tokens), and the
+    // second kernel reads all blocks' counts, so more blocks than SMs buy nothing.
+    const int nb_max = tb.block_rows < sm_count ? tb.block_rows : sm_count;
+    int per = (T + nb_max - 1) / nb_max;
+    if (per < 32) per = 32;
+    const int warps = per < 128 ? (per + 3) / 4 : 32, iters = (per + 4 * warps - 1) / (4 * warps);
+    per = 4 * warps * iters;
+    const int nb = (T + per - 1) / per;
+    if (which == 0) {
+        const size_t smem = sizeof(int32_t) * (size_t)(warps + 1) * E;
+#define BIGMAC_TOPK_COUNT(Q)                                                                                                       \
+    return launch_chained(topk_count_kernel<Q>, nb, warps * 32, smem, stream, src.logits, src.ld, src.parts, src.part_stride,     \
+                          src.logits_out, b_gate, T, E, k, iters, tb.topk_idx, tb.topk_w, tb.prow_of_slot, tb.block_counts)
+        if (E <= 32) BIGMAC_TOPK_COUNT(1);
+        if (E <= 64) BIGMAC_TOPK_COUNT(2);
+        if (E <= 128) BIGMAC_TOPK_COUNT(4);
+        BIGMAC_TOPK_COUNT(8);
+#undef BIGMAC_TOPK_COUNT
+    }
+    PlaceArgs p{};
+    p.topk_idx = tb.topk_idx; p.block_counts = tb.block_counts;
+    p.T = T; p.E = E; p.k = k; p.nb = nb; p.tokens_per_block = per; p.cap = cap;
+    p.splits = 2 * sm_count / nb;                   // about two blocks per SM, four tokens in each at least
+    if (p.splits > per / 4) p.splits = per / 4;
+    if (p.splits < 1) p.splits = 1;
+    p.counts = tb.counts; p.counts_chosen = tb.counts_chosen; p.offsets = tb.offsets; p.poffsets = tb.poffsets;
+    p.tile_expert = tb.tile_expert; p.n_tiles = tb.n_tiles; p.prow_of_slot = tb.prow_of_slot; p.row_of_slot = tb.row_of_slot;
+    p.slot_of_row = tb.slot_of_row; p.slot_of_prow = tb.slot_of_prow; p.zero_word = zero_word; p.status = status;
+    p.src = (const uint4*)mv.src; p.partial = mv.partial; p.parts = mv.parts; p.ld = mv.ld; p.part_stride = mv.part_stride;
+    p.grouped = (uint4*)mv.grouped; p.vecs = mv.row_bytes / 16; p.zero_padding = mv.zero_padding;
+    if (!mv.grouped) return launch_chained(place_kernel<0>, nb * p.splits, kPlaceThreads, 0, stream, p);
+    if (!mv.partial) return launch_chained(place_kernel<1>, nb * p.splits, kPlaceThreads, 0, stream, p);
+    return launch_chained(place_kernel<2>, nb * p.splits, kPlaceThreads, 0, stream, p);
 }
 
 }  // namespace bigmac
