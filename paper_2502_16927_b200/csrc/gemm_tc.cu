@@ -115,7 +115,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
     } else if (warp == 0 && GATHER) {
         // ------------------------------------------------------------------ TMA producer of B beside the gathered A rows
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t s = 0, phase = 1;
             for (int t = blockIdx.x; t < total; t += gridDim.x) {
                 const Tile tl = get_tile(p, BN, t, tiles_m, tiles_n);
@@ -128,7 +128,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
     } else if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t s = 0, phase = 1;                     // stage and the parity its "empty" barrier is waited on with
             // the next tile is looked up (a global load for grouped rows) before this tile's loads are issued, so
             // that its latency does not sit between two tiles
@@ -165,7 +165,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (one thread)
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = instr_desc(BN, !A_KMAJOR, !B_KMAJOR);
             // descriptors of stage 0; the address field (16-byte units, bits 0-13) takes stage and k-step offsets by addition
             const uint64_t da0 = A_KMAJOR ? smem_desc(smem_u32(smem_a), 16, 1024) : smem_desc(smem_u32(smem_a), CHUNK_BYTES, 1024);
@@ -212,7 +212,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         uint64_t* my_z_bar = &z_bar[warp - 2];
         uint32_t z_count = 0;
         auto issue_z = [&](const Tile& tile) {
-            if (lane == 0) {
+            if (elect_one()) {
                 mbar_expect_tx(my_z_bar, kBoxBytesZ);
                 tma_load_2d(box_z, &map_z, my_z_bar, tile.n0 + part * COLS_PER_WARP, tile.m0 + quad * 32);
             }
@@ -254,7 +254,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 if (col0 >= p.N) continue;             // uniform across the warp
                 if (p.bias) add_bias32(v, p.bias + (int64_t)tl.expert * p.bias_stride + col0);   // N is a multiple of 32 here
                 if (TMA_EPI) {
-                    if (lane == 0) tma_store_wait_read();        // previous boxes of this warp have left smem
+                    if (elect_one()) tma_store_wait_read();        // previous boxes of this warp have left smem
                     __syncwarp();
                     if (z_prefetch) {
                         if (c == 0) {
@@ -273,7 +273,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     stage_row_chunk(p, v, box_c, box_z, lane, c);
                     fence_async_smem();
                     __syncwarp();
-                    if (lane == 0) {
+                    if (elect_one()) {
                         const int row0 = tl.expert * p.c_rows_per_expert + tl.m0 + quad * 32;
                         tma_store_2d(&map_c, box_c, col0, row0);
                         if (p.epilogue == EPI_ACT && p.Z && c == CHUNKS - 1) tma_store_2d(&map_z, box_z, col0 - 32, row0);
@@ -293,7 +293,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 }
             }
         }
-        if (TMA_EPI && lane == 0) tma_store_wait_read();          // the boxes have left shared memory; the writes land before the grid ends
+        if (TMA_EPI && elect_one()) tma_store_wait_read();          // the boxes have left shared memory; the writes land before the grid ends
     }
     tc_fence_before();
     __syncthreads();

@@ -196,7 +196,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (both CTAs)
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t s = 0, phase = 1;                     // stage and the parity its "empty" barrier is waited on with
             TileWalk tw;
             for (walk_init(tw, cluster_id, tiles_n); tw.w < total; walk_next(tw, num_clusters, step_pair, step_n, tiles_n)) {
@@ -231,7 +231,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (one thread of the leader CTA)
-        if (leader && lane == 0) {
+        if (leader && elect_one()) {
             constexpr uint32_t idesc = instr_desc_pair(BN, !A_KMAJOR, !B_KMAJOR);
             // descriptors of stage 0; the address field (16-byte units, bits 0-13) takes stage and k-step offsets by addition
             const uint64_t da0 = A_KMAJOR ? smem_desc(smem_u32(smem_a), 16, 1024) : smem_desc(smem_u32(smem_a), CHUNK_BYTES, 1024);
@@ -280,7 +280,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         uint32_t z_count = 0;
         static_assert(!TMA_EPI || CHUNKS == 2, "the sigma' box holds two 32-column chunks");
         auto issue_z = [&](const PairTile& tile) {           // the warp's 32 rows x 64 columns of saved sigma'
-            if (lane == 0) {
+            if (elect_one()) {
                 mbar_expect_tx(my_z_bar, kBoxBytesZ);
                 tma_load_2d(box_z, &map_z, my_z_bar, tile.n0 + part * COLS_PER_WARP, tile.m0 + (int)rank * BM + quad * 32);
             }
@@ -329,7 +329,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                 if (col0 >= p.N) continue;             // uniform across the warp
                 if (p.bias) add_bias32(v, p.bias + (int64_t)tl.expert * p.bias_stride + col0);   // N is a multiple of 32 here
                 if (TMA_EPI) {
-                    if (lane == 0) tma_store_wait_read();
+                    if (elect_one()) tma_store_wait_read();
                     __syncwarp();
                     if (z_prefetch) {
                         if (c == 0) {
@@ -348,7 +348,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                     stage_row_chunk(p, v, box_c, box_z, lane, c);
                     fence_async_smem();
                     __syncwarp();
-                    if (lane == 0 && half_ok && my_m0 < tl.m_limit) {
+                    if (half_ok && my_m0 < tl.m_limit && elect_one()) {
                         const int row0 = tl.expert * p.c_rows_per_expert + my_m0 + quad * 32;
                         tma_store_2d(&map_c, box_c, col0, row0);
                         if (p.epilogue == EPI_ACT && p.Z && c == CHUNKS - 1) tma_store_2d(&map_z, box_z, col0 - 32, row0);
@@ -369,7 +369,7 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
             }
             }
         }
-        if (TMA_EPI && lane == 0) tma_store_wait_read();          // the boxes have left shared memory; the writes land before the grid ends
+        if (TMA_EPI && elect_one()) tma_store_wait_read();          // the boxes have left shared memory; the writes land before the grid ends
     }
     tc_fence_before();
     __syncthreads();

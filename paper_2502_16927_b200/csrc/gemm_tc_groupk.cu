@@ -65,7 +65,7 @@ __device__ void groupk_plan(const int32_t* poffsets, int E, int per, int pairs, 
         if (slots <= kGroupKSlots) break;
         len += len / 2;
     }
-    if (lane == 0) {
+    if (elect_one()) {
         int run = 0, slot = 0, lo = poffsets[0];
         for (int e = 0; e < E; ++e) {
             const int hi = poffsets[e + 1];
@@ -201,7 +201,7 @@ gemm_tc_groupk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
         }
     } else if (GATHER && warp == 1 && !leader) {
         // ---------------------------------------------------------- relay (peer CTA): gathered rows landed -> leader's barrier
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t leader_full = map_to_cta(full_bar, 0);
             uint32_t it = 0;
             for (uint32_t i = 0;; ++i) {
@@ -217,7 +217,7 @@ gemm_tc_groupk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
             }
         }
     } else if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0;
             if (leader) {
                 // ---------------------------------------------------------- scheduler + TMA producer (leader)
@@ -275,7 +275,7 @@ gemm_tc_groupk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (one thread of the leader CTA)
-        if (leader && lane == 0) {
+        if (leader && elect_one()) {
             constexpr uint32_t idesc = instr_desc_pair(BN, true, true);
             const uint64_t da0 = smem_desc(smem_u32(smem_a), CHUNK_BYTES, 1024), db0 = smem_desc(smem_u32(smem_b), CHUNK_BYTES, 1024);
             constexpr uint32_t kStep = (UMMA_K * 128) >> 4;
