@@ -1,26 +1,23 @@
-// Inference forward of the experts in one kernel: u = sigma(xg W1_e^T) W2_e^T per 128-row tile of an expert's
-// segment (Eq. 4), with the hidden activations never leaving the SM.  For low widths r <= 256.
+// Inference forward of the experts in one kernel: u = W2_e sigma(W1_e x') for the rows of every expert's segment (Eq. 4),
+// the hidden activations never leaving the SM.
 //
-// The hidden width h is walked in chunks of 64.  Per chunk c, on one CTA:
-//   GEMM1   acc1[c % 4] (128 x 64 fp32, tensor memory) = X (128 x r, shared memory, loaded once per tile)
-//                                                        x W1_e[64 c .. 64 c + 63, :]^T
-//   sigma   16 epilogue warps read acc1 (tcgen05.ld), apply the activation, and write the bf16 result into shared
-//           memory in the K-major 128-byte-swizzled layout a tcgen05.mma A operand has (A2[c % 2], 128 x 64)
-//   GEMM2   acc2 (128 x r fp32, tensor memory) += A2[c % 2] x W2_e[:, 64 c .. 64 c + 63]^T
-// GEMM1 runs two chunks ahead of GEMM2 (four acc1 buffers), so that the activation of two chunks is in flight
-// while the tensor pipe works on a third.  Tensor memory: 4 x 64 + r <= 512 columns.  Shared memory at
-// r = 256: X 64 KB, W1 and W2 chunks double-buffered 2 x 32 KB each, A2 2 x 16 KB = 224 KB.  After the last chunk
-// the 16 warps store acc2 as bf16 rows of u; the next tile's GEMM1s run meanwhile, only its first GEMM2 waits.
-// All waits are bounded (status word); the tile -> expert table is read one tile ahead.
-// Limit (measured with clock stamps around every wait of the MMA warp): a chunk takes about 1.8 us where the
-// tensor pipe needs 0.5.  The waits are short; the time goes into issuing the chunk's 16 + 4 tcgen05.mma
-// instructions, about 100 cycles each whatever their size, and GEMM1's are only N = 64 wide (32-64 cycles of
-// tensor work each).  A variant on CTA pairs (half the weight bytes per SM, four chunks in flight) ran at the same
-// speed, so loads are not what limits it.  A 128-wide chunk would halve the instruction count but leaves no room to
-// double-buffer the activated chunk beside X in shared memory at r = 256.  The layer therefore uses this kernel
-// only on short tile lists (decode-sized batches), where it saves a launch and the HBM round trip of the
-// activations; on long lists the two separate GEMMs (N = 256 instructions) are faster.
-#include "tc_pair.cuh"
+// The weights are the A operand: 128 rows of W1_e (hidden units) or of W2_e (columns of u) are the M of an MMA and the
+// tokens of a row tile its N, so an expert with 8 rows costs MMAs of N = 16 and not a 128-row tile of padding, and all
+// weight traffic is one stream of 16 KB boxes through one ring.  A work item is (row tile of up to NT tokens, slice of the
+// hidden width); it walks its slice in chunks of 128 hidden units:
+//   GEMM1   acc1[c % 2] (128 hidden x n tokens, tensor memory) = W1_e[chunk, :] X^T        r / 64 boxes
+//   sigma   16 epilogue warps read acc1, apply the activation and write it as bf16 to shared memory in the MN-major layout
+//           of a B operand (a[c % 2], 128 hidden x n): lane = hidden unit = contraction row, so a lane's values are adjacent
+//   GEMM2   acc2 (r x n, tensor memory, r / 128 tiles) += W2_e[:, chunk] a[c % 2]          2 r / 128 boxes
+// GEMM1 runs one chunk ahead of GEMM2.  After the last chunk acc2 leaves as rows of `out`, addressed by slot: fp32 partial
+// results [slices][slots][r], or bf16 rows where there is one slice.  The combine kernel adds a token's k slots and the
+// slices in order, so slices need no other exchange, and padding rows are never written.
+//
+// What bounds it: few tokens, the stream of weights (67 MB at 64 experts of 2 x 256 x 1024); many tokens, the MMAs
+// (M = 128, N = 128: shared memory delivers both operands at just the rate of the tensor pipe) and the activation.
+// Ring of 16 KB stages: NT = 128: 6 (96 KB in flight per SM; about 44 KB cover the DRAM latency at the full rate), beside X
+// 64 KB and two activation buffers of 32 KB at r = 256; NT = 64: 8, for r up to 512 (X 64 KB, activations 2 x 16 KB).
+#include "tc_common.cuh"
 
 namespace bigmac {
 
@@ -28,348 +25,311 @@ using namespace tc;
 
 namespace {
 
-constexpr int BH = 64;                                   // hidden chunk
+constexpr int HC = 128;                                  // hidden units per chunk
+constexpr uint32_t BOX_BYTES = 128 * BK * 2;             // one ring stage: 128 weight rows x 64 contraction elements
 constexpr int kMlpEpiWarps = 16;
-constexpr int kAcc1 = 4;                                 // acc1 buffers; GEMM1 runs kAhead chunks ahead of GEMM2
-constexpr int kAhead = 2;
-constexpr int kFirstEpiWarp = 3;                         // warp 0: X and W1 loads, warp 1: MMA issue, warp 2: W2 loads
-constexpr int kMlpThreads = (kFirstEpiWarp + kMlpEpiWarps) * 32;
+constexpr int kMlpThreads = (2 + kMlpEpiWarps) * 32;
 
 struct MlpParams {
-    void* U;             // [rows, r] bf16
+    void* out;               // [slices][slots][r] fp32, or [slots][r] bf16 if there is one slice
+    int64_t slots;
     int r, h, act;
-    int b1_rows_per_expert, b2_rows_per_expert;          // h, r
-    const int32_t* tile_expert;
-    const int32_t* n_tiles;
+    MlpSlicing sl;
+    const int32_t *tile_expert, *n_tiles, *poffsets, *counts, *slot_of_prow;
     int max_tiles;
     int* status;
 };
 
-// Arrive on a barrier of another CTA of the cluster, making this thread's earlier stores into that CTA visible to
-// whoever acquires the barrier at cluster scope.
-__device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-__device__ __forceinline__ void st_cluster_16B(uint32_t cluster_addr, float a, float b, float c, float d) {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+// A work item as every role sees it; n = 0: nothing to do (the second half of a short tile).
+struct MlpItem {
+    int expert, row0, rows, n, c0, chunks, slice;
+};
+
+template <int NT>
+__device__ __forceinline__ MlpItem mlp_item(const MlpParams& p, int tiles, int slices, int i) {
+    // all first halves of the tiles come before the second ones (NT = 64), most of which are empty where experts are short
+    MlpItem t;
+    const int half = NT < 128 && i >= tiles * slices ? 1 : 0, j = i - half * tiles * slices, tile = j / slices;
+    t.slice = j - tile * slices;
+    t.expert = p.tile_expert[tile];
+    t.row0 = tile * kPad + half * NT;
+    t.rows = min(NT, p.poffsets[t.expert] + p.counts[t.expert] - t.row0);
+    t.n = t.rows > 0 ? (t.rows + 15) / 16 * 16 : 0;
+    t.chunks = p.sl.chunks / slices;
+    t.c0 = t.slice * t.chunks;
+    return t;
 }
 
-// SPLIT: a pair of CTAs (a cluster) shares every tile: CTA 0 walks the first half of the hidden chunks, CTA 1 the
-// second, so that a short tile list (a few hundred tokens: one tile per expert, far fewer tiles than SMs) streams
-// its weights through twice as many SMs.  CTA 1 hands its 128 x r fp32 partial result to CTA 0 through CTA 0's
-// shared memory (the X and W1 buffers, free once CTA 0's last GEMM1 of the tile is done: 128 r 2 + 2 x 64 r 2 bytes
-// = 128 r 4), CTA 0 adds it to its own and stores the tile.
-template <bool SPLIT>
-__device__ __forceinline__ void fused_mlp_body(const CUtensorMap& map_x, const CUtensorMap& map_w1, const CUtensorMap& map_w2,
-                                               const MlpParams& p) {
-    const int KB1 = p.r / BK;                            // 64-deep k slices of GEMM1
-    const uint32_t X_BYTES = (uint32_t)KB1 * BM * BK * 2;
-    const uint32_t W1_BYTES = (uint32_t)KB1 * BH * BK * 2;
-    const uint32_t W2_BYTES = (uint32_t)p.r * BH * 2;
-    constexpr uint32_t A2_BYTES = BM * BH * 2;
-    constexpr uint32_t TMEM_COLS = 512;
+template <int NT, int STAGES>
+__global__ void __launch_bounds__(kMlpThreads, 1)
+fused_mlp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w1,
+                 const __grid_constant__ CUtensorMap map_w2, const MlpParams p) {
+    constexpr uint32_t A_CHUNKS = NT / 64;               // 64-token column blocks of an activation buffer
+    constexpr uint32_t ACT_BYTES = A_CHUNKS * HC * 128;
+    constexpr uint32_t XKB_BYTES = NT * BK * 2;          // one 64-deep k slice of X
+    const int KB1 = p.r / BK, MT = (p.r + 127) / 128;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* s_x = smem;
-    uint8_t* s_w1 = s_x + X_BYTES;                       // [2]
-    uint8_t* s_w2 = s_w1 + 2 * W1_BYTES;                 // [2]
-    uint8_t* s_a2 = s_w2 + 2 * W2_BYTES;                 // [2]
-    uint64_t* bars = (uint64_t*)(s_a2 + 2 * A2_BYTES);
-    uint64_t* x_full = bars;            uint64_t* x_empty = bars + 1;
-    uint64_t* w1_full = bars + 2;       uint64_t* w1_empty = bars + 4;
-    uint64_t* w2_full = bars + 6;       uint64_t* w2_empty = bars + 8;
-    uint64_t* acc1_full = bars + 10;    uint64_t* acc1_empty = bars + 14;      // [kAcc1] each
-    uint64_t* a2_full = bars + 18;      uint64_t* a2_empty = bars + 20;
-    uint64_t* acc2_full = bars + 22;    uint64_t* acc2_empty = bars + 23;
-    uint64_t* peer_free = bars + 24;                     // SPLIT, in CTA 1: CTA 0's X and W1 buffers may be written
-    uint64_t* partial_full = bars + 25;                  // SPLIT, in CTA 0: CTA 1's partial result has arrived
-    uint64_t* tile_done = bars + 26;                     // SPLIT, in CTA 0: the partial result has been read
-    uint32_t* tmem_slot = (uint32_t*)(bars + 27);
+    uint8_t* s_ring = smem;
+    uint8_t* s_act = s_ring + STAGES * BOX_BYTES;        // [2]
+    uint8_t* s_x = s_act + 2 * ACT_BYTES;
+    uint64_t* bars = (uint64_t*)(s_x + (uint32_t)KB1 * XKB_BYTES);
+    uint64_t* full = bars;              uint64_t* empty = bars + STAGES;
+    uint64_t* x_full = bars + 2 * STAGES;
+    uint64_t* x_empty = x_full + 1;
+    uint64_t* acc1_full = x_full + 2;   uint64_t* acc1_empty = x_full + 4;       // [2] each
+    uint64_t* act_full = x_full + 6;    uint64_t* act_empty = x_full + 8;        // [2] each
+    uint64_t* acc2_full = x_full + 10;  uint64_t* acc2_empty = x_full + 11;
+    uint32_t* tmem_slot = (uint32_t*)(x_full + 12);
     volatile int* dead = (volatile int*)(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 32) {                                 // the maps are on their way while the barriers are set up
+    if (threadIdx.x == 32) {                             // the maps are on their way while the barriers are set up
         prefetch_tensormap(&map_x);
         prefetch_tensormap(&map_w1);
         prefetch_tensormap(&map_w2);
     }
-
     if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         mbar_init(x_full, 1); mbar_init(x_empty, 1);
         for (int s = 0; s < 2; ++s) {
-            mbar_init(&w1_full[s], 1); mbar_init(&w1_empty[s], 1);
-            mbar_init(&w2_full[s], 1); mbar_init(&w2_empty[s], 1);
-            mbar_init(&a2_full[s], kMlpEpiWarps); mbar_init(&a2_empty[s], 1);
+            mbar_init(&acc1_full[s], 1); mbar_init(&acc1_empty[s], kMlpEpiWarps);
+            mbar_init(&act_full[s], kMlpEpiWarps); mbar_init(&act_empty[s], 1);
         }
-        for (int s = 0; s < kAcc1; ++s) { mbar_init(&acc1_full[s], 1); mbar_init(&acc1_empty[s], kMlpEpiWarps); }
         mbar_init(acc2_full, 1); mbar_init(acc2_empty, kMlpEpiWarps);
-        mbar_init(peer_free, 1); mbar_init(partial_full, kMlpEpiWarps); mbar_init(tile_done, kMlpEpiWarps);
         *dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc(tmem_slot, TMEM_COLS);
+    if (warp == 1) tmem_alloc(tmem_slot, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (SPLIT) cluster_sync_all();                        // the peer's barriers exist before anything signals them
     // Chained launch: everything above touched no global memory and may have run while the kernel before this one in
     // the stream was still working.  Tensor memory is held, so the next kernel of the stream may be set up in turn;
     // from the wait on, the predecessor's results are complete.
     grid_dependency_launch();
     grid_dependency_wait();
-    const uint32_t tmem_base = *tmem_slot;
-    const int total = min(*p.n_tiles, p.max_tiles);
-    const uint32_t crank = SPLIT ? cluster_ctarank() : 0u;
-    const int first = SPLIT ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, stride = SPLIT ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-    const int chunks = SPLIT ? p.h / BH / 2 : p.h / BH;   // this CTA's chunks of a tile: cbase, cbase + 1, ...
-    const int cbase = SPLIT ? (int)crank * chunks : 0;
+    const uint32_t tmem_base = *tmem_slot, acc2_tmem = tmem_base + 2 * NT;
+    const int tiles = min(*p.n_tiles, p.max_tiles), slices = mlp_slices(p.sl, tiles), total = tiles * (128 / NT) * slices;
 
     if (warp == 0) {
-        // ------------------------------------------------------------------ TMA producer: X and the W1 chunks
-        if (lane == 0) {
-            uint32_t g = 0, tl = 0;
-            int next_e = first < total ? p.tile_expert[first] : 0;
-            for (int t = first; t < total; t += stride, ++tl) {
-                const int e = next_e;
-                if (t + stride < total) next_e = p.tile_expert[t + stride];
-                mbar_wait(x_empty, (tl & 1) ^ 1, dead, p.status);
-                // CTA 0 of a pair: X and W1 buffers hold the peer's partial result until the epilogue has read it
-                if (SPLIT && crank == 0 && tl > 0) mbar_wait(tile_done, (tl - 1) & 1, dead, p.status);
-                mbar_expect_tx(x_full, X_BYTES);
-                for (int kb = 0; kb < KB1; ++kb) tma_load_2d(s_x + kb * (BM * BK * 2), &map_x, x_full, kb * BK, t * BM);
-                for (int c = 0; c < chunks; ++c, ++g) {
-                    const int s = g & 1;
-                    mbar_wait(&w1_empty[s], ((g >> 1) & 1) ^ 1, dead, p.status);
-                    mbar_expect_tx(&w1_full[s], W1_BYTES);
-                    for (int kb = 0; kb < KB1; ++kb)
-                        tma_load_2d(s_w1 + s * W1_BYTES + kb * (BH * BK * 2), &map_w1, &w1_full[s], kb * BK,
-                                    e * p.b1_rows_per_expert + (cbase + c) * BH);
-                }
-            }
-        }
-    } else if (warp == 2) {
-        // ------------------------------------------------------------------ TMA producer: the W2 chunks (its own
-        // thread: a W2 buffer frees only when GEMM2 two chunks back is done, and the W1 loads must not queue behind that)
-        if (lane == 0) {
-            uint32_t g = 0;
-            int next_e = first < total ? p.tile_expert[first] : 0;
-            for (int t = first; t < total; t += stride) {
-                const int e = next_e;
-                if (t + stride < total) next_e = p.tile_expert[t + stride];
-                for (int c = 0; c < chunks; ++c, ++g) {
-                    const int s = g & 1;
-                    mbar_wait(&w2_empty[s], ((g >> 1) & 1) ^ 1, dead, p.status);
-                    mbar_expect_tx(&w2_full[s], W2_BYTES);
-                    tma_load_2d(s_w2 + s * W2_BYTES, &map_w2, &w2_full[s], (cbase + c) * BH, e * p.b2_rows_per_expert);
+        // ------------------------------------------------------------------ TMA producer: X once per item, then the weight boxes
+        if (elect_one()) {
+            uint32_t s = 0, phase = 1, local = 0;
+            auto box = [&](const CUtensorMap* map, int c0, int c1) {
+                mbar_wait_lean(&empty[s], phase, dead, p.status);
+                mbar_expect_tx(&full[s], BOX_BYTES);
+                tma_load_2d(s_ring + s * BOX_BYTES, map, &full[s], c0, c1);
+                if (++s == STAGES) { s = 0; phase ^= 1; }
+            };
+            for (int i = blockIdx.x; i < total; i += gridDim.x) {
+                const MlpItem t = mlp_item<NT>(p, tiles, slices, i);
+                if (t.n == 0) continue;
+                mbar_wait_lean(x_empty, (local & 1) ^ 1, dead, p.status);
+                ++local;
+                mbar_expect_tx(x_full, (uint32_t)(KB1 * t.n) * BK * 2);
+                for (int kb = 0; kb < KB1; ++kb)
+                    for (int j = 0; j < t.n; j += 16) tma_load_2d(s_x + kb * XKB_BYTES + j * 128, &map_x, x_full, kb * BK, t.row0 + j);
+                const int w1_row = t.expert * p.h + t.c0 * HC, w2_row = t.expert * p.r;
+                for (int c = 0; c <= t.chunks; ++c) {    // in the order of the MMAs: W1 of chunk c, W2 of chunk c - 1
+                    if (c < t.chunks)
+                        for (int kb = 0; kb < KB1; ++kb) box(&map_w1, kb * BK, w1_row + c * HC);
+                    if (c > 0)
+                        for (int m = 0; m < MT; ++m)
+                            for (int kh = 0; kh < 2; ++kh) box(&map_w2, (t.c0 + c - 1) * HC + kh * BK, w2_row + m * 128);
                 }
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------------ MMA issuer
-        const uint32_t idesc1 = instr_desc(BH, false, false);
-        const uint32_t idesc2 = instr_desc(p.r, false, false);
-        const uint32_t acc2_tmem = tmem_base + kAcc1 * BH;
-        // Descriptors of the buffers' first bytes; the address field (bits 0-13, in 16-byte units) takes offsets by plain
-        // addition, which keeps the instruction stream of this warp short: it shares its scheduler with four busy
-        // epilogue warps, and with descriptors rebuilt per MMA the issue of one chunk's MMAs took longer than the MMAs.
-        const uint64_t desc_x = smem_desc(smem_u32(s_x), 16, 1024), desc_w1 = smem_desc(smem_u32(s_w1), 16, 1024);
-        const uint64_t desc_w2 = smem_desc(smem_u32(s_w2), 16, 1024), desc_a2 = smem_desc(smem_u32(s_a2), 16, 1024);
-        uint32_t g = 0, tl = 0;
-        // GEMM2 of global chunk gp (chunk cp of tile number tile_no)
-        auto gemm2 = [&](uint32_t gp, int cp, uint32_t tile_no) {
-            const int s = gp & 1;
-            const uint32_t ph = (gp >> 1) & 1;
-            mbar_spin(&w2_full[s], ph, dead, p.status);
-            mbar_spin(&a2_full[s], ph, dead, p.status);
-            if (cp == 0) mbar_spin(acc2_empty, (tile_no & 1) ^ 1, dead, p.status);
-            tc_fence_after();
-            if (lane == 0) {
-                const uint64_t da = desc_a2 + ((s * A2_BYTES) >> 4), db = desc_w2 + ((s * W2_BYTES) >> 4);
+        // ------------------------------------------------------------------ MMA issuer (one thread)
+        if (elect_one()) {
+            const uint64_t d_ring = smem_desc(smem_u32(s_ring), 16, 1024), d_x = smem_desc(smem_u32(s_x), 16, 1024);
+            const uint64_t d_act = smem_desc(smem_u32(s_act), HC * 128, 1024);   // MN-major, 64-token blocks HC rows of 128 bytes apart
+            uint32_t s = 0, phase = 0, g = 0, local = 0; // g: chunks so far, over all items
+            for (int i = blockIdx.x; i < total; i += gridDim.x) {
+                const MlpItem t = mlp_item<NT>(p, tiles, slices, i);
+                if (t.n == 0) continue;
+                const uint32_t idesc1 = instr_desc(t.n, false, false), idesc2 = instr_desc(t.n, false, true);
+                mbar_wait_lean(x_full, local & 1, dead, p.status);
+                for (int c = 0; c <= t.chunks; ++c) {
+                    if (c < t.chunks) {                  // GEMM1 of chunk c
+                        const uint32_t gc = g + c, a = gc & 1;
+                        mbar_wait_lean(&acc1_empty[a], ((gc >> 1) & 1) ^ 1, dead, p.status);
+                        tc_fence_after();
+                        for (int kb = 0; kb < KB1; ++kb) {
+                            mbar_wait_lean(&full[s], phase, dead, p.status);
+                            tc_fence_after();
+                            const uint64_t da = d_ring + s * (BOX_BYTES >> 4), db = d_x + kb * (XKB_BYTES >> 4);
 #pragma unroll
-                for (int kk = 0; kk < BH / UMMA_K; ++kk)
-                    umma_bf16(acc2_tmem, da + ((kk * UMMA_K * 2) >> 4), db + ((kk * UMMA_K * 2) >> 4), idesc2, (cp | kk) != 0);
-                umma_commit(&a2_empty[s]);
-                umma_commit(&w2_empty[s]);
-            }
-            __syncwarp();
-        };
-        // GEMM1 of global chunk gc (chunk c of the current tile)
-        auto gemm1 = [&](uint32_t gc, int c) {
-            const int s = gc & 1, a = gc & (kAcc1 - 1);
-            mbar_spin(&w1_full[s], (gc >> 1) & 1, dead, p.status);
-            mbar_spin(&acc1_empty[a], ((gc / kAcc1) & 1) ^ 1, dead, p.status);
-            tc_fence_after();
-            if (lane == 0) {
-                const uint32_t d_tmem = tmem_base + a * BH;
-                for (int kb = 0; kb < KB1; ++kb) {
-                    const uint64_t da = desc_x + ((kb * (BM * BK * 2)) >> 4);
-                    const uint64_t db = desc_w1 + ((s * W1_BYTES + kb * (BH * BK * 2)) >> 4);
+                            for (int kk = 0; kk < BK / UMMA_K; ++kk)
+                                umma_bf16(tmem_base + a * NT, da + ((kk * UMMA_K * 2) >> 4), db + ((kk * UMMA_K * 2) >> 4), idesc1, (kb | kk) != 0);
+                            umma_commit(&empty[s]);
+                            if (++s == STAGES) { s = 0; phase ^= 1; }
+                        }
+                        umma_commit(&acc1_full[a]);
+                        if (c == t.chunks - 1) umma_commit(x_empty);
+                    }
+                    if (c > 0) {                         // GEMM2 of chunk c - 1
+                        const uint32_t gc = g + c - 1, a = gc & 1;
+                        mbar_wait_lean(&act_full[a], (gc >> 1) & 1, dead, p.status);
+                        if (c == 1) mbar_wait_lean(acc2_empty, (local & 1) ^ 1, dead, p.status);
+                        tc_fence_after();
+                        for (int m = 0; m < MT; ++m)
+                            for (int kh = 0; kh < 2; ++kh) {
+                                mbar_wait_lean(&full[s], phase, dead, p.status);
+                                tc_fence_after();
+                                const uint64_t da = d_ring + s * (BOX_BYTES >> 4), db = d_act + ((a * ACT_BYTES + kh * BK * 128) >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < BK / UMMA_K; ++kk)
-                        umma_bf16(d_tmem, da + ((kk * UMMA_K * 2) >> 4), db + ((kk * UMMA_K * 2) >> 4), idesc1, (kb | kk) != 0);
+                                for (int kk = 0; kk < BK / UMMA_K; ++kk)
+                                    umma_bf16(acc2_tmem + m * NT, da + ((kk * UMMA_K * 2) >> 4), db + ((kk * UMMA_K * 128) >> 4), idesc2,
+                                              (c - 1) | kh | kk);
+                                umma_commit(&empty[s]);
+                                if (++s == STAGES) { s = 0; phase ^= 1; }
+                            }
+                        umma_commit(&act_empty[a]);
+                    }
                 }
-                umma_commit(&w1_empty[s]);
-                umma_commit(&acc1_full[a]);
-                if (c == chunks - 1) umma_commit(x_empty);
+                umma_commit(acc2_full);
+                g += t.chunks;
+                ++local;
             }
-            __syncwarp();
-        };
-        for (int t = first; t < total; t += stride, ++tl) {
-            mbar_spin(x_full, tl & 1, dead, p.status);
-            for (int c = 0; c < kAhead && c < chunks; ++c) gemm1(g + c, c);
-            for (int c = 0; c < chunks; ++c, ++g) {
-                if (c + kAhead < chunks) gemm1(g + kAhead, c + kAhead);
-                gemm2(g, c, tl);
-            }
-            if (lane == 0) umma_commit(acc2_full);
-            __syncwarp();
         }
     } else {
-        // ------------------------------------------------------------------ epilogue (warps 3..18)
-        const int quad = warp & 3;                       // TMEM lanes 32*quad ..
-        const int cpart = (warp - kFirstEpiWarp) >> 2;   // 16 of the chunk's 64 columns
-        const int row_in_tile = quad * 32 + lane;
-        uint32_t g = 0, tl = 0;
-        for (int t = first; t < total; t += stride, ++tl) {
-            for (int c = 0; c < chunks; ++c, ++g) {
-                const int s = g & 1, a = g & (kAcc1 - 1);
-                const uint32_t ph = (g >> 1) & 1;
-                mbar_spin(&acc1_full[a], (g / kAcc1) & 1, dead, p.status);
+        // ------------------------------------------------------------------ epilogue (warps 2..17)
+        const int quad = warp & 3, part = (warp - 2) >> 2;     // tensor-memory lanes 32 quad .., 16-token groups part, part + 4
+        const uint32_t lanes = (uint32_t)(quad * 32) << 16;
+        const int hid = quad * 32 + lane;                      // hidden unit of the chunk = contraction row of GEMM2
+        uint32_t g = 0, local = 0;
+        for (int i = blockIdx.x; i < total; i += gridDim.x) {
+            const MlpItem t = mlp_item<NT>(p, tiles, slices, i);
+            if (t.n == 0) continue;
+            // lane l keeps the slot of token 16 (part + 4 (l / 16)) + l % 16 of the tile, for the stores at the end
+            const int tok = 16 * (part + 4 * (lane >> 4)) + (lane & 15);
+            const int slot = tok < t.rows ? p.slot_of_prow[t.row0 + tok] : -1;
+            for (int c = 0; c < t.chunks; ++c, ++g) {
+                const uint32_t a = g & 1, ph = (g >> 1) & 1;
+                const bool real = (t.c0 + c) * HC + hid < p.h;   // past the hidden width: the box held another expert's rows
+                mbar_wait_lean(&acc1_full[a], ph, dead, p.status);
                 tc_fence_after();
-                // the tile's last GEMM1 is done: nothing reads this CTA's X and W1 buffers any more, the peer may write
-                if (SPLIT && crank == 0 && c == chunks - 1 && warp == kFirstEpiWarp && lane == 0)
-                    mbar_arrive_cluster(map_to_cta(peer_free, 1));
-                float v[16];
-                tmem_load_16_nowait(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(a * BH + cpart * 16), (uint32_t*)v);
-                tmem_load_wait();
+                uint32_t w[2][8];
+#pragma unroll
+                for (int q = 0; q < (NT > 64 ? 2 : 1); ++q) {
+                    const int grp = part + 4 * q;
+                    if (grp * 16 >= t.n) break;          // uniform
+                    float v[16];
+                    tmem_load_16_nowait(tmem_base + lanes + a * NT + grp * 16, (uint32_t*)v);
+                    tmem_load_wait();
+                    act_chunk_any<false, 16>(p.act, v, nullptr);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) w[q][j] = real ? pack_bf16(v[2 * j], v[2 * j + 1]) : 0u;
+                }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acc1_empty[a]);
-                act_chunk_any<false, 16>(p.act, v, nullptr);
-                uint32_t w[8];
+                mbar_wait_lean(&act_empty[a], ph ^ 1, dead, p.status);       // GEMM2 two chunks back has read this buffer
 #pragma unroll
-                for (int i = 0; i < 8; ++i) w[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-                mbar_spin(&a2_empty[s], ph ^ 1, dead, p.status);       // GEMM2 two chunks back has read this buffer
-                uint8_t* row = s_a2 + s * A2_BYTES + row_in_tile * 128;
-                const int sw = row_in_tile & 7;                         // 128-byte swizzle: 16-byte piece j of a row sits at j ^ (row % 8)
-                st_shared_16B(row + (((2 * cpart) ^ sw) << 4), w[0], w[1], w[2], w[3]);
-                st_shared_16B(row + (((2 * cpart + 1) ^ sw) << 4), w[4], w[5], w[6], w[7]);
+                for (int q = 0; q < (NT > 64 ? 2 : 1); ++q) {
+                    const int grp = part + 4 * q;
+                    if (grp * 16 >= t.n) break;
+                    uint8_t* row = s_act + a * ACT_BYTES + (grp >> 2) * (HC * 128) + hid * 128;
+                    const int piece = 2 * (grp & 3), sw = hid & 7;           // 128-byte swizzle: piece j of row k sits at j ^ (k % 8)
+                    st_shared_16B(row + ((piece ^ sw) << 4), w[q][0], w[q][1], w[q][2], w[q][3]);
+                    st_shared_16B(row + (((piece + 1) ^ sw) << 4), w[q][4], w[q][5], w[q][6], w[q][7]);
+                }
                 fence_async_smem();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&a2_full[s]);
+                if (lane == 0) mbar_arrive(&act_full[a]);
             }
-            // the tile's output: acc2 (128 x r) -> bf16 rows of u
-            mbar_spin(acc2_full, tl & 1, dead, p.status);
+            mbar_wait_lean(acc2_full, local & 1, dead, p.status);
             tc_fence_after();
-            const int cols = p.r / 4;                                   // per warp: 16, 32, 48 or 64
-            __nv_bfloat16* out = (__nv_bfloat16*)p.U + ((int64_t)t * BM + row_in_tile) * p.r + cpart * cols;
-            const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(kAcc1 * BH + cpart * cols);
-            // SPLIT: the partial result sits in CTA 0's X / W1 buffers as 16-byte pieces [column / 4][row] (neighbouring
-            // lanes, i.e. rows, at neighbouring addresses)
-            const int piece0 = cpart * (cols / 4);
-            if (SPLIT && crank == 1) {
-                mbar_wait_cluster(peer_free, tl & 1, dead, p.status);
-                const uint32_t dst = map_to_cta(s_x, 0);
-                for (int j = 0; j < cols; j += 16) {
-                    float v[16];
-                    tmem_load_16_nowait(t_addr + j, (uint32_t*)v);
-                    tmem_load_wait();
+            float* out = (float*)p.out + (int64_t)t.slice * p.slots * p.r;
+            for (int m = 0; m < MT; ++m) {
+                const int col = m * 128 + hid;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        st_cluster_16B(dst + (uint32_t)(((piece0 + j / 4 + q) * BM + row_in_tile) * 16), v[4 * q], v[4 * q + 1],
-                                       v[4 * q + 2], v[4 * q + 3]);
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive_release_cluster(map_to_cta(partial_full, 0));
-            } else {
-                if (SPLIT) mbar_wait_cluster(partial_full, tl & 1, dead, p.status);
-                for (int j = 0; j < cols; j += 16) {
+                for (int q = 0; q < (NT > 64 ? 2 : 1); ++q) {
+                    const int grp = part + 4 * q;
+                    if (grp * 16 >= t.n) break;
                     float v[16];
-                    tmem_load_16_nowait(t_addr + j, (uint32_t*)v);
+                    tmem_load_16_nowait(acc2_tmem + lanes + m * NT + grp * 16, (uint32_t*)v);
                     tmem_load_wait();
-                    if (SPLIT) {
+                    if (slices > 1) {
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const float4 o = *(const float4*)(s_x + ((piece0 + j / 4 + q) * BM + row_in_tile) * 16);
-                            v[4 * q] += o.x; v[4 * q + 1] += o.y; v[4 * q + 2] += o.z; v[4 * q + 3] += o.w;
+                        for (int j = 0; j < 16; ++j) {
+                            const int to = __shfl_sync(0xffffffffu, slot, 16 * q + j);
+                            if (to >= 0 && col < p.r) out[(int64_t)to * p.r + col] = v[j];
+                        }
+                    } else {                             // neighbouring lanes swap halves of a token pair: an even lane has two columns
+#pragma unroll                                           // of the first token, an odd lane of the second
+                        for (int j = 0; j < 16; j += 2) {
+                            const bool odd = lane & 1;
+                            const float other = __shfl_xor_sync(0xffffffffu, odd ? v[j] : v[j + 1], 1);
+                            const int to0 = __shfl_sync(0xffffffffu, slot, 16 * q + j), to1 = __shfl_sync(0xffffffffu, slot, 16 * q + j + 1);
+                            const int to = odd ? to1 : to0;
+                            const uint32_t w = odd ? pack_bf16(other, v[j + 1]) : pack_bf16(v[j], other);
+                            if (to >= 0 && col < p.r) *(uint32_t*)((__nv_bfloat16*)p.out + (int64_t)to * p.r + (col & ~1)) = w;
                         }
                     }
-                    uint32_t w[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) w[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-                    st_global_32B(out + j, w);
-                }
-                if (SPLIT) {                                 // these reads come before the next tile's TMA writes
-                    fence_async_smem();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(tile_done);
                 }
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(acc2_empty);
+            ++local;
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (SPLIT) cluster_sync_all();                        // nobody leaves while the peer may still signal or write here
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, TMEM_COLS);
+        tmem_dealloc(tmem_base, 512);
     }
 }
 
-__global__ void __launch_bounds__(kMlpThreads, 1)
-fused_mlp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w1,
-                 const __grid_constant__ CUtensorMap map_w2, const MlpParams p) {
-    fused_mlp_body<false>(map_x, map_w1, map_w2, p);
-}
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMlpThreads, 1)
-fused_mlp_split_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w1,
-                       const __grid_constant__ CUtensorMap map_w2, const MlpParams p) {
-    fused_mlp_body<true>(map_x, map_w1, map_w2, p);
+template <int NT, int STAGES>
+cudaError_t launch(const CUtensorMap& mx, const CUtensorMap& m1, const CUtensorMap& m2, const MlpParams& p, cudaStream_t stream) {
+    const size_t smem = (size_t)STAGES * BOX_BYTES + 2 * (size_t)(NT / 64) * HC * 128 + (size_t)(p.r / BK) * NT * BK * 2 +
+                        (2 * STAGES + 12) * 8 + 16 + 1024;
+    static PerDeviceOnce once;
+    int dev;
+    if (once.needed(&dev)) {
+        cudaError_t e = cudaFuncSetAttribute(fused_mlp_kernel<NT, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+        if (e != cudaSuccess) return e;
+        once.mark(dev);
+    }
+    const int64_t items = (int64_t)p.max_tiles * (128 / NT) * p.sl.most;
+    return launch_chained(fused_mlp_kernel<NT, STAGES>, (unsigned)(items < sm_count() ? items : sm_count()), kMlpThreads, smem, stream, mx, m1, m2, p);
 }
 
 }  // namespace
 
 bool fused_mlp_supported(int r, int h, int dtype) {
-    return dtype == BIGMAC_BF16 && r >= 64 && r <= 256 && r % 64 == 0 && h >= 64 && h % 64 == 0;
+    return dtype == BIGMAC_BF16 && r >= 64 && r <= 512 && r % 64 == 0 && h >= 64 && h % 64 == 0;
 }
 
-// xg [max_rows, r] grouped padded rows, w1 [E, h, r], w2 [E, r, h], u [max_rows, r]; tiles of 128 rows, tile -> expert
-// and the live tile count on the device.
-cudaError_t launch_fused_mlp(const void* xg, const void* w1, const void* w2, void* u, int64_t max_rows, int r, int h, int E,
-                             int act, const int32_t* tile_expert, const int32_t* n_tiles, int* status, cudaStream_t stream) {
-    if (max_rows <= 0) return cudaSuccess;
+// Slices are limited to what fits the activation buffer [P, h] of bf16 that the separate GEMMs would use.
+MlpSlicing fused_mlp_slicing(int r, int h, int64_t N, int64_t P) {
+    MlpSlicing m{sm_count(), (h + HC - 1) / HC, 1, r <= 256 ? 1 : 2};
+    while (m.most < 8 && 2 * m.most * N * r * 4 <= P * h * 2) m.most *= 2;
+    return m;
+}
+
+// xg [max_rows, r] grouped padded rows, w1 [E, h, r], w2 [E, r, h], out [slices][slots][r]; tiles of 128 rows and the tables
+// on the device.
+cudaError_t launch_fused_mlp(const void* xg, const void* w1, const void* w2, void* out, int64_t max_rows, int64_t slots,
+                             const MlpSlicing& sl, int r, int h, int E, int act, const Tables& tb, int* status, cudaStream_t stream) {
+    if (max_rows < kPad) return cudaSuccess;
     CUtensorMap mx, m1, m2;
-    bool ok = make_map(&mx, xg, (uint64_t)r, (uint64_t)max_rows, (uint64_t)r, BK, BM);
-    ok &= make_map(&m1, w1, (uint64_t)r, (uint64_t)E * h, (uint64_t)r, BK, BH);
-    ok &= make_map(&m2, w2, (uint64_t)h, (uint64_t)E * r, (uint64_t)h, BH, (uint32_t)r);
+    bool ok = make_map(&mx, xg, (uint64_t)r, (uint64_t)max_rows, (uint64_t)r, BK, 16);
+    ok &= make_map(&m1, w1, (uint64_t)r, (uint64_t)E * h, (uint64_t)r, BK, 128);
+    ok &= make_map(&m2, w2, (uint64_t)h, (uint64_t)E * r, (uint64_t)h, BK, 128);
     if (!ok) return cudaErrorInvalidValue;
     MlpParams p{};
-    p.U = u; p.r = r; p.h = h; p.act = act; p.b1_rows_per_expert = h; p.b2_rows_per_expert = r;
-    p.tile_expert = tile_expert; p.n_tiles = n_tiles; p.max_tiles = (int)(max_rows / BM); p.status = status;
-    const int kb1 = r / BK;
-    const size_t smem = (size_t)kb1 * BM * BK * 2 + 2 * (size_t)kb1 * BH * BK * 2 + 2 * (size_t)r * BH * 2 + 2 * (size_t)BM * BH * 2 +
-                        27 * 8 + 16 + 1024;
-    static PerDeviceOnce once;
-    int dev;
-    if (once.needed(&dev)) {
-        cudaError_t e = cudaFuncSetAttribute(fused_mlp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_mlp_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-        if (e != cudaSuccess) return e;
-        once.mark(dev);
-    }
-    if (p.max_tiles <= 0) return cudaSuccess;
-    // at most one tile per SM and an even number of hidden chunks: two SMs per tile, half of the chunks each
-    if (p.max_tiles <= sm_count() && (h / BH) % 2 == 0) {
-        const int pairs = p.max_tiles < sm_count() / 2 ? p.max_tiles : sm_count() / 2;
-        return launch_chained(fused_mlp_split_kernel, 2 * pairs, kMlpThreads, smem, stream, mx, m1, m2, p);
-    }
-    const int grid = p.max_tiles < sm_count() ? p.max_tiles : sm_count();
-    return launch_chained(fused_mlp_kernel, grid, kMlpThreads, smem, stream, mx, m1, m2, p);
+    p.out = out; p.slots = slots; p.r = r; p.h = h; p.act = act; p.sl = sl;
+    p.tile_expert = tb.tile_expert; p.n_tiles = tb.n_tiles; p.poffsets = tb.poffsets; p.counts = tb.counts; p.slot_of_prow = tb.slot_of_prow;
+    p.max_tiles = (int)(max_rows / kPad); p.status = status;
+    return r <= 256 ? launch<128, 6>(mx, m1, m2, p, stream) : launch<64, 8>(mx, m1, m2, p, stream);
 }
 
 }  // namespace bigmac

@@ -106,11 +106,35 @@ bool gemm_tc_groupk_supported(const GemmArgs& g);
 size_t gemm_tc_groupk_ws_bytes(int M, int N, int E);
 cudaError_t gemm_tc_groupk(const GemmArgs& g, int* status, int* sched, void* ws, cudaStream_t stream);
 cudaError_t gemm_tc_groupk_finish(const GemmArgs& g, void* ws, cudaStream_t stream);   // always after gemm_tc_groupk
-// Inference forward of the experts in one kernel for r <= 256 (gemm_tc_mlp.cu): u = sigma(xg W1_e^T) W2_e^T per
-// 128-row tile, hidden activations kept on the SM.
+// Inference forward of the experts in one kernel (gemm_tc_mlp.cu): fp32 rows of u = sigma(xg W1_e^T) W2_e^T by slot,
+// out [slices][slots][r] (the slices of the hidden width add up to u; a single slice is written as bf16), hidden activations
+// kept on the SM.
+// How many slices is a function of the number of row tiles, which only the device knows: every kernel concerned
+// evaluates mlp_slices for itself.
+struct MlpSlicing {
+    int units;       // SMs
+    int chunks;      // 128-wide chunks of the hidden width
+    int most;        // slices that the output buffer has room for
+    int per_tile;    // work items per 128-row tile and slice
+};
+// The slices s (a power of two that divides the chunks) with the shortest longest SM: rounds of items, times an item's
+// chunks and what its start and its output take in units of a chunk (fp32 partial results: twice the bytes of bf16).
+// Few tiles: more slices put idle SMs to work (64 tiles of 8 chunks: two slices, 17 -> 12 us); more than one tile per SM:
+// one slice (220 tiles of 8 chunks: the fp32 rows of two slices cost what the better last round gains).
+__host__ __device__ inline int mlp_slices(const MlpSlicing& m, int tiles) {
+    int best = 1, best_cost = 0x7fffffff;
+    for (int s = 1; s <= m.most && m.chunks % s == 0; s *= 2) {
+        const long long items = (long long)tiles * m.per_tile * s;
+        const long long cost = (items + m.units - 1) / m.units * (m.chunks / s + (s > 1 ? 3 : 2));
+        if (cost < best_cost) { best = s; best_cost = (int)(cost < 0x7ffffffe ? cost : 0x7ffffffe); }
+    }
+    return best;
+}
+struct Tables;
 bool fused_mlp_supported(int r, int h, int dtype);
-cudaError_t launch_fused_mlp(const void* xg, const void* w1, const void* w2, void* u, int64_t max_rows, int r, int h, int E,
-                             int act, const int32_t* tile_expert, const int32_t* n_tiles, int* status, cudaStream_t stream);
+MlpSlicing fused_mlp_slicing(int r, int h, int64_t N, int64_t P);
+cudaError_t launch_fused_mlp(const void* xg, const void* w1, const void* w2, void* out, int64_t max_rows, int64_t slots,
+                             const MlpSlicing& sl, int r, int h, int E, int act, const Tables& tb, int* status, cudaStream_t stream);
 // CTA-pair variant (tcgen05 cta_group::2) for outputs at least 256 wide.
 bool gemm_tc_pair_supported(const GemmArgs& g);
 bool gemm_tc_pair_preferred(const GemmArgs& g);
@@ -203,6 +227,10 @@ cudaError_t launch_dispatch(const void* src, void* grouped, const Tables& tb, in
 // dst rows are `dst_ld` elements apart (0: dense, = width).
 cudaError_t launch_combine(const void* grouped, void* dst, const float* w, const int32_t* prow_of_slot, int T,
                            int k, int width, int dtype, cudaStream_t stream, int dst_ld = 0, bool may_drop = false);
+// The same from the fp32 rows of the fused expert kernel: dst[t,:] = sum_j w[t*k+j] * sum_s parts[s][t*k+j][:], bf16 result;
+// with may_drop, slots without a row are left out.
+cudaError_t launch_combine_parts(const void* parts, const MlpSlicing& sl, const int32_t* n_tiles, void* dst, const float* w,
+                                 const int32_t* prow_of_slot, int T, int k, int width, cudaStream_t stream, bool may_drop);
 // Backward of the combine: du[prow,:] = p[s] * dy_lo[t,:] (zeros on padding), dp[s] = <dy_lo[t,:], u[prow,:]>.
 cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float* dp, const Tables& tb, int k,
                                int width, int dtype, int64_t max_prows, cudaStream_t stream);

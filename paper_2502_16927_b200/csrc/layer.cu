@@ -129,12 +129,24 @@ void carve_backward_scratch(Carver& cv, const Dims& m, Buffers& b) {
     b.bias_ws = bias_ws ? (float*)cv.take_bytes(bias_ws) : nullptr;
 }
 
-// Few tokens: the descend + gate-logits launch has a handful of output tiles, each walking all of d; its contraction
-// is then cut into parts (fp32 partial results, added by a small kernel) so that the SMs share the weight streaming.
-// A function of the shape only: every call of a handle with the same T takes the same path.
+// The descend + gate-logits launch has few output tiles where there are few tokens, each walking all of d; its contraction
+// is then cut into parts (fp32 partial results, added by the routing kernels on the way) so that the SMs share the work.
+// Cost of s parts in k slices of tensor work (0.35 us): the longest SM pair's slices, plus what writing and reading the
+// partial results takes (0.8 us per MB).  At d = 2048, r + E = 320: 8 parts at 64 tokens, 4 at 512, 3 at 1200, none from
+// 1800 on (at 3001, three parts: launch 19.3 -> 16.3 us, placement 6.9 -> 10.4).  A function of the shape only: every call of a handle with the same T takes the same path.
 int descend_split_parts(const Dims& m) {
-    if (m.T > 1024 || m.E % 4 || m.dtype != BIGMAC_BF16) return 1;
-    return choose_split_k(m.T, m.r + m.E, m.d);
+    if (m.E % 4 || m.dtype != BIGMAC_BF16) return 1;
+    const int n = m.r + m.E, bn = n >= 256 ? 256 : 128, bm = n >= 256 ? 256 : 128;
+    const int64_t tiles = (int64_t)((m.T + bm - 1) / bm) * ((n + bn - 1) / bn);
+    const int num_kb = m.d / 64, units = n >= 256 ? gemm_tc_sm_count() / 2 : gemm_tc_sm_count();
+    int best = 1;
+    double best_cost = 0;
+    for (int s = 1; s <= kMaxSplitK && s <= num_kb; ++s) {
+        double cost = (double)((tiles * s + units - 1) / units) * ((num_kb + s - 1) / s);
+        if (s > 1) cost += (double)s * m.T * n * 4.0 / 0.44e6;
+        if (s == 1 || cost < best_cost) { best = s; best_cost = cost; }
+    }
+    return best;
 }
 void carve_descend_split(Carver& cv, const Dims& m, Buffers& b) {
     const int parts = descend_split_parts(m);
@@ -316,6 +328,13 @@ GemmArgs dw1_request(const Dims& m, const void* dz, const void* rows, const Tabl
     return g;
 }
 
+// Do the experts of an inference forward run in one kernel?  (The fused_mlp debug switch: 0 never, 2 wherever it can.)
+bool uses_fused_mlp(const bigmac_layer* L, const Dims& m) {
+    const int mode = switches().fused_mlp;
+    if (mode == 0 || m.bias || !sigma_as_bytes(L) || !fused_mlp_supported(m.r, m.h, m.dtype) || m.N * m.r * 4 > m.P * m.h * 2) return false;
+    return mode == 2 || m.P / kPad <= 2 * (int64_t)gemm_tc_sm_count();
+}
+
 // Is the dispatch fused into its consumers' operand loads (F5 of the forward disappears as a launch, the grouped
 // copy xg of x' is never written)?  Inference: expert GEMM1 gathers the rows of x' itself.  Training: so does the
 // weight gradient dW1, when it runs on the balanced kernel (the statically scheduled kernels read a grouped copy).
@@ -324,10 +343,7 @@ GemmArgs dw1_request(const Dims& m, const void* dz, const void* rows, const Tabl
 bool dispatch_is_fused(const bigmac_layer* L, const Dims& m, bool training) {
     if (!switches().fuse_dispatch || !sigma_as_bytes(L) || m.r % 64) return false;
     if (!training) {
-        const bool short_list = m.P / kPad <= 2 * (int64_t)gemm_tc_sm_count();
-        const bool mlp_fused = !m.bias && (switches().fused_mlp == 2 || (switches().fused_mlp == 1 && short_list)) &&
-                               fused_mlp_supported(m.r, m.h, m.dtype);
-        return !mlp_fused;
+        return !uses_fused_mlp(L, m);
     }
     if (m.r % 128) return false;
     Tables shape_only{};                                     // the kernel choice depends on shapes and alignment only:
@@ -534,17 +550,12 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
     }
     BIGMAC_TRY(route_from_logits(L, m, W, b, src, mv, aux_word_to_zero(m, routing_out), st));
     BIGMAC_TRY(export_routing(L, m, b, routing_out, st));
-    const bool short_list = m.P / kPad <= 2 * (int64_t)gemm_tc_sm_count();
-    const bool mlp_fused_ = !training && !m.bias && (switches().fused_mlp == 2 || (switches().fused_mlp == 1 && short_list)) &&
-                            sigma_as_bytes(L) && fused_mlp_supported(m.r, m.h, m.dtype);
-    // Inference, low width r <= 256, up to two row tiles per SM: F6 + F7 in one kernel, the hidden activations stay on
-    // the SM.  On long tile lists the two separate GEMMs are faster (the fused kernel is bound by the issue of its many
-    // narrow MMA instructions): measured 0.375 vs 0.329 ms forward at the medium workload, 0.099 vs 0.106 ms at 512
-    // decode tokens.  The fused_mlp debug switch forces it off (0) / on (2).
-    if (mlp_fused_) {
+    // Inference: F6 + F7 in one kernel, the hidden activations stay on the SM (uses_fused_mlp has the rule).
+    const bool mlp_fused = !training && uses_fused_mlp(L, m);
+    const MlpSlicing slicing = fused_mlp_slicing(m.r, m.h, m.N, m.P);
+    if (mlp_fused) {
         Stage s(L, S_FUSED_MLP, st);
-        BIGMAC_CUDA(launch_fused_mlp(b.xg, W->w1, W->w2, b.u, m.P, m.r, m.h, m.E, c.act, b.tb.tile_expert, b.tb.n_tiles,
-                                     L->status, st));
+        BIGMAC_CUDA(launch_fused_mlp(b.xg, W->w1, W->w2, b.a, m.P, m.N, slicing, m.r, m.h, m.E, c.act, b.tb, L->status, st));
     } else {
         {                                                                             // F6 a = sigma(xg W1_e^T); saves sigma'(z)
             GemmArgs g;
@@ -566,7 +577,10 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
         }
     }
     if (m.cdac) b.y_lo = y;                                                       // Eq. 3: the weighted sum is the output
-    { Stage s(L, S_COMBINE, st); BIGMAC_CUDA(launch_combine(b.u, b.y_lo, b.tb.topk_w, b.tb.prow_of_slot, m.T, m.k, m.r, m.dtype, st, 0, m.cap != kNoCapacity)); }  // F8
+    if (mlp_fused) {                                                              // F8
+        Stage s(L, S_COMBINE, st);
+        BIGMAC_CUDA(launch_combine_parts(b.a, slicing, b.tb.n_tiles, b.y_lo, b.tb.topk_w, b.tb.prow_of_slot, m.T, m.k, m.r, st, m.cap != kNoCapacity));
+    } else { Stage s(L, S_COMBINE, st); BIGMAC_CUDA(launch_combine(b.u, b.y_lo, b.tb.topk_w, b.tb.prow_of_slot, m.T, m.k, m.r, m.dtype, st, 0, m.cap != kNoCapacity)); }  // F8
     if (!m.cdac) {                                                                // F9 ascend: y = y' W'_up
         GemmArgs g;
         g.A = b.y_lo; g.lda = m.r; g.B = W->w_up; g.ldb = m.r; g.C = y; g.ldc = m.d;

@@ -79,8 +79,10 @@ __global__ void __launch_bounds__(256) dispatch_kernel(const uint4* __restrict__
     }
 }
 
-// MAY_DROP: slots may carry row -1 (dropped under a capacity limit) and are then left out; without it the loop has no
-// branch and the k row loads of a token are issued together.
+// A warp per token.  The rows of eight slots are fetched together (lane j reads the place and weight of slot j, all row
+// loads of a batch are issued before the first is used), then added in slot order: with one dependent load per slot the
+// kernel waited for eight round trips to L2 in a row.  MAY_DROP: slots may carry row -1 (dropped under a capacity limit)
+// and are then left out.
 template <typename T, bool MAY_DROP>
 __global__ void __launch_bounds__(256) combine_kernel(const uint4* __restrict__ grouped, uint4* __restrict__ dst,
                                                       const float* __restrict__ w,
@@ -88,27 +90,100 @@ __global__ void __launch_bounds__(256) combine_kernel(const uint4* __restrict__ 
                                                       int vecs_per_row, int dst_vecs_per_row) {
     grid_dependency_wait();
     grid_dependency_launch();
-    constexpr int V = Vec<T>::kElems;
+    constexpr int V = Vec<T>::kElems, B = 8;
     const int t = warp_global_id();
     if (t >= n_tokens) return;
     const int lane = threadIdx.x & 31;
-    for (int c = lane; c < vecs_per_row; c += 32) {
+    for (int c0 = 0; c0 < vecs_per_row; c0 += 32) {
+        const int c = c0 + lane;
+        const bool mine = c < vecs_per_row;
         float acc[V];
 #pragma unroll
         for (int i = 0; i < V; ++i) acc[i] = 0.0f;
-        for (int j = 0; j < k; ++j) {                      // slot order: fixed summation order
-            const int64_t s = (int64_t)t * k + j;
-            int prow = prow_of_slot[s];
-            if (MAY_DROP && prow < 0) continue;             // dropped under a capacity limit: absent from the sum
-            if (!MAY_DROP) prow = max(prow, 0);             // dropless rows are never negative; keeps the address in range if one were
-            const float p = w ? w[s] : 1.0f;
-            float f[V];
-            Vec<T>::unpack(grouped[(int64_t)prow * vecs_per_row + c], f);
+        for (int j0 = 0; j0 < k; j0 += B) {
+            int place = -1;
+            float weight = 1.0f;
+            if (lane < B && j0 + lane < k) {
+                const int64_t s = (int64_t)t * k + j0 + lane;
+                place = prow_of_slot[s];
+                if (!MAY_DROP) place = max(place, 0);        // dropless rows are never negative; keeps the address in range if one were
+                if (w) weight = w[s];
+            }
+            uint4 v[B];
 #pragma unroll
-            for (int i = 0; i < V; ++i) acc[i] = fmaf(p, f[i], acc[i]);
+            for (int j = 0; j < B; ++j) {
+                const int prow = __shfl_sync(kFull, place, j);
+                v[j] = (mine && prow >= 0) ? grouped[(int64_t)prow * vecs_per_row + c] : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int j = 0; j < B; ++j) {                      // slot order: fixed summation order
+                if (__shfl_sync(kFull, place, j) < 0) continue;
+                const float p = __shfl_sync(kFull, weight, j);
+                float f[V];
+                Vec<T>::unpack(v[j], f);
+#pragma unroll
+                for (int i = 0; i < V; ++i) acc[i] = fmaf(p, f[i], acc[i]);
+            }
         }
-        dst[(int64_t)t * dst_vecs_per_row + c] = Vec<T>::pack(acc);
+        if (mine) dst[(int64_t)t * dst_vecs_per_row + c] = Vec<T>::pack(acc);
     }
+}
+
+// Combine of the fused expert kernel's fp32 rows, [parts][T k][r]: the rows of a token's slots lie side by side, a thread
+// owns four columns of one token.  The loads of eight slots of one slice are in flight together.
+template <bool MAY_DROP>
+__global__ void __launch_bounds__(128) combine_parts_kernel(const float4* __restrict__ src, const int32_t* __restrict__ n_tiles,
+                                                            MlpSlicing sl, int64_t part_stride, uint2* __restrict__ dst,
+                                                            const float* __restrict__ w, const int32_t* __restrict__ prow_of_slot,
+                                                            int T, int k, int quads) {
+    grid_dependency_wait();
+    grid_dependency_launch();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)T * quads) return;
+    const int parts = mlp_slices(sl, *n_tiles);
+    const int64_t t = i / quads;
+    const int c = (int)(i - t * quads);
+    float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float4* row = src + t * k * quads + c;
+    for (int j0 = 0; j0 < k; j0 += 8) {
+        float4 u[8];
+        float p[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            p[j] = j0 + j < k ? w[t * k + j0 + j] : 0.0f;
+            if (MAY_DROP && j0 + j < k && prow_of_slot[t * k + j0 + j] < 0) p[j] = 0.0f;
+            u[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        if (parts == 1) {                                // bf16 rows
+            uint2 v[8];
+            const uint2* from = reinterpret_cast<const uint2*>(src) + t * k * quads + c;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const bool there = j0 + j < k && (!MAY_DROP || prow_of_slot[t * k + j0 + j] >= 0);
+                v[j] = there ? from[(int64_t)(j0 + j) * quads] : make_uint2(0, 0);
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                u[j] = make_float4(__uint_as_float(v[j].x << 16), __uint_as_float(v[j].x & 0xffff0000u), __uint_as_float(v[j].y << 16),
+                                   __uint_as_float(v[j].y & 0xffff0000u));
+        }
+        else for (int s = 0; s < parts; ++s) {           // slices in order inside a slot
+            float4 v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const bool there = j0 + j < k && (!MAY_DROP || prow_of_slot[t * k + j0 + j] >= 0);
+                v[j] = there ? row[s * part_stride + (int64_t)(j0 + j) * quads] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { u[j].x += v[j].x; u[j].y += v[j].y; u[j].z += v[j].z; u[j].w += v[j].w; }
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {                    // slot order
+            acc.x = fmaf(p[j], u[j].x, acc.x); acc.y = fmaf(p[j], u[j].y, acc.y); acc.z = fmaf(p[j], u[j].z, acc.z); acc.w = fmaf(p[j], u[j].w, acc.w);
+        }
+    }
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y), hi = __floats2bfloat162_rn(acc.z, acc.w);
+    dst[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
 }
 
 template <typename T>
@@ -379,6 +454,16 @@ cudaError_t launch_combine(const void* grouped, void* dst, const float* w, const
         return launch_chained(combine_kernel<float, false>, warp_blocks(T), 256, 0, stream, src, out, w, prow_of_slot, T, k, vecs, dvecs);
     }
     return cudaGetLastError();
+}
+
+cudaError_t launch_combine_parts(const void* parts, const MlpSlicing& sl, const int32_t* n_tiles, void* dst, const float* w,
+                                 const int32_t* prow_of_slot, int T, int k, int width, cudaStream_t stream, bool may_drop) {
+    if (T == 0) return cudaSuccess;
+    const int quads = width / 4;
+    const int64_t n = (int64_t)T * quads, stride = (int64_t)T * k * quads;
+    const unsigned blocks = (unsigned)((n + 127) / 128);
+    if (may_drop) return launch_chained(combine_parts_kernel<true>, blocks, 128, 0, stream, (const float4*)parts, n_tiles, sl, stride, (uint2*)dst, w, prow_of_slot, T, k, quads);
+    return launch_chained(combine_parts_kernel<false>, blocks, 128, 0, stream, (const float4*)parts, n_tiles, sl, stride, (uint2*)dst, w, prow_of_slot, T, k, quads);
 }
 
 cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float* dp, const Tables& tb, int k,

@@ -342,6 +342,8 @@ __global__ void __launch_bounds__(1024) tables_small_kernel(const int32_t* __res
     }
 }
 
+constexpr int kMaxParts = 8;                        // parts of a split descend contraction
+
 // ---- Routing in two launches (k <= 8, E a multiple of 4 up to 256: every configuration of the paper) -------------
 // A forward used to spend six launches between the gate logits and the experts (top-k, fill, three passes of the
 // counting sort, dispatch): about 2.5 us each for work of well under a microsecond, 20 us of 128 at 3001 tokens of the
@@ -378,9 +380,14 @@ __global__ void __launch_bounds__(1024) topk_count_kernel(const float* __restric
             float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             if (e0 < E) {
                 x = *reinterpret_cast<const float4*>(row + e0);
-                for (int s = 1; s < parts; ++s) {
-                    const float4 y = *reinterpret_cast<const float4*>(row + s * part_stride + e0);
-                    x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+                if (parts > 1) {                     // all parts' loads in flight together, added in part order
+                    float4 y[kMaxParts - 1];
+#pragma unroll
+                    for (int s = 1; s < kMaxParts; ++s)
+                        if (s < parts) y[s - 1] = *reinterpret_cast<const float4*>(row + s * part_stride + e0);
+#pragma unroll
+                    for (int s = 1; s < kMaxParts; ++s)
+                        if (s < parts) { x.x += y[s - 1].x; x.y += y[s - 1].y; x.z += y[s - 1].z; x.w += y[s - 1].w; }
                 }
                 if (logits_out && live) *reinterpret_cast<float4*>(logits_out + t * E + e0) = x;
                 if (b_gate) { x.x += b_gate[e0]; x.y += b_gate[e0 + 1]; x.z += b_gate[e0 + 2]; x.w += b_gate[e0 + 3]; }
@@ -476,21 +483,36 @@ template <int MOVE>
 __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p) {
     grid_dependency_wait();
     grid_dependency_launch();
-    __shared__ int4 s_all[kPlaceThreads], s_below[kPlaceThreads];           // [parts][E / 4]
+    __shared__ int32_t s_all[kPlaceThreads], s_below[kPlaceThreads];        // [parts][E]
     __shared__ int32_t s_base[kPlaceMaxExperts], s_total[kPlaceMaxExperts], s_off[kPlaceMaxExperts + 1], s_poff[kPlaceMaxExperts + 1];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kWarps = kPlaceThreads / 32;
-    const int E = p.E, groups = E >> 2, nparts = min(32, kPlaceThreads / groups);
+    const int E = p.E, nparts = min(16, kPlaceThreads / E);
     const int b = blockIdx.x / p.splits;             // the block of kernel 1 whose slots these are
+    const int per_split = (p.tokens_per_block + p.splits - 1) / p.splits;
+    const int64_t first = (int64_t)b * p.tokens_per_block + (int64_t)(blockIdx.x - b * p.splits) * per_split;
+    const int64_t last = min(min(first + per_split, (int64_t)(b + 1) * p.tokens_per_block), (int64_t)p.T);
+    // the warp's first token: its experts and ranks are on their way while the counts are added up
+    int next_e = 0, next_rank = 0;
+    if (first + warp < last && lane < p.k) {
+        next_e = p.topk_idx[(first + warp) * p.k + lane];
+        next_rank = p.prow_of_slot[(first + warp) * p.k + lane];
+    }
     {
-        const int g = tid % groups, part = tid / groups;
-        int4 all = make_int4(0, 0, 0, 0), below = all;
-        if (part < nparts)
-            for (int row = part; row < p.nb; row += nparts) {
-                const int4 c = *reinterpret_cast<const int4*>(p.block_counts + (size_t)row * E + 4 * g);
-                all.x += c.x; all.y += c.y; all.z += c.z; all.w += c.w;
-                if (row < b) { below.x += c.x; below.y += c.y; below.z += c.z; below.w += c.w; }
+        const int e = tid % E, part = tid / E;       // neighbouring threads on neighbouring experts
+        int all = 0, below = 0;
+        if (part < nparts) {
+            for (int row = part; row < p.nb; row += 16 * nparts) {
+                int c[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) c[i] = row + i * nparts < p.nb ? p.block_counts[(size_t)(row + i * nparts) * E + e] : 0;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    all += c[i];
+                    if (row + i * nparts < b) below += c[i];
+                }
             }
+        }
         s_all[tid] = all;
         s_below[tid] = below;
     }
@@ -498,8 +520,8 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p)
     if (tid < E) {
         int all = 0, below = 0;
         for (int q = 0; q < nparts; ++q) {
-            all += reinterpret_cast<const int32_t*>(s_all)[q * E + tid];
-            below += reinterpret_cast<const int32_t*>(s_below)[q * E + tid];
+            all += s_all[q * E + tid];
+            below += s_below[q * E + tid];
         }
         s_total[tid] = all;
         s_base[tid] = below;
@@ -531,9 +553,6 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p)
     }
     __syncthreads();
     // ---- this block's tokens
-    const int per_split = (p.tokens_per_block + p.splits - 1) / p.splits;
-    const int64_t first = (int64_t)b * p.tokens_per_block + (int64_t)(blockIdx.x - b * p.splits) * per_split;
-    const int64_t last = min(min(first + per_split, (int64_t)(b + 1) * p.tokens_per_block), (int64_t)p.T);
     for (int64_t t = first + warp; t < last; t += kWarps) {
         uint4 v0 = make_uint4(0, 0, 0, 0), v1 = v0;
         if (MOVE == 1) {                             // the first 64 pieces of the row are on their way before its place is known
@@ -543,12 +562,13 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p)
         int prow = -1;
         if (lane < p.k) {
             const int64_t s = t * p.k + lane;
-            const int e = p.topk_idx[s];
+            const int e = next_e, rank = next_rank;
+            if (t + kWarps < last) { next_e = p.topk_idx[s + kWarps * p.k]; next_rank = p.prow_of_slot[s + kWarps * p.k]; }
             int row = -1;
             if ((unsigned)e >= (unsigned)E) {        // second line of defence: the slot goes nowhere, the call reports it
                 if (p.status) atomicExch(p.status, 2);
             } else {
-                const int within = s_base[e] + p.prow_of_slot[s];
+                const int within = s_base[e] + rank;
                 if (within < p.cap) {                // else dropped under a capacity limit
                     row = s_off[e] + within;
                     prow = s_poff[e] + within;
@@ -572,13 +592,19 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p)
                     const int cc = c + 32 * h;
                     if (cc >= p.vecs) continue;
                     const float* from = p.partial + t * p.ld + 8 * cc;
-                    float4 a = *reinterpret_cast<const float4*>(from), d = *reinterpret_cast<const float4*>(from + 4);
-#pragma unroll 4
-                    for (int s = 1; s < p.parts; ++s) {
-                        const float4 x = *reinterpret_cast<const float4*>(from + s * p.part_stride), y = *reinterpret_cast<const float4*>(from + s * p.part_stride + 4);
-                        a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
-                        d.x += y.x; d.y += y.y; d.z += y.z; d.w += y.w;
-                    }
+                    float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), d = a, x[kMaxParts], y[kMaxParts];
+#pragma unroll
+                    for (int s = 0; s < kMaxParts; ++s)
+                        if (s < p.parts) {
+                            x[s] = *reinterpret_cast<const float4*>(from + s * p.part_stride);
+                            y[s] = *reinterpret_cast<const float4*>(from + s * p.part_stride + 4);
+                        }
+#pragma unroll
+                    for (int s = 0; s < kMaxParts; ++s)
+                        if (s < p.parts) {
+                            a.x += x[s].x; a.y += x[s].y; a.z += x[s].z; a.w += x[s].w;
+                            d.x += y[s].x; d.y += y[s].y; d.z += y[s].z; d.w += y[s].w;
+                        }
                     __nv_bfloat162 o[4] = {__floats2bfloat162_rn(a.x, a.y), __floats2bfloat162_rn(a.z, a.w),
                                            __floats2bfloat162_rn(d.x, d.y), __floats2bfloat162_rn(d.z, d.w)};
                     (h ? v1 : v0) = *reinterpret_cast<uint4*>(o);

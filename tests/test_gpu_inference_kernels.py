@@ -1,0 +1,71 @@
+"""Kernels of the inference forward at the sizes where their tiling can go wrong: the experts in one kernel (token counts
+around its 16-token groups, 64- and 128-token tiles, hidden widths that end inside a 128-wide chunk, one to eight slices
+of the hidden width) and the two routing launches (one to many blocks, expert counts around the lanes' loads)."""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import margin
+from paper_2502_16927_b200 import workloads as wl
+from helpers import make_layer, to_device, to_numpy
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(w, skew):
+    inp = wl.make_inputs(w)
+    inp["b_gate"] = (skew * np.linspace(1.0, -1.0, w.E) ** 3).astype(np.float32)
+    margin.enforce_margin(w, inp, 1e-3)
+    return inp
+
+
+def _check_tables(R, rt):
+    for name in ("topk_idx", "counts", "counts_chosen", "offsets", "row_of_slot", "slot_of_row"):
+        np.testing.assert_array_equal(to_numpy(R[name]), getattr(rt, name).reshape(-1), err_msg=name)
+    # softmax of fp32 logits (rounding about 1e-6 of values of order one)
+    np.testing.assert_allclose(to_numpy(R["topk_w"]), rt.topk_p.reshape(-1), rtol=0, atol=2e-5)
+
+
+@pytest.mark.parametrize("r,h", [(64, 64), (128, 192), (192, 512), (256, 1024), (320, 256), (512, 384)])
+@pytest.mark.parametrize("T,skew", [(17, 0.0), (40, 4.0), (129, 0.0), (333, 2.0)])
+def test_experts_in_one_kernel(r, h, T, skew):
+    import torch
+    from paper_2502_16927_b200 import binding
+
+    w = wl.Workload("mlp", T=T, d=128, r=r, h=h, E=12, k=3, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=500 + T)
+    inp = _inputs(w, skew)
+    dev = to_device(w, inp)
+    layer = make_layer(w)
+    try:
+        binding.bigmac_debug_set("fused_mlp", 2)
+        y, R = layer.forward(dev["x"], dev, want_routing=True)
+        again = layer.forward(dev["x"], dev)
+        torch.cuda.synchronize()
+    finally:
+        binding.bigmac_debug_set("defaults")
+    assert layer.status() == 0
+    rt = oracle.route(inp, w.k)
+    _check_tables(R, rt)
+    ref = oracle.forward_tokens(inp, rt, w.act)["y"]
+    # four bf16 stores (x', a, y', y; u too with one slice) of unit roundoff 2^-8 each, i.e. about 0.17 % of the rms per store
+    err = np.linalg.norm(to_numpy(y) - ref) / np.linalg.norm(ref)
+    assert err <= 8e-3, err
+    assert torch.equal(y, again)
+    layer.close()
+
+
+@pytest.mark.parametrize("E,k", [(4, 1), (8, 8), (36, 3), (64, 8), (100, 5), (256, 8)])
+@pytest.mark.parametrize("T", [1, 4, 31, 33, 128, 4737, 20003])
+def test_routing_in_two_launches(E, k, T):
+    import torch
+
+    w = wl.Workload("route", T=T, d=32, r=8, h=8, E=E, k=k, dtype=wl.DTYPE_F32, act=wl.ACT_RELU, seed=33)
+    inp = _inputs(w, 1.0)
+    dev = to_device(w, inp)
+    for f in (0.0, 0.6):
+        layer = make_layer(w, capacity_factor=f)
+        R = layer.route(dev["x"], dev)
+        torch.cuda.synchronize()
+        assert layer.status() == 0
+        _check_tables(R, oracle.route(inp, w.k, capacity_factor=f))
+        layer.close()
