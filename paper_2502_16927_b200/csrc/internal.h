@@ -69,10 +69,10 @@ struct GemmArgs {
     const int32_t* tile_expert = nullptr;
     const int32_t* n_tiles = nullptr;
     const int32_t* poffsets = nullptr;
-    // Tensor-core path only, dense problems only:
+    // Dense problems only:
     const void* B2 = nullptr;           // second MN-major B: contraction rows k >= b2_first_k read B2[(k - b2_first_k)*ldb2 + n]
     int64_t ldb2 = 0;
-    int b2_first_k = 0;                 // multiple of 64
+    int b2_first_k = 0;                 // multiple of 64 on the tensor-core path
     // ... or, with K-major B: output columns n >= n_split use rows of B2 (n - n_split) and are written as fp32 to
     // C2[m*ldc2 + n - n_split] for n - n_split < N2 (n_split a multiple of the tile width; N = n_split + N2).
     int n_split = -1;
@@ -95,6 +95,9 @@ struct GemmArgs {
 
 // fp32-FMA GEMM for either dtype (dtype: bigmac_dtype_t of A, B, Z and - unless out_f32 - C).
 cudaError_t gemm_simt(const GemmArgs& g, int dtype, cudaStream_t stream);
+// Up to kSimtBatch independent contractions in one launch (none may read what another writes).
+constexpr int kSimtBatch = 3;
+cudaError_t gemm_simt_batch(const GemmArgs* g, int count, int dtype, cudaStream_t stream);
 // tcgen05 / TMEM / TMA GEMM, bf16 inputs, fp32 accumulation.  `status` is the device status word.
 cudaError_t gemm_tc(const GemmArgs& g, int* status, cudaStream_t stream);
 bool gemm_tc_available();

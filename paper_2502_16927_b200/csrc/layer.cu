@@ -197,6 +197,29 @@ int gemm(const bigmac_layer* L, int id, const GemmArgs& g, cudaStream_t st) {
     return err == cudaSuccess ? BIGMAC_OK : BIGMAC_ERR_CUDA;
 }
 
+// Contractions that do not depend on each other.  On the FMA path (small layers, where a launch costs more than most
+// contractions) they go out in one launch, by flush(); on the tensor cores one by one, at once.
+struct Together {
+    const bigmac_layer* L;
+    bool batch;
+    cudaStream_t st;
+    GemmArgs g[kSimtBatch];
+    int n = 0, first_id = 0;
+    int add(int id, const GemmArgs& q, cudaStream_t stream) {
+        if (!batch) return gemm(L, id, q, stream);
+        if (n == 0) first_id = id;
+        g[n++] = q;
+        return BIGMAC_OK;
+    }
+    int flush() {
+        if (n == 0) return BIGMAC_OK;
+        Stage stage(L, first_id, st);
+        const cudaError_t err = gemm_simt_batch(g, n, L->cfg.dtype, st);
+        n = 0;
+        return err == cudaSuccess ? BIGMAC_OK : BIGMAC_ERR_CUDA;
+    }
+};
+
 // Number of parts to cut a dense contraction of `num_kb` k slices into so that tiles * parts fills the SMs:
 // minimises waves * slices-per-part (ties: fewer parts).
 int choose_split_k(int M, int N, int K) {
@@ -236,7 +259,8 @@ int route_from_logits(const bigmac_layer* L, const Dims& m, const bigmac_weights
 }
 
 // Step F1 as a launch of its own: gate logits on x (a gate on x': descend first, logits from its stored value).
-int run_logits(const bigmac_layer* L, const Dims& m, const void* x, const bigmac_weights_t* W, Buffers& b, cudaStream_t st) {
+int run_logits(const bigmac_layer* L, const Dims& m, const void* x, const bigmac_weights_t* W, Buffers& b, cudaStream_t st,
+               Together* with = nullptr) {
     GemmArgs g;
     if (m.gate_low) {
         GemmArgs q;
@@ -248,7 +272,7 @@ int run_logits(const bigmac_layer* L, const Dims& m, const void* x, const bigmac
         g.A = x; g.lda = m.d; g.B = W->w_gate; g.ldb = m.d; g.K = m.d;
     }
     g.C = b.logits; g.ldc = m.E; g.M = m.T; g.N = m.E; g.out_f32 = true;
-    return gemm(L, G_LOGITS, g, st);
+    return with ? with->add(G_LOGITS, g, st) : gemm(L, G_LOGITS, g, st);
 }
 
 // The word of a caller's aux_loss table that has to be set to zero because the layer has no such loss.
@@ -534,13 +558,15 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
             BIGMAC_TRY(gemm(L, G_DESCEND, g, st));
         }
     } else {
-        BIGMAC_TRY(run_logits(L, m, x, W, b, st));                                // F1
+        Together both{L, !L->use_tc && !m.gate_low, st};
+        BIGMAC_TRY(run_logits(L, m, x, W, b, st, &both));                         // F1
         if (!m.cdac && !m.gate_low) {                                             // F4 descend: x' = x W'_down
             GemmArgs g;
             g.A = x; g.lda = m.d; g.B = W->w_down; g.ldb = m.d; g.C = b.x_lo; g.ldc = m.r;
             g.M = m.T; g.N = m.r; g.K = m.d;
-            BIGMAC_TRY(gemm(L, G_DESCEND, g, st));
+            BIGMAC_TRY(both.add(G_DESCEND, g, st));
         }
+        BIGMAC_TRY(both.flush());
     }
     // F2, F3 and F5 (dispatch at width r) - unless the dispatch is fused into its consumers: expert GEMM1's producer warp
     // then gathers the rows of x' itself (slot_of_prow names the token of every grouped row, -1 the zero padding rows) and
@@ -639,7 +665,10 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
     // do not depend on.  Everything that shares the fp32 workspace stays ordered.
     const bool overlap_on = switches().overlap != 0;
     // (not while per-stage events are recorded: a stage timed beside another stream's launches would not be its own time)
-    const bool overlap = overlap_on && L->side && !L->prof_on && !m.cdac;
+    // (nor on the FMA path, which puts what could overlap into one launch)
+    const bool batch = !L->use_tc && !m.cdac && !m.gate_low;
+    const bool overlap = overlap_on && L->side && !L->prof_on && !m.cdac && !batch;
+    Together together{L, batch, st};
     cudaStream_t sd = st;
     if (overlap) {
         sd = L->side;
@@ -652,7 +681,7 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         GemmArgs g;
         g.A = dy; g.lda = m.d; g.B = W->w_up; g.ldb = m.r; g.b_kmajor = false; g.C = b.dy_lo; g.ldc = m.r;
         g.M = m.T; g.N = m.r; g.K = m.d;
-        BIGMAC_TRY(gemm(L, G_DY_LO, g, st));
+        BIGMAC_TRY(together.add(G_DY_LO, g, st));
     }
     const bool fused = L->cfg.dtype == BIGMAC_BF16 && L->use_tc && L->tc_mask == ~0u;
     const int ldcat = m.ldcat;
@@ -666,9 +695,10 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
             Stage s(L, S_SPLITK_REDUCE, sd);
             BIGMAC_CUDA(launch_splitk_reduce(b.splitk_ws, g.split_k, m.d, m.r, G->dw_up, m.d, nullptr, 0, m.dtype, acc, sd));
         } else {
-            BIGMAC_TRY(gemm(L, G_DW_UP, g, sd));
+            BIGMAC_TRY(together.add(G_DW_UP, g, sd));
         }
     }
+    BIGMAC_TRY(together.flush());
     if (overlap) BIGMAC_CUDA(cudaEventRecord(L->fork_join[1], sd));          // dW_up done: the fp32 workspace is free again
     // du = p dy'[t], dp = <dy'[t], u>; then the softmax-over-k backward
     { Stage s(L, S_COMBINE_BWD, st); BIGMAC_CUDA(launch_combine_bwd(b.dy_lo, b.u, b.du, b.dp, b.tb, m.k, m.r, m.dtype, m.P, st)); }
@@ -725,14 +755,14 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         g.A = b.du; g.lda = m.r; g.a_kmajor = false; g.B = b.a; g.ldb = m.h; g.b_kmajor = false;
         g.C = G->dw2; g.ldc = m.h; g.c_stride = (int64_t)m.r * m.h; g.M = m.r; g.N = m.h; g.K = (int)m.P;
         g.group = GROUP_K; g.num_experts = m.E; g.poffsets = b.tb.poffsets; g.accumulate = acc;
-        BIGMAC_TRY(expert_weight_grad(L, G_DW2, g, b.splitk_ws, st));
+        BIGMAC_TRY(batch ? together.add(G_DW2, g, st) : expert_weight_grad(L, G_DW2, g, b.splitk_ws, st));
     }
     {   // dxg = dz W1_e
         GemmArgs g;
         g.A = dz; g.lda = m.h; g.B = W->w1; g.ldb = m.r; g.b_kmajor = false; g.b_stride = (int64_t)m.h * m.r;
         g.C = b.dxg; g.ldc = m.r; g.M = (int)m.P; g.N = m.r; g.K = m.h;
         g.group = GROUP_M; g.num_experts = m.E; g.tile_expert = b.tb.tile_expert; g.n_tiles = b.tb.n_tiles; g.poffsets = b.tb.poffsets;
-        BIGMAC_TRY(gemm(L, G_DXG, g, st));
+        BIGMAC_TRY(together.add(G_DXG, g, st));
     }
     if (overlap) {   // dx'[t] = sum_j dxg[row of slot (t,j)]: an HBM-bound gather beside the tensor-bound dW1
         BIGMAC_CUDA(cudaEventRecord(L->fork_join[4], st));
@@ -747,8 +777,9 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
             g.gather_rows = b.tb.slot_of_prow;
             g.gather_div = m.k;
         }
-        BIGMAC_TRY(expert_weight_grad(L, G_DW1, g, b.splitk_ws, st));
+        BIGMAC_TRY(batch ? together.add(G_DW1, g, st) : expert_weight_grad(L, G_DW1, g, b.splitk_ws, st));
     }
+    BIGMAC_TRY(together.flush());
     if (m.cdac) {
         // Eq. 3: dx = sum_j dxg[row of slot (t,j)] + dl W_gate; dW_gate = dl^T x
         { Stage s(L, S_DXLO_GATHER, st); BIGMAC_CUDA(launch_combine(b.dxg, dx, nullptr, b.tb.prow_of_slot, m.T, m.k, m.d, m.dtype, st, 0, m.cap != kNoCapacity)); }
@@ -860,30 +891,39 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
             BIGMAC_CUDA(cudaStreamWaitEvent(st, L->fork_join[7], 0));
         }
     } else {
-        {   // dx = dx' W_down
+        if (batch) {   // dx = [dx' | dl] [W_down ; W_gate]: one contraction over r + E
             GemmArgs g;
-            g.A = b.dx_lo; g.lda = ldcat; g.B = W->w_down; g.ldb = m.d; g.b_kmajor = false; g.C = dx; g.ldc = m.d;
-            g.M = m.T; g.N = m.d; g.K = m.r;
-            BIGMAC_TRY(gemm(L, G_DX, g, st));
-        }
-        {   // dx += dl W_gate
-            GemmArgs g;
-            g.A = b.dlogits; g.lda = ldcat; g.B = W->w_gate; g.ldb = m.d; g.b_kmajor = false; g.C = dx; g.ldc = m.d;
-            g.M = m.T; g.N = m.d; g.K = m.E; g.accumulate = true;
-            BIGMAC_TRY(gemm(L, G_DX_GATE, g, st));
+            g.A = b.dcat; g.lda = ldcat; g.B = W->w_down; g.ldb = m.d; g.b_kmajor = false;
+            g.B2 = W->w_gate; g.ldb2 = m.d; g.b2_first_k = m.r;
+            g.C = dx; g.ldc = m.d; g.M = m.T; g.N = m.d; g.K = m.r + m.E;
+            BIGMAC_TRY(together.add(G_DX, g, st));
+        } else {
+            {   // dx = dx' W_down
+                GemmArgs g;
+                g.A = b.dx_lo; g.lda = ldcat; g.B = W->w_down; g.ldb = m.d; g.b_kmajor = false; g.C = dx; g.ldc = m.d;
+                g.M = m.T; g.N = m.d; g.K = m.r;
+                BIGMAC_TRY(gemm(L, G_DX, g, st));
+            }
+            {   // dx += dl W_gate
+                GemmArgs g;
+                g.A = b.dlogits; g.lda = ldcat; g.B = W->w_gate; g.ldb = m.d; g.b_kmajor = false; g.C = dx; g.ldc = m.d;
+                g.M = m.T; g.N = m.d; g.K = m.E; g.accumulate = true;
+                BIGMAC_TRY(gemm(L, G_DX_GATE, g, st));
+            }
         }
         if (G->dw_down) {   // dW_down[c',c] = sum_t dx'[t,c'] x[t,c]
             GemmArgs g;
             g.A = b.dx_lo; g.lda = ldcat; g.a_kmajor = false; g.B = x; g.ldb = m.d; g.b_kmajor = false;
             g.C = G->dw_down; g.ldc = m.d; g.M = m.r; g.N = m.d; g.K = m.T; g.accumulate = acc;
-            BIGMAC_TRY(gemm(L, G_DW_DOWN, g, st));
+            BIGMAC_TRY(together.add(G_DW_DOWN, g, st));
         }
         if (G->dw_gate) {   // dW_gate[e,c] = sum_t dl[t,e] x[t,c]
             GemmArgs g;
             g.A = b.dlogits; g.lda = ldcat; g.a_kmajor = false; g.B = x; g.ldb = m.d; g.b_kmajor = false;
             g.C = G->dw_gate; g.ldc = m.d; g.M = m.E; g.N = m.d; g.K = m.T; g.accumulate = acc;
-            BIGMAC_TRY(gemm(L, G_DW_GATE, g, st));
+            BIGMAC_TRY(together.add(G_DW_GATE, g, st));
         }
+        BIGMAC_TRY(together.flush());
     }
     if (!colsum_done && G->db_gate) {
         Stage s(L, S_COLSUM, st, 2);
