@@ -170,8 +170,9 @@ typedef struct {
     float *aux_loss;        /* [1]   */
 } bigmac_routing_t;
 
-/* Validate the configuration and create a handle on the current CUDA device.  Allocates one small
- * device status word (no other device memory is owned by the handle), one stream and ten events.
+/* Validate the configuration and create a handle on the current CUDA device.  Allocates a few
+ * device words, with them (BF16 configurations whose small batches run in one kernel) up to 8 MB of words in which that
+ * kernel's blocks hand values to each other (1.1 MB at d 2048, r 256, h 1024, k 8), one stream and ten events.
  * Errors: INVALID_ARG (null pointers, non-positive sizes, k > E, unknown enums, a negative or non-finite
  * capacity_factor or aux_loss_coef), UNSUPPORTED (BF16
  * with d, r or h not a multiple of 64; E > 1024), CUDA. */

@@ -1,20 +1,25 @@
 // Small-batch (decode-shaped) inference forward of the BigMac layer in ONE cooperative kernel.
 //
-// For a handful of tokens the layer is a chain of matrix-vector products that is bound by streaming the touched
-// weights once (W'_down, W_gate, the selected experts' W1/W2, W'_up) and by launch latency; ten separate launches
-// cost far more than the arithmetic.  All SMs walk five phases with three grid-wide barriers (after A, C and D):
-//   A  [x' | logits] = x [W'_down ; W_gate]^T           a CTA owns a few weight rows, its sixteen warps a sixteenth of
-//                                                        the contraction each, tokens four at a time
-//   B  top-k + softmax gate values                       one warp per token, repeated by every CTA into its own
-//                                                        shared memory (a few KB of logits from L2: cheaper than a barrier)
-//   C  a = sigma(W1_e x')  for every routed slot          sixteen weight rows per warp task
-//   D  u = W2_e a                                         four weight rows per warp task
-//   E  y' = sum_j p_j u_j ;  y = W'_up y'                 two weight rows per warp task
-// Weights are read as 16-byte vectors, up to sixteen of them in flight per lane before the first is used (the
-// kernel is bound by latency chains and by instruction fetch, not by arithmetic); products accumulate in fp32,
-// intermediates stay fp32 in scratch.
-// The grid barrier is a bounded spin on a global counter (cooperative launch guarantees co-residency); if the
-// bound is ever hit the kernel records BIGMAC_ERR_TIMEOUT in the status word and runs on, so it always ends.
+// For a handful of tokens the layer is a chain of matrix-vector products that is bound by streaming the touched weights
+// once (W'_down, W_gate, the selected experts' W1/W2, W'_up) and by latency; separate launches cost far more than the
+// arithmetic.  All SMs walk five phases:
+//   A  [x' | logits] = x [W'_down ; W_gate]^T   a CTA owns a few weight rows, a warp takes 32 16-byte pieces of one
+//   B  top-k + softmax gate values               by rank counting, repeated by every CTA in its own shared memory
+//   C  a = sigma(W1_e x') per routed slot         a CTA owns a range of hidden units, a warp takes a few rows
+//   D  y' = sum_j p_j W2_{e_j} a_j                a CTA owns some columns of one token, a warp takes (column, slot) rows
+//   E  y = W'_up y'                               a CTA owns a few rows
+// Values that cross from one CTA to another (x', logits, a, y') travel as 8-byte words (fp32 value, tag of this launch):
+// the consumer polls the very words it needs until their tags match, so a hand-over is one store and one load through
+// L2.  With a grid-wide barrier (arrive, spin, then load) each of the three hand-overs took 2.2-2.7 us, 7 of the 15 us of
+// one token.  The words live in memory of the handle that is zero at first and written by this kernel only, and the tag
+// counts the handle's launches on the device (a captured launch can be replayed), so a stale word never matches.
+// Code is executed once or a few times per launch, and a first execution waits for instruction fetch: phases are small
+// loops, ranges and divisors come ready from the host.  (Four extra warps that ran through the later phases' code
+// beforehand, without effect, gained nothing: what is left is the latency of the hand-overs and of the weights.)
+// Weights do not depend on the hand-overs: W'_up rows are fetched into shared memory at the start, the first rows of A
+// before x is staged, the first W2 rows before the wait for a; C fetches a step's rows ahead.
+// Products accumulate in fp32, intermediates stay fp32.  The cooperative launch guarantees that all CTAs run at the same
+// time; every wait is bounded (status word), so the kernel always ends.
 #include "internal.h"
 #include "act.cuh"
 
@@ -23,22 +28,52 @@ namespace bigmac {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kDecodeThreads = 512;
-constexpr int kDecodeMaxExperts = 256;      // top-k keeps a token's logits in registers: 8 per lane
-constexpr int kDecodeMaxSlots = 2048;        // T k: every CTA keeps all slots' expert ids and gate values
+constexpr int kDecodeThreads = 512, kWarps = kDecodeThreads / 32;
 constexpr int kDecodeMaxTokens = 16;
+constexpr int kDecodeMaxExperts = 256;
+constexpr int kDecodeMaxHidden = 16384;     // k h: the hidden activations of one token are staged in shared memory (64 KB)
+constexpr int kDecodeMaxUpBytes = 32768;    // W'_up rows of a CTA kept in shared memory
+constexpr size_t kDecodeMaxWords = 1u << 20; // hand-over words (8 MB) a handle keeps at most
+
+// n / d for 0 <= n < 2^31 by a multiplication (d >= 1; round-up method with a 31-bit dividend).
+struct Divisor {
+    uint32_t d, m, s;
+    Divisor() = default;
+    explicit Divisor(int v) : d((uint32_t)v), m(0), s(0) {
+        while (s < 31 && (1u << s) < d) ++s;
+        m = (uint32_t)(((1ull << (31 + s)) + d - 1) / d);
+    }
+    __device__ __forceinline__ int div(int n) const { return (int)(uint32_t)(((unsigned long long)(uint32_t)n * m) >> (31 + s)); }
+};
+// Share b of `total` things dealt out over the grid in contiguous ranges.
+struct Split {
+    int per, rest;
+    Split() = default;
+    Split(int total, int grid) : per(total / grid), rest(total % grid) {}
+    __device__ __forceinline__ int first(int b) const { return b * per + min(b, rest); }
+};
 
 struct DecodeArgs {
     const __nv_bfloat16 *x, *w_gate, *w_down, *w1, *w2, *w_up;
     const float* b_gate;
     __nv_bfloat16* y;
-    float *logits, *x_lo, *a, *u;      // scratch: [T,E], [T,r], [T*k,h], [T*k,r]
+    unsigned long long *x_lo, *logits, *a, *y_lo;      // hand-over words: [T,r], [T,LE], [T*k,h], [T,r]
     int32_t* topk_idx;
     float* topk_w;
-    unsigned* barrier;                 // zero before the launch; the kernel leaves it zero
+    unsigned* epoch;                   // [grid] launches of this handle so far, a word of its own for every CTA
     int* status;
     int T, d, r, h, E, k, act;
+    int copies, copy_words;            // x', logits and y' are written `copies` times, copy_words apart; CTA b reads copy b % copies
+    int LE;                            // row length of the logits' words: E up to a multiple of four
+    Split rows_a, groups_c, rows_e;    // who does what in phases A, C (groups of rows of all slots) and E
+    Split cols_d;                      // phase D: columns of a token over its CTAs
+    int ctas_d;                        // phase D: CTAs per token
+    Divisor by_parts, by_pieces, by_k, by_slot, by_ctas, by_lanes;   // parts of a row in A; pieces of x; k; groups of a slot in C; ctas_d; 32-expert groups
+    // shared memory, offsets in floats: region (x; then x'; then a of a token; then y'), W'_up rows, logits, slots, sums
+    int up_rows, off_up, off_log, off_idx, off_val, off_w, off_sums;
 };
+extern __shared__ float4 decode_smem_raw[];
+__device__ __forceinline__ float* smem_at(int off) { return reinterpret_cast<float*>(decode_smem_raw) + off; }
 
 __device__ __forceinline__ void unpack8(const uint4& v, float* f) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -49,74 +84,69 @@ __device__ __forceinline__ void unpack8(const uint4& v, float* f) {
     }
 }
 
-// All CTAs of the (cooperative) grid meet here; `phase` counts the barriers passed so far.  One thread per CTA arrives
-// with a release at GPU scope (the block barrier before it makes the CTA's writes part of what is released) and
-// spins with acquire loads; the block barrier after it hands what was acquired to the other threads.
-__device__ __forceinline__ void grid_barrier(unsigned* counter, unsigned phase, int* status) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
-        const unsigned target = (phase + 1) * gridDim.x;
-        unsigned seen = 0;
-        for (uint32_t i = 0; i < (1u << 24); ++i) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
-            if (seen >= target) break;
-        }
-        if (seen < target) atomicExch(status, 1);
-    }
-    __syncthreads();
+// ---- hand-over words.  Value and tag share one 64-bit access, so neither needs an ordering with anything else.
+__device__ __forceinline__ void put_word(unsigned long long* p, float v, uint32_t tag) {
+    const unsigned long long w = ((unsigned long long)tag << 32) | __float_as_uint(v);
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
 }
-
-// Partial dot products of ROWS consecutive weight rows (bf16, row-major, `ld` apart) over their 16-byte pieces
-// [piece0, piece0 + npieces) with the fp32 vectors vp[0 .. nv); lanes stride over the pieces, U pieces per row and
-// round: the ROWS * U loads of a round are issued before any of them is used.  With SPLIT the vectors are in the
-// two-plane layout of split_index (elements 8c .. 8c+3 of a vector at float4 number c, elements 8c+4 .. 8c+7 at
-// float4 number `plane` + c): neighbouring lanes then read neighbouring 16 bytes of shared memory, where the natural
-// layout costs a two-way bank conflict on every load.  out[row * NV + t] is this lane's share; the caller sums
-// over the lanes (warp_reduce_scatter).
-template <int ROWS, int NV, int U, bool SPLIT>
-__device__ __forceinline__ void rows_dot(const __nv_bfloat16* w, int64_t ld, int piece0, int npieces, const float* const (&vp)[NV],
-                                         int plane, int nv, float (&out)[ROWS * NV]) {
-    const int lane = threadIdx.x & 31, end = piece0 + npieces;
+__device__ __forceinline__ void put_copies(const DecodeArgs& a, unsigned long long* p, float v, uint32_t tag) {
+#pragma unroll 1
+    for (int i = 0; i < a.copies; ++i) put_word(p + i * a.copy_words, v, tag);
+}
+// Thread `tid` of `threads` waits for its share of n words (n even, 16-byte aligned) and puts the values into dst, in the
+// words' own order.  A thread asks for four pairs at a time, and only for its own: a pair that everybody reads holds all of
+// them up.
+__device__ __noinline__ void get_words(float* dst, const unsigned long long* words, int n, int tid, int threads, uint32_t tag, int* status) {
+    constexpr int U = 4;
+#pragma unroll 1
+    for (int i0 = 2 * tid; i0 < n; i0 += 2 * U * threads) {
+        unsigned long long w[2 * U];
+        bool ok = false;
+#pragma unroll 1
+        for (uint32_t spin = 0; spin < (1u << 20) && !ok; ++spin) {
+            ok = true;
 #pragma unroll
-    for (int i = 0; i < ROWS * NV; ++i) out[i] = 0.0f;
-    for (int c0 = piece0 + lane; c0 < end; c0 += 32 * U) {
-        uint4 wv[U][ROWS];
+            for (int u = 0; u < U; ++u)
+                if (i0 + 2 * u * threads < n)
+                    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w[2 * u]), "=l"(w[2 * u + 1]) : "l"(words + i0 + 2 * u * threads) : "memory");
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int c = c0 + 32 * u;
-#pragma unroll
-            for (int i = 0; i < ROWS; ++i)
-                wv[u][i] = c < end ? __ldg(reinterpret_cast<const uint4*>(w + i * ld) + c) : make_uint4(0u, 0u, 0u, 0u);
+            for (int u = 0; u < U; ++u)
+                if (i0 + 2 * u * threads < n) ok = ok && (uint32_t)(w[2 * u] >> 32) == tag && (uint32_t)(w[2 * u + 1] >> 32) == tag;
         }
+        if (!ok) atomicExch(status, 1);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int c = c0 + 32 * u;
-            if (c < end) {
-#pragma unroll
-                for (int t = 0; t < NV; ++t) {
-                    if (t < nv) {
-                        const float4* vt = reinterpret_cast<const float4*>(vp[t]);
-                        const float4 v0 = SPLIT ? vt[c] : vt[2 * c];
-                        const float4 v1 = SPLIT ? vt[plane + c] : vt[2 * c + 1];
-#pragma unroll
-                        for (int i = 0; i < ROWS; ++i) {
-                            float wf[8];
-                            unpack8(wv[u][i], wf);
-                            float acc = out[i * NV + t];
-                            acc = fmaf(wf[0], v0.x, acc); acc = fmaf(wf[1], v0.y, acc); acc = fmaf(wf[2], v0.z, acc); acc = fmaf(wf[3], v0.w, acc);
-                            acc = fmaf(wf[4], v1.x, acc); acc = fmaf(wf[5], v1.y, acc); acc = fmaf(wf[6], v1.z, acc); acc = fmaf(wf[7], v1.w, acc);
-                            out[i * NV + t] = acc;
-                        }
-                    }
-                }
-            }
-        }
+        for (int u = 0; u < U; ++u)
+            if (i0 + 2 * u * threads < n)
+                *reinterpret_cast<float2*>(dst + i0 + 2 * u * threads) = make_float2(__uint_as_float((uint32_t)w[2 * u]), __uint_as_float((uint32_t)w[2 * u + 1]));
     }
 }
 
-// Where element e of a staged vector of n elements sits in the two-plane layout (see rows_dot).
+// Where element e of a staged vector of n elements (a multiple of 8) sits: elements 8c .. 8c+3 at float4 number c,
+// elements 8c+4 .. 8c+7 at float4 number n / 8 + c.  Neighbouring lanes, which hold neighbouring 16-byte pieces of a
+// bf16 row, then read neighbouring 16 bytes of shared memory, where the natural layout has a two-way bank conflict.
 __device__ __forceinline__ int split_index(int e, int n) { return ((e >> 2) & 1) * (n >> 1) + ((e >> 3) << 2) + (e & 3); }
+
+// Dot product of one 16-byte piece of a bf16 row (unpacked to four pairs) with elements 8c .. 8c+7 of a vector staged as
+// above (v0, v1), added to a pair of partial sums: packed multiply-adds, two elements an instruction.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) { f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { f32x2 d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d; }
+__device__ __forceinline__ float sum2(f32x2 v) { float a, b; asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); return a + b; }
+struct Piece {
+    f32x2 w[4];
+    __device__ __forceinline__ explicit Piece(const uint4& v) {
+        float f[8];
+        unpack8(v, f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = pack2(f[2 * i], f[2 * i + 1]);
+    }
+};
+__device__ __forceinline__ f32x2 dot8(const Piece& q, const float4& v0, const float4& v1, f32x2 acc) {
+    acc = fma2(q.w[0], pack2(v0.x, v0.y), acc);
+    acc = fma2(q.w[1], pack2(v0.z, v0.w), acc);
+    acc = fma2(q.w[2], pack2(v1.x, v1.y), acc);
+    return fma2(q.w[3], pack2(v1.z, v1.w), acc);
+}
 
 // Sums each of the N values (a power of two, at most 32) over the warp's lanes with N - 1 + log2(32 / N) shuffles
 // instead of 5 N: every halving step a lane hands half of its values to its partner and keeps the sums of the
@@ -141,269 +171,393 @@ __device__ __forceinline__ float warp_reduce_scatter(float* v) {
     return total;
 }
 
-// The kernel runs every piece of its code once or a few times per launch, so code size is time (instruction fetch
-// was the largest stall with one fully unrolled copy per token count): tokens are walked four at a time by a loop
-// around one small copy of each phase, and the weights of a task are read again for each group of four (from L1).
-constexpr int kTokenGroup = 4;
-
-// A: rows of [W'_down ; W_gate] against the tokens staged in `xs` as fp32 [T,d] (two-plane layout).  CTA b owns rows
-// b, b + grid, ...; a warp takes one sixteenth of the contraction of four of them at a time (x leaves shared memory
-// once per four rows), the sixteen pieces meet in shared memory and are added in order.
-__device__ __forceinline__ void phase_a(const DecodeArgs& p, const float* xs, float* part_sums) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kWarps = kDecodeThreads / 32, ROWS = 4;
-    const int R = p.r + p.E, G = gridDim.x, per_cta = (R + G - 1) / G;
-    const int pieces = p.d / 8, per_part = (pieces + kWarps - 1) / kWarps;
-    const int piece0 = min(pieces, warp * per_part), end = min(pieces, piece0 + per_part);
-    for (int first = 0; first < per_cta; first += ROWS) {
-        // rows j0, j0 + G, ...: W'_down and W_gate are two arrays, so the four rows are addressed one by one; a row
-        // past the end is replaced by a valid one and its result dropped
-        const int j0 = blockIdx.x + G * first;
-        const uint4* rows[ROWS];
+// A: the rows of [W'_down ; W_gate] of this CTA (the gate reads x, not x'); a warp takes 32 pieces of one row at a time, the
+// parts of a row meet in shared memory and are added in order.  TG: tokens whose sums a warp keeps at a time.
+template <int TG>
+__device__ __forceinline__ void phase_a(const DecodeArgs& p, uint32_t tag) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x;
+    float* xs = smem_at(0);
+    float* sums = smem_at(p.off_sums);
+    const int pieces = p.d / 8, parts = (int)p.by_parts.d, r0 = p.rows_a.first(b), nrows = p.rows_a.first(b + 1) - r0, tasks = nrows * parts;
+    auto fetch = [&](int i) {
+        const int row = p.by_parts.div(i), c = (i - row * parts) * 32 + lane, j = r0 + row;
+        const uint4* w = reinterpret_cast<const uint4*>(j < p.r ? p.w_down : p.w_gate) + (int64_t)(j < p.r ? j : j - p.r) * pieces;
+        return c < pieces ? __ldg(w + c) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    uint4 wv = make_uint4(0u, 0u, 0u, 0u);
+    if (warp < tasks) wv = fetch(warp);                      // on its way before x
+    constexpr int XU = TG == 1 ? 1 : 4;
+    const int xn = p.T * pieces;
+#pragma unroll 1
+    for (int i0 = tid; i0 < xn; i0 += XU * kDecodeThreads) {
+        uint4 xv[XU];
 #pragma unroll
-        for (int i = 0; i < ROWS; ++i) {
-            int j = j0 + G * i;
-            if (first + i >= per_cta || j >= R) j = 0;
-            rows[i] = reinterpret_cast<const uint4*>(j < p.r ? p.w_down + (int64_t)j * p.d : p.w_gate + (int64_t)(j - p.r) * p.d);
-        }
-        bool first_round = true;                             // at least one round, so that every slot below is written
-        for (int cb = piece0; cb < end || first_round; cb += 32, first_round = false) {
-            const int c = cb + lane;
-            uint4 wv[ROWS];
+        for (int u = 0; u < XU; ++u)
+            if (i0 + u * kDecodeThreads < xn) xv[u] = __ldg(reinterpret_cast<const uint4*>(p.x) + i0 + u * kDecodeThreads);
 #pragma unroll
-            for (int i = 0; i < ROWS; ++i) wv[i] = c < end ? __ldg(rows[i] + c) : make_uint4(0u, 0u, 0u, 0u);
-            for (int t0 = 0; t0 < p.T; t0 += kTokenGroup) {
-                float acc[ROWS * kTokenGroup];
-#pragma unroll
-                for (int i = 0; i < ROWS * kTokenGroup; ++i) acc[i] = 0.0f;
-                if (c < end) {
-#pragma unroll
-                    for (int t = 0; t < kTokenGroup; ++t) {
-                        if (t0 + t < p.T) {
-                            const float4* vt = reinterpret_cast<const float4*>(xs + (int64_t)(t0 + t) * p.d);
-                            const float4 v0 = vt[c], v1 = vt[pieces + c];
-#pragma unroll
-                            for (int i = 0; i < ROWS; ++i) {
-                                float wf[8];
-                                unpack8(wv[i], wf);
-                                float a = 0.0f;
-                                a = fmaf(wf[0], v0.x, a); a = fmaf(wf[1], v0.y, a); a = fmaf(wf[2], v0.z, a); a = fmaf(wf[3], v0.w, a);
-                                a = fmaf(wf[4], v1.x, a); a = fmaf(wf[5], v1.y, a); a = fmaf(wf[6], v1.z, a); a = fmaf(wf[7], v1.w, a);
-                                acc[i * kTokenGroup + t] = a;
-                            }
-                        }
-                    }
-                }
-                const float mine = warp_reduce_scatter<ROWS * kTokenGroup>(acc);   // (row, token) = lane / 2 / 4, % 4
-                if (!(lane & 1)) {
-                    float* slot = part_sums + ((lane >> 3) * kWarps + warp) * 16 + t0 + ((lane >> 1) & 3);
-                    *slot = first_round ? mine : *slot + mine;
-                }
+        for (int u = 0; u < XU; ++u)
+            if (i0 + u * kDecodeThreads < xn) {
+                float f[8];
+                unpack8(xv[u], f);
+                const int t = p.by_pieces.div(i0 + u * kDecodeThreads), q = i0 + u * kDecodeThreads - t * pieces;
+                float4* vt = reinterpret_cast<float4*>(xs + t * p.d);
+                vt[q] = make_float4(f[0], f[1], f[2], f[3]);
+                vt[pieces + q] = make_float4(f[4], f[5], f[6], f[7]);
             }
-        }
-        __syncthreads();
-        if (threadIdx.x < ROWS * 16) {
-            const int i = threadIdx.x / 16, t = threadIdx.x % 16, j = j0 + G * i;
-            if (first + i < per_cta && j < R && t < p.T) {
-                float sum = 0.0f;
-                for (int q = 0; q < kWarps; ++q) sum += part_sums[(i * kWarps + q) * 16 + t];
-                if (j < p.r) p.x_lo[t * p.r + j] = sum;
-                else p.logits[t * p.E + (j - p.r)] = sum + (p.b_gate ? p.b_gate[j - p.r] : 0.0f);
-            }
-        }
-        __syncthreads();
     }
-}
-
-// E: two rows of W'_up per warp task against y' [T,r] staged in `ys` (two-plane layout).
-__device__ __forceinline__ void phase_e(const DecodeArgs& p, const float* ys, int gwarp, int nwarps) {
-    constexpr int ROWS = 2;
-    const int lane = threadIdx.x & 31;
-    for (int task = gwarp; task < p.d / ROWS; task += nwarps) {
-        const int c0 = task * ROWS;
-        for (int t0 = 0; t0 < p.T; t0 += kTokenGroup) {
-            float acc[ROWS * kTokenGroup];
-            const float* vp[kTokenGroup];
-#pragma unroll
-            for (int t = 0; t < kTokenGroup; ++t) vp[t] = ys + (int64_t)min(t0 + t, p.T - 1) * p.r;
-            rows_dot<ROWS, kTokenGroup, 2, true>(p.w_up + (int64_t)c0 * p.r, p.r, 0, p.r / 8, vp, p.r / 8,
-                                                min(kTokenGroup, p.T - t0), acc);
-            const float v = warp_reduce_scatter<ROWS * kTokenGroup>(acc);     // (row, token) = lane / 4 / 4, % 4
-            const int t = t0 + ((lane >> 2) & 3);
-            if (!(lane & 3) && t < p.T) p.y[(int64_t)t * p.d + c0 + (lane >> 4)] = __float2bfloat16(v);
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kDecodeThreads, 1) decode_forward_kernel(const DecodeArgs p) {
-    extern __shared__ float smem_f[];                       // phase A: x as fp32 [T,d]; C: x' [T,r]; E: y' [T,r]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int warps_per_cta = kDecodeThreads / 32;
-    const int gwarp = warp * gridDim.x + blockIdx.x, nwarps = gridDim.x * warps_per_cta;   // neighbouring tasks on different SMs
-    const int T = p.T, N = p.T * p.k;
-
-    int* s_idx = reinterpret_cast<int*>(smem_f + T * max(p.d, p.r));     // [T k] expert of every slot
-    float* s_w = reinterpret_cast<float*>(s_idx + N);                      // [T k] its gate value
-    float* part_sums = s_w + N;                                            // [4 rows][16 warps][16 tokens] phase A's pieces
-
-    // ---- A: descend + gate logits (the gate reads x, not x')
-    // every CTA stages the same bytes: each starts somewhere else in them, or all SMs ask the same L2 lines at once
-    for (int i0 = threadIdx.x; i0 < T * p.d / 8; i0 += kDecodeThreads) {  // d is a multiple of 8, x 16-byte aligned
-        const int i = (i0 + blockIdx.x * 224) % (T * p.d / 8);
-        float f[8];
-        unpack8(__ldg(reinterpret_cast<const uint4*>(p.x) + i), f);
-        const int t = i / (p.d / 8), c = i % (p.d / 8);
-        float4* vt = reinterpret_cast<float4*>(smem_f + (int64_t)t * p.d);
-        vt[c] = make_float4(f[0], f[1], f[2], f[3]);
-        vt[p.d / 8 + c] = make_float4(f[4], f[5], f[6], f[7]);
+    if (p.up_rows > 0) {                                     // W'_up for phase E
+        const int up0 = p.rows_e.first(b), n = (p.rows_e.first(b + 1) - up0) * (p.r / 8);
+        const uint4* from = reinterpret_cast<const uint4*>(p.w_up) + (int64_t)up0 * (p.r / 8);
+        const uint32_t to = (uint32_t)__cvta_generic_to_shared(smem_at(p.off_up));
+#pragma unroll 1
+        for (int i = tid; i < n; i += kDecodeThreads)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + i * 16), "l"(from + i) : "memory");
     }
     __syncthreads();
-    phase_a(p, smem_f, part_sums);
-    grid_barrier(p.barrier, 0, p.status);
-
-    // ---- B: top-k by (logit descending, expert id ascending), softmax over the k kept logits.  Every CTA does all
-    // tokens for itself (warp t: token t); CTA 0 also writes the tables the caller may ask for.
-    if (warp < T) {
-        const int t = warp;
-        const float* l = p.logits + (int64_t)t * p.E;
-        float mine[kDecodeMaxExperts / 32];                  // logits of experts lane, lane + 32, ...
+#pragma unroll 1
+    for (int i = warp; i < tasks; i += kWarps) {
+        const Piece q(wv);
+        const int c = min((i - p.by_parts.div(i) * parts) * 32 + lane, pieces - 1);   // lanes past the end hold zero weights
+        if (i + kWarps < tasks) wv = fetch(i + kWarps);
+#pragma unroll 1
+        for (int t0 = 0; t0 < p.T; t0 += TG) {
+            float acc[TG];
 #pragma unroll
-        for (int i = 0; i < kDecodeMaxExperts / 32; ++i) {
-            const int e = lane + 32 * i;
-            const float v = e < p.E ? __ldcg(l + e) : 0.0f;
-            mine[i] = v == v ? v : -INFINITY;                // NaN is ordered as -inf
-        }
-        uint32_t taken = 0;                                  // bit i: expert lane + 32 i already chosen
-        float top = 0.0f, part = 0.0f;
-        for (int j0 = 0; j0 < p.k; j0 += 32) {               // winner j stays with lane j - j0 until the stores
-            float my_ex = 0.0f;
-            int my_e = 0;
-            for (int j = j0; j < min(p.k, j0 + 32); ++j) {
-                float best = -INFINITY;
-                int best_e = 0x7fffffff;                     // "no candidate yet"; k <= E, so every round ends with a real id
-#pragma unroll
-                for (int i = 0; i < kDecodeMaxExperts / 32; ++i) {
-                    const int e = lane + 32 * i;
-                    if (e < p.E && !((taken >> i) & 1u) && (best_e == 0x7fffffff || mine[i] > best)) { best = mine[i]; best_e = e; }
-                }
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) {
-                    const float ov = __shfl_xor_sync(kFull, best, off);
-                    const int oe = __shfl_xor_sync(kFull, best_e, off);
-                    if (ov > best || (ov == best && oe < best_e)) { best = ov; best_e = oe; }
-                }
-                if (best_e != 0x7fffffff && (best_e & 31) == lane) taken |= 1u << (best_e >> 5);
-                if (j == 0) top = best;
-                const float ex = top == -INFINITY ? 1.0f : expf(best - top);   // only -inf logits kept: 1/k each
-                part += ex;
-                if (lane == j - j0) { my_ex = ex; my_e = best_e; }
+            for (int t = 0; t < TG; ++t) {
+                const float4* vt = reinterpret_cast<const float4*>(xs + min(t0 + t, p.T - 1) * p.d);
+                acc[t] = sum2(dot8(q, vt[c], vt[pieces + c], 0ull));
             }
-            if (j0 + lane < p.k) { s_idx[t * p.k + j0 + lane] = my_e; s_w[t * p.k + j0 + lane] = my_ex; }
+            const float sum = warp_reduce_scatter<TG>(acc);          // token t0 + lane / (32 / TG)
+            if (!(lane & (32 / TG - 1))) sums[i * 16 + t0 + lane / (32 / TG)] = sum;   // tokens past T: slots of their own
         }
-        __syncwarp();
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = tid; i < nrows * 16; i += kDecodeThreads) {
+        const int t = i & 15, j = r0 + (i >> 4), e = j - p.r;
+        if (t >= p.T) continue;
+        float sum = 0.0f;
+#pragma unroll 4
+        for (int q = 0; q < parts; ++q) sum += sums[((i >> 4) * parts + q) * 16 + t];
+        unsigned long long* to = p.x_lo + t * p.r + split_index(j, p.r);
+        if (e >= 0) {
+            if (p.b_gate) sum += p.b_gate[e];
+            sum = sum == sum ? sum : -INFINITY;              // NaN is ordered as -inf
+            to = p.logits + t * p.LE + e;
+            if (e == p.E - 1)                                // words that fill the row up: never counted before anything
+#pragma unroll 1
+                for (int q = p.E; q < p.LE; ++q) put_copies(p, p.logits + t * p.LE + q, __int_as_float(0x7fffffff), tag);
+        }
+        put_copies(p, to, sum, tag);
+    }
+}
+
+// B: top-k by (logit descending, expert id ascending), softmax over the k kept logits; x' takes x's place.
+__device__ __forceinline__ void phase_b(const DecodeArgs& p, uint32_t tag) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int half = kDecodeThreads / 2;
+    const bool logits = tid < half;
+    float* s_log = smem_at(p.off_log);
+    int* s_idx = reinterpret_cast<int*>(smem_at(p.off_idx));
+    float* s_val = smem_at(p.off_val);
+    float* s_w = smem_at(p.off_w);
+    __syncthreads();
+    if (tid < p.T * p.k) { s_idx[tid] = 0; s_val[tid] = 0.0f; }          // (kept if a wait gave up)
+    get_words(smem_at(logits ? p.off_log : 0), (logits ? p.logits : p.x_lo) + blockIdx.x % p.copies * p.copy_words, logits ? p.T * p.LE : p.T * p.r, tid & (half - 1), half, tag, p.status);
+    __syncthreads();
+    // an expert's place in its token's order is the number of experts before it: no rounds of arg-max
+    const int per_token = (int)p.by_lanes.d;
+#pragma unroll 1
+    for (int i = warp; i < p.T * per_token; i += kWarps) {
+        const int t = p.by_lanes.div(i), e = (i - t * per_token) * 32 + lane;
+        const float4* l = reinterpret_cast<const float4*>(s_log + t * p.LE);
+        const float v = s_log[t * p.LE + min(e, p.E - 1)];
+        int before = 0;
+#pragma unroll 2
+        for (int q = 0; q < p.LE; q += 4) {
+            const float4 o = l[q >> 2];
+            before += (o.x > v || (o.x == v && q < e)) ? 1 : 0;
+            before += (o.y > v || (o.y == v && q + 1 < e)) ? 1 : 0;
+            before += (o.z > v || (o.z == v && q + 2 < e)) ? 1 : 0;
+            before += (o.w > v || (o.w == v && q + 3 < e)) ? 1 : 0;
+        }
+        if (e < p.E && before < p.k) { s_idx[t * p.k + before] = e; s_val[t * p.k + before] = v; }
+    }
+    __syncthreads();
+    // a warp per token (T <= 16 warps)
+    if (warp < p.T) {
+        const int at = warp * p.k;
+        const float top = s_val[at];
+        float sum = 0.0f;
+#pragma unroll 1
         for (int j = lane; j < p.k; j += 32) {
-            const float w = s_w[t * p.k + j] / part;
-            s_w[t * p.k + j] = w;
-            if (blockIdx.x == 0) { p.topk_idx[t * p.k + j] = s_idx[t * p.k + j]; p.topk_w[t * p.k + j] = w; }
+            const float ex = top == -INFINITY ? 1.0f : expf(s_val[at + j] - top);      // only -inf logits kept: 1/k each
+            s_w[at + j] = ex;
+            sum += ex;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+#pragma unroll 1
+        for (int j = lane; j < p.k; j += 32) {
+            const float w = s_w[at + j] / sum;
+            s_w[at + j] = w;
+            if (blockIdx.x == 0) { p.topk_idx[at + j] = s_idx[at + j]; p.topk_w[at + j] = w; }
         }
     }
+}
 
-    // ---- C: a = sigma(W1_e x') per routed slot.  (Grouping the slots by expert, so that a weight byte is read once
-    // however many tokens chose the expert, was measured slower at every T <= 16: the repeats are L2 hits, and the
-    // lists, the smaller tasks and the wider reductions cost more than they save.)
-    for (int i = threadIdx.x; i < T * p.r / 4; i += kDecodeThreads) {
-        const int t = i / (p.r / 4), c = 4 * (i % (p.r / 4));
-        *reinterpret_cast<float4*>(smem_f + t * p.r + split_index(c, p.r)) = __ldcg(reinterpret_cast<const float4*>(p.x_lo) + i);
+// C: a = sigma(W1_e x') per routed slot, ROWS rows per warp and step.  (Grouping the slots by expert, so that a weight byte
+// is read once however many tokens chose the expert, was measured slower at every T <= 16: the repeats are L2 hits, and
+// the lists and wider reductions cost more than they save.)
+template <int ROWS>
+__device__ __forceinline__ void phase_c(const DecodeArgs& p, uint32_t tag) {
+    const int lane = threadIdx.x & 31, b = blockIdx.x, rp = p.r / 8;
+    const int* s_idx = reinterpret_cast<const int*>(smem_at(p.off_idx));
+    const int per_slot = (int)p.by_slot.d, g1 = p.groups_c.first(b + 1);     // h is a multiple of 16
+    int g = p.groups_c.first(b) + (int)(threadIdx.x >> 5);
+    uint4 wv[ROWS];
+    const uint4* w = nullptr;
+    auto rows_at = [&](int q) {
+        const int s = p.by_slot.div(q);
+        w = reinterpret_cast<const uint4*>(p.w1) + ((int64_t)s_idx[s] * p.h + (q - s * per_slot) * ROWS) * rp;
+    };
+    auto fetch = [&](int c) {
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) wv[i] = c < rp ? __ldg(w + i * rp + c) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    if (g < g1) { rows_at(g); fetch(lane); }
+#pragma unroll 1
+    for (; g < g1; g += kWarps) {
+        const int s = p.by_slot.div(g), q0 = (g - s * per_slot) * ROWS;
+        const float4* v = reinterpret_cast<const float4*>(smem_at(p.by_k.div(s) * p.r));
+        f32x2 acc2[ROWS] = {};
+#pragma unroll 1
+        for (int c = lane; c - lane < rp; c += 32) {
+            const int cc = min(c, rp - 1);                   // lanes past the end hold zero weights
+            const float4 v0 = v[cc], v1 = v[rp + cc];
+#pragma unroll
+            for (int i = 0; i < ROWS; ++i) acc2[i] = dot8(Piece(wv[i]), v0, v1, acc2[i]);
+            int next = c + 32;                               // the next pieces, or the next step's rows, before the sums are finished
+            if (next - lane >= rp && g + kWarps < g1) { rows_at(g + kWarps); next = lane; }
+            fetch(next);
+        }
+        float acc[ROWS];
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) acc[i] = sum2(acc2[i]);
+        constexpr int L = 32 / ROWS;
+        const float z = act_apply(p.act, warp_reduce_scatter<ROWS>(acc));              // row lane / L
+        if (!(lane & (L - 1))) put_word(p.a + (int64_t)s * p.h + split_index(q0 + lane / L, p.h), z, tag);
+    }
+}
+
+// D: y'[t, c] = sum_j p_j (W2_{e_j}[c, :] a_j): floor(grid / T) CTAs per token, some columns each, ROWS (column, slot) rows per
+// warp and step.
+template <int ROWS>
+__device__ __forceinline__ void phase_d(const DecodeArgs& p, uint32_t tag) {
+    const int tid = threadIdx.x, lane = tid & 31, b = blockIdx.x, hp = p.h / 8;
+    const int* s_idx = reinterpret_cast<const int*>(smem_at(p.off_idx));
+    const float* s_w = smem_at(p.off_w);
+    float* sums = smem_at(p.off_sums);
+    const bool works = b < p.T * p.ctas_d;           // the last grid - T floor(grid / T) CTAs have no columns: rows = 0
+    const int t = works ? p.by_ctas.div(b) : 0, share = works ? b - t * p.ctas_d : 0, c0 = p.cols_d.first(share);
+    const int rows = works ? (p.cols_d.first(share + 1) - c0) * p.k : 0;     // row i: column c0 + i / k, slot i % k
+    uint4 wv[ROWS][4];
+    const uint4* w[ROWS];
+    int slot[ROWS];
+    auto rows_at = [&](int i) {                              // rows i, i + kWarps, ...
+#pragma unroll
+        for (int n = 0; n < ROWS; ++n) {
+            const int row = min(i + n * kWarps, max(rows - 1, 0)), col = p.by_k.div(row);
+            slot[n] = row - col * p.k;
+            w[n] = reinterpret_cast<const uint4*>(p.w2) + ((int64_t)s_idx[t * p.k + slot[n]] * p.r + c0 + col) * hp;
+        }
+    };
+    auto fetch = [&](int c) {                                // four pieces of a lane
+#pragma unroll
+        for (int n = 0; n < ROWS; ++n)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) wv[n][u] = c + 32 * u < hp ? __ldg(w[n] + c + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    int i = tid >> 5;
+    rows_at(i);
+    if (i < rows) fetch(lane);                               // the first rows are on their way before the wait for a
+    __syncthreads();                                         // x' is not read any more, its place takes a
+    if (rows > 0) get_words(smem_at(0), p.a + (int64_t)t * p.k * p.h, p.k * p.h, tid, kDecodeThreads, tag, p.status);
+    __syncthreads();
+    const float4* v = reinterpret_cast<const float4*>(smem_at(0));
+#pragma unroll 1
+    for (; i < rows; i += ROWS * kWarps) {
+        f32x2 acc2[ROWS] = {};
+        int from[ROWS];
+#pragma unroll
+        for (int n = 0; n < ROWS; ++n) from[n] = 2 * slot[n] * hp;
+#pragma unroll 1
+        for (int c = lane; c - lane < hp; c += 128) {
+#pragma unroll
+            for (int n = 0; n < ROWS; ++n)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int at = from[n] + min(c + 32 * u, hp - 1);        // past the end: zero weights
+                    acc2[n] = dot8(Piece(wv[n][u]), v[at], v[at + hp], acc2[n]);
+                }
+            int next = c + 128;
+            if (next - lane >= hp && i + ROWS * kWarps < rows) { rows_at(i + ROWS * kWarps); next = lane; }
+            fetch(next);
+        }
+        float acc[ROWS];
+#pragma unroll
+        for (int n = 0; n < ROWS; ++n) acc[n] = sum2(acc2[n]);
+        constexpr int L = 32 / ROWS;
+        const float u = warp_reduce_scatter<ROWS>(acc);                      // row lane / L
+        const int row = i + lane / L * kWarps;
+        if (!(lane & (L - 1)) && row < rows) sums[row] = u;
     }
     __syncthreads();
-    {
-        constexpr int ROWS = 16;
-        const int groups = p.h / ROWS;                       // h is a multiple of 16
-        for (int task = gwarp; task < N * groups; task += nwarps) {
-            const int s = task / groups, q0 = (task % groups) * ROWS;
-            const int e = s_idx[s];
-            const float* vp[1] = {smem_f + (s / p.k) * p.r};
-            float acc[ROWS];
-            rows_dot<ROWS, 1, 1, true>(p.w1 + ((int64_t)e * p.h + q0) * p.r, p.r, 0, p.r / 8, vp, p.r / 8, 1, acc);
-            const float z = warp_reduce_scatter<ROWS>(acc);            // row lane / 2
-            if (!(lane & 1)) p.a[(int64_t)s * p.h + q0 + lane / 2] = act_apply(p.act, z);
-        }
+#pragma unroll 1
+    for (int c = tid; c * p.k < rows; c += kDecodeThreads) {       // combine in slot order
+        float acc = 0.0f;
+#pragma unroll 4
+        for (int j = 0; j < p.k; ++j) acc = fmaf(s_w[t * p.k + j], sums[c * p.k + j], acc);
+        put_copies(p, p.y_lo + t * p.r + split_index(c0 + c, p.r), acc, tag);
     }
-    grid_barrier(p.barrier, 1, p.status);
+}
 
-    // ---- D: u = W2_e a per routed slot
-    {
-        const int groups = p.r / 4;
-        for (int task = gwarp; task < N * groups; task += nwarps) {
-            const int s = task / groups, c0 = (task % groups) * 4;
-            const int e = s_idx[s];
-            const float* vp[1] = {p.a + (int64_t)s * p.h};
-            float acc[4];
-            rows_dot<4, 1, 4, false>(p.w2 + ((int64_t)e * p.r + c0) * p.h, p.h, 0, p.h / 8, vp, 0, 1, acc);
-            const float v = warp_reduce_scatter<4>(acc);               // row lane / 8
-            if (!(lane & 7)) p.u[(int64_t)s * p.r + c0 + lane / 8] = v;
-        }
-    }
-    grid_barrier(p.barrier, 2, p.status);
-
-    // ---- E: combine in slot order, then ascend
-    for (int i0 = threadIdx.x; i0 < T * p.r / 4; i0 += kDecodeThreads) {   // four columns per thread, 16-byte loads
-        const int i = (i0 + blockIdx.x * 224) % (T * p.r / 4);              // as in phase A: CTAs start at different places
-        const int t = i / (p.r / 4), c = 4 * (i % (p.r / 4));
-        float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        for (int j0 = 0; j0 < p.k; j0 += 8) {                // eight loads in flight, added in slot order
-            float4 uj[8];
+// E: ascend, one row of W'_up per warp and step (a is not read any more: the barrier before the combine of D).
+template <int TG>
+__device__ __forceinline__ void phase_e(const DecodeArgs& p, uint32_t tag) {
+    const int tid = threadIdx.x, lane = tid & 31, b = blockIdx.x, rp = p.r / 8;
+    get_words(smem_at(0), p.y_lo + b % p.copies * p.copy_words, p.T * p.r, tid, kDecodeThreads, tag, p.status);
+    asm volatile("cp.async.wait_all;" ::: "memory");     // the rows of W'_up
+    __syncthreads();
+    const int up0 = p.rows_e.first(b), up1 = p.rows_e.first(b + 1);
+#pragma unroll 1
+    for (int row = up0 + (tid >> 5); row < up1; row += kWarps) {
+        const uint4* w = p.up_rows > 0 ? reinterpret_cast<const uint4*>(smem_at(p.off_up)) + (row - up0) * rp : reinterpret_cast<const uint4*>(p.w_up) + (int64_t)row * rp;
+#pragma unroll 1
+        for (int t0 = 0; t0 < p.T; t0 += TG) {
+            f32x2 acc2[TG] = {};
+#pragma unroll 1
+            for (int c = lane; c < rp; c += 32) {
+                const Piece q(w[c]);
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-                uj[q] = j0 + q < p.k ? __ldcg(reinterpret_cast<const float4*>(p.u + (int64_t)(t * p.k + j0 + q) * p.r + c))
-                                     : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                if (j0 + q < p.k) {
-                    const float w = s_w[t * p.k + j0 + q];
-                    acc.x = fmaf(w, uj[q].x, acc.x); acc.y = fmaf(w, uj[q].y, acc.y);
-                    acc.z = fmaf(w, uj[q].z, acc.z); acc.w = fmaf(w, uj[q].w, acc.w);
+                for (int t = 0; t < TG; ++t) {
+                    const float4* v = reinterpret_cast<const float4*>(smem_at(min(t0 + t, p.T - 1) * p.r));
+                    acc2[t] = dot8(q, v[c], v[rp + c], acc2[t]);
                 }
             }
+            float acc[TG];
+#pragma unroll
+            for (int t = 0; t < TG; ++t) acc[t] = sum2(acc2[t]);
+            constexpr int L = 32 / TG;
+            const float sum = warp_reduce_scatter<TG>(acc);                  // token t0 + lane / L
+            if (!(lane & (L - 1)) && t0 + lane / L < p.T) p.y[(int64_t)(t0 + lane / L) * p.d + row] = __float2bfloat16(sum);
         }
-        *reinterpret_cast<float4*>(smem_f + t * p.r + split_index(c, p.r)) = acc;
     }
-    __syncthreads();
-    phase_e(p, smem_f, gwarp, nwarps);
-    // a fourth round of arrivals: whoever comes last knows that nobody reads the word any more and zeroes it for the
-    // next launch (also after a wait that gave up: every CTA arrives four times whatever happens)
-    __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(p.barrier, 1u) == 4u * gridDim.x - 1u) atomicExch(p.barrier, 0u);
+}
+
+// TG 1: for one or two tokens, where every phase is a single chain of latencies; TG 4: four tokens' sums at a time, more
+// loads in flight per warp.
+template <int TG>
+__global__ void __launch_bounds__(kDecodeThreads, 1) decode_forward_kernel(const __grid_constant__ DecodeArgs p) {
+    constexpr int ROWS_C = TG == 1 ? 4 : 8, ROWS_D = TG == 1 ? 1 : 2;
+    uint32_t tag;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(tag) : "l"(p.epoch + blockIdx.x) : "memory");
+    ++tag;
+    phase_a<TG>(p, tag);
+    phase_b(p, tag);
+    phase_c<ROWS_C>(p, tag);
+    phase_d<ROWS_D>(p, tag);
+    phase_e<TG>(p, tag);
+    if (threadIdx.x == 0) p.epoch[blockIdx.x] = tag;         // nobody else reads or writes this CTA's word
+}
+
+// Shared memory of a launch, offsets in floats: the region that x, x', a and y' take in turn, rows of
+// W'_up, and the rest.
+size_t decode_smem(DecodeArgs& p, int grid) {
+    const int T = p.T, d = p.d, r = p.r, h = p.h, E = p.E, k = p.k;
+    int region = T * (d > r ? d : r);
+    if (k * h > region) region = k * h;
+    const int up = (d + grid - 1) / grid;
+    p.LE = (E + 3) / 4 * 4;
+    p.up_rows = (size_t)up * r * 2 <= kDecodeMaxUpBytes ? up : 0;
+    const int per_token = grid / T > 1 ? grid / T : 1, rows = ((r + per_token - 1) / per_token) * k;     // phase D's rows of a CTA
+    const int sums_a = ((r + E + grid - 1) / grid) * ((d / 8 + 31) / 32) * 16, sums = rows > sums_a ? rows : sums_a;   // phase A's parts
+    p.off_up = (region + 3) / 4 * 4;
+    p.off_log = p.off_up + p.up_rows * r / 2;                // r is a multiple of 8
+    p.off_idx = p.off_log + T * p.LE;
+    p.off_val = p.off_idx + T * k;
+    p.off_w = p.off_val + T * k;
+    p.off_sums = p.off_w + T * k;
+    return sizeof(float) * ((size_t)p.off_sums + sums);
+}
+constexpr size_t kDecodeSmemLimit = 220 * 1024;
+
+// Where x', logits and y' are a few lines of memory that all CTAs poll, copies keep the readers from queueing up (14.2 -> 13.9 us
+// for one token, 19.4 -> 18.7 for four at r = 256; nothing for eight).
+constexpr int decode_copies(int T, int r) { return T * r <= 512 ? 4 : T * r <= 1024 ? 2 : 1; }
+
+DecodeArgs decode_shape(int T, int d, int r, int h, int E, int k) {
+    DecodeArgs p{};
+    p.T = T; p.d = d; p.r = r; p.h = h; p.E = E; p.k = k;
+    return p;
 }
 
 }  // namespace
 
-bool decode_forward_supported(int T, int d, int r, int h, int E, int k, int dtype) {
-    return dtype == BIGMAC_BF16 && T >= 1 && T <= kDecodeMaxTokens && (int64_t)T * d <= 32768 && d % 8 == 0 && r % 8 == 0 &&
-           h % 16 == 0 && E <= kDecodeMaxExperts && T * k <= kDecodeMaxSlots;
+bool decode_forward_supported(int T, int d, int r, int h, int E, int k, int dtype, int num_sms) {
+    if (dtype != BIGMAC_BF16 || T < 1 || T > kDecodeMaxTokens || (int64_t)T * d > 32768 || d % 8 || r % 8 || h % 16 ||
+        E > kDecodeMaxExperts || (int64_t)k * h > kDecodeMaxHidden || T * k > kDecodeThreads || T > num_sms ||
+        decode_forward_words(T, r, h, E, k) > kDecodeMaxWords)
+        return false;
+    DecodeArgs p = decode_shape(T, d, r, h, E, k);
+    return decode_smem(p, num_sms) <= kDecodeSmemLimit;
 }
 
-cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void* y, float* logits, float* x_lo, float* a,
-                                  float* u, int32_t* topk_idx, float* topk_w, unsigned* barrier, int* status, int T, int d,
-                                  int r, int h, int E, int k, int act, int num_sms, cudaStream_t stream) {
-    DecodeArgs p;
+// Hand-over words of batches of up to T tokens.
+size_t decode_forward_words(int T, int r, int h, int E, int k) {
+    size_t most = 0;
+    for (int t = 1; t <= T; ++t) {
+        const size_t words = (size_t)t * (decode_copies(t, r) * (2 * (size_t)r + (E + 3) / 4 * 4) + (size_t)k * h);
+        if (words > most) most = words;
+    }
+    return most;
+}
+
+// The largest batch of at most max_tokens tokens that the kernel takes at these widths (0: none).
+int decode_forward_max_tokens(int max_tokens, int d, int r, int h, int E, int k, int dtype, int num_sms) {
+    int T = max_tokens < kDecodeMaxTokens ? max_tokens : kDecodeMaxTokens;
+    while (T > 0 && !decode_forward_supported(T, d, r, h, E, k, dtype, num_sms)) --T;
+    return T;
+}
+
+cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void* y, void* words, int32_t* topk_idx, float* topk_w,
+                                  unsigned* epoch, int* status, int T, int d, int r, int h, int E, int k, int act,
+                                  int num_sms, cudaStream_t stream) {
+    DecodeArgs p = decode_shape(T, d, r, h, E, k);
+    const size_t smem = decode_smem(p, num_sms);
     p.x = (const __nv_bfloat16*)x; p.w_gate = (const __nv_bfloat16*)W->w_gate; p.w_down = (const __nv_bfloat16*)W->w_down;
     p.w1 = (const __nv_bfloat16*)W->w1; p.w2 = (const __nv_bfloat16*)W->w2; p.w_up = (const __nv_bfloat16*)W->w_up;
-    p.b_gate = W->b_gate; p.y = (__nv_bfloat16*)y; p.logits = logits; p.x_lo = x_lo; p.a = a; p.u = u;
-    p.topk_idx = topk_idx; p.topk_w = topk_w; p.barrier = barrier; p.status = status;
-    p.T = T; p.d = d; p.r = r; p.h = h; p.E = E; p.k = k; p.act = act;
-    const size_t smem = sizeof(float) * (size_t)T * (d > r ? d : r) + (size_t)T * k * (sizeof(int) + sizeof(float)) +
-                        sizeof(float) * 4 * (kDecodeThreads / 32) * 16;
+    p.b_gate = W->b_gate; p.y = (__nv_bfloat16*)y;
+    p.x_lo = (unsigned long long*)words; p.logits = p.x_lo + (size_t)T * r; p.y_lo = p.logits + (size_t)T * p.LE; p.copies = decode_copies(T, r); p.copy_words = T * (2 * r + p.LE); p.a = p.x_lo + (size_t)p.copies * p.copy_words;
+    p.topk_idx = topk_idx; p.topk_w = topk_w; p.epoch = epoch; p.status = status; p.act = act;
+    const bool few = T <= 2;
+    const int rows_c = few ? 4 : 8;
+    p.rows_a = Split(r + E, num_sms); p.rows_e = Split(d, num_sms); p.groups_c = Split(T * k * (h / rows_c), num_sms);
+    p.ctas_d = num_sms / T > 1 ? num_sms / T : 1; p.cols_d = Split(r, p.ctas_d);
+    p.by_parts = Divisor((d / 8 + 31) / 32); p.by_pieces = Divisor(d / 8); p.by_k = Divisor(k); p.by_slot = Divisor(h / rows_c);
+    p.by_ctas = Divisor(p.ctas_d); p.by_lanes = Divisor((E + 31) / 32);
     static PerDeviceOnce once;
     int dev;
+    const void* kernel1 = (const void*)decode_forward_kernel<1>;
+    const void* kernel4 = (const void*)decode_forward_kernel<4>;
     if (once.needed(&dev)) {
-        cudaError_t e = cudaFuncSetAttribute(decode_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768 * 4 + kDecodeMaxSlots * 8 + 4 * (kDecodeThreads / 32) * 16 * 4);
+        cudaError_t e = cudaFuncSetAttribute(kernel1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemLimit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemLimit);
         if (e != cudaSuccess) return e;
         once.mark(dev);
     }
-    void* args[] = {(void*)&p};
-    return cudaLaunchCooperativeKernel((const void*)decode_forward_kernel, dim3(num_sms), dim3(kDecodeThreads), args, smem,
-                                       stream);
+    void* ptrs[] = {(void*)&p};
+    return cudaLaunchCooperativeKernel(few ? kernel1 : kernel4, dim3(num_sms), dim3(kDecodeThreads), ptrs, smem, stream);
 }
 
 }  // namespace bigmac

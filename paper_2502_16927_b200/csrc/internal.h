@@ -283,11 +283,14 @@ struct WordCopies {
 };
 cudaError_t launch_word_copies(const WordCopies& c, cudaStream_t stream);
 
-// Small-batch inference forward in one cooperative kernel (bf16, T <= 16): scratch logits [T,E], x_lo [T,r],
-// a [T*k,h], u [T*k,r] fp32; writes y, topk_idx, topk_w.  `barrier` is one device word owned by the handle.
-bool decode_forward_supported(int T, int d, int r, int h, int E, int k, int dtype);
-cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void* y, float* logits, float* x_lo, float* a,
-                                  float* u, int32_t* topk_idx, float* topk_w, unsigned* barrier, int* status, int T, int d,
-                                  int r, int h, int E, int k, int act, int num_sms, cudaStream_t stream);
+// Small-batch inference forward in one cooperative kernel (bf16, T <= 16): writes y, topk_idx, topk_w.  words:
+// decode_forward_words() 8-byte words of the handle for the values that cross between CTAs, zero when the handle is made
+// and written by this kernel only; epoch: num_sms device words of the handle, zero at first (launches so far, per block).
+bool decode_forward_supported(int T, int d, int r, int h, int E, int k, int dtype, int num_sms);
+size_t decode_forward_words(int T, int r, int h, int E, int k);
+int decode_forward_max_tokens(int max_tokens, int d, int r, int h, int E, int k, int dtype, int num_sms);
+cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void* y, void* words, int32_t* topk_idx, float* topk_w,
+                                  unsigned* epoch, int* status, int T, int d, int r, int h, int E, int k, int act,
+                                  int num_sms, cudaStream_t stream);
 
 }  // namespace bigmac

@@ -419,11 +419,19 @@ int bigmac_layer_create(const bigmac_config_t* cfg, bigmac_layer_t** out) {
     L->cfg = *cfg;
     L->use_tc = cfg->dtype == BIGMAC_BF16 && !(cfg->flags & BIGMAC_FLAG_SIMT_GEMM);
     L->tc_mask = switches().tc_mask;
-    if (cudaGetDevice(&L->device) != cudaSuccess || cudaMalloc((void**)&L->status, 4 * sizeof(int)) != cudaSuccess ||
-        cudaMemset(L->status, 0, 4 * sizeof(int)) != cudaSuccess) {
+    // status words, and behind them the hand-over words of the small-batch kernel where the configuration can reach it
+    const bool plain = L->use_tc && !(cfg->flags & (BIGMAC_FLAG_CDAC | BIGMAC_FLAG_GATE_LOW | BIGMAC_FLAG_EXPERT_BIAS)) &&
+                       cfg->capacity_factor == 0 && cfg->aux_loss_coef == 0;
+    const int few = plain ? decode_forward_max_tokens(cfg->max_tokens, cfg->d, cfg->r, cfg->h, cfg->E, cfg->k, cfg->dtype, gemm_tc_sm_count()) : 0;
+    const size_t words = decode_forward_words(few, cfg->r, cfg->h, cfg->E, cfg->k);
+    const size_t head = words ? 256 + ((size_t)gemm_tc_sm_count() * 4 + 255) / 256 * 256 : 256, bytes = head + 8 * words;
+    if (cudaGetDevice(&L->device) != cudaSuccess || cudaMalloc((void**)&L->status, bytes) != cudaSuccess ||
+        cudaMemset(L->status, 0, bytes) != cudaSuccess) {
+        cudaFree(L->status);
         delete L;
         return BIGMAC_ERR_CUDA;
     }
+    L->decode_words = words ? (char*)L->status + head : nullptr;
     if (L->use_tc && !gemm_tc_available()) {
         cudaFree(L->status);
         delete L;
@@ -514,13 +522,12 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
     const bigmac_config_t& c = L->cfg;
 
     // A few tokens, inference: the whole forward in one cooperative kernel (weight streaming, no tensor cores)
-    if (!training && !m.cdac && !m.gate_low && !m.bias && m.cap == kNoCapacity && m.aux == 0 && sigma_as_bytes(L) &&
-        decode_forward_supported(m.T, m.d, m.r, m.h, m.E, m.k, m.dtype)) {
+    if (!training && !m.cdac && !m.gate_low && !m.bias && m.cap == kNoCapacity && m.aux == 0 && sigma_as_bytes(L) && L->decode_words &&
+        decode_forward_supported(m.T, m.d, m.r, m.h, m.E, m.k, m.dtype, gemm_tc_sm_count())) {
         {
             Stage s(L, S_DECODE, st);
-            BIGMAC_CUDA(launch_decode_forward(x, W, y, b.logits, (float*)b.xg, (float*)b.a, (float*)b.u, b.tb.topk_idx,
-                                              b.tb.topk_w, (unsigned*)(L->status + 1), L->status, m.T, m.d, m.r, m.h, m.E,
-                                              m.k, c.act, gemm_tc_sm_count(), st));
+            BIGMAC_CUDA(launch_decode_forward(x, W, y, L->decode_words, b.tb.topk_idx, b.tb.topk_w, (unsigned*)(L->status + 64),
+                                              L->status, m.T, m.d, m.r, m.h, m.E, m.k, c.act, gemm_tc_sm_count(), st));
         }
         if (routing_out) {
             { Stage s(L, S_TABLES, st, tables_kernel_count(m.N, m.E)); BIGMAC_CUDA(launch_tables(b.tb, m.T, m.E, m.k, m.cap, st, L->status)); }

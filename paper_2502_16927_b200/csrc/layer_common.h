@@ -11,8 +11,9 @@
 struct bigmac_layer {
     bigmac_config_t cfg;
     int device;
-    int* status;        // device status word; status[1] is the grid-barrier counter of the small-batch kernel,
-                        // status[2..3] the work counters of the per-expert weight-gradient kernel (zero at rest)
+    int* status = nullptr;  // device status word; status[2..3] are the work counters of the per-expert weight-gradient kernel
+                        // (zero at rest), status[64 ..] the small-batch kernel's launch counts, one per block
+    void* decode_words = nullptr;   // hand-over words of the small-batch kernel (same allocation), or null
     bool use_tc;        // bf16 contractions on tcgen05
     unsigned tc_mask;   // debug: bit i set = contraction i runs on tcgen05 (the tc_mask switch at creation)
     // second stream of the backward pass (created on first use): launches that do not depend on each other and lean
