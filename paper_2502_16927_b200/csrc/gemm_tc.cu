@@ -72,6 +72,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    if (p.prefetch_bytes && threadIdx.x == 64) {             // a CTA without a tile: its share of what a later launch streams
+        const int tiles = ((p.M + BM - 1) / BM) * ((p.N + BN - 1) / BN) * p.split_k;
+        constexpr uint32_t kPiece = 32768;
+        if ((int)blockIdx.x >= tiles)
+            for (int q = 0; q < 2; ++q)
+                for (uint32_t at = (blockIdx.x - tiles) * kPiece; at < p.prefetch_bytes; at += (gridDim.x - tiles) * kPiece)
+                    prefetch_l2(p.prefetch[q] + at, min(kPiece, p.prefetch_bytes - at));
+    }
     if (warp == 1) tmem_alloc(tmem_slot, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
@@ -316,7 +324,7 @@ cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorM
         if (e != cudaSuccess) return e;
         once.mark(dev);
     }
-    const int grid = max_tiles < sm_count() ? max_tiles : sm_count();
+    const int grid = max_tiles < sm_count() && !p.prefetch_bytes ? max_tiles : sm_count();
     return launch_chained(kernel, grid, GATHER ? kThreadsGather : kThreadsV2, smem, stream, ma, mb, mc, mz, mb2, p);
 }
 
@@ -383,6 +391,10 @@ cudaError_t dispatch(const GemmArgs& g, int* status, cudaStream_t stream) {
     p.epi_parts = 4;
     p.bias = g.group == GROUP_M ? g.bias : nullptr; p.bias_stride = g.bias_stride;
     if (p.bias && (g.N % 32 || ((uintptr_t)g.bias % 16) || g.bias_stride % 4)) return cudaErrorInvalidValue;
+    if (g.prefetch_bytes && g.group == GROUP_NONE && g.prefetch_bytes < ((size_t)1 << 30)) {
+        p.prefetch[0] = (const uint8_t*)g.prefetch[0]; p.prefetch[1] = (const uint8_t*)g.prefetch[1];
+        p.prefetch_bytes = (uint32_t)g.prefetch_bytes;
+    }
     p.gather_rows = g.gather_rows; p.gather_src = g.A; p.gather_ld = g.lda; p.gather_div = g.gather_div > 0 ? g.gather_div : 1;
     const int64_t tiles = (int64_t)((g.N + BN - 1) / BN) * ((g.M + BM - 1) / BM) * (g.group == GROUP_K ? E : p.split_k);
     const int max_tiles = tiles > (1 << 30) ? (1 << 30) : (int)tiles;
@@ -418,8 +430,17 @@ cudaError_t launch_expire_wait(int* status, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
+// Up to as many 128 x 128 tiles as there are SMs: four times the CTAs of the 256 x 256 pair tiles, which leave most of the
+// chip idle there (descend + logits at 3001 tokens, 320 columns, K = 2048: 24 pairs, 19 us -> 72 CTAs, 13 us; dy' 21 -> 14).
+bool gemm_tc_one_round(int M, int N, int split_k) {
+    return (int64_t)((M + 127) / 128) * ((N + 127) / 128) * split_k <= sm_count();
+}
+
 cudaError_t gemm_tc(const GemmArgs& g, int* status, cudaStream_t stream) {
     if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+    if (g.group == GROUP_NONE && g.a_kmajor && !g.force_kernel && g.epilogue == EPI_NONE && gemm_tc_one_round(g.M, g.N, g.split_k) &&
+        (!g.C2 || g.n_split % 128 == 0))
+        return dispatch<128, 6, false>(g, status, stream);
     // Where it pays, the problem runs on CTA pairs (each SM stages half of B); the tc_pair debug switch disables that.
     const bool pair_enabled = switches().tc_pair != 0;
     const bool want_pair = g.gather_rows ? false          // gathered rows: the one-CTA kernel

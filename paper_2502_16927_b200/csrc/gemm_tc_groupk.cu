@@ -365,17 +365,36 @@ gemm_tc_groupk_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
 
 // C_e = sum of the parts of a split expert, in part order (+ C_e when accumulating); C_e = 0 for an expert
 // without rows (unless accumulating).  plan = [pp (E+1) | ss (E+1)] as left by the contraction kernel.
+// Most experts need nothing, usually all of them: a small grid lists the others and shares their elements out.  (A block
+// per expert and 16 KB of it, 4096 blocks for 64 experts and 8192 for 128, held the next launch up by 5 and 14 us.)
 __global__ void __launch_bounds__(256) groupk_finish_kernel(const float* __restrict__ ws, const int32_t* __restrict__ plan,
                                                             __nv_bfloat16* __restrict__ C, int64_t c_stride, int64_t mn,
                                                             int E, int accumulate) {
     grid_dependency_wait();
     grid_dependency_launch();
-    const int e = blockIdx.y;
-    const int parts = plan[e + 1] - plan[e];
-    if (parts == 1 || (parts == 0 && accumulate)) return;
-    const float* base = ws + (int64_t)plan[E + 1 + e] * mn;
-    __nv_bfloat16* dst = C + (int64_t)e * c_stride;
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; i < mn; i += (int64_t)gridDim.x * blockDim.x * 8) {
+    __shared__ int32_t s_list[kMaxExperts];
+    __shared__ int s_count;
+    if (threadIdx.x < 32) {
+        int n = 0;
+        for (int e0 = 0; e0 < E; e0 += 32) {
+            const int e = e0 + (int)threadIdx.x;
+            const int parts = e < E ? plan[e + 1] - plan[e] : 1;
+            const bool need = !(parts == 1 || (parts == 0 && accumulate));
+            const unsigned votes = __ballot_sync(0xffffffffu, need);
+            if (need) s_list[n + __popc(votes & ((1u << threadIdx.x) - 1u))] = e;
+            n += __popc(votes);
+        }
+        if (threadIdx.x == 0) s_count = n;
+    }
+    __syncthreads();
+    const int64_t per = (mn / 8 + blockDim.x - 1) / blockDim.x;               // pieces of an expert, eight elements a thread
+    for (int64_t q = blockIdx.x; q < s_count * per; q += gridDim.x) {
+        const int e = s_list[q / per];
+        const int64_t i = ((q % per) * blockDim.x + threadIdx.x) * 8;
+        if (i >= mn) continue;
+        const int parts = plan[e + 1] - plan[e];
+        const float* base = ws + (int64_t)plan[E + 1 + e] * mn;
+        __nv_bfloat16* dst = C + (int64_t)e * c_stride;
         float acc[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
@@ -452,8 +471,7 @@ cudaError_t gemm_tc_groupk_finish(const GemmArgs& g, void* ws, cudaStream_t stre
     float* slots = (float*)ws;
     int32_t* plan = (int32_t*)((char*)ws + (((size_t)kGroupKSlots * g.M * g.N * sizeof(float) + 255) & ~(size_t)255));
     const int64_t mn = (int64_t)g.M * g.N;
-    dim3 grid((unsigned)((mn / 8 + 255) / 256 < 64 ? (mn / 8 + 255) / 256 : 64), (unsigned)E);
-    return launch_chained(groupk_finish_kernel, grid, 256, 0, stream, slots, plan, (__nv_bfloat16*)g.C, g.c_stride, mn, E, g.accumulate ? 1 : 0);
+    return launch_chained(groupk_finish_kernel, 4 * sm_count(), 256, 0, stream, slots, plan, (__nv_bfloat16*)g.C, g.c_stride, mn, E, g.accumulate ? 1 : 0);
 }
 
 }  // namespace bigmac

@@ -91,6 +91,10 @@ struct GemmArgs {
     // bias[e*bias_stride + n] (16-byte aligned, bias_stride a multiple of 4)
     const float* bias = nullptr;
     int64_t bias_stride = 0;
+    // Dense problems: memory that a later launch streams (16-byte aligned, multiples of 16 bytes); SMs that have no tile of
+    // this problem ask for it to be brought to L2.  A hint, without effect on results.
+    const void* prefetch[2] = {nullptr, nullptr};
+    size_t prefetch_bytes = 0;          // of each
 };
 
 // fp32-FMA GEMM for either dtype (dtype: bigmac_dtype_t of A, B, Z and - unless out_f32 - C).
@@ -101,6 +105,8 @@ cudaError_t gemm_simt_batch(const GemmArgs* g, int count, int dtype, cudaStream_
 // tcgen05 / TMEM / TMA GEMM, bf16 inputs, fp32 accumulation.  `status` is the device status word.
 cudaError_t gemm_tc(const GemmArgs& g, int* status, cudaStream_t stream);
 bool gemm_tc_available();
+// Does a dense contraction with these output sizes and parts run in one round of 128 x 128 tiles, one CTA each?
+bool gemm_tc_one_round(int M, int N, int split_k);
 // Per-expert weight-gradient contraction (GROUP_K, both operands MN-major, bf16 output) with dynamically scheduled
 // work items and long experts cut into parts (gemm_tc_groupk.cu).  ws: gemm_tc_groupk_ws_bytes() bytes, 256-byte
 // aligned; sched: two device ints that are zero between launches (the kernel leaves them so).

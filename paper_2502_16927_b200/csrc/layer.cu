@@ -131,19 +131,20 @@ void carve_backward_scratch(Carver& cv, const Dims& m, Buffers& b) {
 
 // The descend + gate-logits launch has few output tiles where there are few tokens, each walking all of d; its contraction
 // is then cut into parts (fp32 partial results, added by the routing kernels on the way) so that the SMs share the work.
-// Cost of s parts in k slices of tensor work (0.35 us): the longest SM pair's slices, plus what writing and reading the
+// Cost of s parts: the longest SM's k slices (0.35 us each on a pair of SMs, 0.2 on one), plus what writing and reading the
 // partial results takes (0.8 us per MB).  At d = 2048, r + E = 320: 8 parts at 64 tokens, 4 at 512, 3 at 1200, none from
 // 1800 on (at 3001, three parts: launch 19.3 -> 16.3 us, placement 6.9 -> 10.4).  A function of the shape only: every call of a handle with the same T takes the same path.
 int descend_split_parts(const Dims& m) {
     if (m.E % 4 || m.dtype != BIGMAC_BF16) return 1;
-    const int n = m.r + m.E, bn = n >= 256 ? 256 : 128, bm = n >= 256 ? 256 : 128;
-    const int64_t tiles = (int64_t)((m.T + bm - 1) / bm) * ((n + bn - 1) / bn);
-    const int num_kb = m.d / 64, units = n >= 256 ? gemm_tc_sm_count() / 2 : gemm_tc_sm_count();
+    const int n = m.r + m.E, num_kb = m.d / 64;
     int best = 1;
     double best_cost = 0;
     for (int s = 1; s <= kMaxSplitK && s <= num_kb; ++s) {
-        double cost = (double)((tiles * s + units - 1) / units) * ((num_kb + s - 1) / s);
-        if (s > 1) cost += (double)s * m.T * n * 4.0 / 0.44e6;
+        const bool pairs = n >= 256 && !(m.r % 128 == 0 && gemm_tc_one_round(m.T, n, s));
+        const int b = pairs ? 256 : 128, units = gemm_tc_sm_count() / (pairs ? 2 : 1);
+        const int64_t tiles = (int64_t)((m.T + b - 1) / b) * ((n + b - 1) / b);
+        double cost = (double)((tiles * s + units - 1) / units) * ((num_kb + s - 1) / s) * (pairs ? 0.35 : 0.2);
+        if (s > 1) cost += (double)s * m.T * n * 4.0 * 0.8e-6;
         if (s == 1 || cost < best_cost) { best = s; best_cost = cost; }
     }
     return best;
@@ -548,6 +549,12 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
         g.A = x; g.lda = m.d; g.B = W->w_down; g.ldb = m.d; g.C = b.x_lo; g.ldc = m.r;
         g.B2 = W->w_gate; g.ldb2 = m.d; g.n_split = m.r; g.C2 = b.logits; g.ldc2 = m.E; g.N2 = m.E;
         g.M = m.T; g.N = m.r + m.E; g.K = m.d;
+        // Where a batch touches nearly all experts (two slots for each), their weights stream from DRAM to L2 while the
+        // routing runs, which leaves memory idle for 20 us.  Up to 80 MB: beside the rest they fit in L2 (126 MB).
+        const size_t expert_bytes = (size_t)m.E * m.h * m.r * esize(m.dtype);
+        if (!training && uses_fused_mlp(L, m) && m.N >= 2 * (int64_t)m.E && 2 * expert_bytes <= ((size_t)80 << 20)) {
+            g.prefetch[0] = W->w1; g.prefetch[1] = W->w2; g.prefetch_bytes = expert_bytes;
+        }
         if (b.descend_ws) {                                   // few tokens: contraction in parts, added by the routing kernels
             const int ld = m.r + m.E, parts = descend_split_parts(m);
             const int64_t part_stride = (int64_t)m.T * ld;
