@@ -180,14 +180,8 @@ gemm_tc_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
         int32_t* s_off = s_pp + p.num_experts + 1;
         for (int e = threadIdx.x; e <= p.num_experts; e += blockDim.x) s_off[e] = p.poffsets[e];
         __syncthreads();
-        if (threadIdx.x == 0 && p.group == GROUP_M) {
-            int run = 0;
-            for (int e = 0; e < p.num_experts; ++e) {
-                s_pp[e] = run;
-                run += ((s_off[e + 1] - s_off[e]) / kPad + 1) / 2;
-            }
-            s_pp[p.num_experts] = run;
-        }
+        if (warp == 0 && p.group == GROUP_M)
+            warp_prefix(p.num_experts, s_pp, [&](int e) { return ((s_off[e + 1] - s_off[e]) / kPad + 1) / 2; });
     }
     __syncthreads();                                         // the pair prefix is in shared memory
     if (p.group == GROUP_M) pairs_m = s_pp[p.num_experts];

@@ -65,25 +65,13 @@ __device__ void groupk_plan(const int32_t* poffsets, int E, int per, int pairs, 
         if (slots <= kGroupKSlots) break;
         len += len / 2;
     }
-    if (elect_one()) {
-        int run = 0, slot = 0, lo = poffsets[0];
-        for (int e = 0; e < E; ++e) {
-            const int hi = poffsets[e + 1];
-            const int kb = (hi - lo) / BK;
-            lo = hi;
-            int parts = kb == 0 ? 0 : 1;
-            if (kb > len) {
-                const int want = (kb + len - 1) / len;
-                if (slot + want <= kGroupKSlots) parts = want;
-            }
-            pp[e] = run;
-            ss[e] = slot;
-            run += parts;
-            if (parts > 1) slot += parts;
-        }
-        pp[E] = run;
-        ss[E] = slot;
-    }
+    // (the loop above ends with the slots in their number: it stops at the latest when no expert is longer than len)
+    auto parts = [&](int e) {
+        const int kb = (poffsets[e + 1] - poffsets[e]) / BK;
+        return kb > len ? (kb + len - 1) / len : kb > 0;
+    };
+    warp_prefix(E, pp, parts);
+    warp_prefix(E, ss, [&](int e) { const int n = parts(e); return n > 1 ? n : 0; });
 }
 
 template <bool GATHER>
