@@ -403,8 +403,8 @@ int bigmac_ep_route(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_we
     if (route_fused_supported(m.E, m.k)) {
         const RouteSource src{b.logits, m.E, 1, 0, nullptr};
         const int sms = gemm_tc_sm_count();
-        { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_route_fused(src, RouteMove{}, W->b_gate, b.tb, m.T, m.E, m.k, kNoCapacity, nullptr, sms, st, L->status, 0)); }
-        { Stage s(L, S_TABLES, st); BIGMAC_CUDA(launch_route_fused(src, RouteMove{}, W->b_gate, b.tb, m.T, m.E, m.k, kNoCapacity, nullptr, sms, st, L->status, 1)); }
+        { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_route_fused(src, RouteMove{}, RouteExport{}, W->b_gate, b.tb, m.T, m.E, m.k, kNoCapacity, nullptr, sms, st, L->status, 0)); }
+        { Stage s(L, S_TABLES, st); BIGMAC_CUDA(launch_route_fused(src, RouteMove{}, RouteExport{}, W->b_gate, b.tb, m.T, m.E, m.k, kNoCapacity, nullptr, sms, st, L->status, 1)); }
     } else {
         { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_topk(b.logits, W->b_gate, m.T, m.E, m.k, b.tb.topk_idx, b.tb.topk_w, st)); }
         { Stage s(L, S_TABLES, st, tables_kernel_count(m.N, m.E)); BIGMAC_CUDA(launch_tables(b.tb, m.T, m.E, m.k, kNoCapacity, st, L->status)); }

@@ -206,12 +206,20 @@ inline int tables_kernel_count(int64_t N, int E) {
 // is placed nowhere (row -1) and recorded there as 2.
 cudaError_t launch_tables(const Tables& tb, int T, int E, int k, int cap, cudaStream_t stream, int* status = nullptr);
 
-// Top-k, tables and (if mv.grouped is set) the dispatch in two launches, for the (E, k) of route_fused_supported.
+// Top-k, tables, the load-balancing loss and (if mv.grouped is set) the dispatch in two launches, for the (E, k) of route_fused_supported.
 struct RouteSource {                    // gate logits [T, ld]; parts > 1: the sum of `parts` such matrices, part_stride apart
     const float* logits;
     int ld, parts;
     int64_t part_stride;
     float* logits_out;                  // nullable: the logits as [T, E]
+    // load-balancing loss (aux_part null: none): scratch [blocks of the first launch, E] and where the loss goes
+    float *aux_part = nullptr, *aux_loss = nullptr;
+    float aux_coef = 0.0f;
+};
+// Second destinations of the tables (a training call keeps a copy for its backward): the caller's arrays, each nullable.
+struct RouteExport {
+    int32_t *topk_idx, *counts, *counts_chosen, *offsets, *row_of_slot, *slot_of_row;
+    float *topk_w, *aux_loss;
 };
 struct RouteMove {                      // rows of row_bytes bytes to the expert-grouped matrix `grouped` (null: tables only)
     const void* src;                    // the rows, or
@@ -224,8 +232,8 @@ struct RouteMove {                      // rows of row_bytes bytes to the expert
 };
 bool route_fused_supported(int E, int k);
 // which: 0 = first launch (top-k, gate values, block counts), 1 = second launch (tables, rows).
-cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, const float* b_gate, const Tables& tb, int T, int E,
-                               int k, int cap, float* zero_word, int sm_count, cudaStream_t stream, int* status, int which);
+cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, const RouteExport& ex, const float* b_gate, const Tables& tb,
+                               int T, int E, int k, int cap, float* zero_word, int sm_count, cudaStream_t stream, int* status, int which);
 
 // Row moves.  `width` elements of the dtype per row; all row pointers 16-byte aligned.
 // grouped[prow,:] = src[slot_of_prow[prow]/k,:], zeros on padding rows, for prow < n_tiles*kPad.

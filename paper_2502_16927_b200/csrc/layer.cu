@@ -34,7 +34,7 @@ struct Buffers {
     void* dcat;          // [T, r + E64]: dx' in columns [0, r), the dense gate gradient dl in columns [r, r + E64)
     void *dx_lo, *dlogits;                               // views into dcat (row stride r + E64)
     float* colsum_part;  // [kColsumChunks + kAuxChunks, E]: partial column sums of the top-k part, then of the load-balancing part
-    float* aux_part;     // [kAuxChunks, E] forward scratch of the load-balancing loss
+    float* aux_part;     // [kAuxChunks, E] (the fused routing: [block_rows, E] of it) forward scratch of the load-balancing loss
     float* aux_loss;     // [1] saved: L_aux of the batch
     float* logits_saved; // [T,E] saved copy of the gate logits (only with a load-balancing loss)
     float* splitk_ws;    // fp32 partial results of the split weight-gradient contractions
@@ -238,23 +238,58 @@ int choose_split_k(int M, int N, int K) {
     return best;
 }
 
+// Copies the tables into the caller's arrays (a training forward keeps its own copy in `saved` for the backward), all in
+// one launch; members that alias_routing pointed at the caller's arrays are already in place.
+int export_routing(const bigmac_layer* L, const Dims& m, const Buffers& b, bigmac_routing_t* out, cudaStream_t st) {
+    if (!out) return BIGMAC_OK;
+    WordCopies c{};
+    auto add = [&](void* dst, const void* src, int64_t words) {
+        if (dst && dst != src) { c.dst[c.n] = (uint32_t*)dst; c.src[c.n] = (const uint32_t*)src; c.words[c.n++] = words; }
+    };
+    add(out->topk_idx, b.tb.topk_idx, m.N);
+    add(out->topk_w, b.tb.topk_w, m.N);
+    add(out->counts, b.tb.counts, m.E);
+    add(out->offsets, b.tb.offsets, m.E + 1);
+    add(out->row_of_slot, b.tb.row_of_slot, m.N);
+    add(out->slot_of_row, b.tb.slot_of_row, m.N);
+    add(out->counts_chosen, b.tb.counts_chosen, m.E);
+    if (m.aux > 0) add(out->aux_loss, b.aux_loss, 1);
+    if (c.n == 0) return BIGMAC_OK;
+    Stage s(L, S_TABLES, st);
+    BIGMAC_CUDA(launch_word_copies(c, st));
+    return BIGMAC_OK;
+}
+
 // Steps F2-F3 from the gate logits: top-k with softmax gate values, dispatch layout (under the capacity limit, if
 // any), load-balancing loss; with mv.grouped set also F5, the rows of x' to their places.  zero_word: see launch_route_fused.
+// `out` (nullable): the caller's tables, which leave beside the handle's own.
 int route_from_logits(const bigmac_layer* L, const Dims& m, const bigmac_weights_t* W, Buffers& b, const RouteSource& src,
-                      const RouteMove& mv, float* zero_word, cudaStream_t st) {
+                      const RouteMove& mv, float* zero_word, bigmac_routing_t* out, cudaStream_t st) {
     if (route_fused_supported(m.E, m.k)) {
         const int sms = gemm_tc_sm_count();
-        { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_route_fused(src, mv, W->b_gate, b.tb, m.T, m.E, m.k, m.cap, zero_word, sms, st, L->status, 0)); }
-        { Stage s(L, mv.grouped ? S_DISPATCH : S_TABLES, st); BIGMAC_CUDA(launch_route_fused(src, mv, W->b_gate, b.tb, m.T, m.E, m.k, m.cap, zero_word, sms, st, L->status, 1)); }
+        RouteExport ex{};
+        if (out) {
+            auto other = [](auto* to, auto* own) { return to != own ? to : nullptr; };
+            ex.topk_idx = other(out->topk_idx, b.tb.topk_idx); ex.topk_w = other(out->topk_w, b.tb.topk_w);
+            ex.counts = other(out->counts, b.tb.counts); ex.counts_chosen = other(out->counts_chosen, b.tb.counts_chosen);
+            ex.offsets = other(out->offsets, b.tb.offsets); ex.row_of_slot = other(out->row_of_slot, b.tb.row_of_slot);
+            ex.slot_of_row = other(out->slot_of_row, b.tb.slot_of_row);
+            if (m.aux > 0) ex.aux_loss = other(out->aux_loss, b.aux_loss);
+        }
+        RouteSource with_loss = src;
+        if (m.aux > 0) { with_loss.aux_part = b.aux_part; with_loss.aux_loss = b.aux_loss; with_loss.aux_coef = m.aux; }
+        { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_route_fused(with_loss, mv, ex, W->b_gate, b.tb, m.T, m.E, m.k, m.cap, zero_word, sms, st, L->status, 0)); }
+        { Stage s(L, mv.grouped ? S_DISPATCH : S_TABLES, st); BIGMAC_CUDA(launch_route_fused(with_loss, mv, ex, W->b_gate, b.tb, m.T, m.E, m.k, m.cap, zero_word, sms, st, L->status, 1)); }
     } else {
         { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_topk(src.logits, W->b_gate, m.T, m.E, m.k, b.tb.topk_idx, b.tb.topk_w, st)); }
         { Stage s(L, S_TABLES, st, tables_kernel_count(m.N, m.E)); BIGMAC_CUDA(launch_tables(b.tb, m.T, m.E, m.k, m.cap, st, L->status)); }
         if (zero_word) BIGMAC_CUDA(cudaMemsetAsync(zero_word, 0, sizeof(float), st));
         if (mv.grouped) { Stage s(L, S_DISPATCH, st); BIGMAC_CUDA(launch_dispatch(mv.src, mv.grouped, b.tb, m.k, m.r, m.dtype, m.P, st)); }
-    }
-    if (m.aux > 0) {
-        Stage s(L, S_AUX_LOSS, st, 2);
-        BIGMAC_CUDA(launch_aux_loss(b.logits, W->b_gate, b.tb.counts_chosen, m.T, m.E, m.k, m.aux, b.aux_part, b.aux_loss, st));
+        if (m.aux > 0) {
+            Stage s(L, S_AUX_LOSS, st, 2);
+            BIGMAC_CUDA(launch_aux_loss(b.logits, W->b_gate, b.tb.counts_chosen, m.T, m.E, m.k, m.aux, b.aux_part, b.aux_loss, st));
+        }
+        BIGMAC_TRY(export_routing(L, m, b, out, st));
     }
     return BIGMAC_OK;
 }
@@ -281,9 +316,9 @@ float* aux_word_to_zero(const Dims& m, const bigmac_routing_t* out) { return out
 
 // Steps F1-F3 without the rest of the layer.
 int run_routing(const bigmac_layer* L, const Dims& m, const void* x, const bigmac_weights_t* W, Buffers& b,
-                const bigmac_routing_t* out, cudaStream_t st) {
+                bigmac_routing_t* out, cudaStream_t st) {
     BIGMAC_TRY(run_logits(L, m, x, W, b, st));
-    return route_from_logits(L, m, W, b, RouteSource{b.logits, m.E, 1, 0, nullptr}, RouteMove{}, aux_word_to_zero(m, out), st);
+    return route_from_logits(L, m, W, b, RouteSource{b.logits, m.E, 1, 0, nullptr}, RouteMove{}, aux_word_to_zero(m, out), out, st);
 }
 
 // Calls that keep no saved state (bigmac_route, the inference forward): the tables the caller asked for are produced
@@ -298,28 +333,6 @@ void alias_routing(Buffers& b, const bigmac_routing_t* out) {
     if (out->slot_of_row) b.tb.slot_of_row = out->slot_of_row;
     if (out->counts_chosen) b.tb.counts_chosen = out->counts_chosen;
     if (out->aux_loss) b.aux_loss = out->aux_loss;
-}
-
-// Copies the tables into the caller's arrays (a training forward keeps its own copy in `saved` for the backward), all in
-// one launch; members that alias_routing pointed at the caller's arrays are already in place.
-int export_routing(const bigmac_layer* L, const Dims& m, const Buffers& b, bigmac_routing_t* out, cudaStream_t st) {
-    if (!out) return BIGMAC_OK;
-    WordCopies c{};
-    auto add = [&](void* dst, const void* src, int64_t words) {
-        if (dst && dst != src) { c.dst[c.n] = (uint32_t*)dst; c.src[c.n] = (const uint32_t*)src; c.words[c.n++] = words; }
-    };
-    add(out->topk_idx, b.tb.topk_idx, m.N);
-    add(out->topk_w, b.tb.topk_w, m.N);
-    add(out->counts, b.tb.counts, m.E);
-    add(out->offsets, b.tb.offsets, m.E + 1);
-    add(out->row_of_slot, b.tb.row_of_slot, m.N);
-    add(out->slot_of_row, b.tb.slot_of_row, m.N);
-    add(out->counts_chosen, b.tb.counts_chosen, m.E);
-    if (m.aux > 0) add(out->aux_loss, b.aux_loss, 1);
-    if (c.n == 0) return BIGMAC_OK;
-    Stage s(L, S_TABLES, st);
-    BIGMAC_CUDA(launch_word_copies(c, st));
-    return BIGMAC_OK;
 }
 
 int check_call(const bigmac_layer* L, int32_t T) {
@@ -492,8 +505,7 @@ int bigmac_route(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_weigh
     carve_saved(cv, m, b, false);
     alias_routing(b, out);
     cudaStream_t st = (cudaStream_t)stream;
-    BIGMAC_TRY(run_routing(L, m, x, W, b, out, st));
-    return export_routing(L, m, b, out, st);
+    return run_routing(L, m, x, W, b, out, st);
 }
 
 int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_weights_t* W, void* y,
@@ -588,8 +600,7 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
     if (!gather_dispatch) {
         mv.src = b.x_lo; mv.grouped = b.xg; mv.row_bytes = m.r * (int)esize(m.dtype); mv.zero_padding = training;
     }
-    BIGMAC_TRY(route_from_logits(L, m, W, b, src, mv, aux_word_to_zero(m, routing_out), st));
-    BIGMAC_TRY(export_routing(L, m, b, routing_out, st));
+    BIGMAC_TRY(route_from_logits(L, m, W, b, src, mv, aux_word_to_zero(m, routing_out), routing_out, st));
     // Inference: F6 + F7 in one kernel, the hidden activations stay on the SM (uses_fused_mlp has the rule).
     const bool mlp_fused = !training && uses_fused_mlp(L, m);
     const MlpSlicing slicing = fused_mlp_slicing(m.r, m.h, m.N, m.P);
@@ -1071,8 +1082,7 @@ int bigmac_route_static(bigmac_layer_t* L, const void* x, int32_t T, const bigma
     carve_route_only(cv, m, b);
     alias_routing(b, out);
     cudaStream_t st = (cudaStream_t)stream;
-    BIGMAC_TRY(run_routing(L, m, x, W, b, out, st));
-    return export_routing(L, m, b, out, st);
+    return run_routing(L, m, x, W, b, out, st);
 }
 
 int bigmac_profile_enable(bigmac_layer_t* L, int on) {

@@ -355,18 +355,23 @@ constexpr int kMaxParts = 8;                        // parts of a split descend 
 // Kernel 1: top-k with gate values as topk8_kernel, four tokens per warp, plus pass 1 of the counting sort.  Block b owns
 // tokens [b TB, (b + 1) TB), TB = 4 warps iters.  Lane 8 g + j of a warp holds slot j of the warp's token g, so the lane
 // order is the slot order: ranks inside a warp by match_any, across the warps by a scan over per-warp counts.
-template <int Q>   // float4 loads per lane: E <= 32 Q
-__global__ void __launch_bounds__(1024) topk_count_kernel(const float* __restrict__ logits, int ld, int parts, int64_t part_stride,
+// AUX: also the block's column sums of the softmax over all E experts, for the load-balancing loss (launches of their own for
+// these sums, the loss and the copies of the tables put 16 us between the logits and the experts at 2999 tokens).
+constexpr int kTopkAuxWarps = 16;
+template <int Q, bool AUX>   // Q float4 loads per lane: E <= 32 Q
+__global__ void __launch_bounds__(AUX ? 32 * kTopkAuxWarps : 1024) topk_count_kernel(const float* __restrict__ logits, int ld, int parts, int64_t part_stride,
                                                           float* __restrict__ logits_out, const float* __restrict__ b_gate, int T,
                                                           int E, int k, int iters, int32_t* __restrict__ topk_idx,
                                                           float* __restrict__ topk_w, int32_t* __restrict__ local_rank,
-                                                          int32_t* __restrict__ block_counts) {
+                                                          int32_t* __restrict__ block_counts, int32_t* __restrict__ ex_idx,
+                                                          float* __restrict__ ex_w, float* __restrict__ aux_part) {
     grid_dependency_wait();
     grid_dependency_launch();
     extern __shared__ int32_t warp_run[];            // [warps][E], then [E] the block's totals so far
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5, sub = lane & 7;
     int32_t* total = warp_run + warps * E;
-    for (int i = threadIdx.x; i < (warps + 1) * E; i += blockDim.x) warp_run[i] = 0;
+    float* prob_sums = reinterpret_cast<float*>(total + E);      // AUX: [warps][E]
+    for (int i = threadIdx.x; i < (AUX ? 2 * warps + 1 : warps + 1) * E; i += blockDim.x) warp_run[i] = 0;   // (0 is 0.0f)
     __syncthreads();
     for (int it = 0; it < iters; ++it) {
         const int64_t t = ((int64_t)blockIdx.x * iters + it) * (4 * warps) + 4 * warp + (lane >> 3);
@@ -395,6 +400,30 @@ __global__ void __launch_bounds__(1024) topk_count_kernel(const float* __restric
                 taken |= 15u << (4 * i);
             }
             v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
+        }
+        if (AUX) {                                   // a token's softmax over its eight lanes, then the warp's four tokens together
+            float mx = -INFINITY, sum = 0.0f, pr[4 * Q];
+#pragma unroll
+            for (int i = 0; i < 4 * Q; ++i)
+                if (!((taken >> i) & 1u)) mx = fmaxf(mx, v[i]);
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, off));
+#pragma unroll
+            for (int i = 0; i < 4 * Q; ++i) {
+                pr[i] = !((taken >> i) & 1u) && live ? expf(v[i] - mx) : 0.0f;
+                sum += pr[i];
+            }
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) sum += __shfl_xor_sync(kFull, sum, off);
+            const float inv = live ? 1.0f / sum : 0.0f;
+#pragma unroll
+            for (int i = 0; i < 4 * Q; ++i) {
+                float p = pr[i] * inv;
+                p += __shfl_xor_sync(kFull, p, 8);
+                p += __shfl_xor_sync(kFull, p, 16);
+                const int e = 4 * (sub + 8 * (i >> 2)) + (i & 3);
+                if (lane < 8 && e < E) prob_sums[warp * E + e] += p;
+            }
         }
 #pragma unroll
         for (int i = 0; i < 4 * Q; ++i) v[i] = v[i] == v[i] ? v[i] : -INFINITY;     // NaN is ordered as -inf
@@ -445,6 +474,8 @@ __global__ void __launch_bounds__(1024) topk_count_kernel(const float* __restric
             const int64_t s = t * k + sub;
             topk_idx[s] = my_e;
             topk_w[s] = ex / part;
+            if (ex_idx) ex_idx[s] = my_e;
+            if (ex_w) ex_w[s] = ex / part;
             local_rank[s] = warp_run[warp * E + e] + __popc(peers & ((1u << lane) - 1u));
         }
         if (it + 1 < iters) {
@@ -453,7 +484,14 @@ __global__ void __launch_bounds__(1024) topk_count_kernel(const float* __restric
             __syncthreads();
         }
     }
-    for (int x = threadIdx.x; x < E; x += blockDim.x) block_counts[(size_t)blockIdx.x * E + x] = total[x];
+    for (int x = threadIdx.x; x < E; x += blockDim.x) {
+        block_counts[(size_t)blockIdx.x * E + x] = total[x];
+        if (AUX) {
+            float acc = 0.0f;
+            for (int w = 0; w < warps; ++w) acc += prob_sums[w * E + x];
+            aux_part[(size_t)blockIdx.x * E + x] = acc;
+        }
+    }
 }
 
 struct PlaceArgs {
@@ -462,6 +500,10 @@ struct PlaceArgs {
     int32_t *counts, *counts_chosen, *offsets, *poffsets, *tile_expert, *n_tiles;
     int32_t *prow_of_slot /* in: rank inside the block of kernel 1 */, *row_of_slot, *slot_of_row, *slot_of_prow;
     float* zero_word;                                // nullable: set to 0 (the loss of a layer without one)
+    RouteExport ex;
+    const float* aux_part;                           // nullable: [nb][E] sums of softmax probabilities
+    float* aux_loss;
+    float aux_coef;
     // the rows to move: [T, 16 vecs bytes] at src, or fp32 partial results [parts][T][ld] rounded to bf16
     const uint4* src;
     const float* partial;
@@ -578,6 +620,8 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p)
             }
             p.row_of_slot[s] = row;
             p.prow_of_slot[s] = prow;
+            if (p.ex.row_of_slot) p.ex.row_of_slot[s] = row;
+            if (p.ex.slot_of_row && row >= 0) p.ex.slot_of_row[row] = (int32_t)s;
         }
         if (MOVE == 0) continue;
         for (int c = lane; c - lane < p.vecs; c += 64) {
@@ -632,12 +676,50 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p)
     }
     if (p.cap < kNoCapacity)                         // rows past the kept ones exist only under a capacity limit
         for (int64_t r = s_off[E] + (int64_t)blockIdx.x * kPlaceThreads + tid; r < (int64_t)p.T * p.k; r += (int64_t)gridDim.x * kPlaceThreads)
+        {
             p.slot_of_row[r] = -1;
+            if (p.ex.slot_of_row) p.ex.slot_of_row[r] = -1;
+        }
+    if (p.aux_part && blockIdx.x == gridDim.x - 1) { // the loss, coef E sum_e f_e P_e, on the block with the fewest tokens
+        __shared__ float s_term[kPlaceMaxExperts];
+        float* sums = reinterpret_cast<float*>(s_all);
+        const int e = tid % E, part = tid / E;
+        float acc = 0.0f;
+        if (part < nparts) {
+#pragma unroll 8
+            for (int row = part; row < p.nb; row += nparts) acc += p.aux_part[(size_t)row * E + e];
+        }
+        sums[tid] = acc;
+        __syncthreads();
+        if (tid < E) {
+            float P = 0.0f;
+            for (int q = 0; q < nparts; ++q) P += sums[q * E + tid];
+            s_term[tid] = ((float)s_total[tid] / ((float)p.T * (float)p.k)) * (P / (float)p.T);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            float v = 0.0f;
+            for (int x = lane; x < E; x += 32) v += s_term[x];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+            if (lane == 0) {
+                const float loss = p.aux_coef * (float)E * v;
+                *p.aux_loss = loss;
+                if (p.ex.aux_loss) *p.ex.aux_loss = loss;
+            }
+        }
+    }
     if (blockIdx.x == 0) {
-        for (int e = tid; e <= E; e += kPlaceThreads) { p.offsets[e] = s_off[e]; p.poffsets[e] = s_poff[e]; }
+        for (int e = tid; e <= E; e += kPlaceThreads) {
+            p.offsets[e] = s_off[e];
+            p.poffsets[e] = s_poff[e];
+            if (p.ex.offsets) p.ex.offsets[e] = s_off[e];
+        }
         for (int e = tid; e < E; e += kPlaceThreads) {
             p.counts[e] = min(s_total[e], p.cap);
             if (p.counts_chosen) p.counts_chosen[e] = s_total[e];
+            if (p.ex.counts) p.ex.counts[e] = min(s_total[e], p.cap);
+            if (p.ex.counts_chosen) p.ex.counts_chosen[e] = s_total[e];
         }
         if (tid == 0) {
             *p.n_tiles = s_poff[E] / kPad;
@@ -702,8 +784,8 @@ cudaError_t launch_tables(const Tables& tb, int T, int E, int k, int cap, cudaSt
 // The two-launch form wants a lane per slot of a token, eight lanes per token, and at most 32 logits per lane.
 bool route_fused_supported(int E, int k) { return k <= 8 && E % 4 == 0 && E <= kPlaceMaxExperts; }
 
-cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, const float* b_gate, const Tables& tb, int T, int E,
-                               int k, int cap, float* zero_word, int sm_count, cudaStream_t stream, int* status,
+cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, const RouteExport& ex, const float* b_gate, const Tables& tb,
+                               int T, int E, int k, int cap, float* zero_word, int sm_count, cudaStream_t stream, int* status,
                                int which) {
     // As many blocks as there are SMs (and rows in block_counts) at most, 32 tokens in each at least: top-k is bound by
     // issue and latency inside a block, so few fat blocks are slow (128 tokens a block: 2 us more at 512 tokens), and the
@@ -711,14 +793,15 @@ cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, cons
     const int nb_max = tb.block_rows < sm_count ? tb.block_rows : sm_count;
     int per = (T + nb_max - 1) / nb_max;
     if (per < 32) per = 32;
-    const int warps = per < 128 ? (per + 3) / 4 : 32, iters = (per + 4 * warps - 1) / (4 * warps);
+    const int most = src.aux_part ? kTopkAuxWarps : 32, warps = per < 4 * most ? (per + 3) / 4 : most, iters = (per + 4 * warps - 1) / (4 * warps);
     per = 4 * warps * iters;
     const int nb = (T + per - 1) / per;
     if (which == 0) {
-        const size_t smem = sizeof(int32_t) * (size_t)(warps + 1) * E;
+        const size_t smem = sizeof(int32_t) * (size_t)(src.aux_part ? 2 * warps + 1 : warps + 1) * E;     // 33 KB at most
 #define BIGMAC_TOPK_COUNT(Q)                                                                                                       \
-    return launch_chained(topk_count_kernel<Q>, nb, warps * 32, smem, stream, src.logits, src.ld, src.parts, src.part_stride,     \
-                          src.logits_out, b_gate, T, E, k, iters, tb.topk_idx, tb.topk_w, tb.prow_of_slot, tb.block_counts)
+    return launch_chained(src.aux_part ? topk_count_kernel<Q, true> : topk_count_kernel<Q, false>, nb, warps * 32, smem, stream,   \
+                          src.logits, src.ld, src.parts, src.part_stride, src.logits_out, b_gate, T, E, k, iters, tb.topk_idx,    \
+                          tb.topk_w, tb.prow_of_slot, tb.block_counts, ex.topk_idx, ex.topk_w, src.aux_part)
         if (E <= 32) BIGMAC_TOPK_COUNT(1);
         if (E <= 64) BIGMAC_TOPK_COUNT(2);
         if (E <= 128) BIGMAC_TOPK_COUNT(4);
@@ -734,6 +817,7 @@ cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, cons
     p.counts = tb.counts; p.counts_chosen = tb.counts_chosen; p.offsets = tb.offsets; p.poffsets = tb.poffsets;
     p.tile_expert = tb.tile_expert; p.n_tiles = tb.n_tiles; p.prow_of_slot = tb.prow_of_slot; p.row_of_slot = tb.row_of_slot;
     p.slot_of_row = tb.slot_of_row; p.slot_of_prow = tb.slot_of_prow; p.zero_word = zero_word; p.status = status;
+    p.ex = ex; p.aux_part = src.aux_part; p.aux_loss = src.aux_loss; p.aux_coef = src.aux_coef;
     p.src = (const uint4*)mv.src; p.partial = mv.partial; p.parts = mv.parts; p.ld = mv.ld; p.part_stride = mv.part_stride;
     p.grouped = (uint4*)mv.grouped; p.vecs = mv.row_bytes / 16; p.zero_padding = mv.zero_padding;
     if (!mv.grouped) return launch_chained(place_kernel<0>, nb * p.splits, kPlaceThreads, 0, stream, p);
