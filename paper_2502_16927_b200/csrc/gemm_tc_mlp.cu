@@ -9,9 +9,13 @@
 //   sigma   16 epilogue warps read acc1, apply the activation and write it as bf16 to shared memory in the MN-major layout
 //           of a B operand (a[c % 2], 128 hidden x n): lane = hidden unit = contraction row, so a lane's values are adjacent
 //   GEMM2   acc2 (r x n, tensor memory, r / 128 tiles) += W2_e[:, chunk] a[c % 2]          2 r / 128 boxes
-// GEMM1 runs one chunk ahead of GEMM2.  After the last chunk acc2 leaves as rows of `out`, addressed by slot: fp32 partial
-// results [slices][slots][r], or bf16 rows where there is one slice.  The combine kernel adds a token's k slots and the
-// slices in order, so slices need no other exchange, and padding rows are never written.
+// GEMM1 runs one chunk ahead of GEMM2.  After the last chunk acc2 leaves as rows of `out`, by slot: bf16 [slots][r], or fp32 [slices][slots][r].  The
+// combine kernel adds a token's k slots and the slices in order, so slices need no other exchange, and padding rows are never
+// written.  (An issuing thread, a producer thread and a ring for either GEMM, so that their MMAs overlap: 1.9 -> 1.65 us for a
+// chunk of 128 tokens, which is what shared memory delivers operands, weights and activations at, but longer until the
+// first activation; 64 tokens 45.7 -> 47.2 us a forward, 512 53.9 -> 56.1, 3001 the same.)
+// The experts' row offsets are brought to shared memory in one round trip and looked up there: from the number of tiles to a
+// tile's expert to its rows, three dependent loads stood before the first box.
 //
 // What bounds it: few tokens, the stream of weights (67 MB at 64 experts of 2 x 256 x 1024); many tokens, the MMAs
 // (M = 128, N = 128: shared memory delivers both operands at just the rate of the tensor pipe) and the activation.
@@ -33,9 +37,9 @@ constexpr int kMlpThreads = (2 + kMlpEpiWarps) * 32;
 struct MlpParams {
     void* out;               // [slices][slots][r] fp32, or [slots][r] bf16 if there is one slice
     int64_t slots;
-    int r, h, act;
+    int r, h, act, E;
     MlpSlicing sl;
-    const int32_t *tile_expert, *n_tiles, *poffsets, *counts, *slot_of_prow;
+    const int32_t *poffsets, *counts, *slot_of_prow;
     int max_tiles;
     int* status;
 };
@@ -45,17 +49,23 @@ struct MlpItem {
     int expert, row0, rows, n, c0, chunks, slice;
 };
 
+// s_off: padded row offsets of the experts, s_pad: padding rows behind each (both in shared memory)
 template <int NT>
-__device__ __forceinline__ MlpItem mlp_item(const MlpParams& p, int tiles, int slices, int i) {
+__device__ __forceinline__ MlpItem mlp_item(const MlpParams& p, int tiles, int slices, const int32_t* s_off, const uint8_t* s_pad, int i) {
     // all first halves of the tiles come before the second ones (NT = 64), most of which are empty where experts are short
     MlpItem t;
-    const int half = NT < 128 && i >= tiles * slices ? 1 : 0, j = i - half * tiles * slices, tile = j / slices;
+    const int half = NT < 128 && i >= tiles * slices ? 1 : 0, j = i - half * tiles * slices, tile = j >> (__ffs(slices) - 1);
     t.slice = j - tile * slices;
-    t.expert = p.tile_expert[tile];
     t.row0 = tile * kPad + half * NT;
-    t.rows = min(NT, p.poffsets[t.expert] + p.counts[t.expert] - t.row0);
+    int lo = 0, hi = p.E;                                // largest expert whose rows begin at or before the tile
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (s_off[mid] <= tile * kPad) lo = mid; else hi = mid;
+    }
+    t.expert = lo;
+    t.rows = min(NT, s_off[lo + 1] - (int)s_pad[lo] - t.row0);
     t.n = t.rows > 0 ? (t.rows + 15) / 16 * 16 : 0;
-    t.chunks = p.sl.chunks / slices;
+    t.chunks = p.sl.chunks >> (__ffs(slices) - 1);
     t.c0 = t.slice * t.chunks;
     return t;
 }
@@ -83,6 +93,8 @@ fused_mlp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     uint64_t* acc2_full = x_full + 10;  uint64_t* acc2_empty = x_full + 11;
     uint32_t* tmem_slot = (uint32_t*)(x_full + 12);
     volatile int* dead = (volatile int*)(tmem_slot + 1);
+    int32_t* s_off = (int32_t*)(tmem_slot + 4);          // [E + 1]
+    uint8_t* s_pad = (uint8_t*)(s_off + p.E + 1);        // [E]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 32) {                             // the maps are on their way while the barriers are set up
@@ -111,8 +123,13 @@ fused_mlp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     // from the wait on, the predecessor's results are complete.
     grid_dependency_launch();
     grid_dependency_wait();
+    for (int e = threadIdx.x; e <= p.E; e += kMlpThreads) {
+        s_off[e] = p.poffsets[e];
+        if (e < p.E) s_pad[e] = (uint8_t)((kPad - p.counts[e] % kPad) % kPad);
+    }
+    __syncthreads();
     const uint32_t tmem_base = *tmem_slot, acc2_tmem = tmem_base + 2 * NT;
-    const int tiles = min(*p.n_tiles, p.max_tiles), slices = mlp_slices(p.sl, tiles), total = tiles * (128 / NT) * slices;
+    const int tiles = min(s_off[p.E] / kPad, p.max_tiles), slices = mlp_slices(p.sl, tiles), total = tiles * (128 / NT) * slices;
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer: X once per item, then the weight boxes
@@ -125,7 +142,7 @@ fused_mlp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 if (++s == STAGES) { s = 0; phase ^= 1; }
             };
             for (int i = blockIdx.x; i < total; i += gridDim.x) {
-                const MlpItem t = mlp_item<NT>(p, tiles, slices, i);
+                const MlpItem t = mlp_item<NT>(p, tiles, slices, s_off, s_pad, i);
                 if (t.n == 0) continue;
                 mbar_wait_lean(x_empty, (local & 1) ^ 1, dead, p.status);
                 ++local;
@@ -149,7 +166,7 @@ fused_mlp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             const uint64_t d_act = smem_desc(smem_u32(s_act), HC * 128, 1024);   // MN-major, 64-token blocks HC rows of 128 bytes apart
             uint32_t s = 0, phase = 0, g = 0, local = 0; // g: chunks so far, over all items
             for (int i = blockIdx.x; i < total; i += gridDim.x) {
-                const MlpItem t = mlp_item<NT>(p, tiles, slices, i);
+                const MlpItem t = mlp_item<NT>(p, tiles, slices, s_off, s_pad, i);
                 if (t.n == 0) continue;
                 const uint32_t idesc1 = instr_desc(t.n, false, false), idesc2 = instr_desc(t.n, false, true);
                 mbar_wait_lean(x_full, local & 1, dead, p.status);
@@ -203,7 +220,7 @@ fused_mlp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         const int hid = quad * 32 + lane;                      // hidden unit of the chunk = contraction row of GEMM2
         uint32_t g = 0, local = 0;
         for (int i = blockIdx.x; i < total; i += gridDim.x) {
-            const MlpItem t = mlp_item<NT>(p, tiles, slices, i);
+            const MlpItem t = mlp_item<NT>(p, tiles, slices, s_off, s_pad, i);
             if (t.n == 0) continue;
             // lane l keeps the slot of token 16 (part + 4 (l / 16)) + l % 16 of the tile, for the stores at the end
             const int tok = 16 * (part + 4 * (lane >> 4)) + (lane & 15);
@@ -290,7 +307,8 @@ fused_mlp_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
 template <int NT, int STAGES>
 cudaError_t launch(const CUtensorMap& mx, const CUtensorMap& m1, const CUtensorMap& m2, const MlpParams& p, cudaStream_t stream) {
     const size_t smem = (size_t)STAGES * BOX_BYTES + 2 * (size_t)(NT / 64) * HC * 128 + (size_t)(p.r / BK) * NT * BK * 2 +
-                        (2 * STAGES + 12) * 8 + 16 + 1024;
+                        (2 * STAGES + 12) * 8 + 16 + (size_t)(p.E + 1) * 4 + p.E + 1024;
+    if (smem > 232448) return cudaErrorInvalidConfiguration;
     static PerDeviceOnce once;
     int dev;
     if (once.needed(&dev)) {
@@ -310,7 +328,8 @@ bool fused_mlp_supported(int r, int h, int dtype) {
 
 // Slices are limited to what fits the activation buffer [P, h] of bf16 that the separate GEMMs would use.
 MlpSlicing fused_mlp_slicing(int r, int h, int64_t N, int64_t P) {
-    MlpSlicing m{sm_count(), (h + HC - 1) / HC, 1, r <= 256 ? 1 : 2};
+    const int units = sm_count();
+    MlpSlicing m{units, (h + HC - 1) / HC, 1, r <= 256 ? 1 : 2, ((1ull << 40) + units - 1) / units};
     while (m.most < 8 && 2 * m.most * N * r * 4 <= P * h * 2) m.most *= 2;
     return m;
 }
@@ -326,10 +345,12 @@ cudaError_t launch_fused_mlp(const void* xg, const void* w1, const void* w2, voi
     ok &= make_map(&m2, w2, (uint64_t)h, (uint64_t)E * r, (uint64_t)h, BK, 128);
     if (!ok) return cudaErrorInvalidValue;
     MlpParams p{};
-    p.out = out; p.slots = slots; p.r = r; p.h = h; p.act = act; p.sl = sl;
-    p.tile_expert = tb.tile_expert; p.n_tiles = tb.n_tiles; p.poffsets = tb.poffsets; p.counts = tb.counts; p.slot_of_prow = tb.slot_of_prow;
+    p.out = out; p.E = E; p.slots = slots; p.r = r; p.h = h; p.act = act; p.sl = sl;
+    p.poffsets = tb.poffsets; p.counts = tb.counts; p.slot_of_prow = tb.slot_of_prow;
     p.max_tiles = (int)(max_rows / kPad); p.status = status;
-    return r <= 256 ? launch<128, 6>(mx, m1, m2, p, stream) : launch<64, 8>(mx, m1, m2, p, stream);
+    // the tables of more than 300 experts take the place of a stage
+    if (r <= 256) return E <= 300 ? launch<128, 6>(mx, m1, m2, p, stream) : launch<128, 5>(mx, m1, m2, p, stream);
+    return E <= 300 ? launch<64, 8>(mx, m1, m2, p, stream) : launch<64, 7>(mx, m1, m2, p, stream);
 }
 
 }  // namespace bigmac

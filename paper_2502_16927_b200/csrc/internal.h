@@ -125,17 +125,19 @@ struct MlpSlicing {
     int chunks;      // 128-wide chunks of the hidden width
     int most;        // slices that the output buffer has room for
     int per_tile;    // work items per 128-row tile and slice
+    unsigned long long inv;   // 2^40 / units, rounded up: division by a multiplication (exact below 2^40 / units^2)
 };
 // The slices s (a power of two that divides the chunks) with the shortest longest SM: rounds of items, times an item's
 // chunks and what its start and its output take in units of a chunk (fp32 partial results: twice the bytes of bf16).
 // Few tiles: more slices put idle SMs to work (64 tiles of 8 chunks: two slices, 17 -> 12 us); more than one tile per SM:
-// one slice (220 tiles of 8 chunks: the fp32 rows of two slices cost what the better last round gains).
-__host__ __device__ inline int mlp_slices(const MlpSlicing& m, int tiles) {
+// one slice (220 tiles of 8 chunks: the fp32 rows of two slices cost what the better last round gains; so does leaving the whole
+// rounds uncut and cutting the rest only, 88 -> 90 us at 3001 tokens and no difference up to 13000).
+__device__ __forceinline__ int mlp_slices(const MlpSlicing& m, int tiles) {
     int best = 1, best_cost = 0x7fffffff;
-    for (int s = 1; s <= m.most && m.chunks % s == 0; s *= 2) {
-        const long long items = (long long)tiles * m.per_tile * s;
-        const long long cost = (items + m.units - 1) / m.units * (m.chunks / s + (s > 1 ? 3 : 2));
-        if (cost < best_cost) { best = s; best_cost = (int)(cost < 0x7ffffffe ? cost : 0x7ffffffe); }
+    for (int j = 0; (1 << j) <= m.most && !(m.chunks & ((1 << j) - 1)); ++j) {
+        const int rounds = (int)(((unsigned)(tiles * m.per_tile << j) + m.units - 1) * m.inv >> 40);
+        const int cost = rounds * ((m.chunks >> j) + (j > 0 ? 3 : 2));
+        if (cost < best_cost) { best = 1 << j; best_cost = cost; }
     }
     return best;
 }

@@ -370,7 +370,11 @@ GemmArgs dw1_request(const Dims& m, const void* dz, const void* rows, const Tabl
 bool uses_fused_mlp(const bigmac_layer* L, const Dims& m) {
     const int mode = switches().fused_mlp;
     if (mode == 0 || m.bias || !sigma_as_bytes(L) || !fused_mlp_supported(m.r, m.h, m.dtype) || m.N * m.r * 4 > m.P * m.h * 2) return false;
-    return mode == 2 || m.P / kPad <= 2 * (int64_t)gemm_tc_sm_count();
+    if (mode == 2) return true;
+    // r <= 256: always.  Wider rows leave room for 64 tokens in tensor memory, and the weights are streamed again for every 64
+    // tokens of an expert: as long as most experts have one such unit (d 4096, 128 experts, r 512: 600 tokens 139 us, separate
+    // contractions 183; 1200 tokens 208 and 190).
+    return m.r <= 256 || m.N <= 48 * (int64_t)m.E;
 }
 
 // Is the dispatch fused into its consumers' operand loads (F5 of the forward disappears as a launch, the grouped
@@ -561,10 +565,12 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
         g.A = x; g.lda = m.d; g.B = W->w_down; g.ldb = m.d; g.C = b.x_lo; g.ldc = m.r;
         g.B2 = W->w_gate; g.ldb2 = m.d; g.n_split = m.r; g.C2 = b.logits; g.ldc2 = m.E; g.N2 = m.E;
         g.M = m.T; g.N = m.r + m.E; g.K = m.d;
-        // Where a batch touches nearly all experts (two slots for each), their weights stream from DRAM to L2 while the
-        // routing runs, which leaves memory idle for 20 us.  Up to 80 MB: beside the rest they fit in L2 (126 MB).
+        // Where a batch touches nearly all experts (two slots for each) and its experts are bound by the stream of their
+        // weights (up to 128 rows each), the weights come from DRAM to L2 while the routing runs, which leaves memory idle for
+        // 20 us.  Up to 80 MB: beside the rest they fit in L2 (126 MB).  At 3001 tokens, 375 rows an expert, the hint only
+        // slowed the descend launch (13 -> 19 us).
         const size_t expert_bytes = (size_t)m.E * m.h * m.r * esize(m.dtype);
-        if (!training && uses_fused_mlp(L, m) && m.N >= 2 * (int64_t)m.E && 2 * expert_bytes <= ((size_t)80 << 20)) {
+        if (!training && uses_fused_mlp(L, m) && m.N >= 2 * (int64_t)m.E && m.N <= 128 * (int64_t)m.E && 2 * expert_bytes <= ((size_t)80 << 20)) {
             g.prefetch[0] = W->w1; g.prefetch[1] = W->w2; g.prefetch_bytes = expert_bytes;
         }
         if (b.descend_ws) {                                   // few tokens: contraction in parts, added by the routing kernels
