@@ -355,6 +355,10 @@ constexpr int kMaxParts = 8;                        // parts of a split descend 
 // Kernel 1: top-k with gate values as topk8_kernel, four tokens per warp, plus pass 1 of the counting sort.  Block b owns
 // tokens [b TB, (b + 1) TB), TB = 4 warps iters.  Lane 8 g + j of a warp holds slot j of the warp's token g, so the lane
 // order is the slot order: ranks inside a warp by match_any, across the warps by a scan over per-warp counts.
+// Rounds of arg-max over a token's eight lanes: a lane keeps the maxima of its Q quads in registers and the quads themselves in
+// shared memory, where the winner alone strikes its element out (NaN: never a maximum, never equal) and looks its quad over
+// again.  With the values in registers every lane scanned all of them in every round: issue slots bound the kernel, 34 us at
+// 32768 tokens of 128 experts.
 // AUX: also the block's column sums of the softmax over all E experts, for the load-balancing loss (launches of their own for
 // these sums, the loss and the copies of the tables put 16 us between the logits and the experts at 2999 tokens).
 constexpr int kTopkAuxWarps = 16;
@@ -371,6 +375,7 @@ __global__ void __launch_bounds__(AUX ? 32 * kTopkAuxWarps : 1024) topk_count_ke
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5, sub = lane & 7;
     int32_t* total = warp_run + warps * E;
     float* prob_sums = reinterpret_cast<float*>(total + E);      // AUX: [warps][E]
+    float4* quads = reinterpret_cast<float4*>(prob_sums + (AUX ? warps * E : 0)) + threadIdx.x;   // [Q][threads]; E is a multiple of 4
     for (int i = threadIdx.x; i < (AUX ? 2 * warps + 1 : warps + 1) * E; i += blockDim.x) warp_run[i] = 0;   // (0 is 0.0f)
     __syncthreads();
     for (int it = 0; it < iters; ++it) {
@@ -378,7 +383,7 @@ __global__ void __launch_bounds__(AUX ? 32 * kTopkAuxWarps : 1024) topk_count_ke
         const bool live = t < T;
         const float* row = logits + (live ? t : 0) * ld;
         float v[4 * Q];
-        uint32_t taken = 0;                          // bit i: this lane's i-th expert already chosen (or past E)
+        uint32_t past = 0;                           // bit i: this lane's i-th expert is past E
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const int e0 = 4 * (sub + 8 * i);
@@ -397,7 +402,7 @@ __global__ void __launch_bounds__(AUX ? 32 * kTopkAuxWarps : 1024) topk_count_ke
                 if (logits_out && live) *reinterpret_cast<float4*>(logits_out + t * E + e0) = x;
                 if (b_gate) { x.x += b_gate[e0]; x.y += b_gate[e0 + 1]; x.z += b_gate[e0 + 2]; x.w += b_gate[e0 + 3]; }
             } else {
-                taken |= 15u << (4 * i);
+                past |= 15u << (4 * i);
             }
             v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
         }
@@ -405,12 +410,12 @@ __global__ void __launch_bounds__(AUX ? 32 * kTopkAuxWarps : 1024) topk_count_ke
             float mx = -INFINITY, sum = 0.0f, pr[4 * Q];
 #pragma unroll
             for (int i = 0; i < 4 * Q; ++i)
-                if (!((taken >> i) & 1u)) mx = fmaxf(mx, v[i]);
+                if (!((past >> i) & 1u)) mx = fmaxf(mx, v[i]);
 #pragma unroll
             for (int off = 4; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, off));
 #pragma unroll
             for (int i = 0; i < 4 * Q; ++i) {
-                pr[i] = !((taken >> i) & 1u) && live ? expf(v[i] - mx) : 0.0f;
+                pr[i] = !((past >> i) & 1u) && live ? expf(v[i] - mx) : 0.0f;
                 sum += pr[i];
             }
 #pragma unroll
@@ -425,26 +430,52 @@ __global__ void __launch_bounds__(AUX ? 32 * kTopkAuxWarps : 1024) topk_count_ke
                 if (lane < 8 && e < E) prob_sums[warp * E + e] += p;
             }
         }
+        const float none = __int_as_float(0x7fffffff);
+        float most[Q];                               // maximum of each quad
 #pragma unroll
-        for (int i = 0; i < 4 * Q; ++i) v[i] = v[i] == v[i] ? v[i] : -INFINITY;     // NaN is ordered as -inf
+        for (int i = 0; i < 4 * Q; ++i) v[i] = (past >> i) & 1u ? none : v[i] == v[i] ? v[i] : -INFINITY;     // NaN is ordered as -inf
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            most[q] = fmaxf(fmaxf(v[4 * q], v[4 * q + 1]), fmaxf(v[4 * q + 2], v[4 * q + 3]));
+            quads[q * blockDim.x] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        }
         float my_v = -INFINITY;
         int my_e = 0;
         for (int j = 0; j < k; ++j) {
-            float best = -INFINITY;
-            int best_e = kNoExpert;
+            float mine = most[0];
 #pragma unroll
-            for (int i = 0; i < 4 * Q; ++i) {        // ascending expert id within the lane: strict > keeps the lowest id
-                const int e = 4 * (sub + 8 * (i >> 2)) + (i & 3);
-                if (!((taken >> i) & 1u) && (best_e == kNoExpert || v[i] > best)) { best = v[i]; best_e = e; }
-            }
+            for (int q = 1; q < Q; ++q) mine = fmaxf(mine, most[q]);
+            float best = mine;
 #pragma unroll
-            for (int off = 4; off > 0; off >>= 1) {
-                const float ov = __shfl_xor_sync(kFull, best, off);
-                const int oe = __shfl_xor_sync(kFull, best_e, off);
-                if (ov > best || (ov == best && oe < best_e)) { best = ov; best_e = oe; }
+            for (int off = 4; off > 0; off >>= 1) best = fmaxf(best, __shfl_xor_sync(kFull, best, off));
+            bool wins = mine == best;
+            int e = kNoExpert, at = 0, c = 0;
+            float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (wins) {                              // its lowest expert id with that value: ids ascend with the quad and inside it
+#pragma unroll
+                for (int q = Q - 1; q >= 0; --q) at = most[q] == best ? q : at;
+                x = quads[at * blockDim.x];
+                c = x.x == best ? 0 : x.y == best ? 1 : x.z == best ? 2 : 3;
+                e = 4 * (sub + 8 * at) + c;
             }
-            if (((best_e >> 2) & 7) == sub) taken |= 1u << (((best_e >> 5) << 2) | (best_e & 3));
-            if (sub == j) { my_v = best; my_e = best_e; }
+            const unsigned votes = __ballot_sync(kFull, wins), group = (votes >> (lane & 24)) & 0xffu;
+            int from = __ffs(group) - 1;
+            if (__any_sync(kFull, __popc(group) > 1)) {      // equal logits in several lanes: the lowest id of all
+                int low = e;
+#pragma unroll
+                for (int off = 4; off > 0; off >>= 1) low = min(low, __shfl_xor_sync(kFull, low, off));
+                wins = wins && e == low;
+                from = (low >> 2) & 7;
+            }
+            if (wins) {
+                x.x = c == 0 ? none : x.x; x.y = c == 1 ? none : x.y; x.z = c == 2 ? none : x.z; x.w = c == 3 ? none : x.w;
+                quads[at * blockDim.x] = x;
+                const float left = fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w));
+#pragma unroll
+                for (int q = 0; q < Q; ++q) most[q] = at == q ? left : most[q];
+            }
+            const int chosen = __shfl_sync(kFull, e, (lane & 24) + from);
+            if (sub == j) { my_v = best; my_e = chosen; }
         }
         const float top = __shfl_sync(kFull, my_v, lane & 24);
         const float ex = sub < k ? (top == -INFINITY ? 1.0f : expf(my_v - top)) : 0.0f;
@@ -666,11 +697,11 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p)
     const int share = max(1, (int)gridDim.x / E);    // blocks per expert
     for (int e = blockIdx.x / share; e < E; e += gridDim.x / share) {
         const int r0 = s_poff[e] + (s_off[e + 1] - s_off[e]), r1 = s_poff[e + 1];
-        for (int r = r0 + (int)(blockIdx.x % share) * kWarps + warp; r < r1; r += share * kWarps) {
-            if (lane == 0) p.slot_of_prow[r] = -1;
-            if (MOVE != 0 && p.zero_padding)
+        if (MOVE == 0 || p.zero_padding)             // (nothing after the dispatch of an inference forward looks at a padding row)
+            for (int r = r0 + (int)(blockIdx.x % share) * kPlaceThreads + tid; r < r1; r += share * kPlaceThreads) p.slot_of_prow[r] = -1;
+        if (MOVE != 0 && p.zero_padding)
+            for (int r = r0 + (int)(blockIdx.x % share) * kWarps + warp; r < r1; r += share * kWarps)
                 for (int c = lane; c < p.vecs; c += 32) p.grouped[(int64_t)r * p.vecs + c] = make_uint4(0, 0, 0, 0);
-        }
         if (blockIdx.x % share == 0)
             for (int tile = s_poff[e] / kPad + tid; tile < s_poff[e + 1] / kPad; tile += kPlaceThreads) p.tile_expert[tile] = e;
     }
@@ -797,11 +828,23 @@ cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, cons
     per = 4 * warps * iters;
     const int nb = (T + per - 1) / per;
     if (which == 0) {
-        const size_t smem = sizeof(int32_t) * (size_t)(src.aux_part ? 2 * warps + 1 : warps + 1) * E;     // 33 KB at most
+        const int quads = E <= 32 ? 1 : E <= 64 ? 2 : E <= 128 ? 4 : 8;          // 160 KB at most
+        const size_t smem = sizeof(int32_t) * (size_t)(src.aux_part ? 2 * warps + 1 : warps + 1) * E + (size_t)quads * warps * 32 * sizeof(float4);
 #define BIGMAC_TOPK_COUNT(Q)                                                                                                       \
-    return launch_chained(src.aux_part ? topk_count_kernel<Q, true> : topk_count_kernel<Q, false>, nb, warps * 32, smem, stream,   \
-                          src.logits, src.ld, src.parts, src.part_stride, src.logits_out, b_gate, T, E, k, iters, tb.topk_idx,    \
-                          tb.topk_w, tb.prow_of_slot, tb.block_counts, ex.topk_idx, ex.topk_w, src.aux_part)
+    do {                                                                                                                           \
+        const auto kernel = src.aux_part ? topk_count_kernel<Q, true> : topk_count_kernel<Q, false>;                              \
+        static PerDeviceOnce once;                                                                                                 \
+        int dev;                                                                                                                   \
+        if (once.needed(&dev)) {                                                                                                   \
+            cudaError_t e = cudaFuncSetAttribute(topk_count_kernel<Q, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 163840); \
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_count_kernel<Q, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 172032); \
+            if (e != cudaSuccess) return e;                                                                                        \
+            once.mark(dev);                                                                                                        \
+        }                                                                                                                          \
+        return launch_chained(kernel, nb, warps * 32, smem, stream, src.logits, src.ld, src.parts, src.part_stride,               \
+                              src.logits_out, b_gate, T, E, k, iters, tb.topk_idx, tb.topk_w, tb.prow_of_slot, tb.block_counts,    \
+                              ex.topk_idx, ex.topk_w, src.aux_part);                                                               \
+    } while (0)
         if (E <= 32) BIGMAC_TOPK_COUNT(1);
         if (E <= 64) BIGMAC_TOPK_COUNT(2);
         if (E <= 128) BIGMAC_TOPK_COUNT(4);

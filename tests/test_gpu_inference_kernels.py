@@ -92,3 +92,27 @@ def test_routing_in_two_launches(E, k, T):
         assert layer.status() == 0
         _check_tables(R, oracle.route(inp, w.k, capacity_factor=f))
         layer.close()
+
+
+@pytest.mark.parametrize("E,k", [(4, 4), (36, 8), (64, 8), (128, 8), (256, 8)])
+def test_equal_and_nonfinite_logits(E, k):
+    """Logits that are nothing but the gate bias: a handful of values that many experts share (in one lane's quad, across its
+    quads, across lanes), both zeros, infinities and NaN: order by value, then by id, NaN as -inf."""
+    import torch
+
+    T = 70
+    w = wl.Workload("ties", T=T, d=32, r=8, h=8, E=E, k=k, dtype=wl.DTYPE_F32, act=wl.ACT_RELU, seed=3)
+    inp = wl.make_inputs(w)
+    inp["x"] = np.zeros_like(inp["x"])
+    rng = np.random.default_rng(E)
+    for values in ([1.0], [0.0, -0.0, -1.0], [2.0, 2.0, -3.0], [-np.inf, np.nan], [np.inf, 1.0, np.nan, -np.inf]):
+        bias = rng.choice(np.array(values, dtype=np.float32), E)
+        inp["b_gate"] = bias
+        layer = make_layer(w)
+        R = layer.route(to_device(w, inp)["x"], to_device(w, inp))
+        torch.cuda.synchronize()
+        assert layer.status() == 0
+        key = np.where(np.isnan(bias), -np.inf, bias)
+        want = np.array(sorted(range(E), key=lambda e: (-key[e], e))[:k])
+        np.testing.assert_array_equal(to_numpy(R["topk_idx"]).reshape(T, k), np.tile(want, (T, 1)))
+        layer.close()
