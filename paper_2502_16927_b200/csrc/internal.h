@@ -19,16 +19,23 @@ namespace bigmac {
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// chained = false: a plain launch, which takes no place on an SM before its predecessor is done (the place may be of use to
+// a kernel of another stream).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+inline cudaError_t launch_maybe_chained(bool chained, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                   Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = switches().chain ? 1 : 0;
+    cfg.attrs = attr; cfg.numAttrs = chained && switches().chain ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                  Args&&... args) {
+    return launch_maybe_chained(true, kernel, grid, block, smem, stream, static_cast<Args&&>(args)...);
 }
 #endif
 
@@ -252,7 +259,7 @@ cudaError_t launch_combine_parts(const void* parts, const MlpSlicing& sl, const 
                                  const int32_t* prow_of_slot, int T, int k, int width, cudaStream_t stream, bool may_drop);
 // Backward of the combine: du[prow,:] = p[s] * dy_lo[t,:] (zeros on padding), dp[s] = <dy_lo[t,:], u[prow,:]>.
 cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float* dp, const Tables& tb, int k,
-                               int width, int dtype, int64_t max_prows, cudaStream_t stream);
+                               int width, int dtype, int64_t max_prows, cudaStream_t stream, bool chained = true);
 // Softmax-over-k backward: g = sum_i p_i dp_i, dl_j = p_j (dp_j - g); writes the dense [T,E] matrix
 // (zeros off the top-k set, and in the padding columns E..width-1) in the dtype, rows `ld` elements apart, and
 // leaves the fp32 dl_j in dp[slot].  may_drop: the dp of a slot without a row (prow_of_slot < 0) is taken as 0.

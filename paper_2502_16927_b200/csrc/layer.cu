@@ -37,7 +37,9 @@ struct Buffers {
     float* aux_part;     // [kAuxChunks, E] (the fused routing: [block_rows, E] of it) forward scratch of the load-balancing loss
     float* aux_loss;     // [1] saved: L_aux of the batch
     float* logits_saved; // [T,E] saved copy of the gate logits (only with a load-balancing loss)
-    float* splitk_ws;    // fp32 partial results of the split weight-gradient contractions
+    // fp32 partial results, apart because their users run on different streams: of the split dense weight gradients on the
+    // caller's stream, of dW_up, and of the parts of long experts in dW1 / dW2
+    float *splitk_ws, *up_ws, *expert_ws;
     float* descend_ws;   // few tokens: fp32 partial results [parts][T][r + E] of the split descend + logits launch
     float* bias_ws;      // fp32 row-slice sums of the expert-bias gradients (a region of their own: they run on the second stream)
 };
@@ -121,11 +123,12 @@ void carve_backward_scratch(Carver& cv, const Dims& m, Buffers& b) {
     b.dlogits = (b.dcat && !m.cdac) ? (char*)b.dcat + (size_t)m.r * es : b.dcat;
     b.dp = cv.take<float>(m.N);
     b.colsum_part = cv.take<float>((size_t)(kColsumChunks + kAuxChunks) * m.E);
-    // fp32 partial results: of the split dense contractions, and of the parts of long experts in dW1 / dW2
     const size_t dense_ws = (size_t)kMaxSplitK * m.ldcat * m.d * sizeof(float);
     const size_t expert_ws = m.dtype == BIGMAC_BF16 ? gemm_tc_groupk_ws_bytes(m.r, m.h, m.E) : 0;
     const size_t bias_ws = m.bias ? (size_t)m.E * kColsumSlices * (m.h > m.r ? m.h : m.r) * sizeof(float) : 0;
-    b.splitk_ws = (float*)cv.take_bytes(dense_ws > expert_ws ? dense_ws : expert_ws);
+    b.splitk_ws = (float*)cv.take_bytes(dense_ws);
+    b.up_ws = m.cdac ? nullptr : cv.take<float>((size_t)kMaxSplitK * m.r * m.d);
+    b.expert_ws = expert_ws ? (float*)cv.take_bytes(expert_ws) : nullptr;
     b.bias_ws = bias_ws ? (float*)cv.take_bytes(bias_ws) : nullptr;
 }
 
@@ -691,9 +694,9 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
     const bigmac_config_t& c = L->cfg;
     const bool acc = accumulate != 0;
 
-    // Overlap (the overlap debug switch turns it off): dW_up, the gate backward with the bias-gradient column sums, the dx' gather
-    // and [dW_down ; dW_gate] go to a second stream, forked from and joined back into the caller's stream with events, so that they run beside launches they
-    // do not depend on.  Everything that shares the fp32 workspace stays ordered.
+    // Overlap (the overlap debug switch turns it off): dW_up, the gate bias's column sums and dW1 go to a second stream, forked
+    // from and joined back into the caller's stream with events, so that they run beside launches they do not depend on and that
+    // leave a part of the chip; each stream has fp32 workspaces of its own.
     const bool overlap_on = switches().overlap != 0;
     // (not while per-stage events are recorded: a stage timed beside another stream's launches would not be its own time)
     // (nor on the FMA path, which puts what could overlap into one launch)
@@ -721,41 +724,34 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         g.A = dy; g.lda = m.d; g.a_kmajor = false; g.B = b.y_lo; g.ldb = m.r; g.b_kmajor = false;
         g.C = G->dw_up; g.ldc = m.r; g.M = m.d; g.N = m.r; g.K = m.T; g.accumulate = acc;
         if (fused) {   // contraction over all tokens, few output tiles: split it, reduce the parts in order
-            g.split_k = choose_split_k(g.M, g.N, g.K); g.C = b.splitk_ws; g.out_f32 = true; g.accumulate = false;
+            g.split_k = choose_split_k(g.M, g.N, g.K); g.C = b.up_ws; g.out_f32 = true; g.accumulate = false;
             BIGMAC_TRY(gemm(L, G_DW_UP, g, sd));
             Stage s(L, S_SPLITK_REDUCE, sd);
-            BIGMAC_CUDA(launch_splitk_reduce(b.splitk_ws, g.split_k, m.d, m.r, G->dw_up, m.d, nullptr, 0, m.dtype, acc, sd));
+            BIGMAC_CUDA(launch_splitk_reduce(b.up_ws, g.split_k, m.d, m.r, G->dw_up, m.d, nullptr, 0, m.dtype, acc, sd));
         } else {
             BIGMAC_TRY(together.add(G_DW_UP, g, sd));
         }
     }
     BIGMAC_TRY(together.flush());
-    if (overlap) BIGMAC_CUDA(cudaEventRecord(L->fork_join[1], sd));          // dW_up done: the fp32 workspace is free again
-    // du = p dy'[t], dp = <dy'[t], u>; then the softmax-over-k backward
-    { Stage s(L, S_COMBINE_BWD, st); BIGMAC_CUDA(launch_combine_bwd(b.dy_lo, b.u, b.du, b.dp, b.tb, m.k, m.r, m.dtype, m.P, st)); }
-    // The gate backward (dp -> dl) and the gate-bias column sums feed only dx, dW_gate and db_gate at the end of the pass:
-    // with the second stream they run beside the expert contractions instead of in front of them.
-    if (overlap) {
-        BIGMAC_CUDA(cudaEventRecord(L->fork_join[2], st));
-        BIGMAC_CUDA(cudaStreamWaitEvent(sd, L->fork_join[2], 0));
-    }
+    // du = p dy'[t], dp = <dy'[t], u>; then the softmax-over-k backward.  Chained to dy', the first would hold every SM's thread
+    // slots while it waits, and dW_up would find none beside a dy' of a few CTAs (2999 tokens: 48).
+    { Stage s(L, S_COMBINE_BWD, st); BIGMAC_CUDA(launch_combine_bwd(b.dy_lo, b.u, b.du, b.dp, b.tb, m.k, m.r, m.dtype, m.P, st, !overlap)); }
     float* aux_part = nullptr;                                                    // column sums of dL_aux/dl, for db_gate
     if (m.aux > 0) {
         aux_part = b.colsum_part + (size_t)kColsumChunks * m.E;
-        Stage s(L, S_GATE_BWD, sd);
+        Stage s(L, S_GATE_BWD, st);
         BIGMAC_CUDA(launch_gate_bwd_aux(b.dp, b.tb, b.dlogits, b.logits_saved, W->b_gate, m.aux, aux_part, m.T, m.E, m.E64,
-                                        ldcat, m.k, m.dtype, sd, m.cap != kNoCapacity));
+                                        ldcat, m.k, m.dtype, st, m.cap != kNoCapacity));
     } else {
-        Stage s(L, S_GATE_BWD, sd);
-        BIGMAC_CUDA(launch_gate_bwd(b.dp, b.tb, b.dlogits, m.T, m.E, m.E64, ldcat, m.k, m.dtype, sd, m.cap != kNoCapacity));
+        Stage s(L, S_GATE_BWD, st);
+        BIGMAC_CUDA(launch_gate_bwd(b.dp, b.tb, b.dlogits, m.T, m.E, m.E64, ldcat, m.k, m.dtype, st, m.cap != kNoCapacity));
     }
     bool colsum_done = false;
-    if (overlap) {
-        if (G->db_gate) {
-            Stage s(L, S_COLSUM, sd, 2);
-            BIGMAC_CUDA(launch_gate_colsum(b.dp, b.tb, G->db_gate, b.colsum_part, m.N, m.E, acc, sd, aux_part));
-        }
-        BIGMAC_CUDA(cudaEventRecord(L->fork_join[3], sd));
+    if (overlap && G->db_gate) {
+        BIGMAC_CUDA(cudaEventRecord(L->fork_join[2], st));
+        BIGMAC_CUDA(cudaStreamWaitEvent(sd, L->fork_join[2], 0));
+        Stage s(L, S_COLSUM, sd, 2);
+        BIGMAC_CUDA(launch_gate_colsum(b.dp, b.tb, G->db_gate, b.colsum_part, m.N, m.E, acc, sd, aux_part));
         colsum_done = true;
     }
     {   // dz = (du W2_e) * sigma'(z); the forward saved sigma'(z) in the z buffer, dz is written over it
@@ -767,7 +763,6 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         BIGMAC_TRY(gemm(L, G_DZ, g, st));
     }
     void* dz = b.dz ? b.dz : b.z;
-    if (overlap) BIGMAC_CUDA(cudaStreamWaitEvent(st, L->fork_join[1], 0));    // from here on the fp32 workspace is used again
     if (m.bias) {   // db1_e = sum_rows dz[row,:], db2_e = sum_rows du[row,:]  (padding rows hold zeros)
         // Two HBM-bound passes over dz and du that nothing later in the pass reads: with the second stream they run
         // beside the tensor-bound dW2 / dxg (joined with the dx' gather), on slice sums in a region of their own.
@@ -786,7 +781,7 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         g.A = b.du; g.lda = m.r; g.a_kmajor = false; g.B = b.a; g.ldb = m.h; g.b_kmajor = false;
         g.C = G->dw2; g.ldc = m.h; g.c_stride = (int64_t)m.r * m.h; g.M = m.r; g.N = m.h; g.K = (int)m.P;
         g.group = GROUP_K; g.num_experts = m.E; g.poffsets = b.tb.poffsets; g.accumulate = acc;
-        BIGMAC_TRY(batch ? together.add(G_DW2, g, st) : expert_weight_grad(L, G_DW2, g, b.splitk_ws, st));
+        BIGMAC_TRY(batch ? together.add(G_DW2, g, st) : expert_weight_grad(L, G_DW2, g, b.expert_ws, st));
     }
     {   // dxg = dz W1_e
         GemmArgs g;
@@ -795,21 +790,19 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         g.group = GROUP_M; g.num_experts = m.E; g.tile_expert = b.tb.tile_expert; g.n_tiles = b.tb.n_tiles; g.poffsets = b.tb.poffsets;
         BIGMAC_TRY(together.add(G_DXG, g, st));
     }
-    if (overlap) {   // dx'[t] = sum_j dxg[row of slot (t,j)]: an HBM-bound gather beside the tensor-bound dW1
-        BIGMAC_CUDA(cudaEventRecord(L->fork_join[4], st));
-        BIGMAC_CUDA(cudaStreamWaitEvent(sd, L->fork_join[4], 0));
-        { Stage s(L, S_DXLO_GATHER, sd); BIGMAC_CUDA(launch_combine(b.dxg, b.dx_lo, nullptr, b.tb.prow_of_slot, m.T, m.k, m.r, m.dtype, sd, ldcat, m.cap != kNoCapacity)); }
-        BIGMAC_CUDA(cudaEventRecord(L->fork_join[5], sd));
-    }
-    if (G->dw1) {   // dW1_e[q,c'] = sum_rows dz[row,q] xg[row,c']
+    auto dw1 = [&](cudaStream_t stream) -> int {   // dW1_e[q,c'] = sum_rows dz[row,q] xg[row,c']
+        if (!G->dw1) return BIGMAC_OK;
         GemmArgs g = dw1_request(m, dz, b.xg, b.tb, G->dw1, acc);
         if (dispatch_is_fused(L, m, true)) {     // no grouped copy exists: the contraction gathers the rows of x' (Eq. 3: of x)
             g.B = m.cdac ? x : b.x_lo;
             g.gather_rows = b.tb.slot_of_prow;
             g.gather_div = m.k;
         }
-        BIGMAC_TRY(batch ? together.add(G_DW1, g, st) : expert_weight_grad(L, G_DW1, g, b.splitk_ws, st));
-    }
+        return batch ? together.add(G_DW1, g, stream) : expert_weight_grad(L, G_DW1, g, b.expert_ws, stream);
+    };
+    // With the second stream dW1 runs there, beside dx and [dW_down ; dW_gate]: its work items fill what those leave of the chip.
+    const bool dw1_last = fused && !m.cdac && !m.gate_low;
+    if (!dw1_last) BIGMAC_TRY(dw1(st));
     BIGMAC_TRY(together.flush());
     if (m.cdac) {
         // Eq. 3: dx = sum_j dxg[row of slot (t,j)] + dl W_gate; dW_gate = dl^T x
@@ -838,13 +831,17 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         return BIGMAC_OK;
     }
     // dx'[t] = sum_j dxg[row of slot (t,j)]   (the transpose of the dispatch gather)
-    if (overlap) {
-        BIGMAC_CUDA(cudaStreamWaitEvent(st, L->fork_join[5], 0));             // join: the gather ...
-        BIGMAC_CUDA(cudaStreamWaitEvent(st, L->fork_join[3], 0));             // ... and the gate backward with its column sums
-    } else {
+    {
         Stage s(L, S_DXLO_GATHER, st);
         BIGMAC_CUDA(launch_combine(b.dxg, b.dx_lo, nullptr, b.tb.prow_of_slot, m.T, m.k, m.r, m.dtype, st, ldcat, m.cap != kNoCapacity));
     }
+    // Joins the second stream: nothing of this call is left on it.
+    auto join = [&]() -> int {
+        if (!overlap) return BIGMAC_OK;
+        BIGMAC_CUDA(cudaEventRecord(L->fork_join[7], sd));
+        BIGMAC_CUDA(cudaStreamWaitEvent(st, L->fork_join[7], 0));
+        return BIGMAC_OK;
+    };
     if (m.gate_low) {
         // The gate read x': its gradient joins dx' (dx' += dl W_gate, W_gate [E,r]) before the descend projection;
         // dW_gate = dl^T x'.
@@ -889,16 +886,12 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
             }
         }
         if (!colsum_done && G->db_gate) { Stage s(L, S_COLSUM, st, 2); BIGMAC_CUDA(launch_gate_colsum(b.dp, b.tb, G->db_gate, b.colsum_part, m.N, m.E, acc, st, aux_part)); }
-        return BIGMAC_OK;
+        return join();
     }
     if (fused) {
-        // dx and [dW_down ; dW_gate] share only their input [dx' | dl]: with the second stream the weight gradient's CTAs
-        // move in as those of dx leave.  The caller's stream has finished dW1 here, so the fp32 workspace is free.
-        cudaStream_t sw = st;
-        if (overlap && (G->dw_down || G->dw_gate)) {
+        if (overlap) {
             BIGMAC_CUDA(cudaEventRecord(L->fork_join[6], st));
             BIGMAC_CUDA(cudaStreamWaitEvent(sd, L->fork_join[6], 0));
-            sw = sd;
         }
         {   // dx = [dx' | dl] [W_down ; W_gate]: one contraction over r + E
             GemmArgs g;
@@ -912,15 +905,13 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
             g.A = b.dcat; g.lda = ldcat; g.a_kmajor = false; g.B = x; g.ldb = m.d; g.b_kmajor = false;
             g.C = b.splitk_ws; g.ldc = m.d; g.out_f32 = true; g.M = ldcat; g.N = m.d; g.K = m.T;
             g.split_k = choose_split_k(g.M, g.N, g.K);
-            BIGMAC_TRY(gemm(L, G_DW_DOWN, g, sw));
-            Stage s(L, S_SPLITK_REDUCE, sw);
+            BIGMAC_TRY(gemm(L, G_DW_DOWN, g, st));
+            Stage s(L, S_SPLITK_REDUCE, st);
             BIGMAC_CUDA(launch_splitk_reduce(b.splitk_ws, g.split_k, ldcat, m.d, G->dw_down, m.r, G->dw_gate, m.E, m.dtype,
-                                             acc, sw));
+                                             acc, st));
         }
-        if (sw != st) {
-            BIGMAC_CUDA(cudaEventRecord(L->fork_join[7], sd));
-            BIGMAC_CUDA(cudaStreamWaitEvent(st, L->fork_join[7], 0));
-        }
+        BIGMAC_TRY(dw1(sd));
+        BIGMAC_TRY(join());
     } else {
         if (batch) {   // dx = [dx' | dl] [W_down ; W_gate]: one contraction over r + E
             GemmArgs g;
@@ -956,6 +947,7 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         }
         BIGMAC_TRY(together.flush());
     }
+    if (!fused) BIGMAC_TRY(join());
     if (!colsum_done && G->db_gate) {
         Stage s(L, S_COLSUM, st, 2);
         BIGMAC_CUDA(launch_gate_colsum(b.dp, b.tb, G->db_gate, b.colsum_part, m.N, m.E, acc, st, aux_part));

@@ -467,15 +467,15 @@ cudaError_t launch_combine_parts(const void* parts, const MlpSlicing& sl, const 
 }
 
 cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float* dp, const Tables& tb, int k,
-                               int width, int dtype, int64_t max_prows, cudaStream_t stream) {
+                               int width, int dtype, int64_t max_prows, cudaStream_t stream, bool chained) {
     if (max_prows == 0) return cudaSuccess;
     const int vecs = width * elem_bytes(dtype) / 16;
     if (dtype == BIGMAC_BF16)
-        (void)launch_chained(combine_bwd_kernel<__nv_bfloat16>, warp_blocks(max_prows), 256, 0, stream, 
+        (void)launch_maybe_chained(chained, combine_bwd_kernel<__nv_bfloat16>, warp_blocks(max_prows), 256, 0, stream, 
             (const uint4*)dy_lo, (const uint4*)u, (uint4*)du, dp, tb.slot_of_prow, tb.topk_w, tb.n_tiles, k, vecs,
             max_prows);
     else
-        (void)launch_chained(combine_bwd_kernel<float>, warp_blocks(max_prows), 256, 0, stream, 
+        (void)launch_maybe_chained(chained, combine_bwd_kernel<float>, warp_blocks(max_prows), 256, 0, stream, 
             (const uint4*)dy_lo, (const uint4*)u, (uint4*)du, dp, tb.slot_of_prow, tb.topk_w, tb.n_tiles, k, vecs,
             max_prows);
     return cudaGetLastError();
