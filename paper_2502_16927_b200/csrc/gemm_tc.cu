@@ -449,7 +449,7 @@ cudaError_t gemm_tc(const GemmArgs& g, int* status, cudaStream_t stream) {
     if (want_pair) return gemm_tc_pair(g, status, stream);
     // Output-heavy problems (wide rows: activations, ascend, dx) stage their stores through shared memory and
     // TMA, which costs one pipeline stage; contraction-heavy ones keep the deeper pipeline and store directly.
-    const bool staged = switches().staged_stores && !g.C2 && tma_epilogue_possible(g) && g.N >= 1024 && g.N % 256 == 0 &&
+    const bool staged = switches().staged_stores && !g.C2 && tma_epilogue_possible(g) && output_heavy(g) && g.N % 256 == 0 &&
                         (g.epilogue != EPI_DACT || g.group != GROUP_K);
     if (g.N >= 256) return staged ? dispatch<256, 3, true>(g, status, stream) : dispatch<256, 4, false>(g, status, stream);
     return dispatch<128, 6, false>(g, status, stream);

@@ -708,6 +708,9 @@ inline int sm_count() {
     return v;
 }
 
+// Is the problem's time its output's?  Wide rows; and activations of short contractions (d 1024: h = 512 on r = 128).
+inline bool output_heavy(const GemmArgs& g) { return g.N >= 1024 || (g.epilogue != EPI_NONE && g.N >= 512 && g.K <= 256); }
+
 // Can this problem's output leave through shared memory and TMA stores?
 inline bool tma_epilogue_possible(const GemmArgs& g) {
     return !g.out_f32 && !g.accumulate && g.split_k <= 1 && (g.ldc % 8 == 0) && ((uintptr_t)g.C % 16 == 0) &&
