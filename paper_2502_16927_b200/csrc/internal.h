@@ -240,7 +240,9 @@ struct RouteMove {                      // rows of row_bytes bytes to the expert
     bool zero_padding;                  // padding rows are needed as zeros (what an inference forward finds there is never read)
 };
 bool route_fused_supported(int E, int k);
-// which: 0 = first launch (top-k, gate values, block counts), 1 = second launch (tables, rows).
+// which: 0 = first launch (top-k, gate values, block counts), 1 = second launch (tables, rows); 2 = both at once, where
+// route_one_launch says so.
+bool route_one_launch(const RouteSource& src, const RouteMove& mv, int T, int E);
 cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, const RouteExport& ex, const float* b_gate, const Tables& tb,
                                int T, int E, int k, int cap, float* zero_word, int sm_count, cudaStream_t stream, int* status, int which);
 

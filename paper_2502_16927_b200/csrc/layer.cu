@@ -281,6 +281,11 @@ int route_from_logits(const bigmac_layer* L, const Dims& m, const bigmac_weights
         }
         RouteSource with_loss = src;
         if (m.aux > 0) { with_loss.aux_part = b.aux_part; with_loss.aux_loss = b.aux_loss; with_loss.aux_coef = m.aux; }
+        if (route_one_launch(with_loss, mv, m.T, m.E)) {
+            Stage s(L, S_DISPATCH, st);
+            BIGMAC_CUDA(launch_route_fused(with_loss, mv, ex, W->b_gate, b.tb, m.T, m.E, m.k, m.cap, zero_word, sms, st, L->status, 2));
+            return BIGMAC_OK;
+        }
         { Stage s(L, S_TOPK, st); BIGMAC_CUDA(launch_route_fused(with_loss, mv, ex, W->b_gate, b.tb, m.T, m.E, m.k, m.cap, zero_word, sms, st, L->status, 0)); }
         { Stage s(L, mv.grouped ? S_DISPATCH : S_TABLES, st); BIGMAC_CUDA(launch_route_fused(with_loss, mv, ex, W->b_gate, b.tb, m.T, m.E, m.k, m.cap, zero_word, sms, st, L->status, 1)); }
     } else {

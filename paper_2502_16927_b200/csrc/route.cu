@@ -352,13 +352,98 @@ constexpr int kMaxParts = 8;                        // parts of a split descend 
 
 // Where the gate logits (and the rows of x') come from: matrices in memory, or the fp32 partial results
 // [parts][T][ld] of a descend launch whose contraction was cut into parts - then added in part order on the way.
-// Kernel 1: top-k with gate values as topk8_kernel, four tokens per warp, plus pass 1 of the counting sort.  Block b owns
-// tokens [b TB, (b + 1) TB), TB = 4 warps iters.  Lane 8 g + j of a warp holds slot j of the warp's token g, so the lane
-// order is the slot order: ranks inside a warp by match_any, across the warps by a scan over per-warp counts.
+
+// A lane's logits of its token: elements 4 (sub + 8 i) .. + 3 of the row, i < Q.  Returns bit i: element i is past E.
+template <int Q>
+__device__ __forceinline__ uint32_t token_logits(float* v, const float* row, int parts, int64_t part_stride, float* logits_out, int64_t t,
+                                                 bool live, const float* __restrict__ b_gate, int E) {
+    const int sub = threadIdx.x & 7;
+    uint32_t past = 0;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const int e0 = 4 * (sub + 8 * i);
+        float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (e0 < E) {
+            x = *reinterpret_cast<const float4*>(row + e0);
+            if (parts > 1) {                     // all parts' loads in flight together, added in part order
+                float4 y[kMaxParts - 1];
+#pragma unroll
+                for (int s = 1; s < kMaxParts; ++s)
+                    if (s < parts) y[s - 1] = *reinterpret_cast<const float4*>(row + s * part_stride + e0);
+#pragma unroll
+                for (int s = 1; s < kMaxParts; ++s)
+                    if (s < parts) { x.x += y[s - 1].x; x.y += y[s - 1].y; x.z += y[s - 1].z; x.w += y[s - 1].w; }
+            }
+            if (logits_out && live) *reinterpret_cast<float4*>(logits_out + t * E + e0) = x;
+            if (b_gate) { x.x += b_gate[e0]; x.y += b_gate[e0 + 1]; x.z += b_gate[e0 + 2]; x.w += b_gate[e0 + 3]; }
+        } else {
+            past |= 15u << (4 * i);
+        }
+        v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
+    }
+    return past;
+}
+
 // Rounds of arg-max over a token's eight lanes: a lane keeps the maxima of its Q quads in registers and the quads themselves in
 // shared memory, where the winner alone strikes its element out (NaN: never a maximum, never equal) and looks its quad over
 // again.  With the values in registers every lane scanned all of them in every round: issue slots bound the kernel, 34 us at
 // 32768 tokens of 128 experts.
+// Lane j of the eight gets the j-th choice (value, expert id).
+template <int Q>
+__device__ __forceinline__ void token_topk(float* v, uint32_t past, float4* quads, int k, float& my_v, int& my_e) {
+    const int lane = threadIdx.x & 31, sub = lane & 7;
+    my_v = -INFINITY;
+    my_e = 0;
+    const float none = __int_as_float(0x7fffffff);
+    float most[Q];                               // maximum of each quad
+#pragma unroll
+    for (int i = 0; i < 4 * Q; ++i) v[i] = (past >> i) & 1u ? none : v[i] == v[i] ? v[i] : -INFINITY;     // NaN is ordered as -inf
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        most[q] = fmaxf(fmaxf(v[4 * q], v[4 * q + 1]), fmaxf(v[4 * q + 2], v[4 * q + 3]));
+        quads[q * blockDim.x] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    }
+    for (int j = 0; j < k; ++j) {
+        float mine = most[0];
+#pragma unroll
+        for (int q = 1; q < Q; ++q) mine = fmaxf(mine, most[q]);
+        float best = mine;
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) best = fmaxf(best, __shfl_xor_sync(kFull, best, off));
+        bool wins = mine == best;
+        int e = kNoExpert, at = 0, c = 0;
+        float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (wins) {                              // its lowest expert id with that value: ids ascend with the quad and inside it
+#pragma unroll
+            for (int q = Q - 1; q >= 0; --q) at = most[q] == best ? q : at;
+            x = quads[at * blockDim.x];
+            c = x.x == best ? 0 : x.y == best ? 1 : x.z == best ? 2 : 3;
+            e = 4 * (sub + 8 * at) + c;
+        }
+        const unsigned votes = __ballot_sync(kFull, wins), group = (votes >> (lane & 24)) & 0xffu;
+        int from = __ffs(group) - 1;
+        if (__any_sync(kFull, __popc(group) > 1)) {      // equal logits in several lanes: the lowest id of all
+            int low = e;
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) low = min(low, __shfl_xor_sync(kFull, low, off));
+            wins = wins && e == low;
+            from = (low >> 2) & 7;
+        }
+        if (wins) {
+            x.x = c == 0 ? none : x.x; x.y = c == 1 ? none : x.y; x.z = c == 2 ? none : x.z; x.w = c == 3 ? none : x.w;
+            quads[at * blockDim.x] = x;
+            const float left = fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w));
+#pragma unroll
+            for (int q = 0; q < Q; ++q) most[q] = at == q ? left : most[q];
+        }
+        const int chosen = __shfl_sync(kFull, e, (lane & 24) + from);
+        if (sub == j) { my_v = best; my_e = chosen; }
+    }
+}
+
+// Kernel 1: top-k with gate values as topk8_kernel, four tokens per warp, plus pass 1 of the counting sort.  Block b owns
+// tokens [b TB, (b + 1) TB), TB = 4 warps iters.  Lane 8 g + j of a warp holds slot j of the warp's token g, so the lane
+// order is the slot order: ranks inside a warp by match_any, across the warps by a scan over per-warp counts.
 // AUX: also the block's column sums of the softmax over all E experts, for the load-balancing loss (launches of their own for
 // these sums, the loss and the copies of the tables put 16 us between the logits and the experts at 2999 tokens).
 constexpr int kTopkAuxWarps = 16;
@@ -383,29 +468,7 @@ __global__ void __launch_bounds__(AUX ? 32 * kTopkAuxWarps : 1024) topk_count_ke
         const bool live = t < T;
         const float* row = logits + (live ? t : 0) * ld;
         float v[4 * Q];
-        uint32_t past = 0;                           // bit i: this lane's i-th expert is past E
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const int e0 = 4 * (sub + 8 * i);
-            float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (e0 < E) {
-                x = *reinterpret_cast<const float4*>(row + e0);
-                if (parts > 1) {                     // all parts' loads in flight together, added in part order
-                    float4 y[kMaxParts - 1];
-#pragma unroll
-                    for (int s = 1; s < kMaxParts; ++s)
-                        if (s < parts) y[s - 1] = *reinterpret_cast<const float4*>(row + s * part_stride + e0);
-#pragma unroll
-                    for (int s = 1; s < kMaxParts; ++s)
-                        if (s < parts) { x.x += y[s - 1].x; x.y += y[s - 1].y; x.z += y[s - 1].z; x.w += y[s - 1].w; }
-                }
-                if (logits_out && live) *reinterpret_cast<float4*>(logits_out + t * E + e0) = x;
-                if (b_gate) { x.x += b_gate[e0]; x.y += b_gate[e0 + 1]; x.z += b_gate[e0 + 2]; x.w += b_gate[e0 + 3]; }
-            } else {
-                past |= 15u << (4 * i);
-            }
-            v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
-        }
+        const uint32_t past = token_logits<Q>(v, row, parts, part_stride, logits_out, t, live, b_gate, E);
         if (AUX) {                                   // a token's softmax over its eight lanes, then the warp's four tokens together
             float mx = -INFINITY, sum = 0.0f, pr[4 * Q];
 #pragma unroll
@@ -430,53 +493,9 @@ __global__ void __launch_bounds__(AUX ? 32 * kTopkAuxWarps : 1024) topk_count_ke
                 if (lane < 8 && e < E) prob_sums[warp * E + e] += p;
             }
         }
-        const float none = __int_as_float(0x7fffffff);
-        float most[Q];                               // maximum of each quad
-#pragma unroll
-        for (int i = 0; i < 4 * Q; ++i) v[i] = (past >> i) & 1u ? none : v[i] == v[i] ? v[i] : -INFINITY;     // NaN is ordered as -inf
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            most[q] = fmaxf(fmaxf(v[4 * q], v[4 * q + 1]), fmaxf(v[4 * q + 2], v[4 * q + 3]));
-            quads[q * blockDim.x] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-        }
-        float my_v = -INFINITY;
-        int my_e = 0;
-        for (int j = 0; j < k; ++j) {
-            float mine = most[0];
-#pragma unroll
-            for (int q = 1; q < Q; ++q) mine = fmaxf(mine, most[q]);
-            float best = mine;
-#pragma unroll
-            for (int off = 4; off > 0; off >>= 1) best = fmaxf(best, __shfl_xor_sync(kFull, best, off));
-            bool wins = mine == best;
-            int e = kNoExpert, at = 0, c = 0;
-            float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (wins) {                              // its lowest expert id with that value: ids ascend with the quad and inside it
-#pragma unroll
-                for (int q = Q - 1; q >= 0; --q) at = most[q] == best ? q : at;
-                x = quads[at * blockDim.x];
-                c = x.x == best ? 0 : x.y == best ? 1 : x.z == best ? 2 : 3;
-                e = 4 * (sub + 8 * at) + c;
-            }
-            const unsigned votes = __ballot_sync(kFull, wins), group = (votes >> (lane & 24)) & 0xffu;
-            int from = __ffs(group) - 1;
-            if (__any_sync(kFull, __popc(group) > 1)) {      // equal logits in several lanes: the lowest id of all
-                int low = e;
-#pragma unroll
-                for (int off = 4; off > 0; off >>= 1) low = min(low, __shfl_xor_sync(kFull, low, off));
-                wins = wins && e == low;
-                from = (low >> 2) & 7;
-            }
-            if (wins) {
-                x.x = c == 0 ? none : x.x; x.y = c == 1 ? none : x.y; x.z = c == 2 ? none : x.z; x.w = c == 3 ? none : x.w;
-                quads[at * blockDim.x] = x;
-                const float left = fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w));
-#pragma unroll
-                for (int q = 0; q < Q; ++q) most[q] = at == q ? left : most[q];
-            }
-            const int chosen = __shfl_sync(kFull, e, (lane & 24) + from);
-            if (sub == j) { my_v = best; my_e = chosen; }
-        }
+        float my_v;
+        int my_e;
+        token_topk<Q>(v, past, quads, k, my_v, my_e);
         const float top = __shfl_sync(kFull, my_v, lane & 24);
         const float ex = sub < k ? (top == -INFINITY ? 1.0f : expf(my_v - top)) : 0.0f;
         float part = ex;
@@ -547,58 +566,16 @@ struct PlaceArgs {
 };
 
 constexpr int kPlaceThreads = 512, kPlaceMaxExperts = 256;
+// Counts of an expert's slots before this block's, and in all; rows before the expert, unpadded and padded.
+struct PlaceShared { int32_t base[kPlaceMaxExperts], total[kPlaceMaxExperts], off[kPlaceMaxExperts + 1], poff[kPlaceMaxExperts + 1]; };
 
-// Kernel 2: the whole placement, and the dispatch as a scatter: a warp reads the row of a token once and writes it to
-// its k grouped rows (the gather form reads it k times).  Every block adds up the counts of all blocks of kernel 1 for
-// itself (a few tens of KB from L2), which takes less than a launch of a scan kernel.
-// MOVE 0: tables only; 1: rows of a matrix; 2: rows from partial results.
-template <int MOVE>
-__global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p) {
-    grid_dependency_wait();
-    grid_dependency_launch();
-    __shared__ int32_t s_all[kPlaceThreads], s_below[kPlaceThreads];        // [parts][E]
-    __shared__ int32_t s_base[kPlaceMaxExperts], s_total[kPlaceMaxExperts], s_off[kPlaceMaxExperts + 1], s_poff[kPlaceMaxExperts + 1];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// The placement from the counts on: tokens [first, last) of this block, slot_of(t, e, rank) giving lane j < k of a warp its slot's
+// expert and rank behind sh.base; then this block's share of everything else.
+template <int MOVE, typename Slot>
+__device__ __forceinline__ void place_from_counts(const PlaceArgs& p, PlaceShared& sh, int64_t first, int64_t last, Slot slot_of) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, E = p.E, nparts = min(16, kPlaceThreads / E);
     constexpr int kWarps = kPlaceThreads / 32;
-    const int E = p.E, nparts = min(16, kPlaceThreads / E);
-    const int b = blockIdx.x / p.splits;             // the block of kernel 1 whose slots these are
-    const int per_split = (p.tokens_per_block + p.splits - 1) / p.splits;
-    const int64_t first = (int64_t)b * p.tokens_per_block + (int64_t)(blockIdx.x - b * p.splits) * per_split;
-    const int64_t last = min(min(first + per_split, (int64_t)(b + 1) * p.tokens_per_block), (int64_t)p.T);
-    // the warp's first token: its experts and ranks are on their way while the counts are added up
-    int next_e = 0, next_rank = 0;
-    if (first + warp < last && lane < p.k) {
-        next_e = p.topk_idx[(first + warp) * p.k + lane];
-        next_rank = p.prow_of_slot[(first + warp) * p.k + lane];
-    }
-    {
-        const int e = tid % E, part = tid / E;       // neighbouring threads on neighbouring experts
-        int all = 0, below = 0;
-        if (part < nparts) {
-            for (int row = part; row < p.nb; row += 16 * nparts) {
-                int c[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) c[i] = row + i * nparts < p.nb ? p.block_counts[(size_t)(row + i * nparts) * E + e] : 0;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    all += c[i];
-                    if (row + i * nparts < b) below += c[i];
-                }
-            }
-        }
-        s_all[tid] = all;
-        s_below[tid] = below;
-    }
-    __syncthreads();
-    if (tid < E) {
-        int all = 0, below = 0;
-        for (int q = 0; q < nparts; ++q) {
-            all += s_all[q * E + tid];
-            below += s_below[q * E + tid];
-        }
-        s_total[tid] = all;
-        s_base[tid] = below;
-    }
+    int32_t *s_base = sh.base, *s_total = sh.total, *s_off = sh.off, *s_poff = sh.poff;
     __syncthreads();
     if (warp == 0) {                                 // offsets: lane l scans the experts [l per, (l + 1) per)
         const int per = (E + 31) / 32, e0 = min(E, lane * per), e1 = min(E, e0 + per);
@@ -635,8 +612,8 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p)
         int prow = -1;
         if (lane < p.k) {
             const int64_t s = t * p.k + lane;
-            const int e = next_e, rank = next_rank;
-            if (t + kWarps < last) { next_e = p.topk_idx[s + kWarps * p.k]; next_rank = p.prow_of_slot[s + kWarps * p.k]; }
+            int e, rank;
+            slot_of(t, e, rank);
             int row = -1;
             if ((unsigned)e >= (unsigned)E) {        // second line of defence: the slot goes nowhere, the call reports it
                 if (p.status) atomicExch(p.status, 2);
@@ -713,7 +690,7 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p)
         }
     if (p.aux_part && blockIdx.x == gridDim.x - 1) { // the loss, coef E sum_e f_e P_e, on the block with the fewest tokens
         __shared__ float s_term[kPlaceMaxExperts];
-        float* sums = reinterpret_cast<float*>(s_all);
+        __shared__ float sums[kPlaceThreads];
         const int e = tid % E, part = tid / E;
         float acc = 0.0f;
         if (part < nparts) {
@@ -757,6 +734,156 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p)
             if (p.zero_word) *p.zero_word = 0.0f;
         }
     }
+}
+
+
+// Kernel 2: the whole placement, and the dispatch as a scatter: a warp reads the row of a token once and writes it to
+// its k grouped rows (the gather form reads it k times).  Every block adds up the counts of all blocks of kernel 1 for
+// itself (a few tens of KB from L2), which takes less than a launch of a scan kernel.
+// MOVE 0: tables only; 1: rows of a matrix; 2: rows from partial results.
+template <int MOVE>
+__global__ void __launch_bounds__(kPlaceThreads) place_kernel(const PlaceArgs p) {
+    grid_dependency_wait();
+    grid_dependency_launch();
+    __shared__ int32_t s_all[kPlaceThreads], s_below[kPlaceThreads];        // [parts][E]
+    __shared__ PlaceShared sh;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kWarps = kPlaceThreads / 32;
+    const int E = p.E, nparts = min(16, kPlaceThreads / E);
+    const int b = blockIdx.x / p.splits;             // the block of kernel 1 whose slots these are
+    const int per_split = (p.tokens_per_block + p.splits - 1) / p.splits;
+    const int64_t first = (int64_t)b * p.tokens_per_block + (int64_t)(blockIdx.x - b * p.splits) * per_split;
+    const int64_t last = min(min(first + per_split, (int64_t)(b + 1) * p.tokens_per_block), (int64_t)p.T);
+    // the warp's first token: its experts and ranks are on their way while the counts are added up
+    int next_e = 0, next_rank = 0;
+    if (first + warp < last && lane < p.k) {
+        next_e = p.topk_idx[(first + warp) * p.k + lane];
+        next_rank = p.prow_of_slot[(first + warp) * p.k + lane];
+    }
+    {
+        const int e = tid % E, part = tid / E;       // neighbouring threads on neighbouring experts
+        int all = 0, below = 0;
+        if (part < nparts) {
+            for (int row = part; row < p.nb; row += 16 * nparts) {
+                int c[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) c[i] = row + i * nparts < p.nb ? p.block_counts[(size_t)(row + i * nparts) * E + e] : 0;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    all += c[i];
+                    if (row + i * nparts < b) below += c[i];
+                }
+            }
+        }
+        s_all[tid] = all;
+        s_below[tid] = below;
+    }
+    __syncthreads();
+    if (tid < E) {
+        int all = 0, below = 0;
+        for (int q = 0; q < nparts; ++q) {
+            all += s_all[q * E + tid];
+            below += s_below[q * E + tid];
+        }
+        sh.total[tid] = all;
+        sh.base[tid] = below;
+    }
+    place_from_counts<MOVE>(p, sh, first, last, [&](int64_t t, int& e, int& rank) {
+        const int64_t s = t * p.k + lane;
+        e = next_e;
+        rank = next_rank;
+        if (t + kWarps < last) { next_e = p.topk_idx[s + kWarps * p.k]; next_rank = p.prow_of_slot[s + kWarps * p.k]; }
+    });
+}
+
+// Both in one launch, for up to kOneLaunchTokens tokens: a cluster of eight blocks does the top-k of all tokens, an eighth in each
+// block, and the blocks hand each other their counts through distributed shared memory; every cluster does the same and then
+// places and moves its own share of its blocks' tokens.  The repetition costs some L2 reads; the hand-over through memory
+// (a launch's end, the next one's start, the counts and slots read back) cost about 3 us of a forward of 45 to 54.
+constexpr int kOneLaunchTokens = 512, kRouteCluster = 8;
+struct RouteArgs {
+    const float* logits;
+    int ld, parts;
+    int64_t part_stride;
+    const float* b_gate;
+    int32_t* topk_idx;
+    float* topk_w;
+    int per_block;                                   // tokens of a block, at most four for each of its warps
+};
+template <int Q, int MOVE>
+__global__ void __launch_bounds__(kPlaceThreads) route_cluster_kernel(const RouteArgs r, const PlaceArgs p) {
+    constexpr int kWarps = kPlaceThreads / 32;
+    extern __shared__ float4 route_quads[];          // [Q][threads]; then the counts of the warps
+    int32_t* warp_run = reinterpret_cast<int32_t*>(route_quads + Q * kPlaceThreads);      // [kWarps][E]
+    __shared__ PlaceShared sh;
+    __shared__ int32_t counts[kRouteCluster][kPlaceMaxExperts];
+    __shared__ int16_t s_expert[kOneLaunchTokens], s_rank[kOneLaunchTokens];   // slots of this block: 64 tokens of up to eight
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane & 7, E = p.E;
+    const int rank_in = blockIdx.x % kRouteCluster, cluster = blockIdx.x / kRouteCluster, clusters = gridDim.x / kRouteCluster;
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");       // (that all blocks of the cluster have started)
+    for (int i = tid; i < kWarps * E; i += kPlaceThreads) warp_run[i] = 0;
+    grid_dependency_wait();
+    grid_dependency_launch();
+    const int first = rank_in * r.per_block, here = 4 * warp + (lane >> 3), t = first + here;
+    const bool live = here < r.per_block && t < p.T;
+    float v[4 * Q], my_v;
+    int my_e;
+    const uint32_t past = token_logits<Q>(v, r.logits + (int64_t)(live ? t : 0) * r.ld, r.parts, r.part_stride, nullptr, t, live, r.b_gate, E);
+    token_topk<Q>(v, past, route_quads + tid, p.k, my_v, my_e);
+    const float top = __shfl_sync(kFull, my_v, lane & 24);
+    const float ex = sub < p.k ? (top == -INFINITY ? 1.0f : expf(my_v - top)) : 0.0f;
+    float part = ex;
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) part += __shfl_xor_sync(kFull, part, off);
+    const bool slot = live && sub < p.k;
+    const int e = slot ? my_e : -1;
+    const unsigned peers = __match_any_sync(kFull, e);
+    __syncthreads();
+    if (slot && lane == __ffs(peers) - 1) warp_run[warp * E + e] = __popc(peers);
+    __syncthreads();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (tid < E) {                                   // over the warps, then to all blocks of the cluster
+        int run = 0, c[kWarps];
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) c[w] = warp_run[w * E + tid];
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) { warp_run[w * E + tid] = run; run += c[w]; }
+        const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&counts[rank_in][tid]);
+#pragma unroll
+        for (int q = 0; q < kRouteCluster; ++q)
+            asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %0, %1;\n\tst.shared::cluster.b32 [a], %2;\n\t}" ::"r"(mine), "r"(q), "r"(run) : "memory");
+    }
+    __syncthreads();
+    if (slot) {
+        s_expert[here * p.k + sub] = (int16_t)e;
+        s_rank[here * p.k + sub] = (int16_t)(warp_run[warp * E + e] + __popc(peers & ((1u << lane) - 1u)));
+        if (cluster == 0) {
+            const int s = t * p.k + sub;
+            r.topk_idx[s] = my_e;
+            r.topk_w[s] = ex / part;
+            if (p.ex.topk_idx) p.ex.topk_idx[s] = my_e;
+            if (p.ex.topk_w) p.ex.topk_w[s] = ex / part;
+        }
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");   // all counts are here
+    if (tid < E) {
+        int all = 0, below = 0;
+#pragma unroll
+        for (int q = 0; q < kRouteCluster; ++q) {
+            const int c = counts[q][tid];
+            all += c;
+            if (q < rank_in) below += c;
+        }
+        sh.total[tid] = all;
+        sh.base[tid] = below;
+    }
+    const int share = (r.per_block + clusters - 1) / clusters, from = min(first + cluster * share, first + r.per_block);
+    const int to = min(min(from + share, first + r.per_block), p.T);
+    place_from_counts<MOVE>(p, sh, from, to, [&](int64_t tok, int& ex_id, int& rank) {
+        ex_id = s_expert[((int)tok - first) * p.k + lane];
+        rank = s_rank[((int)tok - first) * p.k + lane];
+    });
 }
 
 }  // namespace
@@ -815,6 +942,10 @@ cudaError_t launch_tables(const Tables& tb, int T, int E, int k, int cap, cudaSt
 // The two-launch form wants a lane per slot of a token, eight lanes per token, and at most 32 logits per lane.
 bool route_fused_supported(int E, int k) { return k <= 8 && E % 4 == 0 && E <= kPlaceMaxExperts; }
 
+bool route_one_launch(const RouteSource& src, const RouteMove& mv, int T, int E) {
+    return T <= kOneLaunchTokens && E <= 128 && mv.grouped && !src.aux_part && !src.logits_out;
+}
+
 cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, const RouteExport& ex, const float* b_gate, const Tables& tb,
                                int T, int E, int k, int cap, float* zero_word, int sm_count, cudaStream_t stream, int* status,
                                int which) {
@@ -827,7 +958,7 @@ cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, cons
     const int most = src.aux_part ? kTopkAuxWarps : 32, warps = per < 4 * most ? (per + 3) / 4 : most, iters = (per + 4 * warps - 1) / (4 * warps);
     per = 4 * warps * iters;
     const int nb = (T + per - 1) / per;
-    if (which == 0) {
+    if (which == 0) {                                // (which 2 has no first launch)
         const int quads = E <= 32 ? 1 : E <= 64 ? 2 : E <= 128 ? 4 : 8;          // 160 KB at most
         const size_t smem = sizeof(int32_t) * (size_t)(src.aux_part ? 2 * warps + 1 : warps + 1) * E + (size_t)quads * warps * 32 * sizeof(float4);
 #define BIGMAC_TOPK_COUNT(Q)                                                                                                       \
@@ -863,6 +994,39 @@ cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, cons
     p.ex = ex; p.aux_part = src.aux_part; p.aux_loss = src.aux_loss; p.aux_coef = src.aux_coef;
     p.src = (const uint4*)mv.src; p.partial = mv.partial; p.parts = mv.parts; p.ld = mv.ld; p.part_stride = mv.part_stride;
     p.grouped = (uint4*)mv.grouped; p.vecs = mv.row_bytes / 16; p.zero_padding = mv.zero_padding;
+    if (which == 2) {
+        RouteArgs r{src.logits, src.ld, src.parts, src.part_stride, b_gate, tb.topk_idx, tb.topk_w, (T + kRouteCluster - 1) / kRouteCluster};
+        // about four tokens a block to move, up to twelve clusters (sixteen do not fit the chip at once: 512 tokens 55 -> 61 us)
+        int clusters = (r.per_block + 3) / 4;
+        if (clusters > 12) clusters = 12;
+        const int quads = E <= 32 ? 1 : E <= 64 ? 2 : 4;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = kRouteCluster * clusters; cfg.blockDim = kPlaceThreads; cfg.stream = stream;
+        cfg.dynamicSmemBytes = (size_t)quads * kPlaceThreads * sizeof(float4) + sizeof(int32_t) * (kPlaceThreads / 32) * E;     // 40 KB at most
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kRouteCluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr; cfg.numAttrs = switches().chain ? 2 : 1;
+#define BIGMAC_ROUTE(Q)                                                                                                            \
+    do {                                                                                                                           \
+        const auto kernel = mv.partial ? route_cluster_kernel<Q, 2> : route_cluster_kernel<Q, 1>;                                 \
+        static PerDeviceOnce once;                                                                                                 \
+        int dev;                                                                                                                   \
+        if (once.needed(&dev)) {                                                                                                   \
+            cudaError_t e = cudaFuncSetAttribute(route_cluster_kernel<Q, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 49152);  \
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(route_cluster_kernel<Q, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 49152); \
+            if (e != cudaSuccess) return e;                                                                                        \
+            once.mark(dev);                                                                                                        \
+        }                                                                                                                          \
+        return cudaLaunchKernelEx(&cfg, kernel, r, p);                                                                             \
+    } while (0)
+        if (E <= 32) BIGMAC_ROUTE(1);
+        if (E <= 64) BIGMAC_ROUTE(2);
+        BIGMAC_ROUTE(4);
+#undef BIGMAC_ROUTE
+    }
     if (!mv.grouped) return launch_chained(place_kernel<0>, nb * p.splits, kPlaceThreads, 0, stream, p);
     if (!mv.partial) return launch_chained(place_kernel<1>, nb * p.splits, kPlaceThreads, 0, stream, p);
     return launch_chained(place_kernel<2>, nb * p.splits, kPlaceThreads, 0, stream, p);

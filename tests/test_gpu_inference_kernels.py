@@ -94,6 +94,32 @@ def test_routing_in_two_launches(E, k, T):
         layer.close()
 
 
+@pytest.mark.parametrize("E,k", [(8, 8), (32, 1), (36, 3), (64, 8), (128, 8)])
+@pytest.mark.parametrize("T", [1, 7, 33, 259, 511, 512])
+def test_routing_in_one_launch(E, k, T):
+    """A forward of up to 512 tokens routes in one launch (clusters that share the tokens): rows from a matrix (r 8, fp32) and from
+    partial results (bf16, contraction of d = 1024 in parts), with and without a capacity limit."""
+    import torch
+    from paper_2502_16927_b200 import binding
+
+    for dtype, d, r, h in ((wl.DTYPE_F32, 32, 8, 8), (wl.DTYPE_BF16, 1024, 128, 64)):
+        w = wl.Workload("route", T=T, d=d, r=r, h=h, E=E, k=k, dtype=dtype, act=wl.ACT_RELU, seed=35)
+        inp = _inputs(w, 1.0)
+        dev = to_device(w, inp)
+        for f in (0.0, 0.6):
+            layer = make_layer(w, capacity_factor=f, flags=0)
+            y, R = layer.forward(dev["x"], dev, want_routing=True, training=dtype == wl.DTYPE_F32)
+            torch.cuda.synchronize()
+            assert layer.status() == 0
+            rt = oracle.route(inp, w.k, capacity_factor=f)
+            _check_tables(R, rt)
+            ref = oracle.forward_tokens(inp, rt, w.act)["y"]
+            tol = 1e-4 if dtype == wl.DTYPE_F32 else 8e-3          # bf16: four or five stores of 0.17 % of the rms each
+            err = np.linalg.norm(to_numpy(y) - ref) / max(np.linalg.norm(ref), 1e-30)
+            assert err <= tol, (dtype, f, err)
+            layer.close()
+
+
 @pytest.mark.parametrize("E,k", [(4, 4), (36, 8), (64, 8), (128, 8), (256, 8)])
 def test_equal_and_nonfinite_logits(E, k):
     """Logits that are nothing but the gate bias: a handful of values that many experts share (in one lane's quad, across its
