@@ -22,6 +22,39 @@ Switches& switches() {
 using namespace bigmac;
 using namespace bigmac::detail;
 
+// Memory of the small-batch kernel for a few handles (zero at first, like every __device__ array): one of its own, of more than
+// 1 MB, is a mapping of its own: creation 58 -> 413 us, destruction 51 -> 326 (70 and 68 with the pool).  A place goes from handle to handle as it is: its
+// launch counts go on, so the tags of earlier launches in its words never match.
+constexpr int kDecodePlaces = 4;
+constexpr size_t kDecodePlaceBytes = 1280 * 1024;
+static __device__ __align__(256) unsigned char g_decode_places[kDecodePlaces][kDecodePlaceBytes];
+
+namespace {
+constexpr int kDecodeDevices = 64;
+std::mutex g_decode_mutex;
+bool g_decode_taken[kDecodeDevices][kDecodePlaces] = {};
+
+// A free place of the current device: its number, or -1.
+int take_decode_place(int device, size_t bytes, void** base) {
+    void* all = nullptr;
+    if (bytes > kDecodePlaceBytes || device < 0 || device >= kDecodeDevices) return -1;
+    std::lock_guard<std::mutex> lock(g_decode_mutex);
+    for (int i = 0; i < kDecodePlaces; ++i)
+        if (!g_decode_taken[device][i]) {
+            if (cudaGetSymbolAddress(&all, g_decode_places) != cudaSuccess || !all) { cudaGetLastError(); return -1; }
+            *base = (unsigned char*)all + i * kDecodePlaceBytes;
+            g_decode_taken[device][i] = true;
+            return i;
+        }
+    return -1;
+}
+void give_decode_memory(bigmac_layer* L) {           // after the handle's work on the device is done
+    if (L->decode_place < 0) { cudaFree(L->decode_epochs); return; }
+    std::lock_guard<std::mutex> lock(g_decode_mutex);
+    g_decode_taken[L->device][L->decode_place] = false;
+}
+}  // namespace
+
 namespace bigmac {
 namespace detail {
 
@@ -445,20 +478,30 @@ int bigmac_layer_create(const bigmac_config_t* cfg, bigmac_layer_t** out) {
     L->cfg = *cfg;
     L->use_tc = cfg->dtype == BIGMAC_BF16 && !(cfg->flags & BIGMAC_FLAG_SIMT_GEMM);
     L->tc_mask = switches().tc_mask;
-    // status words, and behind them the hand-over words of the small-batch kernel where the configuration can reach it
+    // memory of the small-batch kernel where the configuration can reach it
     const bool plain = L->use_tc && !(cfg->flags & (BIGMAC_FLAG_CDAC | BIGMAC_FLAG_GATE_LOW | BIGMAC_FLAG_EXPERT_BIAS)) &&
                        cfg->capacity_factor == 0 && cfg->aux_loss_coef == 0;
     const int few = plain ? decode_forward_max_tokens(cfg->max_tokens, cfg->d, cfg->r, cfg->h, cfg->E, cfg->k, cfg->dtype, gemm_tc_sm_count()) : 0;
     const size_t words = decode_forward_words(few, cfg->r, cfg->h, cfg->E, cfg->k);
-    const size_t head = words ? 256 + ((size_t)gemm_tc_sm_count() * 4 + 255) / 256 * 256 : 256, bytes = head + 8 * words;
-    if (cudaGetDevice(&L->device) != cudaSuccess || cudaMalloc((void**)&L->status, bytes) != cudaSuccess ||
-        cudaMemset(L->status, 0, bytes) != cudaSuccess) {
+    const size_t head = ((size_t)gemm_tc_sm_count() * 4 + 255) / 256 * 256, bytes = head + 8 * words;
+    if (cudaGetDevice(&L->device) != cudaSuccess || cudaMalloc((void**)&L->status, 256) != cudaSuccess ||
+        cudaMemset(L->status, 0, 256) != cudaSuccess) {
         cudaFree(L->status);
         delete L;
         return BIGMAC_ERR_CUDA;
     }
-    L->decode_words = words ? (char*)L->status + head : nullptr;
+    if (words) {
+        L->decode_place = take_decode_place(L->device, bytes, (void**)&L->decode_epochs);
+        if (L->decode_place < 0 && (cudaMalloc((void**)&L->decode_epochs, bytes) != cudaSuccess || cudaMemset(L->decode_epochs, 0, bytes) != cudaSuccess)) {
+            cudaFree(L->decode_epochs);
+            cudaFree(L->status);
+            delete L;
+            return BIGMAC_ERR_CUDA;
+        }
+        L->decode_words = (char*)L->decode_epochs + head;
+    }
     if (L->use_tc && !gemm_tc_available()) {
+        give_decode_memory(L);
         cudaFree(L->status);
         delete L;
         return BIGMAC_ERR_UNSUPPORTED;
@@ -483,7 +526,9 @@ int bigmac_layer_destroy(bigmac_layer_t* L) {
     for (cudaEvent_t e : L->fork_join)
         if (e) cudaEventDestroy(e);
     if (L->side) cudaStreamDestroy(L->side);
+    if (L->decode_place >= 0) cudaDeviceSynchronize();   // nothing of this handle runs when another takes its place in the pool
     cudaFree(L->status);
+    give_decode_memory(L);
     delete L;
     return BIGMAC_OK;
 }
@@ -551,7 +596,7 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
         decode_forward_supported(m.T, m.d, m.r, m.h, m.E, m.k, m.dtype, gemm_tc_sm_count())) {
         {
             Stage s(L, S_DECODE, st);
-            BIGMAC_CUDA(launch_decode_forward(x, W, y, L->decode_words, b.tb.topk_idx, b.tb.topk_w, (unsigned*)(L->status + 64),
+            BIGMAC_CUDA(launch_decode_forward(x, W, y, L->decode_words, b.tb.topk_idx, b.tb.topk_w, L->decode_epochs,
                                               L->status, m.T, m.d, m.r, m.h, m.E, m.k, c.act, gemm_tc_sm_count(), st));
         }
         if (routing_out) {

@@ -12,8 +12,12 @@ struct bigmac_layer {
     bigmac_config_t cfg;
     int device;
     int* status = nullptr;  // device status word; status[2..3] are the work counters of the per-expert weight-gradient kernel
-                        // (zero at rest), status[64 ..] the small-batch kernel's launch counts, one per block
-    void* decode_words = nullptr;   // hand-over words of the small-batch kernel (same allocation), or null
+                        // (zero at rest)
+    // the small-batch kernel's memory, or null: launch counts, one per block, and hand-over words; a place of the library's
+    // static pool (its number) or an allocation of the handle's own (-1)
+    unsigned* decode_epochs = nullptr;
+    void* decode_words = nullptr;
+    int decode_place = -1;
     bool use_tc;        // bf16 contractions on tcgen05
     unsigned tc_mask;   // debug: bit i set = contraction i runs on tcgen05 (the tc_mask switch at creation)
     // second stream of the backward pass (created on first use): launches that do not depend on each other and lean
