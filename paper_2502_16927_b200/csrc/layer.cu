@@ -22,9 +22,10 @@ Switches& switches() {
 using namespace bigmac;
 using namespace bigmac::detail;
 
-// Memory of the small-batch kernel for a few handles (zero at first, like every __device__ array): one of its own, of more than
-// 1 MB, is a mapping of its own: creation 58 -> 413 us, destruction 51 -> 326 (70 and 68 with the pool).  A place goes from handle to handle as it is: its
-// launch counts go on, so the tags of earlier launches in its words never match.
+// Memory of the small-batch kernel for a few handles (zero at first, like every __device__ array).  An allocation of its own, of
+// more than 1 MB, is a mapping of its own: creation of a handle 58 -> 413 us, destruction 51 -> 326 (70 and 68 with the pool).
+// A place goes from handle to handle as it is: its launch counts go on, so the tags of earlier launches in its words
+// never match.
 constexpr int kDecodePlaces = 4;
 constexpr size_t kDecodePlaceBytes = 1280 * 1024;
 static __device__ __align__(256) unsigned char g_decode_places[kDecodePlaces][kDecodePlaceBytes];
