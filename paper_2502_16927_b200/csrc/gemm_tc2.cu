@@ -468,8 +468,15 @@ bool gemm_tc_pair_supported(const GemmArgs& g) {
 // are 3-20 % faster on every shape (each SM stages half of B) but one: the training expert GEMM1, whose epilogue
 // (activation, sigma' quantisation, two output streams) keeps the issue slots so busy that one MMA-issuing thread per
 // SM instead of one per pair is worth 2.5 % (0.615-0.626 vs 0.633-0.642 ms in three interleaved runs).
+// So is a short contraction whose output leaves through staging (ascend, dx, dz) up to eight rounds of tiles: with four or five k
+// slices a tile there is little of B to share, and a pair's start, hand-over and exit take 2 to 3 us more (2999 tokens:
+// ascend 11.3 -> 8.9 us, dx 11.7 -> 9.6, dz 29.7 -> 26.3; d 1024, 4096 tokens: 8.9 -> 6.0, 9.7 -> 6.9, 15.1 -> 14.4; 16384 tokens of
+// d 2048: within 10 % either way).
 bool gemm_tc_pair_preferred(const GemmArgs& g) {
-    return gemm_tc_pair_supported(g) && !(g.epilogue == EPI_ACT && g.Z != nullptr);
+    const int64_t tiles = (int64_t)((g.M + BM - 1) / BM) * ((g.N + 255) / 256);
+    const bool short_staged = output_heavy(g) && tma_epilogue_possible(g) && !g.C2 && g.N % 256 == 0 && g.group != GROUP_K &&
+                              g.K <= 320 && tiles <= 8 * (int64_t)sm_count();
+    return gemm_tc_pair_supported(g) && !(g.epilogue == EPI_ACT && g.Z != nullptr) && !short_staged;
 }
 
 cudaError_t gemm_tc_pair(const GemmArgs& g, int* status, cudaStream_t stream) {

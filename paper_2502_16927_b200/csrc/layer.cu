@@ -390,11 +390,11 @@ int check_call(const bigmac_layer* L, int32_t T) {
 bool uses_groupk(const bigmac_layer* L, int id, const GemmArgs& g) {
     const bool enabled = switches().groupk != 0;
     const bool tc = L->cfg.dtype == BIGMAC_BF16 && L->use_tc && ((L->tc_mask >> id) & 1u);
-    // below about 16 k slices of work per CTA pair the items are too short for dynamic hand-out to pay (measured:
-    // +10 us per launch at 1024 tokens of the medium shape, -31 % at 16384 tokens with Zipf loads)
-    const int64_t tiles = (int64_t)((g.M + 255) / 256) * ((g.N + 255) / 256);
-    const bool enough = (L->cfg.flags & BIGMAC_FLAG_DYNAMIC_WGRAD) ||
-                        (int64_t)(g.K / 64) * tiles >= 16 * (int64_t)(gemm_tc_sm_count() / 2);
+    // Dynamic hand-out and the parts' addition pay from about 1500 rows an expert on.  A training step with even / Zipf loads,
+    // dynamic against static, us: d 2048, 375 rows 282 / 322 and 267 / 296, 1125 rows 501 / 571 and 486 / 555, 1500 rows 650 / 705
+    // and 638 / 711, 2048 rows 778 / 877 and 837 / 892; d 4096, 500 rows 1350 / 1508 and 1325 / 1455; d 1024, 2048 rows 303 / 329 and
+    // 297 / 363.  (g.K: the rows with at most 128 of padding for each expert.)
+    const bool enough = (L->cfg.flags & BIGMAC_FLAG_DYNAMIC_WGRAD) || g.K >= (int64_t)(1536 + kPad) * g.num_experts;
     return enabled && tc && enough && gemm_tc_groupk_supported(g);
 }
 

@@ -811,7 +811,7 @@ struct RouteArgs {
     int per_block;                                   // tokens of a block, at most four for each of its warps
 };
 template <int Q, int MOVE>
-__global__ void __launch_bounds__(kPlaceThreads) route_cluster_kernel(const RouteArgs r, const PlaceArgs p) {
+__global__ void __cluster_dims__(kRouteCluster, 1, 1) __launch_bounds__(kPlaceThreads) route_cluster_kernel(const RouteArgs r, const PlaceArgs p) {
     constexpr int kWarps = kPlaceThreads / 32;
     extern __shared__ float4 route_quads[];          // [Q][threads]; then the counts of the warps
     int32_t* warp_run = reinterpret_cast<int32_t*>(route_quads + Q * kPlaceThreads);      // [kWarps][E]
@@ -1000,15 +1000,7 @@ cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, cons
         int clusters = (r.per_block + 3) / 4;
         if (clusters > 12) clusters = 12;
         const int quads = E <= 32 ? 1 : E <= 64 ? 2 : 4;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = kRouteCluster * clusters; cfg.blockDim = kPlaceThreads; cfg.stream = stream;
-        cfg.dynamicSmemBytes = (size_t)quads * kPlaceThreads * sizeof(float4) + sizeof(int32_t) * (kPlaceThreads / 32) * E;     // 40 KB at most
-        cudaLaunchAttribute attr[2];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = kRouteCluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr; cfg.numAttrs = switches().chain ? 2 : 1;
+        const size_t smem = (size_t)quads * kPlaceThreads * sizeof(float4) + sizeof(int32_t) * (kPlaceThreads / 32) * E;     // 40 KB at most
 #define BIGMAC_ROUTE(Q)                                                                                                            \
     do {                                                                                                                           \
         const auto kernel = mv.partial ? route_cluster_kernel<Q, 2> : route_cluster_kernel<Q, 1>;                                 \
@@ -1020,7 +1012,7 @@ cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, cons
             if (e != cudaSuccess) return e;                                                                                        \
             once.mark(dev);                                                                                                        \
         }                                                                                                                          \
-        return cudaLaunchKernelEx(&cfg, kernel, r, p);                                                                             \
+        return launch_chained(kernel, kRouteCluster * clusters, kPlaceThreads, smem, stream, r, p);                                \
     } while (0)
         if (E <= 32) BIGMAC_ROUTE(1);
         if (E <= 64) BIGMAC_ROUTE(2);
