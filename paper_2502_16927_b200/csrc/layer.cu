@@ -805,6 +805,13 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         BIGMAC_CUDA(launch_gate_colsum(b.dp, b.tb, G->db_gate, b.colsum_part, m.N, m.E, acc, sd, aux_part));
         colsum_done = true;
     }
+    if (G->dw2) {   // dW2_e[c',q] = sum_rows du[row,c'] a[row,q]; before dz, which then is still in L2 for dxg where it fits
+        GemmArgs g;
+        g.A = b.du; g.lda = m.r; g.a_kmajor = false; g.B = b.a; g.ldb = m.h; g.b_kmajor = false;
+        g.C = G->dw2; g.ldc = m.h; g.c_stride = (int64_t)m.r * m.h; g.M = m.r; g.N = m.h; g.K = (int)m.P;
+        g.group = GROUP_K; g.num_experts = m.E; g.poffsets = b.tb.poffsets; g.accumulate = acc;
+        BIGMAC_TRY(batch ? together.add(G_DW2, g, st) : expert_weight_grad(L, G_DW2, g, b.expert_ws, st));
+    }
     {   // dz = (du W2_e) * sigma'(z); the forward saved sigma'(z) in the z buffer, dz is written over it
         GemmArgs g;
         g.A = b.du; g.lda = m.r; g.B = W->w2; g.ldb = m.h; g.b_kmajor = false; g.b_stride = (int64_t)m.r * m.h;
@@ -826,13 +833,6 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         Stage s(L, S_COLSUM, sb, 2 * ((G->db1 ? 1 : 0) + (G->db2 ? 1 : 0)));
         if (G->db1) BIGMAC_CUDA(launch_grouped_colsum(dz, b.tb.poffsets, G->db1, b.bias_ws, m.E, m.h, m.dtype, acc, sb));
         if (G->db2) BIGMAC_CUDA(launch_grouped_colsum(b.du, b.tb.poffsets, G->db2, b.bias_ws, m.E, m.r, m.dtype, acc, sb));
-    }
-    if (G->dw2) {   // dW2_e[c',q] = sum_rows du[row,c'] a[row,q]
-        GemmArgs g;
-        g.A = b.du; g.lda = m.r; g.a_kmajor = false; g.B = b.a; g.ldb = m.h; g.b_kmajor = false;
-        g.C = G->dw2; g.ldc = m.h; g.c_stride = (int64_t)m.r * m.h; g.M = m.r; g.N = m.h; g.K = (int)m.P;
-        g.group = GROUP_K; g.num_experts = m.E; g.poffsets = b.tb.poffsets; g.accumulate = acc;
-        BIGMAC_TRY(batch ? together.add(G_DW2, g, st) : expert_weight_grad(L, G_DW2, g, b.expert_ws, st));
     }
     {   // dxg = dz W1_e
         GemmArgs g;
