@@ -472,7 +472,12 @@ bool gemm_tc_pair_supported(const GemmArgs& g) {
 // slices a tile there is little of B to share, and a pair's start, hand-over and exit take 2 to 3 us more (2999 tokens:
 // ascend 11.3 -> 8.9 us, dx 11.7 -> 9.6, dz 29.7 -> 26.3; d 1024, 4096 tokens: 8.9 -> 6.0, 9.7 -> 6.9, 15.1 -> 14.4; 16384 tokens of
 // d 2048: within 10 % either way).
+// And so are the grouped contractions where most experts have one tile of rows: a pair's second CTA then works on padding.
+// (d 4096, 128 experts, 37 to 125 rows each: GEMM2 79 -> 72, 83 -> 81 us, dz 80 -> 73, 85 -> 80, dxg 74 -> 67, 80 -> 77; at 250 rows
+// within 2 %.)  Of the weight gradients dW2, with its wide rows (81 -> 64, 87 -> 80); dW1 is 3 to 10 % slower that way.
 bool gemm_tc_pair_preferred(const GemmArgs& g) {
+    if (g.group == GROUP_M && g.M <= 2 * kPad * (int64_t)g.num_experts) return false;       // M, K: at most kPad of padding an expert
+    if (g.group == GROUP_K && g.K <= 2 * kPad * (int64_t)g.num_experts && g.N > g.M) return false;
     const int64_t tiles = (int64_t)((g.M + BM - 1) / BM) * ((g.N + 255) / 256);
     const bool short_staged = output_heavy(g) && tma_epilogue_possible(g) && !g.C2 && g.N % 256 == 0 && g.group != GROUP_K &&
                               g.K <= 320 && tiles <= 8 * (int64_t)sm_count();
