@@ -142,3 +142,27 @@ def test_equal_and_nonfinite_logits(E, k):
         want = np.array(sorted(range(E), key=lambda e: (-key[e], e))[:k])
         np.testing.assert_array_equal(to_numpy(R["topk_idx"]).reshape(T, k), np.tile(want, (T, 1)))
         layer.close()
+
+
+@pytest.mark.parametrize("E,k", [(4, 4), (33, 8), (64, 8), (100, 40), (256, 16)])
+@pytest.mark.parametrize("T", [1, 3, 16])
+def test_small_batch_orders_equal_and_nonfinite_logits(E, k, T):
+    """The same order in the one-kernel forward of a few tokens, every token with a bias pattern of its own column order."""
+    import torch
+
+    w = wl.Workload("ties", T=T, d=64, r=64, h=64, E=E, k=k, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=3)
+    inp = wl.make_inputs(w)
+    inp["x"] = np.zeros_like(inp["x"])
+    rng = np.random.default_rng(E)
+    layer = make_layer(w)
+    for values in ([1.0], [0.0, -0.0, -1.0], [2.0, 2.0, -3.0], [-np.inf, np.nan], [np.inf, 1.0, np.nan, -np.inf], None):
+        bias = (rng.standard_normal(E) if values is None else rng.choice(np.array(values), E)).astype(np.float32)
+        inp["b_gate"] = bias
+        dev = to_device(w, inp)
+        R = layer.forward(dev["x"], dev, want_routing=True)[1]
+        torch.cuda.synchronize()
+        assert layer.status() == 0
+        key = np.where(np.isnan(bias), -np.inf, bias)
+        want = np.array(sorted(range(E), key=lambda e: (-key[e], e))[:k])
+        np.testing.assert_array_equal(to_numpy(R["topk_idx"]).reshape(T, k), np.tile(want, (T, 1)))
+    layer.close()
