@@ -29,9 +29,12 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kDecodeThreads = 512, kWarps = kDecodeThreads / 32;
-constexpr int kDecodeMaxTokens = 16;
+constexpr int kDecodeMaxTokens = 16;        // 16 tokens: 18.6 us against 26 of the launch chain at d 1024, 33.0 against 35.7 at d 2048
 constexpr int kDecodeMaxExperts = 256;
-constexpr int kDecodeMaxHidden = 16384;     // k h: the hidden activations of one token are staged in shared memory (64 KB)
+constexpr int kDecodeMaxSlots = 2048;       // T k: every CTA keeps all slots' expert ids and gate values
+// Hidden activations of one token staged in shared memory at a time (128 KB).  (64 KB, two passes for k h = 32768: 2 tokens of d 2048,
+// r 256, h 4096, 64 experts, k 8 24.4 -> 27.8 us.)
+constexpr int kDecodeMaxHidden = 32768;
 constexpr int kDecodeMaxUpBytes = 32768;    // W'_up rows of a CTA kept in shared memory
 constexpr size_t kDecodeMaxWords = 1u << 20; // hand-over words (8 MB) a handle keeps at most
 
@@ -68,7 +71,7 @@ struct DecodeArgs {
     Split rows_a, groups_c, rows_e;    // who does what in phases A, C (groups of rows of all slots) and E
     Split cols_d;                      // phase D: columns of a token over its CTAs
     int ctas_d;                        // phase D: CTAs per token
-    Divisor by_parts, by_pieces, by_k, by_slot, by_ctas;   // parts of a row in A; pieces of x; k; groups of a slot in C; ctas_d
+    Divisor by_parts, by_pieces, by_k, by_slot, by_ctas, by_pass;   // parts of a row in A; pieces of x; k; groups of a slot in C; ctas_d; slots of a pass in D
     // shared memory, offsets in floats: region (x; then x'; then a of a token; then y'), W'_up rows, logits, slots, sums
     int up_rows, off_up, off_log, off_idx, off_val, off_w, off_sums;
 };
@@ -360,7 +363,7 @@ __device__ __forceinline__ void phase_c(const DecodeArgs& p, uint32_t tag) {
 }
 
 // D: y'[t, c] = sum_j p_j (W2_{e_j}[c, :] a_j): floor(grid / T) CTAs per token, some columns each, ROWS (column, slot) rows per
-// warp and step.
+// warp and step; in passes over groups of slots where a token's hidden activations are more than shared memory takes.
 template <int ROWS>
 __device__ __forceinline__ void phase_d(const DecodeArgs& p, uint32_t tag) {
     const int tid = threadIdx.x, lane = tid & 31, b = blockIdx.x, hp = p.h / 8;
@@ -369,16 +372,19 @@ __device__ __forceinline__ void phase_d(const DecodeArgs& p, uint32_t tag) {
     float* sums = smem_at(p.off_sums);
     const bool works = b < p.T * p.ctas_d;           // the last grid - T floor(grid / T) CTAs have no columns: rows = 0
     const int t = works ? p.by_ctas.div(b) : 0, share = works ? b - t * p.ctas_d : 0, c0 = p.cols_d.first(share);
-    const int rows = works ? (p.cols_d.first(share + 1) - c0) * p.k : 0;     // row i: column c0 + i / k, slot i % k
+    const int per_pass = (int)p.by_pass.d;                   // slots of a pass
+    const int rows = works ? (p.cols_d.first(share + 1) - c0) * per_pass : 0;    // row i of a pass: column c0 + i / per_pass, slot i % per_pass
+    const int* experts = s_idx + t * p.k;
     uint4 wv[ROWS][4];
     const uint4* w[ROWS];
     int slot[ROWS];
+    int left = p.k;                                          // slots of this pass and those after it
     auto rows_at = [&](int i) {                              // rows i, i + kWarps, ...
 #pragma unroll
         for (int n = 0; n < ROWS; ++n) {
-            const int row = min(i + n * kWarps, max(rows - 1, 0)), col = p.by_k.div(row);
-            slot[n] = row - col * p.k;
-            w[n] = reinterpret_cast<const uint4*>(p.w2) + ((int64_t)s_idx[t * p.k + slot[n]] * p.r + c0 + col) * hp;
+            const int row = min(i + n * kWarps, max(rows - 1, 0)), col = p.by_pass.div(row);
+            slot[n] = min(row - col * per_pass, left - 1);   // (the last pass may have fewer slots: rows that count for nothing)
+            w[n] = reinterpret_cast<const uint4*>(p.w2) + ((int64_t)experts[slot[n]] * p.r + c0 + col) * hp;
         }
     };
     auto fetch = [&](int c) {                                // four pieces of a lane
@@ -387,46 +393,53 @@ __device__ __forceinline__ void phase_d(const DecodeArgs& p, uint32_t tag) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) wv[n][u] = c + 32 * u < hp ? __ldg(w[n] + c + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
     };
-    int i = tid >> 5;
-    rows_at(i);
-    if (i < rows) fetch(lane);                               // the first rows are on their way before the wait for a
-    __syncthreads();                                         // x' is not read any more, its place takes a
-    if (rows > 0) get_words(smem_at(0), p.a + (int64_t)t * p.k * p.h, p.k * p.h, tid, kDecodeThreads, tag, p.status);
-    __syncthreads();
+    const unsigned long long* words = p.a + (int64_t)t * p.k * p.h;
     const float4* v = reinterpret_cast<const float4*>(smem_at(0));
 #pragma unroll 1
-    for (; i < rows; i += ROWS * kWarps) {
-        f32x2 acc2[ROWS] = {};
-        int from[ROWS];
-#pragma unroll
-        for (int n = 0; n < ROWS; ++n) from[n] = 2 * slot[n] * hp;
+    for (float* pass = sums; left > 0; pass += rows, experts += per_pass, words += per_pass * p.h, left -= per_pass) {
+        int i = tid >> 5;
+        rows_at(i);
+        if (i < rows) fetch(lane);                           // the first rows are on their way before the wait for a
+        __syncthreads();                                     // x' or the slots before are not read any more, their place takes a
+        if (rows > 0) get_words(smem_at(0), words, min(per_pass, left) * p.h, tid, kDecodeThreads, tag, p.status);
+        __syncthreads();
 #pragma unroll 1
-        for (int c = lane; c - lane < hp; c += 128) {
+        for (; i < rows; i += ROWS * kWarps) {
+            f32x2 acc2[ROWS] = {};
+            int from[ROWS];
 #pragma unroll
-            for (int n = 0; n < ROWS; ++n)
+            for (int n = 0; n < ROWS; ++n) from[n] = 2 * slot[n] * hp;
+#pragma unroll 1
+            for (int c = lane; c - lane < hp; c += 128) {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int at = from[n] + min(c + 32 * u, hp - 1);        // past the end: zero weights
-                    acc2[n] = dot8(Piece(wv[n][u]), v[at], v[at + hp], acc2[n]);
-                }
-            int next = c + 128;
-            if (next - lane >= hp && i + ROWS * kWarps < rows) { rows_at(i + ROWS * kWarps); next = lane; }
-            fetch(next);
+                for (int n = 0; n < ROWS; ++n)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int at = from[n] + min(c + 32 * u, hp - 1);        // past the end: zero weights
+                        acc2[n] = dot8(Piece(wv[n][u]), v[at], v[at + hp], acc2[n]);
+                    }
+                int next = c + 128;
+                if (next - lane >= hp && i + ROWS * kWarps < rows) { rows_at(i + ROWS * kWarps); next = lane; }
+                fetch(next);
+            }
+            float acc[ROWS];
+#pragma unroll
+            for (int n = 0; n < ROWS; ++n) acc[n] = sum2(acc2[n]);
+            constexpr int L = 32 / ROWS;
+            const float u = warp_reduce_scatter<ROWS>(acc);                      // row lane / L
+            const int row = i + lane / L * kWarps;
+            if (!(lane & (L - 1)) && row < rows) pass[row] = u;
         }
-        float acc[ROWS];
-#pragma unroll
-        for (int n = 0; n < ROWS; ++n) acc[n] = sum2(acc2[n]);
-        constexpr int L = 32 / ROWS;
-        const float u = warp_reduce_scatter<ROWS>(acc);                      // row lane / L
-        const int row = i + lane / L * kWarps;
-        if (!(lane & (L - 1)) && row < rows) sums[row] = u;
     }
     __syncthreads();
 #pragma unroll 1
-    for (int c = tid; c * p.k < rows; c += kDecodeThreads) {       // combine in slot order
+    for (int c = tid; c * per_pass < rows; c += kDecodeThreads) {  // combine in slot order
         float acc = 0.0f;
+        const float* from = sums + c * per_pass;
+#pragma unroll 1
+        for (int j0 = 0; j0 < p.k; j0 += per_pass, from += rows)
 #pragma unroll 4
-        for (int j = 0; j < p.k; ++j) acc = fmaf(s_w[t * p.k + j], sums[c * p.k + j], acc);
+            for (int j = 0; j < min(per_pass, p.k - j0); ++j) acc = fmaf(s_w[t * p.k + j0 + j], from[j], acc);
         put_copies(p, p.y_lo + t * p.r + split_index(c0 + c, p.r), acc, tag);
     }
 }
@@ -485,11 +498,13 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_forward_kernel(const
 size_t decode_smem(DecodeArgs& p, int grid) {
     const int T = p.T, d = p.d, r = p.r, h = p.h, E = p.E, k = p.k;
     int region = T * (d > r ? d : r);
-    if (k * h > region) region = k * h;
+    const int passes = (k * h + kDecodeMaxHidden - 1) / kDecodeMaxHidden, per_pass = (k + passes - 1) / passes;     // phase D
+    if (per_pass * h > region) region = per_pass * h;
+    p.by_pass = Divisor(per_pass);
     const int up = (d + grid - 1) / grid;
     p.LE = (E + 3) / 4 * 4;
     p.up_rows = (size_t)up * r * 2 <= kDecodeMaxUpBytes ? up : 0;
-    const int per_token = grid / T > 1 ? grid / T : 1, rows = ((r + per_token - 1) / per_token) * k;     // phase D's rows of a CTA
+    const int per_token = grid / T > 1 ? grid / T : 1, rows = ((r + per_token - 1) / per_token) * passes * per_pass;     // phase D's rows of a CTA
     const int sums_a = ((r + E + grid - 1) / grid) * ((d / 8 + 31) / 32) * 16, sums = rows > sums_a ? rows : sums_a;   // phase A's parts
     p.off_up = (region + 3) / 4 * 4;
     p.off_log = p.off_up + p.up_rows * r / 2;                // r is a multiple of 8
@@ -513,9 +528,15 @@ DecodeArgs decode_shape(int T, int d, int r, int h, int E, int k) {
 
 }  // namespace
 
+// Every slot streams its expert's weights for itself, from L2 where another had them before; the launch chain reads them once.
+// From more than two slots an expert and 48 million weights a matrix streamed on the chain is the faster one (d 2048, r 512, h 2048, 64
+// experts, k 16: 8 tokens 79.6 us against 81.2, 12 tokens 110 against 82; d 1024, r 256, h 8192, 16 experts, k 6: 4 tokens 45.4
+// against 52.1, 6 tokens 57.9 against 53.0), with fewer weights it is not (r 128, h 512, 64 experts, k 32: 8 tokens 30.8 against 36.5).
+static bool streams_too_much(int T, int r, int h, int E, int k) { return (int64_t)T * k > 2 * E && (int64_t)T * k * h * r > 48000000; }
+
 bool decode_forward_supported(int T, int d, int r, int h, int E, int k, int dtype, int num_sms) {
     if (dtype != BIGMAC_BF16 || T < 1 || T > kDecodeMaxTokens || (int64_t)T * d > 32768 || d % 8 || r % 8 || h % 16 ||
-        E > kDecodeMaxExperts || (int64_t)k * h > kDecodeMaxHidden || T * k > kDecodeThreads || T > num_sms ||
+        E > kDecodeMaxExperts || h > kDecodeMaxHidden || T * k > kDecodeMaxSlots || streams_too_much(T, r, h, E, k) || T > num_sms ||
         decode_forward_words(T, r, h, E, k) > kDecodeMaxWords)
         return false;
     DecodeArgs p = decode_shape(T, d, r, h, E, k);

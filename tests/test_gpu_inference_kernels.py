@@ -166,3 +166,39 @@ def test_small_batch_orders_equal_and_nonfinite_logits(E, k, T):
         want = np.array(sorted(range(E), key=lambda e: (-key[e], e))[:k])
         np.testing.assert_array_equal(to_numpy(R["topk_idx"]).reshape(T, k), np.tile(want, (T, 1)))
     layer.close()
+
+
+def _small_batch(w, one_kernel):
+    """A forward of a few tokens against the oracle, in one kernel or not."""
+    import torch
+    from paper_2502_16927_b200 import binding
+
+    inp = _inputs(w, 0.0)
+    dev = to_device(w, inp)
+    layer = make_layer(w)
+    binding.bigmac_profile_enable(layer.handle, True)
+    y = layer.forward(dev["x"], dev)
+    launches = binding.bigmac_profile_read(layer.handle)["launches"]
+    assert (launches == 1) == one_kernel, launches
+    binding.bigmac_profile_enable(layer.handle, False)
+    again = layer.forward(dev["x"], dev)
+    torch.cuda.synchronize()
+    assert layer.status() == 0 and torch.equal(y, again)
+    ref = oracle.forward_tokens(inp, oracle.route(inp, w.k), w.act)["y"]
+    err = np.linalg.norm(to_numpy(y) - ref) / np.linalg.norm(ref)
+    # bf16 stores of 0.17 % of the rms each: y alone in the one kernel, x', a, u, y' and y in the launch chain
+    assert err <= (4e-3 if one_kernel else 8e-3), err
+    layer.close()
+
+
+@pytest.mark.parametrize("r,h,E,k,T", [
+    (64, 8192, 8, 4, 1), (64, 8192, 8, 5, 3), (64, 16384, 4, 3, 2), (64, 32768, 4, 1, 2),    # one pass over the slots, two, of unequal length
+    (64, 64, 64, 64, 9),                                                                      # 576 slots
+    (256, 9408, 8, 4, 4)])                                                                    # the last batch in front of the launch chain
+def test_small_batch_with_many_hidden_units(r, h, E, k, T):
+    _small_batch(wl.Workload("hidden", T=T, d=128, r=r, h=h, E=E, k=k, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=900 + T), True)
+
+
+@pytest.mark.parametrize("r,h,E,k,T", [(256, 9408, 8, 4, 5), (64, 32832, 4, 1, 1)])
+def test_small_batch_left_to_the_launch_chain(r, h, E, k, T):
+    _small_batch(wl.Workload("chain", T=T, d=128, r=r, h=h, E=E, k=k, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=900 + T), False)
