@@ -35,7 +35,7 @@ constexpr int kDecodeMaxSlots = 2048;       // T k: every CTA keeps all slots' e
 // Hidden activations of one token staged in shared memory at a time (128 KB).  (64 KB, two passes for k h = 32768: 2 tokens of d 2048,
 // r 256, h 4096, 64 experts, k 8 24.4 -> 27.8 us.)
 constexpr int kDecodeMaxHidden = 32768;
-constexpr int kDecodeMaxUpBytes = 32768;    // W'_up rows of a CTA kept in shared memory
+constexpr int kDecodeMaxUpBytes = 65536;    // W'_up rows of a CTA kept in shared memory (56 KB at d 8192, r 512: 4 tokens 24.0 -> 22.6 us)
 constexpr size_t kDecodeMaxWords = 1u << 20; // hand-over words (8 MB) a handle keeps at most
 
 // n / d for 0 <= n < 2^31 by a multiplication (d >= 1; round-up method with a 31-bit dividend).
@@ -478,7 +478,8 @@ __device__ __forceinline__ void phase_e(const DecodeArgs& p, uint32_t tag) {
 }
 
 // TG 1: for one or two tokens, where every phase is a single chain of latencies; TG 4: four tokens' sums at a time, more
-// loads in flight per warp.
+// loads in flight per warp.  Three tokens: 16.8 us by TG 4, 17.1 by TG 1 at d 2048, 30.9 and 35.7 at d 4096.  Two tokens: 15.2 and
+// 15.1 at d 2048 (k h = 8192), but 25.5 and 27.2 at d 4096 (k h = 16384), 20.6 and 21.1 at d 8192.
 template <int TG>
 __global__ void __launch_bounds__(kDecodeThreads, 1) decode_forward_kernel(const __grid_constant__ DecodeArgs p) {
     constexpr int ROWS_C = TG == 1 ? 4 : 8, ROWS_D = TG == 1 ? 1 : 2;
@@ -493,6 +494,8 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_forward_kernel(const
     if (threadIdx.x == 0) p.epoch[blockIdx.x] = tag;         // nobody else reads or writes this CTA's word
 }
 
+constexpr size_t kDecodeSmemLimit = 220 * 1024;
+
 // Shared memory of a launch, offsets in floats: the region that x, x', a and y' take in turn, rows of
 // W'_up, and the rest.
 size_t decode_smem(DecodeArgs& p, int grid) {
@@ -503,9 +506,11 @@ size_t decode_smem(DecodeArgs& p, int grid) {
     p.by_pass = Divisor(per_pass);
     const int up = (d + grid - 1) / grid;
     p.LE = (E + 3) / 4 * 4;
-    p.up_rows = (size_t)up * r * 2 <= kDecodeMaxUpBytes ? up : 0;
+    p.up_rows = 0;
     const int per_token = grid / T > 1 ? grid / T : 1, rows = ((r + per_token - 1) / per_token) * passes * per_pass;     // phase D's rows of a CTA
     const int sums_a = ((r + E + grid - 1) / grid) * ((d / 8 + 31) / 32) * 16, sums = rows > sums_a ? rows : sums_a;   // phase A's parts
+    const size_t rest = (size_t)((region + 3) / 4 * 4) + T * p.LE + 3 * T * k + sums;
+    if ((size_t)up * r * 2 <= kDecodeMaxUpBytes && sizeof(float) * rest + (size_t)up * r * 2 <= kDecodeSmemLimit) p.up_rows = up;
     p.off_up = (region + 3) / 4 * 4;
     p.off_log = p.off_up + p.up_rows * r / 2;                // r is a multiple of 8
     p.off_idx = p.off_log + T * p.LE;
@@ -514,8 +519,6 @@ size_t decode_smem(DecodeArgs& p, int grid) {
     p.off_sums = p.off_w + T * k;
     return sizeof(float) * ((size_t)p.off_sums + sums);
 }
-constexpr size_t kDecodeSmemLimit = 220 * 1024;
-
 // Where x', logits and y' are a few lines of memory that all CTAs poll, copies keep the readers from queueing up (14.2 -> 13.9 us
 // for one token, 19.4 -> 18.7 for four at r = 256; nothing for eight).
 constexpr int decode_copies(int T, int r) { return T * r <= 512 ? 4 : T * r <= 1024 ? 2 : 1; }
@@ -570,7 +573,7 @@ cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void
     p.b_gate = W->b_gate; p.y = (__nv_bfloat16*)y;
     p.x_lo = (unsigned long long*)words; p.logits = p.x_lo + (size_t)T * r; p.y_lo = p.logits + (size_t)T * p.LE; p.copies = decode_copies(T, r); p.copy_words = T * (2 * r + p.LE); p.a = p.x_lo + (size_t)p.copies * p.copy_words;
     p.topk_idx = topk_idx; p.topk_w = topk_w; p.epoch = epoch; p.status = status; p.act = act;
-    const bool few = T <= 2;
+    const bool few = T == 1 || (T == 2 && k * h <= 8192 && d <= 4096);
     const int rows_c = few ? 4 : 8;
     p.rows_a = Split(r + E, num_sms); p.rows_e = Split(d, num_sms); p.groups_c = Split(T * k * (h / rows_c), num_sms);
     p.ctas_d = num_sms / T > 1 ? num_sms / T : 1; p.cols_d = Split(r, p.ctas_d);

@@ -202,3 +202,11 @@ def test_small_batch_with_many_hidden_units(r, h, E, k, T):
 @pytest.mark.parametrize("r,h,E,k,T", [(256, 9408, 8, 4, 5), (64, 32832, 4, 1, 1)])
 def test_small_batch_left_to_the_launch_chain(r, h, E, k, T):
     _small_batch(wl.Workload("chain", T=T, d=128, r=r, h=h, E=E, k=k, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=900 + T), False)
+
+
+@pytest.mark.parametrize("d,r,h,E,k,T", [
+    (8192, 512, 64, 8, 2, 2), (8192, 512, 64, 8, 2, 4),          # W'_up rows of a block: 57 KB of shared memory ...
+    (8192, 1024, 64, 8, 2, 4),                                    # ... and more than it takes
+    (128, 64, 1024, 16, 8, 2), (128, 64, 1088, 16, 8, 2)])       # two tokens on either side of the change of variant
+def test_small_batch_variants(d, r, h, E, k, T):
+    _small_batch(wl.Workload("var", T=T, d=d, r=r, h=h, E=E, k=k, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=950 + T), True)
