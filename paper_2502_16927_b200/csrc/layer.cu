@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "layer_common.h"
+#include "place_pool.h"
 #include "switches.h"
 
 namespace bigmac {
@@ -31,28 +32,21 @@ constexpr size_t kDecodePlaceBytes = 1280 * 1024;
 static __device__ __align__(256) unsigned char g_decode_places[kDecodePlaces][kDecodePlaceBytes];
 
 namespace {
-constexpr int kDecodeDevices = 64;
-std::mutex g_decode_mutex;
-bool g_decode_taken[kDecodeDevices][kDecodePlaces] = {};
+struct CudaApi {
+    static int get(int* device) { return cudaGetDevice(device); }
+    static int set(int device) { return cudaSetDevice(device); }
+    static int synchronize() { return cudaDeviceSynchronize(); }
+};
+PlacePool<64, kDecodePlaces> g_decode_pool;
 
 // A free place of the current device: its number, or -1.
 int take_decode_place(int device, size_t bytes, void** base) {
     void* all = nullptr;
-    if (bytes > kDecodePlaceBytes || device < 0 || device >= kDecodeDevices) return -1;
-    std::lock_guard<std::mutex> lock(g_decode_mutex);
-    for (int i = 0; i < kDecodePlaces; ++i)
-        if (!g_decode_taken[device][i]) {
-            if (cudaGetSymbolAddress(&all, g_decode_places) != cudaSuccess || !all) { cudaGetLastError(); return -1; }
-            *base = (unsigned char*)all + i * kDecodePlaceBytes;
-            g_decode_taken[device][i] = true;
-            return i;
-        }
-    return -1;
-}
-void give_decode_memory(bigmac_layer* L) {           // after the handle's work on the device is done
-    if (L->decode_place < 0) { cudaFree(L->decode_epochs); return; }
-    std::lock_guard<std::mutex> lock(g_decode_mutex);
-    g_decode_taken[L->device][L->decode_place] = false;
+    if (bytes > kDecodePlaceBytes) return -1;
+    if (cudaGetSymbolAddress(&all, g_decode_places) != cudaSuccess || !all) { cudaGetLastError(); return -1; }
+    const int place = g_decode_pool.take(device);
+    if (place >= 0) *base = (unsigned char*)all + place * kDecodePlaceBytes;
+    return place;
 }
 }  // namespace
 
@@ -502,7 +496,8 @@ int bigmac_layer_create(const bigmac_config_t* cfg, bigmac_layer_t** out) {
         L->decode_words = (char*)L->decode_epochs + head;
     }
     if (L->use_tc && !gemm_tc_available()) {
-        give_decode_memory(L);
+        if (L->decode_place >= 0) g_decode_pool.give_unused(L->device, L->decode_place);
+        else cudaFree(L->decode_epochs);
         cudaFree(L->status);
         delete L;
         return BIGMAC_ERR_UNSUPPORTED;
@@ -527,9 +522,12 @@ int bigmac_layer_destroy(bigmac_layer_t* L) {
     for (cudaEvent_t e : L->fork_join)
         if (e) cudaEventDestroy(e);
     if (L->side) cudaStreamDestroy(L->side);
-    if (L->decode_place >= 0) cudaDeviceSynchronize();   // nothing of this handle runs when another takes its place in the pool
-    cudaFree(L->status);
-    give_decode_memory(L);
+    {
+        OnDevice<CudaApi> on(L->device);             // whatever device the caller is on
+        if (L->decode_place >= 0) g_decode_pool.give<CudaApi>(L->device, L->decode_place);
+        else cudaFree(L->decode_epochs);
+        cudaFree(L->status);
+    }
     delete L;
     return BIGMAC_OK;
 }
