@@ -48,6 +48,26 @@ int take_decode_place(int device, size_t bytes, void** base) {
     if (place >= 0) *base = (unsigned char*)all + place * kDecodePlaceBytes;
     return place;
 }
+
+void free_side(bigmac_layer* L) {
+    for (cudaEvent_t& e : L->fork_join)
+        if (e) { cudaEventDestroy(e); e = nullptr; }
+    if (L->side) { cudaStreamDestroy(L->side); L->side = nullptr; }
+}
+
+// `used`: calls may have run on the handle.
+void free_handle(bigmac_layer* L, bool used) {
+    for (cudaEvent_t e : L->ev) cudaEventDestroy(e);
+    free_side(L);
+    {
+        OnDevice<CudaApi> on(L->device);             // whatever device the caller is on
+        if (L->decode_place < 0) cudaFree(L->decode_epochs);
+        else if (used) g_decode_pool.give<CudaApi>(L->device, L->decode_place);
+        else g_decode_pool.give_unused(L->device, L->decode_place);
+        cudaFree(L->status);
+    }
+    delete L;
+}
 }  // namespace
 
 namespace bigmac {
@@ -479,38 +499,33 @@ int bigmac_layer_create(const bigmac_config_t* cfg, bigmac_layer_t** out) {
     const int few = plain ? decode_forward_max_tokens(cfg->max_tokens, cfg->d, cfg->r, cfg->h, cfg->E, cfg->k, cfg->dtype, gemm_tc_sm_count()) : 0;
     const size_t words = decode_forward_words(few, cfg->r, cfg->h, cfg->E, cfg->k);
     const size_t head = ((size_t)gemm_tc_sm_count() * 4 + 255) / 256 * 256, bytes = head + 8 * words;
-    if (cudaGetDevice(&L->device) != cudaSuccess || cudaMalloc((void**)&L->status, 256) != cudaSuccess ||
-        cudaMemset(L->status, 0, 256) != cudaSuccess) {
-        cudaFree(L->status);
+    if (cudaGetDevice(&L->device) != cudaSuccess) {
         delete L;
         return BIGMAC_ERR_CUDA;
-    }
-    if (words) {
-        L->decode_place = take_decode_place(L->device, bytes, (void**)&L->decode_epochs);
-        if (L->decode_place < 0 && (cudaMalloc((void**)&L->decode_epochs, bytes) != cudaSuccess || cudaMemset(L->decode_epochs, 0, bytes) != cudaSuccess)) {
-            cudaFree(L->decode_epochs);
-            cudaFree(L->status);
-            delete L;
-            return BIGMAC_ERR_CUDA;
-        }
-        L->decode_words = (char*)L->decode_epochs + head;
-    }
-    if (L->use_tc && !gemm_tc_available()) {
-        if (L->decode_place >= 0) g_decode_pool.give_unused(L->device, L->decode_place);
-        else cudaFree(L->decode_epochs);
-        cudaFree(L->status);
-        delete L;
-        return BIGMAC_ERR_UNSUPPORTED;
     }
     // the backward pass's second stream and its fork / join events; without them the pass runs on one stream
     bool side_ok = cudaStreamCreateWithFlags(&L->side, cudaStreamNonBlocking) == cudaSuccess;
     for (cudaEvent_t& e : L->fork_join)
         side_ok = side_ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
     if (!side_ok) {
-        for (cudaEvent_t& e : L->fork_join)
-            if (e) { cudaEventDestroy(e); e = nullptr; }
-        if (L->side) { cudaStreamDestroy(L->side); L->side = nullptr; }
+        free_side(L);
         cudaGetLastError();
+    }
+    bool ok = cudaMalloc((void**)&L->status, 256) == cudaSuccess && cudaMemsetAsync(L->status, 0, 256, L->side) == cudaSuccess;
+    if (ok && words) {
+        L->decode_place = take_decode_place(L->device, bytes, (void**)&L->decode_epochs);
+        if (L->decode_place < 0)
+            ok = cudaMalloc((void**)&L->decode_epochs, bytes) == cudaSuccess && cudaMemsetAsync(L->decode_epochs, 0, bytes, L->side) == cudaSuccess;
+        L->decode_words = (char*)L->decode_epochs + head;
+    }
+    // The first call may come on any stream: the clears are waited for here, on a stream that nothing else is queued on.
+    if (!ok || cudaStreamSynchronize(L->side) != cudaSuccess) {
+        free_handle(L, false);
+        return BIGMAC_ERR_CUDA;
+    }
+    if (L->use_tc && !gemm_tc_available()) {
+        free_handle(L, false);
+        return BIGMAC_ERR_UNSUPPORTED;
     }
     *out = L;
     return BIGMAC_OK;
@@ -518,17 +533,7 @@ int bigmac_layer_create(const bigmac_config_t* cfg, bigmac_layer_t** out) {
 
 int bigmac_layer_destroy(bigmac_layer_t* L) {
     if (!L) return BIGMAC_ERR_INVALID_ARG;
-    for (cudaEvent_t e : L->ev) cudaEventDestroy(e);
-    for (cudaEvent_t e : L->fork_join)
-        if (e) cudaEventDestroy(e);
-    if (L->side) cudaStreamDestroy(L->side);
-    {
-        OnDevice<CudaApi> on(L->device);             // whatever device the caller is on
-        if (L->decode_place >= 0) g_decode_pool.give<CudaApi>(L->device, L->decode_place);
-        else cudaFree(L->decode_epochs);
-        cudaFree(L->status);
-    }
-    delete L;
+    free_handle(L, true);
     return BIGMAC_OK;
 }
 

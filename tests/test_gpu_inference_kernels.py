@@ -210,3 +210,32 @@ def test_small_batch_left_to_the_launch_chain(r, h, E, k, T):
     (128, 64, 1024, 16, 8, 2), (128, 64, 1088, 16, 8, 2)])       # two tokens on either side of the change of variant
 def test_small_batch_variants(d, r, h, E, k, T):
     _small_batch(wl.Workload("var", T=T, d=d, r=r, h=h, E=E, k=k, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=950 + T), True)
+
+
+def test_first_call_on_another_stream_while_the_default_stream_is_busy():
+    """Handles made behind queued work of the default stream, more of them than the pool has places, first used on a stream that
+    is not ordered with it: nothing that making them left behind may come between (or after) their launches."""
+    import torch
+
+    w = wl.Workload("busy", T=3, d=128, r=64, h=128, E=8, k=2, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=41)
+    inp = _inputs(w, 0.0)
+    dev = to_device(w, inp)
+    layer = make_layer(w)
+    want = layer.forward(dev["x"], dev)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    torch.cuda._sleep(200_000_000)                       # about 0.1 s of the default stream
+    layers = [layer]
+    with torch.cuda.stream(side):
+        outs = []
+        for _ in range(8):
+            layers.append(make_layer(w))
+            outs += [layers[-1].forward(dev["x"], dev) for _ in range(3)]
+        side.synchronize()
+    torch.cuda.synchronize()
+    outs += [one.forward(dev["x"], dev) for one in layers]
+    for y in outs:
+        assert torch.equal(y, want)
+    for one in layers:
+        assert one.status() == 0
+        one.close()
