@@ -73,7 +73,7 @@ struct DecodeArgs {
     int ctas_d;                        // phase D: CTAs per token
     Divisor by_parts, by_pieces, by_k, by_slot, by_ctas, by_pass;   // parts of a row in A; pieces of x; k; groups of a slot in C; ctas_d; slots of a pass in D
     // shared memory, offsets in floats: region (x; then x'; then a of a token; then y'), W'_up rows, logits, slots, sums
-    int up_rows, off_up, off_log, off_idx, off_val, off_w, off_sums;
+    int up_rows, off_up, off_log, off_idx, off_w, off_sums;
 };
 extern __shared__ float4 decode_smem_raw[];
 __device__ __forceinline__ float* smem_at(int off) { return reinterpret_cast<float*>(decode_smem_raw) + off; }
@@ -261,6 +261,31 @@ __device__ __forceinline__ uint32_t order_key(float v) {
     return b ^ (uint32_t)((int32_t)b >> 31 | (int32_t)0x80000000);
 }
 
+// The experts of one token by one warp: rounds of arg-max over the lanes' experts lane + 32 q (E <= 32 Q), in registers.  (Counting
+// the experts before each expert takes no rounds, but E^2 T comparisons: 35.1 us instead of 33.5 for 16 tokens of 64 experts, 59
+// instead of 17 for 16 of 256 at d 1024, r 128, h 512, k 2.)
+template <int Q>
+__device__ __forceinline__ void select_experts(const float* l, int* idx, int E, int k) {
+    const int lane = threadIdx.x & 31;
+    uint32_t key[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) key[q] = lane + 32 * q < E ? max(order_key(l[lane + 32 * q]), 1u) : 0u;
+#pragma unroll 1
+    for (int j = 0; j < k; ++j) {
+        uint32_t mine = key[0];
+#pragma unroll
+        for (int q = 1; q < Q; ++q) mine = max(mine, key[q]);
+        const uint32_t best = __reduce_max_sync(kFull, mine);
+        uint32_t e = kDecodeMaxExperts;
+#pragma unroll
+        for (int q = Q - 1; q >= 0; --q) e = key[q] == best ? lane + 32 * q : e;
+        e = __reduce_min_sync(kFull, e);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) key[q] = lane + 32 * q == e ? 0u : key[q];
+        if (lane == 0) idx[j] = (int)e;
+    }
+}
+
 // B: top-k by (logit descending, expert id ascending), softmax over the k kept logits; x' takes x's place.
 __device__ __forceinline__ void phase_b(const DecodeArgs& p, uint32_t tag) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -268,42 +293,24 @@ __device__ __forceinline__ void phase_b(const DecodeArgs& p, uint32_t tag) {
     const bool logits = tid < half;
     float* s_log = smem_at(p.off_log);
     int* s_idx = reinterpret_cast<int*>(smem_at(p.off_idx));
-    float* s_val = smem_at(p.off_val);
     float* s_w = smem_at(p.off_w);
     __syncthreads();
     get_words(smem_at(logits ? p.off_log : 0), (logits ? p.logits : p.x_lo) + blockIdx.x % p.copies * p.copy_words, logits ? p.T * p.LE : p.T * p.r, tid & (half - 1), half, tag, p.status);
     __syncthreads();
-    // A warp per token (T <= 16 warps): rounds of arg-max over the lanes' experts lane + 32 q, all in registers.  (Counting the
-    // experts before each expert takes no rounds, but E^2 T comparisons: 35.1 us instead of 33.5 for 16 tokens of 64 experts, 59
-    // instead of 17 for 16 of 256 at d 1024, r 128, h 512, k 2.)
+    // a warp per token (T <= 16 warps)
     if (warp < p.T) {
-        const float* l = s_log + warp * p.LE;
-        uint32_t key[kDecodeMaxExperts / 32];
-#pragma unroll
-        for (int q = 0; q < kDecodeMaxExperts / 32; ++q) key[q] = lane + 32 * q < p.E ? max(order_key(l[lane + 32 * q]), 1u) : 0u;
-#pragma unroll 1
-        for (int j = 0; j < p.k; ++j) {
-            uint32_t mine = key[0];
-#pragma unroll
-            for (int q = 1; q < kDecodeMaxExperts / 32; ++q) mine = max(mine, key[q]);
-            const uint32_t best = __reduce_max_sync(kFull, mine);
-            uint32_t e = kDecodeMaxExperts;
-#pragma unroll
-            for (int q = kDecodeMaxExperts / 32 - 1; q >= 0; --q) e = key[q] == best ? lane + 32 * q : e;
-            e = __reduce_min_sync(kFull, e);
-#pragma unroll
-            for (int q = 0; q < kDecodeMaxExperts / 32; ++q) key[q] = lane + 32 * q == e ? 0u : key[q];
-            if (lane == 0) { s_idx[warp * p.k + j] = (int)e; s_val[warp * p.k + j] = l[e]; }
-        }
+        if (p.E <= 64) select_experts<2>(s_log + warp * p.LE, s_idx + warp * p.k, p.E, p.k);
+        else select_experts<kDecodeMaxExperts / 32>(s_log + warp * p.LE, s_idx + warp * p.k, p.E, p.k);
     }
     __syncthreads();
     if (warp < p.T) {
         const int at = warp * p.k;
-        const float top = s_val[at];
+        const float* l = s_log + warp * p.LE;
+        const float top = l[s_idx[at]];
         float sum = 0.0f;
 #pragma unroll 1
         for (int j = lane; j < p.k; j += 32) {
-            const float ex = top == -INFINITY ? 1.0f : expf(s_val[at + j] - top);      // only -inf logits kept: 1/k each
+            const float ex = top == -INFINITY ? 1.0f : expf(l[s_idx[at + j]] - top);      // only -inf logits kept: 1/k each
             s_w[at + j] = ex;
             sum += ex;
         }
@@ -364,7 +371,8 @@ __device__ __forceinline__ void phase_c(const DecodeArgs& p, uint32_t tag) {
 
 // D: y'[t, c] = sum_j p_j (W2_{e_j}[c, :] a_j): floor(grid / T) CTAs per token, some columns each, ROWS (column, slot) rows per
 // warp and step; in passes over groups of slots where a token's hidden activations are more than shared memory takes.
-template <int ROWS>
+// MANY: more passes than one.
+template <int ROWS, bool MANY>
 __device__ __forceinline__ void phase_d(const DecodeArgs& p, uint32_t tag) {
     const int tid = threadIdx.x, lane = tid & 31, b = blockIdx.x, hp = p.h / 8;
     const int* s_idx = reinterpret_cast<const int*>(smem_at(p.off_idx));
@@ -372,7 +380,7 @@ __device__ __forceinline__ void phase_d(const DecodeArgs& p, uint32_t tag) {
     float* sums = smem_at(p.off_sums);
     const bool works = b < p.T * p.ctas_d;           // the last grid - T floor(grid / T) CTAs have no columns: rows = 0
     const int t = works ? p.by_ctas.div(b) : 0, share = works ? b - t * p.ctas_d : 0, c0 = p.cols_d.first(share);
-    const int per_pass = (int)p.by_pass.d;                   // slots of a pass
+    const int per_pass = MANY ? (int)p.by_pass.d : p.k;      // slots of a pass
     const int rows = works ? (p.cols_d.first(share + 1) - c0) * per_pass : 0;    // row i of a pass: column c0 + i / per_pass, slot i % per_pass
     const int* experts = s_idx + t * p.k;
     uint4 wv[ROWS][4];
@@ -383,7 +391,8 @@ __device__ __forceinline__ void phase_d(const DecodeArgs& p, uint32_t tag) {
 #pragma unroll
         for (int n = 0; n < ROWS; ++n) {
             const int row = min(i + n * kWarps, max(rows - 1, 0)), col = p.by_pass.div(row);
-            slot[n] = min(row - col * per_pass, left - 1);   // (the last pass may have fewer slots: rows that count for nothing)
+            slot[n] = row - col * per_pass;
+            if (MANY) slot[n] = min(slot[n], left - 1);      // (the last pass may have fewer slots: rows that count for nothing)
             w[n] = reinterpret_cast<const uint4*>(p.w2) + ((int64_t)experts[slot[n]] * p.r + c0 + col) * hp;
         }
     };
@@ -396,12 +405,12 @@ __device__ __forceinline__ void phase_d(const DecodeArgs& p, uint32_t tag) {
     const unsigned long long* words = p.a + (int64_t)t * p.k * p.h;
     const float4* v = reinterpret_cast<const float4*>(smem_at(0));
 #pragma unroll 1
-    for (float* pass = sums; left > 0; pass += rows, experts += per_pass, words += per_pass * p.h, left -= per_pass) {
+    for (float* pass = sums; left > 0; pass += rows, experts += per_pass, words += per_pass * p.h, left = MANY ? left - per_pass : 0) {
         int i = tid >> 5;
         rows_at(i);
         if (i < rows) fetch(lane);                           // the first rows are on their way before the wait for a
         __syncthreads();                                     // x' or the slots before are not read any more, their place takes a
-        if (rows > 0) get_words(smem_at(0), words, min(per_pass, left) * p.h, tid, kDecodeThreads, tag, p.status);
+        if (rows > 0) get_words(smem_at(0), words, (MANY ? min(per_pass, left) : p.k) * p.h, tid, kDecodeThreads, tag, p.status);
         __syncthreads();
 #pragma unroll 1
         for (; i < rows; i += ROWS * kWarps) {
@@ -437,9 +446,9 @@ __device__ __forceinline__ void phase_d(const DecodeArgs& p, uint32_t tag) {
         float acc = 0.0f;
         const float* from = sums + c * per_pass;
 #pragma unroll 1
-        for (int j0 = 0; j0 < p.k; j0 += per_pass, from += rows)
+        for (int j0 = 0; j0 < (MANY ? p.k : 1); j0 += per_pass, from += rows)
 #pragma unroll 4
-            for (int j = 0; j < min(per_pass, p.k - j0); ++j) acc = fmaf(s_w[t * p.k + j0 + j], from[j], acc);
+            for (int j = 0; j < (MANY ? min(per_pass, p.k - j0) : p.k); ++j) acc = fmaf(s_w[t * p.k + j0 + j], from[j], acc);
         put_copies(p, p.y_lo + t * p.r + split_index(c0 + c, p.r), acc, tag);
     }
 }
@@ -480,7 +489,7 @@ __device__ __forceinline__ void phase_e(const DecodeArgs& p, uint32_t tag) {
 // TG 1: for one or two tokens, where every phase is a single chain of latencies; TG 4: four tokens' sums at a time, more
 // loads in flight per warp.  Three tokens: 16.8 us by TG 4, 17.1 by TG 1 at d 2048, 30.9 and 35.7 at d 4096.  Two tokens: 15.2 and
 // 15.1 at d 2048 (k h = 8192), but 25.5 and 27.2 at d 4096 (k h = 16384), 20.6 and 21.1 at d 8192.
-template <int TG>
+template <int TG, bool MANY>
 __global__ void __launch_bounds__(kDecodeThreads, 1) decode_forward_kernel(const __grid_constant__ DecodeArgs p) {
     constexpr int ROWS_C = TG == 1 ? 4 : 8, ROWS_D = TG == 1 ? 1 : 2;
     uint32_t tag;
@@ -489,7 +498,7 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_forward_kernel(const
     phase_a<TG>(p, tag);
     phase_b(p, tag);
     phase_c<ROWS_C>(p, tag);
-    phase_d<ROWS_D>(p, tag);
+    phase_d<ROWS_D, MANY>(p, tag);
     phase_e<TG>(p, tag);
     if (threadIdx.x == 0) p.epoch[blockIdx.x] = tag;         // nobody else reads or writes this CTA's word
 }
@@ -509,13 +518,12 @@ size_t decode_smem(DecodeArgs& p, int grid) {
     p.up_rows = 0;
     const int per_token = grid / T > 1 ? grid / T : 1, rows = ((r + per_token - 1) / per_token) * passes * per_pass;     // phase D's rows of a CTA
     const int sums_a = ((r + E + grid - 1) / grid) * ((d / 8 + 31) / 32) * 16, sums = rows > sums_a ? rows : sums_a;   // phase A's parts
-    const size_t rest = (size_t)((region + 3) / 4 * 4) + T * p.LE + 3 * T * k + sums;
+    const size_t rest = (size_t)((region + 3) / 4 * 4) + T * p.LE + 2 * T * k + sums;
     if ((size_t)up * r * 2 <= kDecodeMaxUpBytes && sizeof(float) * rest + (size_t)up * r * 2 <= kDecodeSmemLimit) p.up_rows = up;
     p.off_up = (region + 3) / 4 * 4;
     p.off_log = p.off_up + p.up_rows * r / 2;                // r is a multiple of 8
     p.off_idx = p.off_log + T * p.LE;
-    p.off_val = p.off_idx + T * k;
-    p.off_w = p.off_val + T * k;
+    p.off_w = p.off_idx + T * k;
     p.off_sums = p.off_w + T * k;
     return sizeof(float) * ((size_t)p.off_sums + sums);
 }
@@ -571,7 +579,12 @@ cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void
     p.x = (const __nv_bfloat16*)x; p.w_gate = (const __nv_bfloat16*)W->w_gate; p.w_down = (const __nv_bfloat16*)W->w_down;
     p.w1 = (const __nv_bfloat16*)W->w1; p.w2 = (const __nv_bfloat16*)W->w2; p.w_up = (const __nv_bfloat16*)W->w_up;
     p.b_gate = W->b_gate; p.y = (__nv_bfloat16*)y;
-    p.x_lo = (unsigned long long*)words; p.logits = p.x_lo + (size_t)T * r; p.y_lo = p.logits + (size_t)T * p.LE; p.copies = decode_copies(T, r); p.copy_words = T * (2 * r + p.LE); p.a = p.x_lo + (size_t)p.copies * p.copy_words;
+    p.copies = decode_copies(T, r);
+    p.copy_words = T * (2 * r + p.LE);
+    p.x_lo = (unsigned long long*)words;
+    p.logits = p.x_lo + (size_t)T * r;
+    p.y_lo = p.logits + (size_t)T * p.LE;
+    p.a = p.x_lo + (size_t)p.copies * p.copy_words;
     p.topk_idx = topk_idx; p.topk_w = topk_w; p.epoch = epoch; p.status = status; p.act = act;
     const bool few = T == 1 || (T == 2 && k * h <= 8192 && d <= 4096);
     const int rows_c = few ? 4 : 8;
@@ -581,16 +594,17 @@ cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void
     p.by_ctas = Divisor(p.ctas_d);
     static PerDeviceOnce once;
     int dev;
-    const void* kernel1 = (const void*)decode_forward_kernel<1>;
-    const void* kernel4 = (const void*)decode_forward_kernel<4>;
+    const void* kernels[2][2] = {{(const void*)decode_forward_kernel<4, false>, (const void*)decode_forward_kernel<4, true>},
+                                 {(const void*)decode_forward_kernel<1, false>, (const void*)decode_forward_kernel<1, true>}};
     if (once.needed(&dev)) {
-        cudaError_t e = cudaFuncSetAttribute(kernel1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemLimit);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemLimit);
-        if (e != cudaSuccess) return e;
+        for (int i = 0; i < 4; ++i) {
+            const cudaError_t e = cudaFuncSetAttribute(kernels[i / 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecodeSmemLimit);
+            if (e != cudaSuccess) return e;
+        }
         once.mark(dev);
     }
     void* ptrs[] = {(void*)&p};
-    return cudaLaunchCooperativeKernel(few ? kernel1 : kernel4, dim3(num_sms), dim3(kDecodeThreads), ptrs, smem, stream);
+    return cudaLaunchCooperativeKernel(kernels[few][(int)p.by_pass.d < k], dim3(num_sms), dim3(kDecodeThreads), ptrs, smem, stream);
 }
 
 }  // namespace bigmac
