@@ -42,6 +42,10 @@ int bigmac_debug_gemm(bigmac_layer_t *L, const bigmac_debug_gemm_t *q, int use_t
  * bigmac_device_status returns BIGMAC_ERR_TIMEOUT and the handle and the context stay usable. */
 int bigmac_debug_expire_wait(bigmac_layer_t *L, void *stream);
 
+/* Test aid: sets the number of launches that the small-batch kernel's memory has counted so far (its tags go on from there), as
+ * if that many one-kernel forwards had run on it; synchronises `stream`.  UNSUPPORTED for a handle without that memory. */
+int bigmac_debug_decode_launches(bigmac_layer_t *L, uint32_t launches, void *stream);
+
 /* Measurement aid for the dispatch/combine stage (Eq. 1: bytes through the exchange are proportional
  * to the row width): run the standalone dispatch and combine kernels on rows of `width` elements of
  * the layer's dtype.  width = r is BigMac's exchange; width = d is what a fine-grained layer of equal

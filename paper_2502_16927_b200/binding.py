@@ -90,6 +90,8 @@ def lib() -> C.CDLL:
         L.bigmac_debug_gemm.argtypes = [vp, C.POINTER(bigmac_debug_gemm_t), C.c_int, vp]
         L.bigmac_debug_expire_wait.argtypes = [vp, vp]
         L.bigmac_debug_expire_wait.restype = C.c_int
+        L.bigmac_debug_decode_launches.argtypes = [vp, C.c_uint32, vp]
+        L.bigmac_debug_decode_launches.restype = C.c_int
         L.bigmac_debug_set.argtypes = [C.c_char_p, C.c_int]
         L.bigmac_debug_set.restype = C.c_int
         L.bigmac_route_static.argtypes = [vp, vp, i32, C.POINTER(bigmac_weights_t), C.POINTER(bigmac_routing_t), vp]
@@ -244,6 +246,11 @@ def bigmac_debug_set(name: str, value: int = 0) -> None:
 def bigmac_debug_expire_wait(handle) -> None:
     """Launch the one-thread kernel whose bounded wait runs out (failure path of the device-side waits)."""
     _check(lib().bigmac_debug_expire_wait(handle, _stream()), "bigmac_debug_expire_wait")
+
+
+def bigmac_debug_decode_launches(handle, launches: int) -> None:
+    """Set the launch count of the small-batch kernel's memory (the tags of its hand-over words go on from there)."""
+    _check(lib().bigmac_debug_decode_launches(handle, launches, _stream()), "bigmac_debug_decode_launches")
 
 
 # ---- expert parallelism: the phase calls, name for name ----------------------------------------------------

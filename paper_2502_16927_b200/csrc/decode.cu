@@ -11,8 +11,10 @@
 // Values that cross from one CTA to another (x', logits, a, y') travel as 8-byte words (fp32 value, tag of this launch):
 // the consumer polls the very words it needs until their tags match, so a hand-over is one store and one load through
 // L2.  With a grid-wide barrier (arrive, spin, then load) each of the three hand-overs took 2.2-2.7 us, 7 of the 15 us of
-// one token.  The words live in memory of the handle that is zero at first and written by this kernel only, and the tag
-// counts the handle's launches on the device (a captured launch can be replayed), so a stale word never matches.
+// one token.  The words are written by this kernel only, in memory that one handle at a time has and that was zero at first;
+// the tag counts the launches on that memory, on the device (a captured launch can be replayed).  A tag has 32 bits and would
+// meet itself after 2^32 launches (17 hours of one-token calls): so every launch also retags one word a block of those that its
+// own batch does not use, in turn, and no word is ever older than a few thousand launches.  A stale word never matches.
 // Code is executed once or a few times per launch, and a first execution waits for instruction fetch: phases are small
 // loops, ranges and divisors come ready from the host.  (Four extra warps that ran through the later phases' code
 // beforehand, without effect, gained nothing: what is left is the latency of the hand-overs and of the weights.)
@@ -63,7 +65,9 @@ struct DecodeArgs {
     unsigned long long *x_lo, *logits, *a, *y_lo;      // hand-over words: [T,r], [T,LE], [T*k,h], [T,r]
     int32_t* topk_idx;
     float* topk_w;
-    unsigned* epoch;                   // [grid] launches of this handle so far, a word of its own for every CTA
+    unsigned* epoch;                   // [grid] launches on this memory so far, a word of its own for every CTA
+    int used, total;                   // hand-over words of this launch, and of the memory that x_lo begins
+    unsigned sweep;                    // launches in which every word has its turn to be retagged, less one (a power of two, less one)
     int* status;
     int T, d, r, h, E, k, act;
     int copies, copy_words;            // x', logits and y' are written `copies` times, copy_words apart; CTA b reads copy b % copies
@@ -496,6 +500,10 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_forward_kernel(const
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(tag) : "l"(p.epoch + blockIdx.x) : "memory");
     ++tag;
     phase_a<TG>(p, tag);
+    if (threadIdx.x == kDecodeThreads - 1) {                 // (while the logits are on their way)
+        const int i = (int)((tag & p.sweep) * gridDim.x + blockIdx.x);
+        if (i >= p.used && i < p.total) put_word(p.x_lo + i, 0.0f, tag);
+    }
     phase_b(p, tag);
     phase_c<ROWS_C>(p, tag);
     phase_d<ROWS_D, MANY>(p, tag);
@@ -571,8 +579,8 @@ int decode_forward_max_tokens(int max_tokens, int d, int r, int h, int E, int k,
     return T;
 }
 
-cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void* y, void* words, int32_t* topk_idx, float* topk_w,
-                                  unsigned* epoch, int* status, int T, int d, int r, int h, int E, int k, int act,
+cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void* y, void* words, size_t word_count, int32_t* topk_idx,
+                                  float* topk_w, unsigned* epoch, int* status, int T, int d, int r, int h, int E, int k, int act,
                                   int num_sms, cudaStream_t stream) {
     DecodeArgs p = decode_shape(T, d, r, h, E, k);
     const size_t smem = decode_smem(p, num_sms);
@@ -585,6 +593,10 @@ cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void
     p.logits = p.x_lo + (size_t)T * r;
     p.y_lo = p.logits + (size_t)T * p.LE;
     p.a = p.x_lo + (size_t)p.copies * p.copy_words;
+    p.used = p.copies * p.copy_words + T * k * h;
+    p.total = (int)word_count;
+    if ((size_t)p.used > word_count || word_count > kDecodeMaxWords) return cudaErrorInvalidValue;
+    while ((size_t)(p.sweep + 1) * num_sms < word_count) p.sweep = 2 * p.sweep + 1;
     p.topk_idx = topk_idx; p.topk_w = topk_w; p.epoch = epoch; p.status = status; p.act = act;
     const bool few = T == 1 || (T == 2 && k * h <= 8192 && d <= 4096);
     const int rows_c = few ? 4 : 8;

@@ -308,14 +308,15 @@ struct WordCopies {
 };
 cudaError_t launch_word_copies(const WordCopies& c, cudaStream_t stream);
 
-// Small-batch inference forward in one cooperative kernel (bf16, T <= 16): writes y, topk_idx, topk_w.  words:
-// decode_forward_words() 8-byte words of the handle for the values that cross between CTAs, zero when the handle is made
-// and written by this kernel only; epoch: num_sms device words of the handle, zero at first (launches so far, per block).
+// Small-batch inference forward in one cooperative kernel (bf16, T <= 16): writes y, topk_idx, topk_w.  words: word_count >=
+// decode_forward_words() 8-byte words for the values that cross between CTAs; epoch: num_sms device words, the launches so far,
+// per block.  Both belong to the same memory, which was zero at first, which only this kernel writes and which one launch at a
+// time uses; handles of any widths may have it one after another.  No word's tag is above its memory's launch count.
 bool decode_forward_supported(int T, int d, int r, int h, int E, int k, int dtype, int num_sms);
 size_t decode_forward_words(int T, int r, int h, int E, int k);
 int decode_forward_max_tokens(int max_tokens, int d, int r, int h, int E, int k, int dtype, int num_sms);
-cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void* y, void* words, int32_t* topk_idx, float* topk_w,
-                                  unsigned* epoch, int* status, int T, int d, int r, int h, int E, int k, int act,
+cudaError_t launch_decode_forward(const void* x, const bigmac_weights_t* W, void* y, void* words, size_t word_count, int32_t* topk_idx,
+                                  float* topk_w, unsigned* epoch, int* status, int T, int d, int r, int h, int E, int k, int act,
                                   int num_sms, cudaStream_t stream);
 
 }  // namespace bigmac

@@ -517,6 +517,7 @@ int bigmac_layer_create(const bigmac_config_t* cfg, bigmac_layer_t** out) {
         if (L->decode_place < 0)
             ok = cudaMalloc((void**)&L->decode_epochs, bytes) == cudaSuccess && cudaMemsetAsync(L->decode_epochs, 0, bytes, L->side) == cudaSuccess;
         L->decode_words = (char*)L->decode_epochs + head;
+        L->decode_word_count = L->decode_place < 0 ? words : (kDecodePlaceBytes - head) / 8;     // of a place all, whoever has it
     }
     // The first call may come on any stream: the clears are waited for here, on a stream that nothing else is queued on.
     if (!ok || cudaStreamSynchronize(L->side) != cudaSuccess) {
@@ -600,7 +601,7 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
         decode_forward_supported(m.T, m.d, m.r, m.h, m.E, m.k, m.dtype, gemm_tc_sm_count())) {
         {
             Stage s(L, S_DECODE, st);
-            BIGMAC_CUDA(launch_decode_forward(x, W, y, L->decode_words, b.tb.topk_idx, b.tb.topk_w, L->decode_epochs,
+            BIGMAC_CUDA(launch_decode_forward(x, W, y, L->decode_words, L->decode_word_count, b.tb.topk_idx, b.tb.topk_w, L->decode_epochs,
                                               L->status, m.T, m.d, m.r, m.h, m.E, m.k, c.act, gemm_tc_sm_count(), st));
         }
         if (routing_out) {
@@ -1202,6 +1203,16 @@ int bigmac_debug_set(const char* name, int value) {
     else if (!std::strcmp(name, "tc_mask")) sw.tc_mask = (unsigned)value;
     else if (!std::strcmp(name, "defaults")) sw = Switches();
     else return BIGMAC_ERR_INVALID_ARG;
+    return BIGMAC_OK;
+}
+
+int bigmac_debug_decode_launches(bigmac_layer_t* L, uint32_t launches, void* stream) {
+    if (!L) return BIGMAC_ERR_INVALID_ARG;
+    if (!L->decode_epochs) return BIGMAC_ERR_UNSUPPORTED;
+    const std::vector<unsigned> counts(gemm_tc_sm_count(), launches);
+    if (cudaMemcpyAsync(L->decode_epochs, counts.data(), counts.size() * sizeof(unsigned), cudaMemcpyHostToDevice, (cudaStream_t)stream) != cudaSuccess ||
+        cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess)
+        return BIGMAC_ERR_CUDA;
     return BIGMAC_OK;
 }
 

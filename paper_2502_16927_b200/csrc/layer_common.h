@@ -17,6 +17,7 @@ struct bigmac_layer {
     // static pool (its number) or an allocation of the handle's own (-1)
     unsigned* decode_epochs = nullptr;
     void* decode_words = nullptr;
+    size_t decode_word_count = 0;
     int decode_place = -1;
     bool use_tc;        // bf16 contractions on tcgen05
     unsigned tc_mask;   // debug: bit i set = contraction i runs on tcgen05 (the tc_mask switch at creation)

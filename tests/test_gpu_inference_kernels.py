@@ -239,3 +239,38 @@ def test_first_call_on_another_stream_while_the_default_stream_is_busy():
     for one in layers:
         assert one.status() == 0
         one.close()
+
+
+@pytest.mark.parametrize("more_handles", [0, 4])
+def test_launch_count_of_the_small_batch_kernel_wraps(more_handles):
+    """Hand-over words carry the low 32 bits of a launch count.  A batch size that was last used 2^32 launches ago, with calls of
+    one token in between, must not find its old words valid; nor may the counts around the wrap.  In the pool and outside it."""
+    import torch
+    from paper_2502_16927_b200 import binding
+
+    w = wl.Workload("wrap", T=16, d=128, r=64, h=128, E=8, k=4, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=43)
+    inp = _inputs(w, 0.0)
+    dev = to_device(w, inp)
+    others = [make_layer(w) for _ in range(more_handles)]
+    layer = make_layer(w)
+    first, single = dev["x"].clone(), dev["x"][:1].clone()
+    second = dev["x"].flip(0).contiguous()
+    want, one = layer.forward(second, dev), layer.forward(single, dev)
+    start = (1 << 30) + (more_handles << 20)                        # far from the counts of other tests
+    for _ in range(2):
+        binding.bigmac_debug_decode_launches(layer.handle, start)
+        layer.forward(first, dev)                                   # its words carry start + 1
+        for _ in range(2500):                                       # in place of 2^32 - 1 calls of one token
+            y = layer.forward(single, dev)
+        assert torch.equal(y, one)
+        binding.bigmac_debug_decode_launches(layer.handle, start)
+        for _ in range(3):
+            assert torch.equal(layer.forward(second, dev), want)
+    binding.bigmac_debug_decode_launches(layer.handle, 2 ** 32 - 3)
+    for _ in range(6):
+        assert torch.equal(layer.forward(second, dev), want)
+        assert torch.equal(layer.forward(single, dev), one)
+    assert layer.status() == 0
+    binding.bigmac_debug_decode_launches(layer.handle, start + 10000)      # above all tags but those around the wrap
+    for each in others + [layer]:
+        each.close()
