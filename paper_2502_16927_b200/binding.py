@@ -145,8 +145,13 @@ def _ptr(t: Optional[torch.Tensor]):
     return t.data_ptr()
 
 
+_raw_stream, _current_device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream() -> int:
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is None or _current_device is None:      # a torch that has the two accessors under other names
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
 
 
 # ---- the C ABI, name for name -------------------------------------------------------------------------

@@ -20,3 +20,15 @@ def test_routing_tables(E, k, T):
     # what a program keeps of a step (its loss, its loads) does not keep the tables of all slots with it
     for name in ("aux_loss", "counts", "counts_chosen", "offsets"):
         assert R[name].untyped_storage().nbytes() <= 4 * (3 * (E + 3) + 5), name
+
+
+def test_stream_handle_without_the_private_accessors(monkeypatch):
+    class Stream:
+        cuda_stream = 1234
+
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: Stream)
+    monkeypatch.setattr(binding, "_raw_stream", None)
+    assert binding._stream() == 1234
+    monkeypatch.setattr(binding, "_raw_stream", lambda device: 10 * device)
+    monkeypatch.setattr(binding, "_current_device", lambda: 7)
+    assert binding._stream() == 70
