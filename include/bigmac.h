@@ -171,12 +171,15 @@ typedef struct {
 } bigmac_routing_t;
 
 /* Validate the configuration and create a handle on the current CUDA device.  Allocates a few
- * device words, with them (BF16 configurations whose small batches run in one kernel) up to 8 MB of words in which that
- * kernel's blocks hand values to each other (1.1 MB at d 2048, r 256, h 1024, k 8), one stream and ten events.
+ * device words, one stream and six events.  BF16 configurations whose small batches run in one kernel also have up to 8 MB
+ * of words in which that kernel's blocks hand values to each other (1.1 MB at d 2048, r 256, h 1024, k 8): up to 1.25 MB one of
+ * four places in static memory of the library (5 MB on every device that it is loaded on), given back when the handle is
+ * destroyed; above that, or with all four taken, an allocation of the handle's own.  Waits until its memory is cleared.
  * Errors: INVALID_ARG (null pointers, non-positive sizes, k > E, unknown enums, a negative or non-finite
  * capacity_factor or aux_loss_coef), UNSUPPORTED (BF16
  * with d, r or h not a multiple of 64; E > 1024), CUDA. */
 int bigmac_layer_create(const bigmac_config_t *cfg, bigmac_layer_t **out);
+/* Releases what create took, on the handle's own device, after the work of that device. */
 int bigmac_layer_destroy(bigmac_layer_t *L);
 
 /* Bytes the caller must provide for a call with T tokens: `scratch_bytes` of scratch (contents

@@ -83,8 +83,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if (warp == 1) tmem_alloc(tmem_slot, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
-    // Chained launch: everything above touched no global memory and may have run while the kernel before this one in
-    // the stream was still working.  Tensor memory is held, so the next kernel of the stream may be set up in turn;
+    // Chained launch: everything above touched no global memory (but for the hint to bring weights to L2, which is coherent) and
+    // may have run while the kernel before this one in the stream was still working.  Tensor memory is held, so the next kernel of the stream may be set up in turn;
     // from the wait on, the predecessor's results are complete.
     grid_dependency_launch();
     grid_dependency_wait();

@@ -26,7 +26,7 @@ using namespace bigmac::detail;
 // Memory of the small-batch kernel for a few handles (zero at first, like every __device__ array).  An allocation of its own, of
 // more than 1 MB, is a mapping of its own: creation of a handle 58 -> 413 us, destruction 51 -> 326 (70 and 68 with the pool).
 // A place goes from handle to handle as it is: its launch counts go on, so the tags of earlier launches in its words
-// never match.
+// never match (decode.cu has the rest).
 constexpr int kDecodePlaces = 4;
 constexpr size_t kDecodePlaceBytes = 1280 * 1024;
 static __device__ __align__(256) unsigned char g_decode_places[kDecodePlaces][kDecodePlaceBytes];
@@ -183,8 +183,9 @@ void carve_backward_scratch(Carver& cv, const Dims& m, Buffers& b) {
 // The descend + gate-logits launch has few output tiles where there are few tokens, each walking all of d; its contraction
 // is then cut into parts (fp32 partial results, added by the routing kernels on the way) so that the SMs share the work.
 // Cost of s parts: the longest SM's k slices (0.35 us each on a pair of SMs, 0.2 on one), plus what writing and reading the
-// partial results takes (0.8 us per MB).  At d = 2048, r + E = 320: 8 parts at 64 tokens, 4 at 512, 3 at 1200, none from
-// 1800 on (at 3001, three parts: launch 19.3 -> 16.3 us, placement 6.9 -> 10.4).  A function of the shape only: every call of a handle with the same T takes the same path.
+// partial results takes (0.8 us per MB).  At d = 2048, r + E = 320: 8 parts up to 195 tokens, 4 up to 585, 3 up to 976, 2 up to
+// 1562, then none (at 3001, three parts: launch 19.3 -> 16.3 us, placement 6.9 -> 10.4).  The times were fitted there and serve
+// every width.  A function of the shape only: every call of a handle with the same T takes the same path.
 int descend_split_parts(const Dims& m) {
     if (m.E % 4 || m.dtype != BIGMAC_BF16) return 1;
     const int n = m.r + m.E, num_kb = m.d / 64;
@@ -454,7 +455,7 @@ bool dispatch_is_fused(const bigmac_layer* L, const Dims& m, bool training) {
 // (dynamic work items, long experts in parts), else the generic grouped contraction.
 int expert_weight_grad(const bigmac_layer* L, int id, const GemmArgs& g, float* splitk_ws, cudaStream_t st) {
     if (uses_groupk(L, id, g)) {
-        { Stage stage(L, id, st); BIGMAC_CUDA(gemm_tc_groupk(g, L->status, L->status + 2, splitk_ws, st)); }
+        { Stage stage(L, id, st); BIGMAC_CUDA(gemm_tc_groupk(g, L->status, L->status + 1, splitk_ws, st)); }
         { Stage stage(L, S_SPLITK_REDUCE, st); BIGMAC_CUDA(gemm_tc_groupk_finish(g, splitk_ws, st)); }
         return BIGMAC_OK;
     }
@@ -717,7 +718,7 @@ int bigmac_backward(bigmac_layer_t* L, const void* x, const void* dy, int32_t T,
     if (rc != BIGMAC_OK && L && L->side_forked) {
         // a launch failed after work was forked to the second stream: join it, so that the caller's stream (and a
         // capture in progress) is not left with an open fork and nothing of this call outlives its return unordered
-        if (cudaEventRecord(L->fork_join[9], L->side) == cudaSuccess) cudaStreamWaitEvent((cudaStream_t)stream, L->fork_join[9], 0);
+        if (cudaEventRecord(L->fork_join[5], L->side) == cudaSuccess) cudaStreamWaitEvent((cudaStream_t)stream, L->fork_join[5], 0);
     }
     return rc;
 }
@@ -803,8 +804,8 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
     }
     bool colsum_done = false;
     if (overlap && G->db_gate) {
-        BIGMAC_CUDA(cudaEventRecord(L->fork_join[2], st));
-        BIGMAC_CUDA(cudaStreamWaitEvent(sd, L->fork_join[2], 0));
+        BIGMAC_CUDA(cudaEventRecord(L->fork_join[1], st));
+        BIGMAC_CUDA(cudaStreamWaitEvent(sd, L->fork_join[1], 0));
         Stage s(L, S_COLSUM, sd, 2);
         BIGMAC_CUDA(launch_gate_colsum(b.dp, b.tb, G->db_gate, b.colsum_part, m.N, m.E, acc, sd, aux_part));
         colsum_done = true;
@@ -830,8 +831,8 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         // beside the tensor-bound dW2 / dxg (joined with the dx' gather), on slice sums in a region of their own.
         cudaStream_t sb = st;
         if (overlap) {
-            BIGMAC_CUDA(cudaEventRecord(L->fork_join[8], st));
-            BIGMAC_CUDA(cudaStreamWaitEvent(sd, L->fork_join[8], 0));
+            BIGMAC_CUDA(cudaEventRecord(L->fork_join[4], st));
+            BIGMAC_CUDA(cudaStreamWaitEvent(sd, L->fork_join[4], 0));
             sb = sd;
         }
         Stage s(L, S_COLSUM, sb, 2 * ((G->db1 ? 1 : 0) + (G->db2 ? 1 : 0)));
@@ -893,8 +894,8 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
     // Joins the second stream: nothing of this call is left on it.
     auto join = [&]() -> int {
         if (!overlap) return BIGMAC_OK;
-        BIGMAC_CUDA(cudaEventRecord(L->fork_join[7], sd));
-        BIGMAC_CUDA(cudaStreamWaitEvent(st, L->fork_join[7], 0));
+        BIGMAC_CUDA(cudaEventRecord(L->fork_join[3], sd));
+        BIGMAC_CUDA(cudaStreamWaitEvent(st, L->fork_join[3], 0));
         return BIGMAC_OK;
     };
     if (m.gate_low) {
@@ -945,8 +946,8 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
     }
     if (fused) {
         if (overlap) {
-            BIGMAC_CUDA(cudaEventRecord(L->fork_join[6], st));
-            BIGMAC_CUDA(cudaStreamWaitEvent(sd, L->fork_join[6], 0));
+            BIGMAC_CUDA(cudaEventRecord(L->fork_join[2], st));
+            BIGMAC_CUDA(cudaStreamWaitEvent(sd, L->fork_join[2], 0));
         }
         {   // dx = [dx' | dl] [W_down ; W_gate]: one contraction over r + E
             GemmArgs g;
@@ -1018,8 +1019,8 @@ int bigmac_device_status(bigmac_layer_t* L, void* stream) {
         cudaMemsetAsync(L->status, 0, sizeof(int), st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
         return BIGMAC_ERR_CUDA;
     if (word != 0) {
-        // a kernel gave up on a wait: its work counters and the grid-barrier word may be mid-count; back to rest
-        if (cudaMemsetAsync(L->status + 1, 0, 3 * sizeof(int), st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+        // a kernel gave up on a wait: its work counters may be mid-count; back to rest
+        if (cudaMemsetAsync(L->status + 1, 0, 2 * sizeof(int), st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
             return BIGMAC_ERR_CUDA;
     }
     if (word == 2) return BIGMAC_ERR_STATE;            // an expert-parallel count matrix that cannot be right, or an expert id outside [0, E)

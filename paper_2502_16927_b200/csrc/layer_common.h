@@ -11,10 +11,10 @@
 struct bigmac_layer {
     bigmac_config_t cfg;
     int device;
-    int* status = nullptr;  // device status word; status[2..3] are the work counters of the per-expert weight-gradient kernel
+    int* status = nullptr;  // device status word; status[1..2] are the work counters of the per-expert weight-gradient kernel
                         // (zero at rest)
     // the small-batch kernel's memory, or null: launch counts, one per block, and hand-over words; a place of the library's
-    // static pool (its number) or an allocation of the handle's own (-1)
+    // static pool (its number; counts and words as the handle before left them) or an allocation of the handle's own (-1)
     unsigned* decode_epochs = nullptr;
     void* decode_words = nullptr;
     size_t decode_word_count = 0;
@@ -24,7 +24,7 @@ struct bigmac_layer {
     // second stream of the backward pass (created on first use): launches that do not depend on each other and lean
     // on different units (a tensor-bound weight gradient beside an HBM-bound row move) run side by side
     cudaStream_t side = nullptr;
-    cudaEvent_t fork_join[10] = {};     // [9]: joins the second stream back when a call fails after its fork
+    cudaEvent_t fork_join[6] = {};     // [5]: joins the second stream back when a call fails after its fork
     bool side_forked = false;          // the running bigmac_backward has put work on `side`
     // measurement aid
     bool prof_on = false;

@@ -57,26 +57,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 // Non-blocking test of a phase (try_wait may park the thread for a while before it looks again; a chain of short
 // dependent steps polls with this one instead).
-__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.b32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-__device__ __forceinline__ void mbar_spin(uint64_t* bar, uint32_t parity, volatile int* dead, int* status) {
-    if (*dead) return;
-    for (uint32_t i = 0; i < (kWaitLimit << 4); ++i) {
-        if (mbar_test_wait(bar, parity)) return;
-        if ((i & 4095u) == 4095u && *dead) return;
-    }
-    *dead = 1;
-    atomicExch(status, 1);
-}
 // Bounded wait.  `dead` is a CTA-wide flag in shared memory: once any wait ran out nobody waits again.
 __device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, volatile int* dead, int* status,
                                           uint32_t limit = kWaitLimit) {
