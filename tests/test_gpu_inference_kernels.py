@@ -7,7 +7,7 @@ import pytest
 import oracle
 from oracle import margin
 from paper_2502_16927_b200 import workloads as wl
-from helpers import make_layer, to_device, to_numpy
+from helpers import empty_grads, make_layer, to_device, to_numpy
 
 pytestmark = pytest.mark.gpu
 
@@ -98,17 +98,26 @@ def test_routing_in_two_launches(E, k, T):
 @pytest.mark.parametrize("T", [1, 7, 33, 259, 511, 512])
 def test_routing_in_one_launch(E, k, T):
     """A forward of up to 512 tokens routes in one launch (clusters that share the tokens): rows from a matrix (r 8, fp32) and from
-    partial results (bf16, contraction of d = 1024 in parts), with and without a capacity limit."""
+    partial results (bf16, contraction of d = 1024 in parts; a training forward also wants the padding rows as zeros, which its
+    weight gradients contract over), with and without a capacity limit."""
     import torch
     from paper_2502_16927_b200 import binding
 
-    for dtype, d, r, h in ((wl.DTYPE_F32, 32, 8, 8), (wl.DTYPE_BF16, 1024, 128, 64)):
+    for dtype, d, r, h, training in ((wl.DTYPE_F32, 32, 8, 8, True), (wl.DTYPE_BF16, 1024, 128, 64, False), (wl.DTYPE_BF16, 1024, 128, 64, True)):
         w = wl.Workload("route", T=T, d=d, r=r, h=h, E=E, k=k, dtype=dtype, act=wl.ACT_RELU, seed=35)
         inp = _inputs(w, 1.0)
         dev = to_device(w, inp)
         for f in (0.0, 0.6):
             layer = make_layer(w, capacity_factor=f, flags=0)
-            y, R = layer.forward(dev["x"], dev, want_routing=True, training=dtype == wl.DTYPE_F32)
+            if training:                                             # what lies in the workspaces must not reach a gradient
+                layer._workspaces(T, True)
+                layer._scratch.fill_(255)
+                layer._saved.fill_(255)
+            y, R = layer.forward(dev["x"], dev, want_routing=True, training=training)
+            if training:
+                G = empty_grads(w, "cuda", fill=float("nan"))
+                dx = layer.backward(dev["x"], dev["dy"], dev, G)
+                assert all(bool(torch.isfinite(v).all()) for v in (*G.values(), dx))
             torch.cuda.synchronize()
             assert layer.status() == 0
             rt = oracle.route(inp, w.k, capacity_factor=f)
@@ -274,3 +283,73 @@ def test_launch_count_of_the_small_batch_kernel_wraps(more_handles):
     binding.bigmac_debug_decode_launches(layer.handle, start + 10000)      # above all tags but those around the wrap
     for each in others + [layer]:
         each.close()
+
+
+def test_small_batch_memory_goes_from_call_to_call_and_from_handle_to_handle():
+    """The kernel's launch counts and hand-over words outlive a call and, in the pool of four places, a handle: batch sizes in any
+    order on one handle, handles of other widths in a place, more handles than places, on two streams at a time.  Bit for bit
+    what a handle that is alone computes."""
+    import torch
+
+    shapes = [dict(d=128, r=64, h=128, E=8, k=4), dict(d=256, r=192, h=320, E=12, k=2), dict(d=64, r=64, h=64, E=33, k=8)]
+    sizes = [16, 1, 3, 8, 2, 16, 5, 1]
+    cases = []
+    for n, shape in enumerate(shapes):
+        w = wl.Workload("pool", T=16, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=60 + n, **shape)
+        dev = to_device(w, _inputs(w, 0.0))
+        xs = {T: dev["x"][16 - T:].contiguous() for T in sizes}
+        want = {}
+        for T in sizes:
+            layer = make_layer(w)
+            want[T] = layer.forward(xs[T], dev)
+            layer.close()
+        cases.append((w, dev, xs, want))
+
+    def run(layer, case, order):
+        return [(layer.forward(case[2][T], case[1]), case[3][T]) for T in order]
+
+    got = []
+    for case in cases * 2:                                           # one handle after another
+        layer = make_layer(case[0])
+        for _ in range(3):
+            got += run(layer, case, sizes)
+        assert layer.status() == 0
+        layer.close()
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    layers = [make_layer(case[0]) for case in cases * 2]           # six at a time, three on each stream
+    for n in range(20):
+        for i, (layer, case) in enumerate(zip(layers, cases * 2)):
+            with torch.cuda.stream(streams[i // 3]):
+                got += run(layer, case, [sizes[(n + i) % len(sizes)]])
+    torch.cuda.synchronize()
+    assert all(torch.equal(y, want) for y, want in got)
+    for layer in layers:
+        assert layer.status() == 0
+        layer.close()
+
+
+@pytest.mark.parametrize("T", [1, 2, 16])
+def test_small_batch_forward_in_a_graph(T):
+    """The launch count is kept on the device: a captured call can be replayed, with other tokens, between plain calls."""
+    import torch
+
+    w = wl.Workload("graph", T=16, d=128, r=64, h=128, E=8, k=4, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=71)
+    dev = to_device(w, _inputs(w, 0.0))
+    batches = [dev["x"][i:i + T].contiguous() for i in range(0, 17 - T, max(1, T // 2))]
+    layer = make_layer(w)
+    want = [layer.forward(x, dev) for x in batches]
+    x, y = batches[0].clone(), torch.empty_like(batches[0])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        layer.forward(x, dev, y=y)
+    for _ in range(3):
+        for batch, ref in zip(batches, want):
+            x.copy_(batch)
+            graph.replay()
+            assert torch.equal(y, ref)
+            assert torch.equal(layer.forward(batches[-1], dev), want[-1])
+    assert layer.status() == 0
+    del graph
+    layer.close()

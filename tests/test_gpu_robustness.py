@@ -301,8 +301,10 @@ def test_chained_launches_equal_plain_launches(case):
 
 
 @pytest.mark.parametrize("case", [
-    dict(dtype=wl.DTYPE_F32, shape=dict(T=200, d=32, r=16, h=24, E=8, k=3)),               # generic top-k kernel
-    dict(dtype=wl.DTYPE_BF16, shape=dict(T=700, d=128, r=64, h=128, E=64, k=8)),            # four-tokens-per-warp kernel, three-pass sort
+    dict(dtype=wl.DTYPE_F32, shape=dict(T=200, d=32, r=16, h=24, E=8, k=3)),               # routing in one launch
+    dict(dtype=wl.DTYPE_BF16, shape=dict(T=700, d=128, r=64, h=128, E=64, k=8)),            # routing in two launches
+    dict(dtype=wl.DTYPE_F32, shape=dict(T=200, d=32, r=16, h=24, E=10, k=3)),              # generic top-k kernel, sort in one block
+    dict(dtype=wl.DTYPE_BF16, shape=dict(T=700, d=128, r=64, h=128, E=64, k=12)),           # generic top-k kernel, three-pass sort
     dict(dtype=wl.DTYPE_BF16, shape=dict(T=9, d=128, r=64, h=128, E=32, k=4), decode=True), # one-kernel small-batch forward
 ])
 def test_non_finite_logits_keep_every_expert_id_in_range(case):
