@@ -688,7 +688,9 @@ inline int sm_count() {
     return v;
 }
 
-// Is the problem's time its output's?  Wide rows; and activations of short contractions (d 1024: h = 512 on r = 128).
+// Is the problem's time its output's?  Wide rows; and activations of short contractions.  A training step of 4096 / 16384 tokens of
+// d 1024 without the second rule and with it: h 512 on r 64 149 -> 130 / 300 -> 270 us, r 128 152 -> 135 / 315 -> 287, r 256 180 -> 164 /
+// 371 -> 347; h 768 on r 128 171 -> 147 / 379 -> 344, r 256 202 -> 181 / 436 -> 400.  (r 384 would gain 3 to 6 % too.)
 inline bool output_heavy(const GemmArgs& g) { return g.N >= 1024 || (g.epilogue != EPI_NONE && g.N >= 512 && g.K <= 256); }
 
 // Can this problem's output leave through shared memory and TMA stores?
