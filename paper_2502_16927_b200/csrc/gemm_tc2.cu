@@ -472,7 +472,7 @@ bool gemm_tc_pair_supported(const GemmArgs& g) {
 // slices a tile there is little of B to share, and a pair's start, hand-over and exit take 2 to 3 us more (2999 tokens:
 // ascend 11.3 -> 8.9 us, dx 11.7 -> 9.6, dz 29.7 -> 26.3; d 1024, 4096 tokens: 8.9 -> 6.0, 9.7 -> 6.9, 15.1 -> 14.4; 16384 tokens of
 // d 2048: within 10 % either way).  The line at 320 is not sharp: training steps of six to ten slices (r 384 to 512 at d 2048 and 4096,
-// 1000 to 16384 tokens) move by 3 % either way with it at 512, 640 or 1024, faster up to 3000 tokens and slower above.
+// 1000 to 16384 tokens) move by less than 3 % with it at 512 or 640, faster up to 3000 tokens and slower above.
 // And so are the grouped contractions where most experts have one tile of rows: a pair's second CTA then works on padding.
 // (d 4096, 128 experts, 37 to 125 rows each: GEMM2 79 -> 72, 83 -> 81 us, dz 80 -> 73, 85 -> 80, dxg 74 -> 67, 80 -> 77; at 250 rows
 // within 2 %.)  Of the weight gradients dW2, with its wide rows (81 -> 64, 87 -> 80); dW1 is 3 to 10 % slower that way.

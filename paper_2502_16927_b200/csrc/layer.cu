@@ -185,7 +185,7 @@ void carve_backward_scratch(Carver& cv, const Dims& m, Buffers& b) {
 // Cost of s parts: the longest SM's k slices (0.35 us each on a pair of SMs, 0.2 on one), plus what writing and reading the
 // partial results takes (0.8 us per MB).  At d = 2048, r + E = 320: 8 parts up to 195 tokens, 4 up to 585, 3 up to 976, 2 up to
 // 1562, then none (at 3001, three parts: launch 19.3 -> 16.3 us, placement 6.9 -> 10.4).  The times were fitted there and serve
-// every width: against the best of 1, 2, 3, 4, 6 and 8 parts a forward of 24 to 512 tokens is within 3 % at d 1024 to 8192 (one of 54
+// every width: against the best of 1, 2, 3, 4, 6 and 8 parts a forward of 24 to 512 tokens is within 3 % at d 1024 to 8192 (one of 24
 // shapes 4.5 %, small layers of d 512 up to 6 %); from 700 to 1500 tokens of d 1024, and 700 to 1000 of d 2048, one part would be the
 // better choice (39.3 against 35.1 us, 57.3 against 52.1).  A function of the shape only: every call of a handle with the same T takes the same path.
 int descend_split_parts(const Dims& m) {
