@@ -65,8 +65,8 @@ __device__ __forceinline__ MlpItem mlp_item(const MlpParams& p, int tiles, int s
     t.expert = lo;
     t.rows = min(NT, s_off[lo + 1] - (int)s_pad[lo] - t.row0);
     t.n = t.rows > 0 ? (t.rows + 15) / 16 * 16 : 0;
-    t.chunks = p.sl.chunks >> (__ffs(slices) - 1);
-    t.c0 = t.slice * t.chunks;
+    t.c0 = t.slice * p.sl.chunks >> (__ffs(slices) - 1);
+    t.chunks = ((t.slice + 1) * p.sl.chunks >> (__ffs(slices) - 1)) - t.c0;
     return t;
 }
 

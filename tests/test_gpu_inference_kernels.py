@@ -371,3 +371,10 @@ def test_weights_hint_beside_few_and_many_descend_tiles(T):
     err = np.linalg.norm(to_numpy(y) - ref) / np.linalg.norm(ref)
     assert err <= 8e-3, err                              # four or five bf16 stores of 0.17 % of the rms each
     layer.close()
+
+
+@pytest.mark.parametrize("r,h", [(64, 3200), (256, 1408), (320, 1664), (512, 1088), (512, 320)])
+@pytest.mark.parametrize("T,skew", [(17, 0.0), (40, 4.0), (333, 2.0)])
+def test_experts_in_slices_of_unequal_length(r, h, T, skew):
+    """Hidden widths of 3 to 25 chunks in one to eight slices, which then differ by a chunk."""
+    test_experts_in_one_kernel(r, h, T, skew)
