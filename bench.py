@@ -52,6 +52,7 @@ GEMM_FLOPS = {   # per launch, algorithmic (unpadded rows)
     "gemm_dw1": lambda w: 2.0 * w.N * w.r * w.h, "gemm_dx": lambda w: 2.0 * w.T * w.d * w.r,
     "gemm_dx_gate": lambda w: 2.0 * w.T * w.d * w.E, "gemm_dw_down": lambda w: 2.0 * w.T * w.d * w.r,
     "gemm_dw_gate": lambda w: 2.0 * w.T * w.d * w.E,
+    "fused_expert_mlp": lambda w: 4.0 * w.N * w.r * w.h, "fused_expert_mlp_bwd": lambda w: 4.0 * w.N * w.r * w.h,
 }
 ROW_MOVE_BYTES = {   # per launch, algorithmic: rows read + rows written (+ the 4-byte tables)
     "dispatch": lambda w, b: (w.T * w.r + w.N * w.r) * b + 4.0 * w.N,
@@ -83,6 +84,9 @@ GEMM_BYTES = {
     "gemm_dx_gate": lambda w, b: (w.T * _e64(w) + w.E * w.d) * b,
     "gemm_dw_down": lambda w, b: (w.T * w.r + w.T * w.d + w.r * w.d) * b,
     "gemm_dw_gate": lambda w, b: (w.T * _e64(w) + w.E * w.d) * b,
+    # both contractions of an expert in one launch; a training step also writes (reads) a or dz and sigma' (BF16 path only)
+    "fused_expert_mlp": lambda w, b: (2.0 * w.N * w.r + 2.0 * w.E * w.h * w.r + w.N * w.h) * b + w.N * w.h,
+    "fused_expert_mlp_bwd": lambda w, b: (2.0 * w.N * w.r + 2.0 * w.E * w.h * w.r + w.N * w.h) * b + w.N * w.h,
 }
 
 # DRAM bytes per launch of the two output-heavy contractions as ncu counted them (dram__bytes_read.sum +
@@ -1027,7 +1031,8 @@ def run_ours(args, w):
             entry["frac_of_measured_hbm"] = round(entry["gbs"] / peaks["hbm_gbs"], 3)
         stages[name] = entry
     # the two groups the target names: the per-expert (grouped) contractions together, the row-move kernels together
-    grouped = [n for n in ("gemm_expert1", "gemm_expert2", "gemm_dz", "gemm_dw2", "gemm_dxg", "gemm_dw1") if n in stages]
+    grouped = [n for n in ("gemm_expert1", "gemm_expert2", "gemm_dz", "gemm_dw2", "gemm_dxg", "gemm_dw1", "fused_expert_mlp",
+                            "fused_expert_mlp_bwd") if n in stages]
     g_ms = sum(stages[n]["ms"] for n in grouped)
     g_tf = sum(flops_of[n] for n in grouped) / (g_ms * 1e-3) / 1e12 if g_ms > 0 else 0.0
     moves = [n for n in ROW_MOVE_BYTES if n in stages]

@@ -159,6 +159,14 @@ bool fused_mlp_supported(int r, int h, int dtype);
 MlpSlicing fused_mlp_slicing(int r, int h, int64_t N, int64_t P);
 cudaError_t launch_fused_mlp(const void* xg, const void* w1, const void* w2, void* out, int64_t max_rows, int64_t slots,
                              const MlpSlicing& sl, int r, int h, int E, int act, const Tables& tb, int* status, cudaStream_t stream);
+// Both contractions of the experts in one kernel on CTA pairs (gemm_tc_ffn.cu), r 128 or 256, over grouped padded rows.
+// Forward: u = sigma(xg W1_e^T) W2_e^T; with `sigma` (training) also a = sigma(.) and the bytes of sigma'(.), in an order of
+// their own.  Backward: dz = (du W2_e) sigma', dxg = dz W1_e.
+bool ffn_pair_supported(int r, int h, int E, int dtype);
+cudaError_t launch_ffn_forward(const void* xg, const void* w1, const void* w2, void* a, void* sigma, void* u, int64_t max_rows, int r, int h,
+                               int E, int act, const int32_t* poffsets, int* status, cudaStream_t stream);
+cudaError_t launch_ffn_backward(const void* du, const void* w1, const void* w2, void* dz, const void* sigma, void* dxg, int64_t max_rows, int r,
+                                int h, int E, const int32_t* poffsets, int* status, cudaStream_t stream);
 // CTA-pair variant (tcgen05 cta_group::2) for outputs at least 256 wide.
 bool gemm_tc_pair_supported(const GemmArgs& g);
 bool gemm_tc_pair_preferred(const GemmArgs& g);

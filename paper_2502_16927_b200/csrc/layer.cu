@@ -436,6 +436,41 @@ bool uses_fused_mlp(const bigmac_layer* L, const Dims& m) {
     return m.r <= 256 || m.N <= 48 * (int64_t)m.E;
 }
 
+// Pairs of 128-row tiles per SM pair if the experts are chosen evenly: an expert then has about N / E rows, give or take
+// sqrt(N / E); the probability that it reaches its j-th pair is taken as a ramp of two deviations to either side.
+double ffn_rounds(const Dims& m) {
+    const double rows = std::fmin((double)m.N / m.E, (double)m.cap), dev = std::sqrt((double)m.N / m.E) + 1e-3, pair = 2.0 * kPad;
+    const int64_t whole = (int64_t)std::fmax(0.0, std::ceil((rows - 2 * dev) / pair));      // reached by all
+    double pairs = (double)whole;
+    for (int64_t j = whole; pair * j < rows + 2 * dev; ++j) pairs += std::fmin(1.0, 0.5 + (rows - pair * j) / (4 * dev));
+    return pairs * m.E / (gemm_tc_sm_count() / 2);
+}
+
+// Do both contractions of the experts run in one kernel on CTA pairs?  A function of the handle, T and the debug switches: a
+// training forward and its backward must see the same (sigma' lies in memory as that kernel wants it).
+// Measured against the separate contractions, us (a training step; even loads; d 2048 r 256 h 1024 64 experts top-8, and d 1024 r 128
+// h 512 32 experts top-4): it wins unless its last round of pairs is nearly empty.
+//   r 256: 1200 tokens 206 -> 188, 1800 211 -> 194, 4000 288 -> 266, 12000 649 -> 640, Zipf 3000 286 -> 275, 16384 907 -> 874 (the SM
+//          clock rises from 1.53 to 1.63 GHz under the power cap); 2100 (1.4 rounds, 71 % of two) 232 -> 232
+//   r 128: 300 103 -> 100, 3000 127 -> 121, 8000 178 -> 174, 20000 348 -> 339; but 4096 (1.1 rounds) 136 -> 146, 6000 (70 %) 159 -> 160,
+//          9000 (72 %) 193 -> 197, 11000 (87 %) 215 -> 216
+// Inference, against the kernel whose tokens are the N of its MMAs (gemm_tc_mlp.cu), which takes a batch's few rows an expert better:
+//   r 256: 800 tokens (100 rows) 61 -> 63, 1200 (150) 64.8 -> 64.2, 3001 83 -> 77, 8000 145 -> 127;  r 128: 2000 (250) 37.1 -> 37.4, 2500
+//   (312) 40.1 -> 40.1, 3500 41.2 -> 40.4, 4096 (1.1 rounds) 41.7 -> 46.2, 5000 (64 %) 54.2 -> 51.2, 12000 77 -> 70.
+// That kernel keeps u in fp32 where it cuts the hidden width (mlp_slices: up to half as many tiles as SMs, with more than ten chunks
+// up to an eighth of the SMs for each chunk), which is more precise than u in bf16 here: such batches stay with it.
+bool uses_ffn(const bigmac_layer* L, const Dims& m, bool training) {
+    const int mode = switches().ffn;
+    if (mode == 0 || m.bias || !sigma_as_bytes(L) || !ffn_pair_supported(m.r, m.h, m.E, m.dtype)) return false;
+    if (mode == 2) return true;
+    const double rounds = ffn_rounds(m), full = rounds / std::ceil(rounds);
+    if (training) return rounds <= 1 || full >= (m.r == 256 ? 0.65 : 0.86);
+    const double rows = std::fmin((double)m.N, (double)m.cap * m.E);
+    const int chunks = m.h / 128, units = gemm_tc_sm_count();
+    const double cut_up_to = 128.0 * units * (chunks <= 10 ? 0.5 : chunks / 8.0);            // rows
+    return switches().fused_mlp == 1 && rows > cut_up_to && rows >= (m.r == 256 ? 150.0 : 320.0) * m.E && (rounds <= 1 || full >= 0.6);
+}
+
 // Is the dispatch fused into its consumers' operand loads (F5 of the forward disappears as a launch, the grouped
 // copy xg of x' is never written)?  Inference: expert GEMM1 gathers the rows of x' itself.  Training: so does the
 // weight gradient dW1, when it runs on the balanced kernel (the statically scheduled kernels read a grouped copy).
@@ -669,11 +704,15 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
     }
     BIGMAC_TRY(route_from_logits(L, m, W, b, src, mv, aux_word_to_zero(m, routing_out), routing_out, st));
     // Inference: F6 + F7 in one kernel, the hidden activations stay on the SM (uses_fused_mlp has the rule).
-    const bool mlp_fused = !training && uses_fused_mlp(L, m);
+    const bool in_pairs = !gather_dispatch && uses_ffn(L, m, training);
+    const bool mlp_fused = !training && !in_pairs && uses_fused_mlp(L, m);
     const MlpSlicing slicing = fused_mlp_slicing(m.r, m.h, m.N, m.P);
     if (mlp_fused) {
         Stage s(L, S_FUSED_MLP, st);
         BIGMAC_CUDA(launch_fused_mlp(b.xg, W->w1, W->w2, b.a, m.P, m.N, slicing, m.r, m.h, m.E, c.act, b.tb, L->status, st));
+    } else if (in_pairs) {
+        Stage s(L, S_FUSED_MLP, st);
+        BIGMAC_CUDA(launch_ffn_forward(b.xg, W->w1, W->w2, b.a, training ? b.z : nullptr, b.u, m.P, m.r, m.h, m.E, c.act, b.tb.poffsets, L->status, st));
     } else {
         {                                                                             // F6 a = sigma(xg W1_e^T); saves sigma'(z)
             GemmArgs g;
@@ -819,7 +858,11 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         g.group = GROUP_K; g.num_experts = m.E; g.poffsets = b.tb.poffsets; g.accumulate = acc;
         BIGMAC_TRY(batch ? together.add(G_DW2, g, st) : expert_weight_grad(L, G_DW2, g, b.expert_ws, st));
     }
-    {   // dz = (du W2_e) * sigma'(z); the forward saved sigma'(z) in the z buffer, dz is written over it
+    const bool in_pairs = b.dz && !dispatch_is_fused(L, m, true) && uses_ffn(L, m, true);
+    if (in_pairs) {   // dz = (du W2_e) * sigma'(z) and dxg = dz W1_e
+        Stage s(L, S_FUSED_MLP_BWD, st);
+        BIGMAC_CUDA(launch_ffn_backward(b.du, W->w1, W->w2, b.dz, b.z, b.dxg, m.P, m.r, m.h, m.E, b.tb.poffsets, L->status, st));
+    } else {   // dz = (du W2_e) * sigma'(z); the forward saved sigma'(z) in the z buffer, dz is written over it
         GemmArgs g;
         g.A = b.du; g.lda = m.r; g.B = W->w2; g.ldb = m.h; g.b_kmajor = false; g.b_stride = (int64_t)m.r * m.h;
         g.C = b.dz ? b.dz : b.z; g.Z = b.z; g.ldc = m.h; g.M = (int)m.P; g.N = m.h; g.K = m.r;
@@ -841,7 +884,7 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         if (G->db1) BIGMAC_CUDA(launch_grouped_colsum(dz, b.tb.poffsets, G->db1, b.bias_ws, m.E, m.h, m.dtype, acc, sb));
         if (G->db2) BIGMAC_CUDA(launch_grouped_colsum(b.du, b.tb.poffsets, G->db2, b.bias_ws, m.E, m.r, m.dtype, acc, sb));
     }
-    {   // dxg = dz W1_e
+    if (!in_pairs) {   // dxg = dz W1_e
         GemmArgs g;
         g.A = dz; g.lda = m.h; g.B = W->w1; g.ldb = m.r; g.b_kmajor = false; g.b_stride = (int64_t)m.h * m.r;
         g.C = b.dxg; g.ldc = m.r; g.M = (int)m.P; g.N = m.r; g.K = m.h;
@@ -1197,6 +1240,7 @@ int bigmac_debug_set(const char* name, int value) {
     Switches& sw = switches();
     if (!std::strcmp(name, "overlap")) sw.overlap = value;
     else if (!std::strcmp(name, "tc_pair")) sw.tc_pair = value;
+    else if (!std::strcmp(name, "ffn")) sw.ffn = value;
     else if (!std::strcmp(name, "groupk")) sw.groupk = value;
     else if (!std::strcmp(name, "fused_mlp")) sw.fused_mlp = value;
     else if (!std::strcmp(name, "epi_parts")) sw.epi_parts = value;

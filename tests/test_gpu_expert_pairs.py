@@ -1,0 +1,48 @@
+"""Both contractions of an expert in one kernel on CTA pairs: one chunk of the hidden width or an odd number of them, experts
+without rows, with one row, with a half-used pair of row tiles, more items than SM pairs, the tables of many experts; forward,
+backward and inference.  The sums are the separate contractions' in the same order, so every result has their bits."""
+import numpy as np
+import pytest
+
+from paper_2502_16927_b200 import workloads as wl
+from helpers import empty_grads, make_layer, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("r,h,E,k,T,skew,act", [
+    (256, 128, 5, 2, 300, 3.0, wl.ACT_GELU_ERF),        # one chunk; loads from a few rows to several pairs
+    (128, 384, 4, 4, 129, 0.0, wl.ACT_GELU_ERF),        # three chunks; every expert has 129 rows
+    (256, 640, 96, 2, 40, 0.0, wl.ACT_GELU_ERF),        # experts without rows, with one
+    (128, 256, 3, 1, 20000, 1.0, wl.ACT_GELU_ERF),      # more items than SM pairs
+    (256, 256, 300, 4, 3000, 2.0, wl.ACT_RELU),         # the tables take the place of a ring stage
+    (256, 256, 200, 2, 777, 1.0, wl.ACT_GELU_TANH),
+    (128, 1024, 1, 1, 257, 0.0, wl.ACT_IDENTITY),
+])
+def test_equals_the_separate_contractions(r, h, E, k, T, skew, act):
+    import torch
+    from paper_2502_16927_b200 import binding
+
+    w = wl.Workload("pairs", T=T, d=128, r=r, h=h, E=E, k=k, dtype=wl.DTYPE_BF16, act=act, seed=900 + T)
+    inp = wl.make_inputs(w)
+    inp["b_gate"] = (skew * np.linspace(1.0, -1.0, w.E) ** 3).astype(np.float32)
+    dev = to_device(w, inp)
+    out = {}
+    for mode in (0, 2):
+        layer = make_layer(w)
+        try:
+            binding.bigmac_debug_set("ffn", mode)
+            binding.bigmac_debug_set("fused_mlp", 0)
+            infer = layer.forward(dev["x"], dev)
+            y = layer.forward(dev["x"], dev, training=True)
+            grads = empty_grads(w, dev)
+            dx = layer.backward(dev["x"], dev["dy"], dev, grads)
+            torch.cuda.synchronize()
+        finally:
+            binding.bigmac_debug_set("defaults")
+        assert layer.status() == 0
+        out[mode] = dict(grads, infer=infer, y=y, dx=dx)
+        layer.close()
+    for name, ref in out[0].items():
+        assert torch.equal(ref, out[2][name]), name
+        assert torch.isfinite(ref.float()).all(), name
