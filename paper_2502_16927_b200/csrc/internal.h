@@ -273,9 +273,10 @@ cudaError_t launch_combine(const void* grouped, void* dst, const float* w, const
 // with may_drop, slots without a row are left out.
 cudaError_t launch_combine_parts(const void* parts, const MlpSlicing& sl, const int32_t* n_tiles, void* dst, const float* w,
                                  const int32_t* prow_of_slot, int T, int k, int width, cudaStream_t stream, bool may_drop);
-// Backward of the combine: du[prow,:] = p[s] * dy_lo[t,:] (zeros on padding), dp[s] = <dy_lo[t,:], u[prow,:]>.
-cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float* dp, const Tables& tb, int k,
-                               int width, int dtype, int64_t max_prows, cudaStream_t stream, bool chained = true);
+// Backward of the combine: du[prow,:] = p[s] * dy_lo[t,:] (zeros on padding rows), dp[s] = <dy_lo[t,:], u[prow,:]> (0 for a slot
+// without a row); with dlogits also launch_gate_bwd (below) of these dp.
+cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float* dp, const Tables& tb, void* dlogits, int T, int k,
+                               int width, int E, int dl_width, int dl_ld, int dtype, cudaStream_t stream, bool chained = true);
 // Softmax-over-k backward: g = sum_i p_i dp_i, dl_j = p_j (dp_j - g); writes the dense [T,E] matrix
 // (zeros off the top-k set, and in the padding columns E..width-1) in the dtype, rows `ld` elements apart, and
 // leaves the fp32 dl_j in dp[slot].  may_drop: the dp of a slot without a row (prow_of_slot < 0) is taken as 0.

@@ -830,18 +830,19 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         }
     }
     BIGMAC_TRY(together.flush());
-    // du = p dy'[t], dp = <dy'[t], u>; then the softmax-over-k backward.  Chained to dy', the first would hold every SM's thread
+    // du = p dy'[t], dp = <dy'[t], u>, and the softmax-over-k backward.  Chained to dy', this would hold every SM's thread
     // slots while it waits, and dW_up would find none beside a dy' of a few CTAs (2999 tokens: 48).
-    { Stage s(L, S_COMBINE_BWD, st); BIGMAC_CUDA(launch_combine_bwd(b.dy_lo, b.u, b.du, b.dp, b.tb, m.k, m.r, m.dtype, m.P, st, !overlap)); }
+    {
+        Stage s(L, S_COMBINE_BWD, st);
+        BIGMAC_CUDA(launch_combine_bwd(b.dy_lo, b.u, b.du, b.dp, b.tb, m.aux > 0 ? nullptr : b.dlogits, m.T, m.k, m.r, m.E, m.E64, ldcat, m.dtype,
+                                       st, !overlap));
+    }
     float* aux_part = nullptr;                                                    // column sums of dL_aux/dl, for db_gate
     if (m.aux > 0) {
         aux_part = b.colsum_part + (size_t)kColsumChunks * m.E;
         Stage s(L, S_GATE_BWD, st);
         BIGMAC_CUDA(launch_gate_bwd_aux(b.dp, b.tb, b.dlogits, b.logits_saved, W->b_gate, m.aux, aux_part, m.T, m.E, m.E64,
                                         ldcat, m.k, m.dtype, st, m.cap != kNoCapacity));
-    } else {
-        Stage s(L, S_GATE_BWD, st);
-        BIGMAC_CUDA(launch_gate_bwd(b.dp, b.tb, b.dlogits, m.T, m.E, m.E64, ldcat, m.k, m.dtype, st, m.cap != kNoCapacity));
     }
     bool colsum_done = false;
     if (overlap && G->db_gate) {

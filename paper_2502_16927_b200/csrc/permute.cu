@@ -186,42 +186,104 @@ __global__ void __launch_bounds__(128) combine_parts_kernel(const float4* __rest
     dst[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
 }
 
+// Sums each of eight values over the warp's lanes: lane 4 j .. 4 j + 3 get the total of v[j] (v is used up).  Fixed order.
+__device__ __forceinline__ float warp_sum8(float* v) {
+    const int lane = threadIdx.x & 31;
+    int off = 16;
+#pragma unroll
+    for (int n = 4; n > 0; n >>= 1, off >>= 1) {
+        const bool upper = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float send = upper ? v[i] : v[i + n], keep = upper ? v[i + n] : v[i];
+            v[i] = keep + __shfl_xor_sync(kFull, send, off);
+        }
+    }
+    v[0] += __shfl_xor_sync(kFull, v[0], 2);
+    return v[0] + __shfl_xor_sync(kFull, v[0], 1);
+}
+
+// Backward of the combine, and (dlogits non-null) of the softmax over the k gate values: a warp per token reads dy' once, the
+// rows of u of eight slots together, writes their rows of du and knows all of the token's dp, from which the gate's gradient
+// follows without another launch.  The blocks behind the tokens' write zeros to the experts' padding rows, a block an expert.
+// A slot without a row (dropped under a capacity limit) counts with dp = 0.
+// Bound by HBM (u read, du written).  A warp per grouped row before, with a chain of three dependent loads for one row, and a
+// launch of its own for the gate: a training step of fp32, 256 tokens, 61.0 -> 59.8 us; d 1024, 4096 tokens 137.4 -> 136.3; d 2048,
+// 2999 tokens 280 -> 277.
 template <typename T>
 __global__ void __launch_bounds__(256) combine_bwd_kernel(const uint4* __restrict__ dy_lo, const uint4* __restrict__ u,
                                                           uint4* __restrict__ du, float* __restrict__ dp,
-                                                          const int32_t* __restrict__ slot_of_prow,
-                                                          const float* __restrict__ topk_w,
-                                                          const int32_t* __restrict__ n_tiles, int k, int vecs_per_row,
-                                                          int64_t max_prows) {
+                                                          const int32_t* __restrict__ prow_of_slot, const float* __restrict__ topk_w,
+                                                          const int32_t* __restrict__ topk_idx, const int32_t* __restrict__ counts,
+                                                          const int32_t* __restrict__ poffsets, T* __restrict__ dlogits, int n_tokens,
+                                                          int k, int vecs_per_row, int E, int width, int ld) {
     grid_dependency_wait();
     grid_dependency_launch();
-    constexpr int V = Vec<T>::kElems;
-    const int64_t prow = warp_global_id();
-    int64_t live = (int64_t)(*n_tiles) * kPad;
-    if (live > max_prows) live = max_prows;
-    if (prow >= live) return;
-    const int lane = threadIdx.x & 31;
-    const int s = slot_of_prow[prow];
-    uint4* out = du + prow * vecs_per_row;
-    if (s < 0) {
-        for (int c = lane; c < vecs_per_row; c += 32) out[c] = make_uint4(0, 0, 0, 0);
+    constexpr int V = Vec<T>::kElems, B = 8;
+    const int lane = threadIdx.x & 31, token_blocks = (n_tokens + 7) / 8;
+    if ((int)blockIdx.x >= token_blocks) {
+        const int e = blockIdx.x - token_blocks;
+        const int64_t first = ((int64_t)poffsets[e] + counts[e]) * vecs_per_row, last = (int64_t)poffsets[e + 1] * vecs_per_row;
+        for (int64_t i = first + threadIdx.x; i < last; i += 256) du[i] = make_uint4(0, 0, 0, 0);
         return;
     }
-    const float p = topk_w[s];
-    const uint4* g = dy_lo + (int64_t)(s / k) * vecs_per_row;
-    const uint4* ur = u + prow * vecs_per_row;
-    float dot = 0.0f;
-    for (int c = lane; c < vecs_per_row; c += 32) {
-        float a[V], b[V], o[V];
-        Vec<T>::unpack(g[c], a);
-        Vec<T>::unpack(ur[c], b);
+    const int t = warp_global_id();
+    if (t >= n_tokens) return;
+    const int64_t s0 = (int64_t)t * k;
+    float mine = 0.0f;                                       // k <= 8: lane j has the j-th slot's dp
+    for (int j0 = 0; j0 < k; j0 += B) {
+        int place = -1;
+        float weight = 0.0f;
+        if (lane < B && j0 + lane < k) {
+            place = prow_of_slot[s0 + j0 + lane];
+            weight = topk_w[s0 + j0 + lane];
+        }
+        float dot[B];
 #pragma unroll
-        for (int i = 0; i < V; ++i) { dot = fmaf(a[i], b[i], dot); o[i] = p * a[i]; }
-        out[c] = Vec<T>::pack(o);
+        for (int j = 0; j < B; ++j) dot[j] = 0.0f;
+        for (int c0 = 0; c0 < vecs_per_row; c0 += 32) {
+            const int c = c0 + lane;
+            const bool there = c < vecs_per_row;
+            const uint4 none = make_uint4(0, 0, 0, 0);
+            const uint4 g = there ? dy_lo[(int64_t)t * vecs_per_row + c] : none;
+            uint4 v[B];
+#pragma unroll
+            for (int j = 0; j < B; ++j) {
+                const int prow = __shfl_sync(kFull, place, j);
+                v[j] = there && prow >= 0 ? u[(int64_t)prow * vecs_per_row + c] : none;
+            }
+            float a[V];
+            Vec<T>::unpack(g, a);
+#pragma unroll
+            for (int j = 0; j < B; ++j) {
+                const int prow = __shfl_sync(kFull, place, j);
+                if (prow < 0) continue;                      // uniform
+                const float p = __shfl_sync(kFull, weight, j);
+                float b[V], o[V];
+                Vec<T>::unpack(v[j], b);
+#pragma unroll
+                for (int i = 0; i < V; ++i) { dot[j] = fmaf(a[i], b[i], dot[j]); o[i] = p * a[i]; }
+                if (there) du[(int64_t)prow * vecs_per_row + c] = Vec<T>::pack(o);
+            }
+        }
+        const float total = warp_sum8(dot);
+        mine = __shfl_sync(kFull, total, 4 * (lane & 7));
+        if (lane < B && j0 + lane < k) dp[s0 + j0 + lane] = mine;
     }
+    if (!dlogits) return;
+    T* row = dlogits + (int64_t)t * ld;
+    for (int e = lane; e < width; e += 32) row[e] = (T)0.0f;
+    __syncwarp();                                            // the zeros, and other lanes' dp, are there
+    float part = 0.0f;
+    for (int j = lane; j < k; j += 32) part = fmaf(topk_w[s0 + j], k <= B ? mine : dp[s0 + j], part);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(kFull, dot, off);
-    if (lane == 0) dp[s] = dot;
+    for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(kFull, part, off);
+    for (int j = lane; j < k; j += 32) {
+        const float dl = topk_w[s0 + j] * ((k <= B ? mine : dp[s0 + j]) - part);
+        const int e = topk_idx[s0 + j];
+        if ((unsigned)e < (unsigned)E) row[e] = (T)dl;
+        dp[s0 + j] = dl;                                     // fp32 copy per slot, for the bias gradient
+    }
 }
 
 template <typename T>
@@ -466,19 +528,18 @@ cudaError_t launch_combine_parts(const void* parts, const MlpSlicing& sl, const 
     return launch_chained(combine_parts_kernel<false>, blocks, 128, 0, stream, (const float4*)parts, n_tiles, sl, stride, (uint2*)dst, w, prow_of_slot, T, k, quads);
 }
 
-cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float* dp, const Tables& tb, int k,
-                               int width, int dtype, int64_t max_prows, cudaStream_t stream, bool chained) {
-    if (max_prows == 0) return cudaSuccess;
+cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float* dp, const Tables& tb, void* dlogits, int T, int k,
+                               int width, int E, int dl_width, int dl_ld, int dtype, cudaStream_t stream, bool chained) {
+    if (T == 0) return cudaSuccess;
     const int vecs = width * elem_bytes(dtype) / 16;
+    const unsigned blocks = warp_blocks(T) + E;
     if (dtype == BIGMAC_BF16)
-        (void)launch_maybe_chained(chained, combine_bwd_kernel<__nv_bfloat16>, warp_blocks(max_prows), 256, 0, stream, 
-            (const uint4*)dy_lo, (const uint4*)u, (uint4*)du, dp, tb.slot_of_prow, tb.topk_w, tb.n_tiles, k, vecs,
-            max_prows);
-    else
-        (void)launch_maybe_chained(chained, combine_bwd_kernel<float>, warp_blocks(max_prows), 256, 0, stream, 
-            (const uint4*)dy_lo, (const uint4*)u, (uint4*)du, dp, tb.slot_of_prow, tb.topk_w, tb.n_tiles, k, vecs,
-            max_prows);
-    return cudaGetLastError();
+        return launch_maybe_chained(chained, combine_bwd_kernel<__nv_bfloat16>, blocks, 256, 0, stream, (const uint4*)dy_lo, (const uint4*)u,
+                                    (uint4*)du, dp, tb.prow_of_slot, tb.topk_w, tb.topk_idx, tb.counts, tb.poffsets, (__nv_bfloat16*)dlogits,
+                                    T, k, vecs, E, dl_width, dl_ld);
+    return launch_maybe_chained(chained, combine_bwd_kernel<float>, blocks, 256, 0, stream, (const uint4*)dy_lo, (const uint4*)u, (uint4*)du,
+                                dp, tb.prow_of_slot, tb.topk_w, tb.topk_idx, tb.counts, tb.poffsets, (float*)dlogits, T, k, vecs, E, dl_width,
+                                dl_ld);
 }
 
 cudaError_t launch_gate_bwd(float* dp, const Tables& tb, void* dlogits, int T, int E, int width, int ld, int k,
