@@ -13,7 +13,8 @@
 //           A operand of the next contraction and the box of a TMA store
 //   B(c)    acc2 (128 rows x r) += mid[c % 2] B2[chunk]                                      K = 128, M = 256, N = r
 // The issuer runs A two chunks ahead of B, across the ends of items too (a group's next accumulator is then ready when it has
-// written its chunk); acc2 is read out beside the first chunks of the next item.  Every SM stages half of each B
+// written its chunk), but issues the first two As of an item behind the B of their turn, so that the rows X of the item, whose place
+// the last A of the item before frees, have two chunks' time to arrive; acc2 is read out beside the first chunks of the next item.  Every SM stages half of each B
 // (cta_group::2).  An extra thread moves the middle to memory (TMA stores of 128-row boxes).  sigma' goes from registers to
 // memory and back in an order of its own, which only this kernel knows: the bytes of (row tile, chunk, warp) in the order of
 // the warp's 16-byte accesses.
@@ -198,8 +199,10 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             next_a();
             next_a();
             for (; wb.i < total; wb.next(p, s_pp, chunks, stride, total)) {
-                next_a();
+                const bool a_first = wa.c > 1;
+                if (a_first) next_a();
                 b2(wb.t, wb.c);
+                if (!a_first) next_a();
             }
         }
     } else if (warp == 1) {
@@ -240,7 +243,8 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             contract_a();
             contract_a();
             for (int gb = 0, cb = 0, nb = 0; gb < all; ++gb) {
-                contract_a();                            // its accumulator is free before the middle that B waits for is written
+                const bool a_first = ca > 1;
+                if (a_first) contract_a();               // its accumulator is free before the middle that B waits for is written
                 const uint32_t a = gb & 1;
                 mbar_wait_cluster(&mid_full[a], (gb >> 1) & 1, dead, p.status);
                 if (cb == 0) mbar_wait_lean(acc2_empty, (nb & 1) ^ 1, dead, p.status);
@@ -258,6 +262,7 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                 }
                 umma_commit_pair(&mid_empty[a]);
                 if (++cb == chunks) { umma_commit_pair(acc2_full); cb = 0; ++nb; }
+                if (!a_first) contract_a();
             }
         }
     } else if (warp == 2 + kEpiWarps) {
