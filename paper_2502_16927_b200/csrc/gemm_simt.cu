@@ -3,7 +3,7 @@
 // tolerance of that path need one) and a debugging reference for the bf16 path.
 //
 // The fp32 layer is used at small sizes, where every contraction is one short chain of latencies: one kernel runs up to
-// three independent contractions (a launch costs more than most of them), a block stages a long k slice of its tile at
+// five independent contractions (a launch costs more than most of them), a block stages a long k slice of its tile at
 // once, its eight warps share the slice (each sums its own part of the k range into a 32 x 32 tile, 4 x 8 outputs per
 // lane), and where the contraction is long a cluster of blocks shares it, the partial tiles meeting in distributed shared
 // memory.  All sums have a fixed order.  Tiles: 32 x 32 with 128-deep slices (eight warps along k) while that many tiles do

@@ -107,7 +107,7 @@ struct GemmArgs {
 // fp32-FMA GEMM for either dtype (dtype: bigmac_dtype_t of A, B, Z and - unless out_f32 - C).
 cudaError_t gemm_simt(const GemmArgs& g, int dtype, cudaStream_t stream);
 // Up to kSimtBatch independent contractions in one launch (none may read what another writes).
-constexpr int kSimtBatch = 3;
+constexpr int kSimtBatch = 5;
 cudaError_t gemm_simt_batch(const GemmArgs* g, int count, int dtype, cudaStream_t stream);
 // tcgen05 / TMEM / TMA GEMM, bf16 inputs, fp32 accumulation.  `status` is the device status word.
 cudaError_t gemm_tc(const GemmArgs& g, int* status, cudaStream_t stream);
@@ -167,6 +167,13 @@ cudaError_t launch_ffn_forward(const void* xg, const void* w1, const void* w2, v
                                int E, int act, const int32_t* poffsets, int* status, cudaStream_t stream);
 cudaError_t launch_ffn_backward(const void* du, const void* w1, const void* w2, void* dz, const void* sigma, void* dxg, int64_t max_rows, int r,
                                 int h, int E, const int32_t* poffsets, int* status, cudaStream_t stream);
+// The same on the fp32 path for narrow experts (ffn_simt.cu); sigma' in the dtype and row-major like a, dz written over it.
+struct Tables;
+bool ffn_simt_supported(int r, int h, int dtype);
+cudaError_t launch_ffn_simt_forward(const void* xg, const void* w1, const void* w2, void* a, void* sigma, void* u, int64_t max_rows, int r, int h,
+                                    int act, const Tables& tb, cudaStream_t stream);
+cudaError_t launch_ffn_simt_backward(const void* du, const void* w1, const void* w2, void* sigma, void* dxg, int64_t max_rows, int r, int h,
+                                     const Tables& tb, cudaStream_t stream);
 // CTA-pair variant (tcgen05 cta_group::2) for outputs at least 256 wide.
 bool gemm_tc_pair_supported(const GemmArgs& g);
 bool gemm_tc_pair_preferred(const GemmArgs& g);

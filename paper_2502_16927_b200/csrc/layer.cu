@@ -471,6 +471,12 @@ bool uses_ffn(const bigmac_layer* L, const Dims& m, bool training) {
     return switches().fused_mlp == 1 && rows > cut_up_to && rows >= (m.r == 256 ? 150.0 : 320.0) * m.E && (rounds <= 1 || full >= 0.6);
 }
 
+// ... or, on the fp32 path, in one launch of FMA blocks?  Everywhere within its widths: a training step / an inference forward, us, with two
+// launches for either direction and dW2, dW1 apart from the last contractions, and so: d 128, r 32, h 128, 8 experts top-2, 32 tokens
+// 52 -> 47 / 23 -> 21, 256 58 -> 52 / 24 -> 22, 2048 105 -> 83 / 39 -> 32; h 256, 32 experts top-4, 100 tokens 126 -> 77 / 45 -> 31; h 64, 4
+// experts top-1, 1024 tokens 72 -> 62 / 26.5 -> 25.4.  With r 64 it is not always the faster one (h 256, 16 experts, 256 tokens 96 -> 99).
+bool uses_ffn_simt(const Dims& m) { return switches().ffn != 0 && !m.bias && ffn_simt_supported(m.r, m.h, m.dtype); }
+
 // Is the dispatch fused into its consumers' operand loads (F5 of the forward disappears as a launch, the grouped
 // copy xg of x' is never written)?  Inference: expert GEMM1 gathers the rows of x' itself.  Training: so does the
 // weight gradient dW1, when it runs on the balanced kernel (the statically scheduled kernels read a grouped copy).
@@ -710,6 +716,9 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
     if (mlp_fused) {
         Stage s(L, S_FUSED_MLP, st);
         BIGMAC_CUDA(launch_fused_mlp(b.xg, W->w1, W->w2, b.a, m.P, m.N, slicing, m.r, m.h, m.E, c.act, b.tb, L->status, st));
+    } else if (uses_ffn_simt(m)) {
+        Stage s(L, S_FUSED_MLP, st);
+        BIGMAC_CUDA(launch_ffn_simt_forward(b.xg, W->w1, W->w2, b.a, training ? b.z : nullptr, b.u, m.P, m.r, m.h, c.act, b.tb, st));
     } else if (in_pairs) {
         Stage s(L, S_FUSED_MLP, st);
         BIGMAC_CUDA(launch_ffn_forward(b.xg, W->w1, W->w2, b.a, training ? b.z : nullptr, b.u, m.P, m.r, m.h, m.E, c.act, b.tb.poffsets, L->status, st));
@@ -859,8 +868,12 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         g.group = GROUP_K; g.num_experts = m.E; g.poffsets = b.tb.poffsets; g.accumulate = acc;
         BIGMAC_TRY(batch ? together.add(G_DW2, g, st) : expert_weight_grad(L, G_DW2, g, b.expert_ws, st));
     }
+    const bool narrow = uses_ffn_simt(m);        // (dz over sigma', which nothing else reads)
     const bool in_pairs = b.dz && !dispatch_is_fused(L, m, true) && uses_ffn(L, m, true);
-    if (in_pairs) {   // dz = (du W2_e) * sigma'(z) and dxg = dz W1_e
+    if (narrow) {
+        Stage s(L, S_FUSED_MLP_BWD, st);
+        BIGMAC_CUDA(launch_ffn_simt_backward(b.du, W->w1, W->w2, b.z, b.dxg, m.P, m.r, m.h, b.tb, st));
+    } else if (in_pairs) {   // dz = (du W2_e) * sigma'(z) and dxg = dz W1_e
         Stage s(L, S_FUSED_MLP_BWD, st);
         BIGMAC_CUDA(launch_ffn_backward(b.du, W->w1, W->w2, b.dz, b.z, b.dxg, m.P, m.r, m.h, m.E, b.tb.poffsets, L->status, st));
     } else {   // dz = (du W2_e) * sigma'(z); the forward saved sigma'(z) in the z buffer, dz is written over it
@@ -885,7 +898,7 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         if (G->db1) BIGMAC_CUDA(launch_grouped_colsum(dz, b.tb.poffsets, G->db1, b.bias_ws, m.E, m.h, m.dtype, acc, sb));
         if (G->db2) BIGMAC_CUDA(launch_grouped_colsum(b.du, b.tb.poffsets, G->db2, b.bias_ws, m.E, m.r, m.dtype, acc, sb));
     }
-    if (!in_pairs) {   // dxg = dz W1_e
+    if (!in_pairs && !narrow) {   // dxg = dz W1_e
         GemmArgs g;
         g.A = dz; g.lda = m.h; g.B = W->w1; g.ldb = m.r; g.b_kmajor = false; g.b_stride = (int64_t)m.h * m.r;
         g.C = b.dxg; g.ldc = m.r; g.M = (int)m.P; g.N = m.r; g.K = m.h;
@@ -905,7 +918,7 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
     // With the second stream dW1 runs there, beside dx and [dW_down ; dW_gate]: its work items fill what those leave of the chip.
     const bool dw1_last = fused && !m.cdac && !m.gate_low;
     if (!dw1_last) BIGMAC_TRY(dw1(st));
-    BIGMAC_TRY(together.flush());
+    if (!narrow) BIGMAC_TRY(together.flush());       // else dW2 and dW1 go out with dx, dW_down and dW_gate
     if (m.cdac) {
         // Eq. 3: dx = sum_j dxg[row of slot (t,j)] + dl W_gate; dW_gate = dl^T x
         { Stage s(L, S_DXLO_GATHER, st); BIGMAC_CUDA(launch_combine(b.dxg, dx, nullptr, b.tb.prow_of_slot, m.T, m.k, m.d, m.dtype, st, 0, m.cap != kNoCapacity)); }

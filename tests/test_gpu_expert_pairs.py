@@ -1,6 +1,7 @@
-"""Both contractions of an expert in one kernel on CTA pairs: one chunk of the hidden width or an odd number of them, experts
+"""Both contractions of an expert in one kernel.  On CTA pairs: one chunk of the hidden width or an odd number of them, experts
 without rows, with one row, with a half-used pair of row tiles, more items than SM pairs, the tables of many experts; forward,
-backward and inference.  The sums are the separate contractions' in the same order, so every result has their bits."""
+backward and inference.  The sums are the separate contractions' in the same order, so every result has their bits.
+On the fp32 path: widths that are no multiple of a tile or of a warp, two chunks, blocks of 16 and of 32 rows, of padding rows alone."""
 import numpy as np
 import pytest
 
@@ -46,3 +47,32 @@ def test_equals_the_separate_contractions(r, h, E, k, T, skew, act):
     for name, ref in out[0].items():
         assert torch.equal(ref, out[2][name]), name
         assert torch.isfinite(ref.float()).all(), name
+
+
+@pytest.mark.parametrize("d,r,h,E,k,T,capacity", [(128, 32, 128, 8, 2, 33, 0.0), (64, 4, 4, 3, 1, 7, 0.0), (64, 12, 132, 5, 2, 130, 0.0),
+                                                 (128, 32, 256, 6, 3, 200, 0.7), (64, 20, 60, 4, 2, 5000, 0.0), (64, 28, 252, 40, 2, 300, 0.0)])
+def test_fp32_in_one_launch(d, r, h, E, k, T, capacity):
+    import torch
+    from paper_2502_16927_b200 import binding
+
+    w = wl.Workload("narrow", T=T, d=d, r=r, h=h, E=E, k=k, dtype=wl.DTYPE_F32, act=wl.ACT_GELU_ERF, seed=40 + T)
+    dev = to_device(w, wl.make_inputs(w))
+    out = {}
+    for mode in (0, 1):
+        layer = make_layer(w, capacity_factor=capacity)
+        try:
+            binding.bigmac_debug_set("ffn", mode)
+            infer = layer.forward(dev["x"], dev)
+            y = layer.forward(dev["x"], dev, training=True)
+            grads = empty_grads(w, dev)
+            dx = layer.backward(dev["x"], dev["dy"], dev, grads)
+            torch.cuda.synchronize()
+        finally:
+            binding.bigmac_debug_set("defaults")
+        out[mode] = dict(grads, infer=infer, y=y, dx=dx)
+        layer.close()
+    # The same products in another order: sums of at most 256 terms, four in a row, of unit roundoff 6e-8, i.e. 16 x 6e-8 x 4 for random
+    # signs; the weight gradients then sum these errors like their terms.
+    for name, ref in out[0].items():
+        err = (ref.double() - out[1][name].double()).norm() / ref.double().norm()
+        assert err <= 4e-6, (name, float(err))
