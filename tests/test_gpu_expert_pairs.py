@@ -72,7 +72,8 @@ def test_fp32_in_one_launch(d, r, h, E, k, T, capacity):
         out[mode] = dict(grads, infer=infer, y=y, dx=dx)
         layer.close()
     # The same products in another order: sums of at most 256 terms, four in a row, of unit roundoff 6e-8, i.e. 16 x 6e-8 x 4 for random
-    # signs; the weight gradients then sum these errors like their terms.
+    # signs; the weight gradients then sum these errors like their terms.  The gate's gradients are differences of dp: ten times that
+    # (and exactly zero with one expert a token).
     for name, ref in out[0].items():
-        err = (ref.double() - out[1][name].double()).norm() / ref.double().norm()
-        assert err <= 4e-6, (name, float(err))
+        err = (ref.double() - out[1][name].double()).norm()
+        assert err <= (4e-5 if "gate" in name else 4e-6) * ref.double().norm(), (name, float(err), float(ref.double().norm()))
