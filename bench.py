@@ -58,7 +58,7 @@ ROW_MOVE_BYTES = {   # per launch, algorithmic: rows read + rows written (+ the 
     "dispatch": lambda w, b: (w.T * w.r + w.N * w.r) * b + 4.0 * w.N,
     "combine": lambda w, b: (w.N * w.r + w.T * w.r) * b + 8.0 * w.N,
     "dxlo_gather": lambda w, b: (w.N * w.r + w.T * w.r) * b + 4.0 * w.N,
-    "combine_bwd": lambda w, b: (2.0 * w.N * w.r + w.N * w.r) * b + 12.0 * w.N,
+    "combine_bwd": lambda w, b: (2.0 * w.N * w.r + w.T * w.r) * b + 12.0 * w.N,     # a token's row of dy' once, u in, du out
 }
 
 
