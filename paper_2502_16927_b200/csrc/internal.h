@@ -286,9 +286,9 @@ cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float
                                int width, int E, int dl_width, int dl_ld, int dtype, cudaStream_t stream, bool chained = true);
 // Softmax-over-k backward: g = sum_i p_i dp_i, dl_j = p_j (dp_j - g); writes the dense [T,E] matrix
 // (zeros off the top-k set, and in the padding columns E..width-1) in the dtype, rows `ld` elements apart, and
-// leaves the fp32 dl_j in dp[slot].  may_drop: the dp of a slot without a row (prow_of_slot < 0) is taken as 0.
+// leaves the fp32 dl_j in dp[slot].  (The expert-parallel form; on one GPU launch_combine_bwd does it.)
 cudaError_t launch_gate_bwd(float* dp, const Tables& tb, void* dlogits, int T, int E, int width, int ld, int k,
-                            int dtype, cudaStream_t stream, bool may_drop = false);
+                            int dtype, cudaStream_t stream);
 // Load-balancing loss (Table 5; conventional form, the paper prints none):
 //   L_aux = coef * E * sum_e f_e P_e,  f_e = counts_chosen[e] / (T k),  P_e = mean_t softmax_E(logits[t,:] + b_gate)[e].
 // Forward: loss[0] = L_aux; `partial` holds kAuxChunks * E floats of scratch.  Deterministic summation order.

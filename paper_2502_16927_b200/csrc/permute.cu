@@ -289,8 +289,7 @@ __global__ void __launch_bounds__(256) combine_bwd_kernel(const uint4* __restric
 template <typename T>
 __global__ void __launch_bounds__(256) gate_bwd_kernel(float* __restrict__ dp, const float* __restrict__ topk_w,
                                                        const int32_t* __restrict__ topk_idx, T* __restrict__ dlogits,
-                                                       int n_tokens, int E, int width, int ld, int k,
-                                                       const int32_t* __restrict__ prow_of_slot /* nullable */) {
+                                                       int n_tokens, int E, int width, int ld, int k) {
     grid_dependency_wait();
     grid_dependency_launch();
     const int t = warp_global_id();
@@ -299,10 +298,7 @@ __global__ void __launch_bounds__(256) gate_bwd_kernel(float* __restrict__ dp, c
     const float* p = topk_w + (int64_t)t * k;
     float* g = dp + (int64_t)t * k;
     float part = 0.0f;
-    for (int j = lane; j < k; j += 32) {
-        if (prow_of_slot && prow_of_slot[(int64_t)t * k + j] < 0) g[j] = 0.0f;   // dropped under a capacity limit
-        part = fmaf(p[j], g[j], part);
-    }
+    for (int j = lane; j < k; j += 32) part = fmaf(p[j], g[j], part);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(kFull, part, off);
     T* row = dlogits + (int64_t)t * ld;
@@ -543,14 +539,13 @@ cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float
 }
 
 cudaError_t launch_gate_bwd(float* dp, const Tables& tb, void* dlogits, int T, int E, int width, int ld, int k,
-                            int dtype, cudaStream_t stream, bool may_drop) {
+                            int dtype, cudaStream_t stream) {
     if (T == 0) return cudaSuccess;
-    const int32_t* prow = may_drop ? tb.prow_of_slot : nullptr;
     if (dtype == BIGMAC_BF16)
         (void)launch_chained(gate_bwd_kernel<__nv_bfloat16>, warp_blocks(T), 256, 0, stream, dp, tb.topk_w, tb.topk_idx,
-                                                                          (__nv_bfloat16*)dlogits, T, E, width, ld, k, prow);
+                                                                          (__nv_bfloat16*)dlogits, T, E, width, ld, k);
     else
-        (void)launch_chained(gate_bwd_kernel<float>, warp_blocks(T), 256, 0, stream, dp, tb.topk_w, tb.topk_idx, (float*)dlogits, T, E, width, ld, k, prow);
+        (void)launch_chained(gate_bwd_kernel<float>, warp_blocks(T), 256, 0, stream, dp, tb.topk_w, tb.topk_idx, (float*)dlogits, T, E, width, ld, k);
     return cudaGetLastError();
 }
 
