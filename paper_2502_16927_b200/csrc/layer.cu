@@ -188,9 +188,8 @@ void carve_backward_scratch(Carver& cv, const Dims& m, Buffers& b) {
 // every width: against the best of 1, 2, 3, 4, 6 and 8 parts a forward of 24 to 512 tokens is within 3 % at d 1024 to 8192 (one of 24
 // shapes 4.5 %, small layers of d 512 up to 6 %); from 700 to 1500 tokens of d 1024, and 700 to 1000 of d 2048, one part would be the
 // better choice (39.3 against 35.1 us, 57.3 against 52.1).  A function of the shape only: every call of a handle with the same T takes the same path.
-int descend_split_parts(const Dims& m) {
-    if (m.E % 4 || m.dtype != BIGMAC_BF16) return 1;
-    const int n = m.r + m.E, num_kb = m.d / 64;
+int split_parts(const Dims& m, int n) {
+    const int num_kb = m.d / 64;
     int best = 1;
     double best_cost = 0;
     for (int s = 1; s <= kMaxSplitK && s <= num_kb; ++s) {
@@ -203,6 +202,7 @@ int descend_split_parts(const Dims& m) {
     }
     return best;
 }
+int descend_split_parts(const Dims& m) { return m.E % 4 || m.dtype != BIGMAC_BF16 ? 1 : split_parts(m, m.r + m.E); }
 void carve_descend_split(Carver& cv, const Dims& m, Buffers& b) {
     const int parts = descend_split_parts(m);
     b.descend_ws = parts > 1 ? cv.take<float>((size_t)parts * m.T * (m.r + m.E)) : nullptr;
@@ -376,6 +376,18 @@ float* aux_word_to_zero(const Dims& m, const bigmac_routing_t* out) { return out
 // Steps F1-F3 without the rest of the layer.
 int run_routing(const bigmac_layer* L, const Dims& m, const void* x, const bigmac_weights_t* W, Buffers& b,
                 bigmac_routing_t* out, cudaStream_t st) {
+    // Few tokens: the logits' contraction in parts too, added by the top-k (a tile of 128 tokens walks all of d, 8 us at d 2048 and 15 at
+    // d 4096).  The parts lie where a forward has the hidden activations, where the call has that room.  With up to 512 tokens in one
+    // launch after it, us: d 2048, 64 experts, 64 tokens 18.8 -> 12.7, 512 18.3 -> 14.4, 1000 19.9 -> 16.8; d 4096, 128 experts 26.4 -> 16.5,
+    // 25.5 -> 18.7, 26.7 -> 20.2; d 1024, 32 experts 13.8 -> 9.6, 13.5 -> 10.4, 15.2 -> 14.1.
+    const int parts = b.a && route_fused_supported(m.E, m.k) && !m.gate_low && L->use_tc && L->tc_mask == ~0u ? split_parts(m, m.E) : 1;
+    if (parts > 1 && (size_t)parts * m.T * m.E * sizeof(float) <= (size_t)m.P * m.h * esize(m.dtype)) {
+        GemmArgs g;
+        g.A = x; g.lda = m.d; g.B = W->w_gate; g.ldb = m.d; g.C = b.a; g.ldc = m.E;
+        g.M = m.T; g.N = m.E; g.K = m.d; g.out_f32 = true; g.split_k = parts;
+        BIGMAC_TRY(gemm(L, G_LOGITS, g, st));
+        return route_from_logits(L, m, W, b, RouteSource{(const float*)b.a, m.E, parts, (int64_t)m.T * m.E, nullptr}, RouteMove{}, aux_word_to_zero(m, out), out, st);
+    }
     BIGMAC_TRY(run_logits(L, m, x, W, b, st));
     return route_from_logits(L, m, W, b, RouteSource{b.logits, m.E, 1, 0, nullptr}, RouteMove{}, aux_word_to_zero(m, out), out, st);
 }

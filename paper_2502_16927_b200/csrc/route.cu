@@ -822,6 +822,7 @@ struct RouteArgs {
     float* topk_w;
     int per_block;                                   // tokens of a block, at most four for each of its warps
 };
+// MOVE as above.
 template <int Q, int MOVE>
 __global__ void __cluster_dims__(kRouteCluster, 1, 1) __launch_bounds__(kPlaceThreads) route_cluster_kernel(const RouteArgs r, const PlaceArgs p) {
     constexpr int kWarps = kPlaceThreads / 32;
@@ -893,8 +894,9 @@ __global__ void __cluster_dims__(kRouteCluster, 1, 1) __launch_bounds__(kPlaceTh
     const int share = (r.per_block + clusters - 1) / clusters, from = min(first + cluster * share, first + r.per_block);
     const int to = min(min(from + share, first + r.per_block), p.T);
     place_from_counts<MOVE>(p, sh, from, to, [&](int64_t tok, int& ex_id, int& rank) {
-        ex_id = s_expert[((int)tok - first) * p.k + lane];
-        rank = s_rank[((int)tok - first) * p.k + lane];
+        const int at = MOVE == 0 ? (int)tok - first * p.k : ((int)tok - first) * p.k + lane;     // MOVE 0: tok is the slot
+        ex_id = s_expert[at];
+        rank = s_rank[at];
     });
 }
 
@@ -955,7 +957,7 @@ cudaError_t launch_tables(const Tables& tb, int T, int E, int k, int cap, cudaSt
 bool route_fused_supported(int E, int k) { return k <= 8 && E % 4 == 0 && E <= kPlaceMaxExperts; }
 
 bool route_one_launch(const RouteSource& src, const RouteMove& mv, int T, int E) {
-    return T <= kOneLaunchTokens && E <= 128 && mv.grouped && !src.aux_part && !src.logits_out;
+    return T <= kOneLaunchTokens && E <= 128 && !src.aux_part && !src.logits_out;
 }
 
 cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, const RouteExport& ex, const float* b_gate, const Tables& tb,
@@ -1015,12 +1017,13 @@ cudaError_t launch_route_fused(const RouteSource& src, const RouteMove& mv, cons
         const size_t smem = (size_t)quads * kPlaceThreads * sizeof(float4) + sizeof(int32_t) * (kPlaceThreads / 32) * E;     // 40 KB at most
 #define BIGMAC_ROUTE(Q)                                                                                                            \
     do {                                                                                                                           \
-        const auto kernel = mv.partial ? route_cluster_kernel<Q, 2> : route_cluster_kernel<Q, 1>;                                 \
+        const auto kernel = !mv.grouped ? route_cluster_kernel<Q, 0> : mv.partial ? route_cluster_kernel<Q, 2> : route_cluster_kernel<Q, 1>; \
         static PerDeviceOnce once;                                                                                                 \
         int dev;                                                                                                                   \
         if (once.needed(&dev)) {                                                                                                   \
             cudaError_t e = cudaFuncSetAttribute(route_cluster_kernel<Q, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 49152);  \
             if (e == cudaSuccess) e = cudaFuncSetAttribute(route_cluster_kernel<Q, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 49152); \
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(route_cluster_kernel<Q, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 49152); \
             if (e != cudaSuccess) return e;                                                                                        \
             once.mark(dev);                                                                                                        \
         }                                                                                                                          \
