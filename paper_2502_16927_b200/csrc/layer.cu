@@ -373,20 +373,52 @@ int run_logits(const bigmac_layer* L, const Dims& m, const void* x, const bigmac
 // The word of a caller's aux_loss table that has to be set to zero because the layer has no such loss.
 float* aux_word_to_zero(const Dims& m, const bigmac_routing_t* out) { return out && m.aux <= 0 ? out->aux_loss : nullptr; }
 
-// Steps F1-F3 without the rest of the layer.
+// Only what routing needs: logits, counting-sort counters and the tables (no float intermediates).
+void carve_route_only(Carver& cv, const Dims& m, Buffers& b) {
+    carve_route_scratch(cv, m, b, false);
+    b.tb.topk_idx = cv.take<int32_t>(m.N);
+    b.tb.topk_w = cv.take<float>(m.N);
+    b.tb.counts = cv.take<int32_t>(m.E);
+    b.tb.offsets = cv.take<int32_t>(m.E + 1);
+    b.tb.poffsets = cv.take<int32_t>(m.E + 1);
+    b.tb.row_of_slot = cv.take<int32_t>(m.N);
+    b.tb.slot_of_row = cv.take<int32_t>(m.N);
+    b.tb.prow_of_slot = cv.take<int32_t>(m.N);
+    b.tb.slot_of_prow = cv.take<int32_t>(m.P);
+    b.tb.tile_expert = cv.take<int32_t>(m.P / kPad);
+    b.tb.n_tiles = cv.take<int32_t>(1);
+    b.tb.counts_chosen = cv.take<int32_t>(m.E);
+    b.aux_loss = cv.take<float>(1);
+    if (m.gate_low) b.x_lo = cv.take_bytes((size_t)m.T * m.r * esize(m.dtype));   // the gate reads x'
+}
+
+// Parts of the logits' contraction in a routing-only call: few tokens are a few tiles, each walking all of d.  A function of the shape: the
+// call with its own scratch (partial results where a forward has the hidden activations) and the one without (a fixed array) have
+// to return the same bits, so both must have the room.
+int route_logits_parts(const bigmac_layer* L, const Dims& m) {
+    if (!L->use_tc || L->tc_mask != ~0u || m.gate_low || !route_fused_supported(m.E, m.k)) return 1;
+    const int parts = split_parts(m, m.E);
+    const size_t bytes = (size_t)parts * m.T * m.E * sizeof(float);
+    Carver measure(nullptr);
+    Buffers b{};
+    carve_route_only(measure, m, b);
+    measure.take_bytes(bytes);
+    return bytes <= (size_t)m.P * m.h * esize(m.dtype) && measure.total() <= (size_t)BIGMAC_STATIC_SCRATCH_BYTES ? parts : 1;
+}
+
+// Steps F1-F3 without the rest of the layer.  parts_room: for the partial results of route_logits_parts.
 int run_routing(const bigmac_layer* L, const Dims& m, const void* x, const bigmac_weights_t* W, Buffers& b,
-                bigmac_routing_t* out, cudaStream_t st) {
-    // Few tokens: the logits' contraction in parts too, added by the top-k (a tile of 128 tokens walks all of d, 8 us at d 2048 and 15 at
-    // d 4096).  The parts lie where a forward has the hidden activations, where the call has that room.  With up to 512 tokens in one
-    // launch after it, us: d 2048, 64 experts, 64 tokens 18.8 -> 12.7, 512 18.3 -> 14.4, 1000 19.9 -> 16.8; d 4096, 128 experts 26.4 -> 16.5,
+                void* parts_room, bigmac_routing_t* out, cudaStream_t st) {
+    // Few tokens: the logits' contraction in parts, added by the top-k (a tile of 128 tokens walked all of d, 8 us at d 2048 and 15 at
+    // d 4096).  With up to 512 tokens in one launch after it, us: d 2048, 64 experts, 64 tokens 18.8 -> 12.7, 512 18.3 -> 14.4, 1000 19.9 -> 16.8; d 4096, 128 experts 26.4 -> 16.5,
     // 25.5 -> 18.7, 26.7 -> 20.2; d 1024, 32 experts 13.8 -> 9.6, 13.5 -> 10.4, 15.2 -> 14.1.
-    const int parts = b.a && route_fused_supported(m.E, m.k) && !m.gate_low && L->use_tc && L->tc_mask == ~0u ? split_parts(m, m.E) : 1;
-    if (parts > 1 && (size_t)parts * m.T * m.E * sizeof(float) <= (size_t)m.P * m.h * esize(m.dtype)) {
+    const int parts = route_logits_parts(L, m);
+    if (parts > 1) {
         GemmArgs g;
-        g.A = x; g.lda = m.d; g.B = W->w_gate; g.ldb = m.d; g.C = b.a; g.ldc = m.E;
+        g.A = x; g.lda = m.d; g.B = W->w_gate; g.ldb = m.d; g.C = parts_room; g.ldc = m.E;
         g.M = m.T; g.N = m.E; g.K = m.d; g.out_f32 = true; g.split_k = parts;
         BIGMAC_TRY(gemm(L, G_LOGITS, g, st));
-        return route_from_logits(L, m, W, b, RouteSource{(const float*)b.a, m.E, parts, (int64_t)m.T * m.E, nullptr}, RouteMove{}, aux_word_to_zero(m, out), out, st);
+        return route_from_logits(L, m, W, b, RouteSource{(const float*)parts_room, m.E, parts, (int64_t)m.T * m.E, nullptr}, RouteMove{}, aux_word_to_zero(m, out), out, st);
     }
     BIGMAC_TRY(run_logits(L, m, x, W, b, st));
     return route_from_logits(L, m, W, b, RouteSource{b.logits, m.E, 1, 0, nullptr}, RouteMove{}, aux_word_to_zero(m, out), out, st);
@@ -636,7 +668,7 @@ int bigmac_route(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_weigh
     carve_saved(cv, m, b, false);
     alias_routing(b, out);
     cudaStream_t st = (cudaStream_t)stream;
-    return run_routing(L, m, x, W, b, out, st);
+    return run_routing(L, m, x, W, b, b.a, out, st);
 }
 
 int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_weights_t* W, void* y,
@@ -1176,25 +1208,6 @@ int static_scratch_address(int device, void** ptr) {
     return BIGMAC_OK;
 }
 
-// Only what routing needs: logits, counting-sort counters and the tables (no float intermediates).
-void carve_route_only(Carver& cv, const Dims& m, Buffers& b) {
-    carve_route_scratch(cv, m, b, false);
-    b.tb.topk_idx = cv.take<int32_t>(m.N);
-    b.tb.topk_w = cv.take<float>(m.N);
-    b.tb.counts = cv.take<int32_t>(m.E);
-    b.tb.offsets = cv.take<int32_t>(m.E + 1);
-    b.tb.poffsets = cv.take<int32_t>(m.E + 1);
-    b.tb.row_of_slot = cv.take<int32_t>(m.N);
-    b.tb.slot_of_row = cv.take<int32_t>(m.N);
-    b.tb.prow_of_slot = cv.take<int32_t>(m.N);
-    b.tb.slot_of_prow = cv.take<int32_t>(m.P);
-    b.tb.tile_expert = cv.take<int32_t>(m.P / kPad);
-    b.tb.n_tiles = cv.take<int32_t>(1);
-    b.tb.counts_chosen = cv.take<int32_t>(m.E);
-    b.aux_loss = cv.take<float>(1);
-    if (m.gate_low) b.x_lo = cv.take_bytes((size_t)m.T * m.r * esize(m.dtype));   // the gate reads x'
-}
-
 }  // namespace
 
 extern "C" {
@@ -1218,9 +1231,10 @@ int bigmac_route_static(bigmac_layer_t* L, const void* x, int32_t T, const bigma
     Carver cv(base);
     Buffers b{};
     carve_route_only(cv, m, b);
+    void* parts_room = cv.take_bytes((size_t)route_logits_parts(L, m) * m.T * m.E * sizeof(float));      // (one part: not used)
     alias_routing(b, out);
     cudaStream_t st = (cudaStream_t)stream;
-    return run_routing(L, m, x, W, b, out, st);
+    return run_routing(L, m, x, W, b, parts_room, out, st);
 }
 
 int bigmac_profile_enable(bigmac_layer_t* L, int on) {

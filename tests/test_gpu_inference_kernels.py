@@ -97,18 +97,21 @@ def test_routing_in_two_launches(E, k, T):
 @pytest.mark.parametrize("E,k,T", [(4, 1, 1), (64, 8, 5), (128, 8, 127), (132, 3, 129), (256, 8, 300), (36, 3, 512), (64, 8, 513), (128, 8, 1500), (32, 4, 3000)])
 def test_routing_call_with_logits_in_parts(E, k, T):
     """bf16, d = 1088 (17 slices: parts of unequal length): the routing call adds the parts of its logits in the top-k; up to 512 tokens
-    and 128 experts in one launch."""
+    and 128 experts in one launch.  The call without scratch of its own returns the same bits."""
     import torch
+    from paper_2502_16927_b200 import binding
 
     w = wl.Workload("route", T=T, d=1088, r=64, h=64, E=E, k=k, dtype=wl.DTYPE_BF16, act=wl.ACT_RELU, seed=36)
     inp = _inputs(w, 1.0)
     dev = to_device(w, inp)
     for f in (0.0, 0.6):
         layer = make_layer(w, capacity_factor=f)
-        R = layer.route(dev["x"], dev)
+        R, S = layer.route(dev["x"], dev), layer.empty_routing(T)
+        binding.bigmac_route_static(layer.handle, dev["x"], T, dev, S)
         torch.cuda.synchronize()
         assert layer.status() == 0
         _check_tables(R, oracle.route(inp, w.k, capacity_factor=f))
+        assert all(torch.equal(R[name], S[name]) for name in ("topk_idx", "topk_w", "counts", "offsets", "row_of_slot", "slot_of_row"))
         layer.close()
 
 
