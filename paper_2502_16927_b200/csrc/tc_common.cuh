@@ -338,10 +338,10 @@ __device__ __forceinline__ void gelu_pair2(float z0, float z1, float& a0, float&
     upk2(P, p0, p1);
     const f32x2_t cdf = pk2(fma_sat(z0, p0, 0.5f), fma_sat(z1, p1, 0.5f));
     float x0, x1;
-    upk2(fma2(w, pk2(-0.72134752f, -0.72134752f), pk2(-1.32574806f, -1.32574806f)), x0, x1);
-    const f32x2_t e = pk2(fast_ex2(x0), fast_ex2(x1));                                   // exp(-z^2 / 2) / sqrt(2 pi), the factor as 2^-1.3257
+    upk2(mul2(w, pk2(-0.72134752f, -0.72134752f)), x0, x1);
+    const f32x2_t e = pk2(fast_ex2(x0), fast_ex2(x1));                                   // exp(-z^2 / 2)
     upk2(mul2(z, cdf), a0, a1);
-    upk2(fma2(z, e, cdf), g0, g1);
+    upk2(fma2(mul2(z, e), pk2(0.39894228f, 0.39894228f), cdf), g0, g1);
 }
 
 // sigma' is saved as one byte per element: q = round(200 sigma' + 27), i.e. sigma' = (q - 27) / 200 on [-0.135, 1.14]

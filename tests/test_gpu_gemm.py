@@ -121,6 +121,32 @@ def test_gelu_epilogue_error_bound_over_a_sweep_of_z():
     assert np.max(np.abs(got_z - _dgelu(z64))) <= 0.0026
 
 
+def _sigma_byte_checksum():
+    """CRC of the saved sigma' of GELU over 8 M fp32 values across [-8, 8), each given as the exact sum of three bf16 parts."""
+    import zlib
+    import torch
+    M, N, K = 131072, 64, 192
+    n = (np.arange(M * N, dtype=np.int64) * 40503 + 11) % 2 ** 24
+    rest = ((n - 2 ** 23).astype(np.float64) * 2.0 ** -20).astype(np.float32).reshape(M, N)      # 24 bits: exact
+    A = np.empty((M, K), dtype=np.float32)
+    for part in range(3):                               # the upper 8 significant bits of what is left
+        A[:, part * N:(part + 1) * N] = (rest.view(np.uint32) & np.uint32(0xFFFF0000)).view(np.float32)
+        rest = rest - A[:, part * N:(part + 1) * N]
+    assert not rest.any()
+    C = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")
+    Z = torch.zeros((M, N), dtype=torch.uint8, device="cuda")
+    _run(_layer(), _q(A=_dev_bf16(A), B=_dev_bf16(np.tile(np.eye(N, dtype=np.float32), 3)), C=C, Z=Z, lda=K, ldb=K, ldc=N, M=M, N=N, K=K,
+                      a_kmajor=1, b_kmajor=1, epilogue=1, act=1))
+    return zlib.crc32(Z.cpu().numpy().tobytes())
+
+
+def test_saved_gelu_derivative_keeps_its_bits():
+    """A training step of equal inputs has equal gradients from one version of the library to the next: the bytes of sigma' are
+    pinned.  (Another order of its roundings, as exact as this one, moves one byte in some 500000 and with it the last bit of one bf16
+    gradient in 50.)"""
+    assert _sigma_byte_checksum() == 0xD0C8B78A
+
+
 @pytest.mark.parametrize("N", [32, 8, 5])
 def test_dense_fp32_output_with_narrow_n(N):
     import torch
