@@ -326,13 +326,7 @@ bool fused_mlp_supported(int r, int h, int dtype) {
     return dtype == BIGMAC_BF16 && r >= 64 && r <= 512 && r % 64 == 0 && h >= 64 && h % 64 == 0;
 }
 
-// Slices are limited to what fits the activation buffer [P, h] of bf16 that the separate GEMMs would use.
-MlpSlicing fused_mlp_slicing(int r, int h, int64_t N, int64_t P) {
-    const int units = sm_count();
-    MlpSlicing m{units, (h + HC - 1) / HC, 1, r <= 256 ? 1 : 2, ((1ull << 40) + units - 1) / units};
-    while (m.most < 8 && 2 * m.most * N * r * 4 <= P * h * 2) m.most *= 2;
-    return m;
-}
+MlpSlicing fused_mlp_slicing(int r, int h, int64_t N, int64_t P) { return mlp_slicing(sm_count(), r, h, N, P); }
 
 // xg [max_rows, r] grouped padded rows, w1 [E, h, r], w2 [E, r, h], out [slices][slots][r]; tiles of 128 rows and the tables
 // on the device.

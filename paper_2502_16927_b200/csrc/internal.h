@@ -6,6 +6,7 @@
 #include <stddef.h>
 
 #include "bigmac.h"
+#include "expert_choice.h"
 #include "switches.h"
 
 namespace bigmac {
@@ -39,7 +40,6 @@ inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
 }
 #endif
 
-constexpr int kPad = 128;          // expert segments are padded to multiples of this many rows internally
 constexpr int kMaxExperts = 1024;
 
 // ---------------------------------------------------------------------------------------------
@@ -125,35 +125,6 @@ cudaError_t gemm_tc_groupk_finish(const GemmArgs& g, void* ws, cudaStream_t stre
 // Inference forward of the experts in one kernel (gemm_tc_mlp.cu): fp32 rows of u = sigma(xg W1_e^T) W2_e^T by slot,
 // out [slices][slots][r] (the slices of the hidden width add up to u; a single slice is written as bf16), hidden activations
 // kept on the SM.
-// How many slices is a function of the number of row tiles, which only the device knows: every kernel concerned
-// evaluates mlp_slices for itself.
-struct MlpSlicing {
-    int units;       // SMs
-    int chunks;      // 128-wide chunks of the hidden width
-    int most;        // slices that the output buffer has room for
-    int per_tile;    // work items per 128-row tile and slice
-    unsigned long long inv;   // 2^40 / units, rounded up: division by a multiplication (exact below 2^40 / units^2)
-};
-// The slices s (a power of two) with the shortest longest SM: rounds of items, times an item's
-// chunks and what its start and its output take in units of a chunk (fp32 partial results: twice the bytes of bf16).
-// Few tiles: more slices put idle SMs to work (64 tiles of 8 chunks: two slices, 17 -> 12 us); more than one tile per SM:
-// one slice (220 tiles of 8 chunks: the fp32 rows of two slices cost what the better last round gains; so does leaving the whole
-// rounds uncut and cutting the rest only, 88 -> 90 us at 3001 tokens and no difference up to 13000).  The units were fitted at
-// d 2048; against the best of 1, 2, 4 and 8 slices a forward of 24 to 4096 tokens is within 4.4 % at eight widths (r 64 to 512, h 256 to
-// 2048, 8 to 128 experts), most within 1.5 %, but for d 4096 at 24 tokens (107.8 us, one slice 97.5).
-// Slices that differ by a chunk, of at least three, are taken where one slice would leave half of the SMs idle (2 experts of
-// h 2112, r 512, 64 tokens: 65 -> 41 us a forward, 32 experts 72 -> 60); with more tiles their fp32 rows cost more (100 experts, 600
-// tokens: 106 -> 121), and slices of one or two chunks bring nothing at 500 tokens and more.
-__device__ __forceinline__ int mlp_slices(const MlpSlicing& m, int tiles) {
-    int best = 1, best_cost = 0x7fffffff;
-    for (int j = 0; (1 << j) <= m.most; ++j) {
-        if ((m.chunks & ((1 << j) - 1)) && ((m.chunks >> j) < 3 || 2 * tiles > m.units)) break;
-        const int rounds = (int)(((unsigned)(tiles * m.per_tile << j) + m.units - 1) * m.inv >> 40);
-        const int cost = rounds * (((m.chunks - 1) >> j) + 1 + (j > 0 ? 3 : 2));
-        if (cost < best_cost) { best = 1 << j; best_cost = cost; }
-    }
-    return best;
-}
 struct Tables;
 bool fused_mlp_supported(int r, int h, int dtype);
 MlpSlicing fused_mlp_slicing(int r, int h, int64_t N, int64_t P);

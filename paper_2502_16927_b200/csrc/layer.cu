@@ -480,52 +480,14 @@ bool uses_fused_mlp(const bigmac_layer* L, const Dims& m) {
     return m.r <= 256 || m.N <= 48 * (int64_t)m.E;
 }
 
-// Rounds of pairs of 128-row tiles on the SM pairs: if the experts are chosen evenly, an expert has about N / E rows, give or take
-// sqrt(N / E), and the probability that it reaches its j-th pair is taken as a ramp of two deviations to either side; if they
-// are chosen as unevenly as Zipf's law has it, full pairs and 0.85 (few rows an expert) to 0.55 (2048) pairs an expert more, a fit within
-// 2 % of the pairs to such loads of 32 and 64 experts.
-double ffn_rounds(const Dims& m, bool even) {
-    const double pair = 2.0 * kPad, units = gemm_tc_sm_count() / 2;
-    if (!even) return (std::fmin((double)m.N, (double)m.cap * m.E) / pair + (0.5 + 0.42 / (1 + (double)m.N / m.E / 300)) * m.E) / units;
-    const double rows = std::fmin((double)m.N / m.E, (double)m.cap), dev = std::sqrt((double)m.N / m.E) + 1e-3;
-    const int64_t whole = (int64_t)std::fmax(0.0, std::ceil((rows - 2 * dev) / pair));      // reached by all
-    double pairs = (double)whole;
-    for (int64_t j = whole; pair * j < rows + 2 * dev; ++j) pairs += std::fmin(1.0, 0.5 + (rows - pair * j) / (4 * dev));
-    return pairs * m.E / units;
-}
-
 // Do both contractions of the experts run in one kernel on CTA pairs?  A function of the handle, T and the debug switches: a
-// training forward and its backward must see the same (sigma' lies in memory as that kernel wants it).
-// Measured against the separate contractions, us (a training step; even loads; d 2048 r 256 h 1024 64 experts top-8, and d 1024 r 128
-// h 512 32 experts top-4): it wins unless its last round of pairs is nearly empty.  How full that is depends on the loads, which only the
-// device knows, so both estimates have to allow it.
-//   r 256: 600 tokens 176 -> 172, 4000 288 -> 266, 12000 649 -> 640, Zipf 600 185 -> 179, 3000 286 -> 275, 16384 907 -> 874 (the SM clock rises
-//          from 1.53 to 1.63 GHz under the power cap); 2048 (65 % of two rounds) 227 -> 229, Zipf 3500 (68 % of three) 303 -> 312.  1400: 207 ->
-//          190 even, but Zipf (91 pairs for 64) 223 -> 232, and 850 Zipf (78) 196 -> 221
-//   r 128: 300 103 -> 100, 3000 127 -> 121, 8000 178 -> 174, 20000 348 -> 339; but 4096 (1.1 rounds) 136 -> 146, 6000 (70 %) 159 -> 160,
-//          9000 (72 %) 193 -> 197, 11000 (87 %) 215 -> 216; Zipf 3300 138 -> 132, 3600 142 -> 155
-// Inference, against the kernel whose tokens are the N of its MMAs (gemm_tc_mlp.cu), which takes a batch's few rows an expert better:
-//   r 256: 800 tokens (100 rows) 61 -> 63, 1200 (150) 64.8 -> 64.2, 3001 83 -> 77, 8000 145 -> 127, Zipf 1500 64 -> 75, 2300 (79 %) 80 -> 77, 3950 (73 %)
-//   88 -> 95, 4200 (78 %) 100 -> 95;  r 128: 2000 (250) 37.1 -> 37.4, 2500 (312) 40.1 -> 40.1, 3500 41.2 -> 40.4, 4096 (1.1 rounds) 41.7 -> 46.2, 5000 (64 %)
-//   54.2 -> 51.2, 12000 77 -> 70, Zipf 3300 40.9 -> 40.4, 3600 41 -> 47, 5000 53 -> 51.
-// That kernel keeps u in fp32 where it cuts the hidden width (mlp_slices: up to half as many tiles as SMs, with more than ten chunks
-// up to an eighth of the SMs for each chunk), which is more precise than u in bf16 here: such batches stay with it.
+// training forward and its backward must see the same (sigma' lies in memory as that kernel wants it).  ffn_pair_pays has the rule.
 bool uses_ffn(const bigmac_layer* L, const Dims& m, bool training) {
     const int mode = switches().ffn;
     if (mode == 0 || m.bias || !sigma_as_bytes(L) || !ffn_pair_supported(m.r, m.h, m.E, m.dtype)) return false;
     if (mode == 2) return true;
-    if (!training) {
-        const double rows = std::fmin((double)m.N, (double)m.cap * m.E);
-        const int chunks = m.h / 128, units = gemm_tc_sm_count();
-        const double cut_up_to = 128.0 * units * (chunks <= 10 ? 0.5 : chunks / 8.0);        // rows
-        if (switches().fused_mlp != 1 || rows <= cut_up_to || rows < (m.r == 256 ? 150.0 : 320.0) * m.E) return false;
-    }
-    const double least = training ? (m.r == 256 ? 0.72 : 0.87) : (m.r == 256 ? 0.77 : 0.63);      // of all rounds' pairs
-    for (int even = 0; even < 2; ++even) {
-        const double rounds = ffn_rounds(m, even != 0), whole = std::ceil(1.03 * rounds);        // an estimate
-        if (whole > 1 && rounds < least * whole) return false;
-    }
-    return true;
+    if (!training && switches().fused_mlp != 1) return false;
+    return ffn_pair_pays(ExpertCall{m.T, m.k, m.r, m.h, m.E, m.cap, gemm_tc_sm_count(), training});
 }
 
 // ... or, on the fp32 path, in one launch of FMA blocks?  Everywhere within its widths: a training step / an inference forward, us, with two

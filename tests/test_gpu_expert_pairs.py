@@ -77,3 +77,27 @@ def test_fp32_in_one_launch(d, r, h, E, k, T, capacity):
     for name, ref in out[0].items():
         err = (ref.double() - out[1][name].double()).norm()
         assert err <= (4e-5 if "gate" in name else 4e-6) * ref.double().norm(), (name, float(err), float(ref.double().norm()))
+
+
+def test_inference_under_a_capacity_limit_keeps_u_in_fp32():
+    """1250 tokens of 16 experts top-8, eight of them favoured: the capacity limit leaves 48 row tiles, for which the experts' kernel of
+    few rows cuts the hidden width and keeps u in fp32.  Such a call does not go to the pairs, which would round u to bf16."""
+    import torch
+    from paper_2502_16927_b200 import binding
+
+    w = wl.Workload("limit", T=1250, d=128, r=256, h=1024, E=16, k=8, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=77)
+    inp = wl.make_inputs(w)
+    inp["b_gate"] = np.where(np.arange(w.E) < 8, 30.0, 0.0).astype(np.float32)
+    dev = to_device(w, inp)
+    out = {}
+    for mode in (0, 1):
+        try:
+            binding.bigmac_debug_set("ffn", mode)
+            layer = make_layer(w, capacity_factor=1.2)
+            out[mode] = layer.forward(dev["x"], dev)
+            torch.cuda.synchronize()
+        finally:
+            binding.bigmac_debug_set("defaults")
+        assert layer.status() == 0
+        layer.close()
+    assert torch.equal(out[0], out[1])
