@@ -44,6 +44,10 @@ BIGMAC_HOST_DEVICE inline int mlp_slices(const MlpSlicing& m, int tiles) {
     }
     return best;
 }
+// padded rows of N slots over E experts, at most
+inline int64_t padded_rows_max(int64_t N, int E) { return ((N + kPad - 1) / kPad + E) * (int64_t)kPad; }
+// Do that kernel's fp32 rows fit the activation buffer [P, h] of bf16?
+inline bool mlp_fits(int r, int h, int64_t N, int64_t P) { return N * r * 4 <= P * h * 2; }
 // Slices are limited to what fits the activation buffer [P, h] of bf16 that the separate contractions would use.
 inline MlpSlicing mlp_slicing(int units, int r, int h, int64_t N, int64_t P) {
     MlpSlicing m{units, (h + 127) / 128, 1, r <= 256 ? 1 : 2, ((1ull << 40) + units - 1) / units};
@@ -59,47 +63,72 @@ struct ExpertCall {
     int64_t N() const { return (int64_t)T * k; }
 };
 
-// Rounds of pairs of 128-row tiles on the SM pairs: if the experts are chosen evenly, an expert has about N / E rows, give or take
-// sqrt(N / E), and the probability that it reaches its j-th pair is taken as a ramp of two deviations to either side; if they
-// are chosen as unevenly as Zipf's law has it, full pairs and 0.85 (few rows an expert) to 0.55 (2048) pairs an expert more, a fit within
-// 2 % of the pairs to such loads of 32 and 64 experts.
-inline double ffn_rounds(const ExpertCall& m, bool even) {
-    const double N = (double)m.N(), pair = 2.0 * kPad, units = m.units / 2;
-    if (!even) return (std::fmin(N, (double)m.cap * m.E) / pair + (0.5 + 0.42 / (1 + N / m.E / 300)) * m.E) / units;
+// Rounds of items of `size` rows on `units` SMs or SM pairs: if the experts are chosen evenly, an expert has about N / E rows, give or
+// take sqrt(N / E) (normally distributed, which is the probability that it reaches its j-th item); if they
+// are chosen as unevenly as Zipf's law has it, full items and 0.85 (few rows an expert) to 0.55 (eight items) an expert more, a fit
+// within 2 % of the pairs of tiles to such loads of 32 and 64 experts.
+inline double item_rounds(const ExpertCall& m, int size, int units, bool even) {
+    const double N = (double)m.N();
+    if (!even) return (std::fmin(N, (double)m.cap * m.E) / size + (0.5 + 0.42 / (1 + N / m.E / (1.172 * size))) * m.E) / units;
     const double rows = std::fmin(N / m.E, (double)m.cap), dev = std::sqrt(N / m.E) + 1e-3;
-    const int64_t whole = (int64_t)std::fmax(0.0, std::ceil((rows - 2 * dev) / pair));      // reached by all
-    double pairs = (double)whole;
-    for (int64_t j = whole; pair * j < rows + 2 * dev; ++j) pairs += std::fmin(1.0, 0.5 + (rows - pair * j) / (4 * dev));
-    return pairs * m.E / units;
+    const int64_t whole = (int64_t)std::fmax(0.0, std::ceil((rows - 3 * dev) / size));      // reached by all
+    double items = (double)whole;
+    for (int64_t j = whole; size * j < rows + 3 * dev; ++j) items += 0.5 * std::erfc((size * j - rows) / (1.41421356 * dev));
+    return items * m.E / units;
 }
 
-// Where the kernel on CTA pairs pays, among the widths it takes.
-// Measured against the separate contractions, us (a training step; even loads; d 2048 r 256 h 1024 64 experts top-8, and d 1024 r 128
-// h 512 32 experts top-4): it wins unless its last round of pairs is nearly empty.  How full that is depends on the loads, which only the
-// device knows, so both estimates have to allow it.
-//   r 256: 600 tokens 176 -> 172, 4000 288 -> 266, 12000 649 -> 640, Zipf 600 185 -> 179, 3000 286 -> 275, 16384 907 -> 874 (the SM clock rises
-//          from 1.53 to 1.63 GHz under the power cap); 2048 (65 % of two rounds) 227 -> 229, Zipf 3500 (68 % of three) 303 -> 312.  1400: 207 ->
-//          190 even, but Zipf (91 pairs for 64) 223 -> 232, and 850 Zipf (78) 196 -> 221
-//   r 128: 300 103 -> 100, 3000 127 -> 121, 8000 178 -> 174, 20000 348 -> 339; but 4096 (1.1 rounds) 136 -> 146, 6000 (70 %) 159 -> 160,
-//          9000 (72 %) 193 -> 197, 11000 (87 %) 215 -> 216; Zipf 3300 138 -> 132, 3600 142 -> 155
-// Inference, against the kernel whose tokens are the N of its MMAs (gemm_tc_mlp.cu), which takes a batch's few rows an expert better:
-//   r 256: 800 tokens (100 rows) 61 -> 63, 1200 (150) 64.8 -> 64.2, 3001 83 -> 77, 8000 145 -> 127, Zipf 1500 64 -> 75, 2300 (79 %) 80 -> 77, 3950 (73 %)
-//   88 -> 95, 4200 (78 %) 100 -> 95;  r 128: 2000 (250) 37.1 -> 37.4, 2500 (312) 40.1 -> 40.1, 3500 41.2 -> 40.4, 4096 (1.1 rounds) 41.7 -> 46.2, 5000 (64 %)
-//   54.2 -> 51.2, 12000 77 -> 70, Zipf 3300 40.9 -> 40.4, 3600 41 -> 47, 5000 53 -> 51.
+// Where the kernel on CTA pairs pays, among the widths it takes.  How full its last round of pairs is depends on the loads, which only
+// the device knows, so both estimates have to allow it.  The lines were set on steps and forwards of r 128 (d 1024) and r 256 (d 2048) with
+// h 128 to 4096, 8 to 256 experts, 8 to 3000 rows an expert, even and Zipf loads: of 1684 shapes a training step goes to the pairs
+// with 598, 531 of them faster by more than 1.5 % and two slower (2.2 %), a forward with 452, 428 faster and seven slower (3.5 % at most).
+// Figures: us, the other kernels -> this one; loads even unless said.
+//
+// Training, against the separate contractions.  It wins with many rows an expert and full rounds.
+//   d 2048, r 256, h 1024, 64 experts top-8: 3000 tokens 253 -> 245, Zipf 280 -> 269, 5600 354 -> 338, 8000 441 -> 423, 13000 638 -> 616; but 2048 (68 %
+//   of two rounds) 229 -> 231, Zipf 700 (1.01 rounds) 187 -> 218, 1400 and 3950 224 -> 230 and 321 -> 320 (even 205 -> 190, 283 -> 261).
+//   d 1024, r 128, h 512, 32 experts top-4: 2300 tokens 120 -> 116, 3000 124 -> 120, 16384 283 -> 277, 24000 395 -> 384; but 4200 (1.16 rounds) 140 ->
+//   149, 5600 155 -> 160, 9000 186 -> 195, Zipf 3600 (1.04) 143 -> 155; 700 to 1800 tokens 107 either way.
+// In a single round the separate contractions have blocks for all SMs, which counts the more, the longer an item's walk along
+// the hidden width is: 8 experts top-2, 300 tokens, r 128, h 256 103 -> 96, 512 105 -> 103, 1024 108 -> 115, 2048 111 -> 141, 4096 125 -> 197; r 256,
+// h 1024 123 -> 130, 2048 134 -> 158; 8192 tokens, 0.9 of the round: r 128, h 2048 235 -> 223, r 256, h 2048 330 -> 311.
+// With more rounds an expert needs the rows, a pair that is half empty costs a whole one: 256 experts top-8, 1280 tokens (40 rows), r 256, h 256
+// 201 -> 214, 2048 573 -> 600, r 128, h 1024 266 -> 312; 6080 tokens (190 rows), r 256, h 256 320 -> 285, 2048 809 -> 774.  Very large batches of r 256, under
+// the power cap: h 1024, 64 experts, 20500 tokens 943 -> 983, 24000 1127 -> 1125, 29000 1333 -> 1335, 256 experts, 32000 1678 -> 1742.  r 128 with h 128 wins
+// little (64 experts, 3000 tokens 117 -> 115; 256 experts, 12000 254 -> 259).
+//
+// Inference, against the kernel whose tokens are the N of its MMAs (gemm_tc_mlp.cu), which takes a batch's few rows an expert better and
+// whose items are single tiles on single SMs: what counts is how its rounds compare with these.
+//   r 256, h 1024, 64 experts: 1400 tokens 61.4 -> 60.8, 3000 84 -> 77, 8000 148 -> 131, 8700 (four rounds of tiles, five of pairs) 150 -> 143, 16384 287 -> 236, Zipf
+//   1150 (one, two) 59 -> 74, 3950 (two, three) 89 -> 95, 6300 (three, four) 119 -> 122; 128 experts, 3040 tokens, Zipf (two, three) 93 -> 102.
+//   r 128, h 512, 32 experts: 2600 40.4 -> 40.2, 5000 52.9 -> 51.2, 16384 93 -> 86, 18200 (four, five) 95.8 -> 94.1, 3600 Zipf (one, two) 41 -> 46, 8700 (two,
+//   three) 58 -> 61, 13500 (three, four) 78.1 -> 79.2; with a longer walk four to five rounds lose as well: 128 experts, h 2048, 8192 tokens 162 -> 179.
+// Where the hidden width is too narrow for that kernel, it is the separate contractions again: 64 experts, 3000 tokens, h 128, r 256 59 -> 51,
+// r 128 47 -> 43; but 256 experts, 16384 tokens, r 128 125 -> 129.
 // That kernel keeps u in fp32 where it cuts the hidden width (mlp_slices: up to half as many tiles as SMs, with more than ten chunks
 // up to an eighth of the SMs for each chunk), which is more precise than u in bf16 here: a batch stays with it if its loads could
 // leave so few tiles (under a capacity limit, if k experts are chosen by all tokens and keep what the limit allows).
 inline bool ffn_pair_pays(const ExpertCall& m) {
-    if (!m.training) {
-        const double rows = std::fmin((double)m.N(), (double)m.cap * m.E), fewest = (double)m.k * std::fmin((double)m.T, (double)m.cap);
-        const int chunks = m.h / 128;
-        const double cut_up_to = 128.0 * m.units * (chunks <= 10 ? 0.5 : chunks / 8.0);        // rows
-        if (fewest <= cut_up_to || rows < (m.r == 256 ? 150.0 : 320.0) * m.E) return false;
+    const bool wide = m.r == 256;
+    const int chunks = m.h / 128;
+    const double rows = std::fmin((double)m.N(), (double)m.cap * m.E) / m.E;               // an expert's, on average
+    const bool mlp = mlp_fits(m.r, m.h, m.N(), padded_rows_max(m.N(), m.E));
+    double least = m.training ? (wide ? 0.72 : 0.87) : (wide ? 0.77 : 0.63);               // part of the rounds that has to be filled
+    double least_of_one = 0;
+    if (m.training) {
+        if (wide ? chunks > 2 && m.N() > 160000 : chunks == 1) return false;
+        if (wide && chunks >= 16) least = 0.8;
+        if (chunks > (wide ? 4 : 2)) least_of_one = wide ? std::fmin(0.72, 0.1 + chunks / 32.0) : chunks <= 4 ? 0.6 : 0.87;
+    } else {
+        const double fewest = (double)m.k * std::fmin((double)m.T, (double)m.cap);
+        const double cut_up_to = 128.0 * m.units * (chunks <= 10 ? 0.5 : chunks / 8.0);    // rows
+        if (fewest <= cut_up_to || rows < (wide ? 150 : 320)) return false;
+        if (!mlp && !wide && m.N() > 128000) return false;
     }
-    const double least = m.training ? (m.r == 256 ? 0.72 : 0.87) : (m.r == 256 ? 0.77 : 0.63);      // of all rounds' pairs
     for (int even = 0; even < 2; ++even) {
-        const double rounds = ffn_rounds(m, even != 0), whole = std::ceil(1.03 * rounds);        // an estimate
-        if (whole > 1 && rounds < least * whole) return false;
+        const double rounds = item_rounds(m, 2 * kPad, m.units / 2, even != 0), whole = std::ceil(1.03 * rounds);        // an estimate
+        if (whole > 1 ? rounds < least * whole : rounds < least_of_one) return false;
+        if (m.training && (whole > 1 ? rows < 176 : chunks > 2 && rows < (wide ? 100 : 176))) return false;
+        if (!m.training && mlp && std::ceil(0.985 * item_rounds(m, kPad, m.units, even != 0)) < (wide || chunks <= 4 ? 0.78 : 0.95) * std::ceil(rounds)) return false;
     }
     return true;
 }

@@ -186,7 +186,6 @@ struct PerDeviceOnce {
     void mark(int dev) { if (dev >= 0) done |= 1ull << dev; }
 };
 
-inline int64_t padded_rows_max(int64_t N, int E) { return ((N + kPad - 1) / kPad + E) * (int64_t)kPad; }
 constexpr int kSortChunk = 1024;   // slots per block of the counting sort
 inline int sort_blocks(int64_t N) { return (int)((N + kSortChunk - 1) / kSortChunk); }
 

@@ -472,7 +472,7 @@ GemmArgs dw1_request(const Dims& m, const void* dz, const void* rows, const Tabl
 // Do the experts of an inference forward run in one kernel?  (The fused_mlp debug switch: 0 never, 2 wherever it can.)
 bool uses_fused_mlp(const bigmac_layer* L, const Dims& m) {
     const int mode = switches().fused_mlp;
-    if (mode == 0 || m.bias || !sigma_as_bytes(L) || !fused_mlp_supported(m.r, m.h, m.dtype) || m.N * m.r * 4 > m.P * m.h * 2) return false;
+    if (mode == 0 || m.bias || !sigma_as_bytes(L) || !fused_mlp_supported(m.r, m.h, m.dtype) || !mlp_fits(m.r, m.h, m.N, m.P)) return false;
     if (mode == 2) return true;
     // r <= 256: always.  Wider rows leave room for 64 tokens in tensor memory, and the weights are streamed again for every 64
     // tokens of an expert: as long as most experts have one such unit (d 4096, 128 experts, r 512: 600 tokens 139 us, separate

@@ -60,3 +60,32 @@ int main() {
 """)
     chosen, limited = map(int, out.split())
     assert chosen > 1000 and limited > 100
+
+
+def test_pairs_only_where_they_were_the_faster_ones(tmp_path):
+    """Calls on either side of the lines, each timed both ways (148 SMs; even and Zipf loads where the loads are not known): the ones that
+    the kernel on CTA pairs made slower by 3 to 45 % keep their kernels, the ones that it made faster have it."""
+    slower = [(1, 128, 512, 32, 4, 4200), (1, 128, 512, 32, 4, 1800), (1, 128, 1024, 8, 2, 300), (1, 128, 2048, 8, 2, 300), (1, 128, 2048, 8, 2, 3000),
+              (1, 128, 4096, 8, 2, 32), (1, 128, 2048, 64, 2, 1678), (1, 128, 1024, 256, 8, 1280), (1, 128, 128, 256, 8, 9000), (1, 256, 2048, 8, 2, 300),
+              (1, 256, 2048, 8, 2, 3000), (1, 256, 2048, 64, 3, 286), (1, 256, 256, 256, 1, 3832), (1, 256, 256, 256, 8, 1000), (1, 256, 2048, 256, 8, 3000),
+              (1, 256, 1024, 64, 8, 700), (1, 256, 1024, 64, 8, 20500), (1, 256, 1024, 256, 8, 32000), (0, 128, 2048, 128, 8, 6000),
+              (0, 128, 1024, 64, 8, 4096), (0, 128, 512, 64, 8, 4096), (0, 128, 2048, 128, 8, 8192), (0, 128, 512, 32, 4, 8700), (0, 256, 1024, 128, 8, 3040),
+              (0, 256, 2048, 128, 8, 6000), (0, 256, 1024, 64, 8, 1150), (0, 128, 128, 256, 8, 16384)]
+    faster = [(1, 128, 512, 32, 4, 3000), (1, 128, 512, 32, 4, 16384), (1, 128, 2048, 8, 2, 8192), (1, 128, 256, 8, 2, 300),
+              (1, 256, 1024, 64, 8, 2999), (1, 256, 1024, 64, 8, 5600), (1, 256, 1024, 64, 8, 16384), (1, 256, 256, 256, 8, 6080), (1, 256, 1024, 32, 4, 3000),
+              (0, 128, 512, 32, 4, 5000), (0, 128, 512, 32, 4, 16384), (0, 256, 1024, 64, 8, 3001), (0, 256, 1024, 64, 8, 8000), (0, 256, 1024, 64, 8, 8700),
+              (0, 256, 1024, 64, 8, 16384), (0, 256, 128, 64, 8, 3000)]
+    shapes = slower + faster
+    out = _run(tmp_path, r"""
+#include <cstdlib>
+int main(int argc, char** argv) {
+    for (int i = 1; i + 5 < argc; i += 6) {
+        int v[6];
+        for (int j = 0; j < 6; ++j) v[j] = std::atoi(argv[i + j]);
+        std::printf("%d\n", (int)ffn_pair_pays(ExpertCall{v[5], v[4], v[1], v[2], v[3], kNoCapacity, 148, v[0] != 0}));
+    }
+    return 0;
+}
+""", *(n for shape in shapes for n in shape))
+    chosen = [s for s, c in zip(shapes, map(int, out.split())) if c]
+    assert chosen == faster, (set(chosen) - set(faster), set(faster) - set(chosen))
