@@ -210,7 +210,9 @@ __device__ __forceinline__ float warp_sum8(float* v) {
 // Bound by HBM (u read, du written).  A warp per grouped row before, with a chain of three dependent loads for one row, and a
 // launch of its own for the gate: a training step of fp32, 256 tokens, 61.0 -> 59.8 us; d 1024, 4096 tokens 137.4 -> 136.3; d 2048,
 // 2999 tokens 280 -> 277.
-template <typename T>
+// B slots of a token at once, C pieces of 32 vectors of each: B = 8, C = 1; with one or two slots a token B = 2, C = 2 (20000 tokens, one
+// slot, with the gate: r 512 31.2 us with B = 8, 21.8 so, r 256 22.9 and 18.3; as two kernels 27 and 23).
+template <typename T, int B, int C>
 __global__ void __launch_bounds__(256) combine_bwd_kernel(const uint4* __restrict__ dy_lo, const uint4* __restrict__ u,
                                                           uint4* __restrict__ du, float* __restrict__ dp,
                                                           const int32_t* __restrict__ prow_of_slot, const float* __restrict__ topk_w,
@@ -219,7 +221,7 @@ __global__ void __launch_bounds__(256) combine_bwd_kernel(const uint4* __restric
                                                           int k, int vecs_per_row, int E, int width, int ld) {
     grid_dependency_wait();
     grid_dependency_launch();
-    constexpr int V = Vec<T>::kElems, B = 8;
+    constexpr int V = Vec<T>::kElems;
     const int lane = threadIdx.x & 31, token_blocks = (n_tokens + 7) / 8;
     if ((int)blockIdx.x >= token_blocks) {
         const int e = blockIdx.x - token_blocks;
@@ -230,59 +232,83 @@ __global__ void __launch_bounds__(256) combine_bwd_kernel(const uint4* __restric
     const int t = warp_global_id();
     if (t >= n_tokens) return;
     const int64_t s0 = (int64_t)t * k;
-    float mine = 0.0f;                                       // k <= 8: lane j has the j-th slot's dp
+    T* row = dlogits ? dlogits + (int64_t)t * ld : nullptr;
+    if (row)
+        for (int e = lane; e < width; e += 32) row[e] = (T)0.0f;
+    float mine = 0.0f, weight = 0.0f;                        // k <= B: lane j has the j-th slot's dp, weight and expert
+    int expert = -1;
     for (int j0 = 0; j0 < k; j0 += B) {
         int place = -1;
-        float weight = 0.0f;
+        weight = 0.0f;
         if (lane < B && j0 + lane < k) {
             place = prow_of_slot[s0 + j0 + lane];
             weight = topk_w[s0 + j0 + lane];
+            expert = topk_idx[s0 + j0 + lane];
         }
         float dot[B];
 #pragma unroll
         for (int j = 0; j < B; ++j) dot[j] = 0.0f;
-        for (int c0 = 0; c0 < vecs_per_row; c0 += 32) {
-            const int c = c0 + lane;
-            const bool there = c < vecs_per_row;
+        for (int c0 = 0; c0 < vecs_per_row; c0 += 32 * C) {
             const uint4 none = make_uint4(0, 0, 0, 0);
-            const uint4 g = there ? dy_lo[(int64_t)t * vecs_per_row + c] : none;
-            uint4 v[B];
+            uint4 g[C], v[C][B];
 #pragma unroll
-            for (int j = 0; j < B; ++j) {
-                const int prow = __shfl_sync(kFull, place, j);
-                v[j] = there && prow >= 0 ? u[(int64_t)prow * vecs_per_row + c] : none;
+            for (int q = 0; q < C; ++q) {
+                const int c = c0 + 32 * q + lane;
+                g[q] = c < vecs_per_row ? dy_lo[(int64_t)t * vecs_per_row + c] : none;
+#pragma unroll
+                for (int j = 0; j < B; ++j) {
+                    const int prow = __shfl_sync(kFull, place, j);
+                    v[q][j] = c < vecs_per_row && prow >= 0 ? u[(int64_t)prow * vecs_per_row + c] : none;
+                }
             }
-            float a[V];
-            Vec<T>::unpack(g, a);
 #pragma unroll
-            for (int j = 0; j < B; ++j) {
-                const int prow = __shfl_sync(kFull, place, j);
-                if (prow < 0) continue;                      // uniform
-                const float p = __shfl_sync(kFull, weight, j);
-                float b[V], o[V];
-                Vec<T>::unpack(v[j], b);
+            for (int q = 0; q < C; ++q) {
+                const int c = c0 + 32 * q + lane;
+                float a[V];
+                Vec<T>::unpack(g[q], a);
 #pragma unroll
-                for (int i = 0; i < V; ++i) { dot[j] = fmaf(a[i], b[i], dot[j]); o[i] = p * a[i]; }
-                if (there) du[(int64_t)prow * vecs_per_row + c] = Vec<T>::pack(o);
+                for (int j = 0; j < B; ++j) {
+                    const int prow = __shfl_sync(kFull, place, j);
+                    if (prow < 0) continue;                  // uniform
+                    const float p = __shfl_sync(kFull, weight, j);
+                    float b[V], o[V];
+                    Vec<T>::unpack(v[q][j], b);
+#pragma unroll
+                    for (int i = 0; i < V; ++i) { dot[j] = fmaf(a[i], b[i], dot[j]); o[i] = p * a[i]; }
+                    if (c < vecs_per_row) du[(int64_t)prow * vecs_per_row + c] = Vec<T>::pack(o);
+                }
             }
         }
-        const float total = warp_sum8(dot);
-        mine = __shfl_sync(kFull, total, 4 * (lane & 7));
+        if (B == 8) {
+            const float total = warp_sum8(dot);
+            mine = __shfl_sync(kFull, total, 4 * (lane & 7));
+        } else {                                             // the same order of additions
+#pragma unroll
+            for (int j = 0; j < B; ++j) {
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) dot[j] += __shfl_xor_sync(kFull, dot[j], off);
+                if (lane == j) mine = dot[j];
+            }
+        }
         if (lane < B && j0 + lane < k) dp[s0 + j0 + lane] = mine;
     }
-    if (!dlogits) return;
-    T* row = dlogits + (int64_t)t * ld;
-    for (int e = lane; e < width; e += 32) row[e] = (T)0.0f;
+    if (!row) return;
     __syncwarp();                                            // the zeros, and other lanes' dp, are there
     float part = 0.0f;
-    for (int j = lane; j < k; j += 32) part = fmaf(topk_w[s0 + j], k <= B ? mine : dp[s0 + j], part);
+    if (k <= B) part = fmaf(weight, mine, part);             // (weight 0 beyond k)
+    else
+        for (int j = lane; j < k; j += 32) part = fmaf(topk_w[s0 + j], dp[s0 + j], part);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(kFull, part, off);
-    for (int j = lane; j < k; j += 32) {
-        const float dl = topk_w[s0 + j] * ((k <= B ? mine : dp[s0 + j]) - part);
-        const int e = topk_idx[s0 + j];
+    auto give = [&](int j, float w, float g, int e) {
+        const float dl = w * (g - part);
         if ((unsigned)e < (unsigned)E) row[e] = (T)dl;
         dp[s0 + j] = dl;                                     // fp32 copy per slot, for the bias gradient
+    };
+    if (k <= B) {
+        if (lane < k) give(lane, weight, mine, expert);
+    } else {
+        for (int j = lane; j < k; j += 32) give(j, topk_w[s0 + j], dp[s0 + j], topk_idx[s0 + j]);
     }
 }
 
@@ -529,13 +555,13 @@ cudaError_t launch_combine_bwd(const void* dy_lo, const void* u, void* du, float
     if (T == 0) return cudaSuccess;
     const int vecs = width * elem_bytes(dtype) / 16;
     const unsigned blocks = warp_blocks(T) + E;
+    auto launch = [&](auto kernel, auto* dl) {
+        return launch_maybe_chained(chained, kernel, blocks, 256, 0, stream, (const uint4*)dy_lo, (const uint4*)u, (uint4*)du, dp, tb.prow_of_slot,
+                                    tb.topk_w, tb.topk_idx, tb.counts, tb.poffsets, dl, T, k, vecs, E, dl_width, dl_ld);
+    };
     if (dtype == BIGMAC_BF16)
-        return launch_maybe_chained(chained, combine_bwd_kernel<__nv_bfloat16>, blocks, 256, 0, stream, (const uint4*)dy_lo, (const uint4*)u,
-                                    (uint4*)du, dp, tb.prow_of_slot, tb.topk_w, tb.topk_idx, tb.counts, tb.poffsets, (__nv_bfloat16*)dlogits,
-                                    T, k, vecs, E, dl_width, dl_ld);
-    return launch_maybe_chained(chained, combine_bwd_kernel<float>, blocks, 256, 0, stream, (const uint4*)dy_lo, (const uint4*)u, (uint4*)du,
-                                dp, tb.prow_of_slot, tb.topk_w, tb.topk_idx, tb.counts, tb.poffsets, (float*)dlogits, T, k, vecs, E, dl_width,
-                                dl_ld);
+        return k <= 2 ? launch(combine_bwd_kernel<__nv_bfloat16, 2, 2>, (__nv_bfloat16*)dlogits) : launch(combine_bwd_kernel<__nv_bfloat16, 8, 1>, (__nv_bfloat16*)dlogits);
+    return k <= 2 ? launch(combine_bwd_kernel<float, 2, 2>, (float*)dlogits) : launch(combine_bwd_kernel<float, 8, 1>, (float*)dlogits);
 }
 
 cudaError_t launch_gate_bwd(float* dp, const Tables& tb, void* dlogits, int T, int E, int width, int ld, int k,
