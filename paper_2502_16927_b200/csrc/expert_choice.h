@@ -63,14 +63,14 @@ struct ExpertCall {
     int64_t N() const { return (int64_t)T * k; }
 };
 
-// Rounds of items of `size` rows on `units` SMs or SM pairs: if the experts are chosen evenly, an expert has about N / E rows, give or
-// take sqrt(N / E) (normally distributed, which is the probability that it reaches its j-th item); if they
-// are chosen as unevenly as Zipf's law has it, full items and 0.85 (few rows an expert) to 0.55 (eight items) an expert more, a fit
-// within 2 % of the pairs of tiles to such loads of 32 and 64 experts.
+// Rounds of items of `size` rows on `units` SMs or SM pairs.  If the experts are chosen evenly, an expert has about N / E rows, give or
+// take 1.5 sqrt(N / E) (a gate without a bias has some preferences of its own; 32 experts top-4 pass three rounds of pairs at 13050
+// tokens), and reaches its j-th item with the normal distribution's probability.  If they are chosen as unevenly as Zipf's law has
+// it: full items and 0.85 (few rows an expert) to 0.55 (eight items) an expert more, within 2 % of the pairs of tiles for 32 and 64 experts.
 inline double item_rounds(const ExpertCall& m, int size, int units, bool even) {
     const double N = (double)m.N();
     if (!even) return (std::fmin(N, (double)m.cap * m.E) / size + (0.5 + 0.42 / (1 + N / m.E / (1.172 * size))) * m.E) / units;
-    const double rows = std::fmin(N / m.E, (double)m.cap), dev = std::sqrt(N / m.E) + 1e-3;
+    const double rows = std::fmin(N / m.E, (double)m.cap), dev = 1.5 * std::sqrt(N / m.E) + 1e-3;
     const int64_t whole = (int64_t)std::fmax(0.0, std::ceil((rows - 3 * dev) / size));      // reached by all
     double items = (double)whole;
     for (int64_t j = whole; size * j < rows + 3 * dev; ++j) items += 0.5 * std::erfc((size * j - rows) / (1.41421356 * dev));
@@ -80,14 +80,16 @@ inline double item_rounds(const ExpertCall& m, int size, int units, bool even) {
 // Where the kernel on CTA pairs pays, among the widths it takes.  How full its last round of pairs is depends on the loads, which only
 // the device knows, so both estimates have to allow it.  The lines were set on steps and forwards of r 128 (d 1024) and r 256 (d 2048) with
 // h 128 to 4096, 8 to 256 experts, 8 to 3000 rows an expert, even and Zipf loads: of 1684 shapes a training step goes to the pairs
-// with 598, 531 of them faster by more than 1.5 % and two slower (2.2 %), a forward with 452, 428 faster and seven slower (3.5 % at most).
+// with 624, 553 of them faster by more than 1.5 % and two slower (2.2 %), a forward with 452, 428 faster and seven slower (3.5 % at most; up
+// to 10 % where loads just miss the estimated number of rounds).
 // Figures: us, the other kernels -> this one; loads even unless said.
 //
 // Training, against the separate contractions.  It wins with many rows an expert and full rounds.
 //   d 2048, r 256, h 1024, 64 experts top-8: 3000 tokens 253 -> 245, Zipf 280 -> 269, 5600 354 -> 338, 8000 441 -> 423, 13000 638 -> 616; but 2048 (68 %
 //   of two rounds) 229 -> 231, Zipf 700 (1.01 rounds) 187 -> 218, 1400 and 3950 224 -> 230 and 321 -> 320 (even 205 -> 190, 283 -> 261).
 //   d 1024, r 128, h 512, 32 experts top-4: 2300 tokens 120 -> 116, 3000 124 -> 120, 16384 283 -> 277, 24000 395 -> 384; but 4200 (1.16 rounds) 140 ->
-//   149, 5600 155 -> 160, 9000 186 -> 195, Zipf 3600 (1.04) 143 -> 155; 700 to 1800 tokens 107 either way.
+//   149, 5600 155 -> 160, 9000 186 -> 195, Zipf 3600 (1.04) 143 -> 155; 1000 to 1800 tokens lose 1 to 3 %,
+//   512 to 880 (one tile an expert) win as much.
 // In a single round the separate contractions have blocks for all SMs, which counts the more, the longer an item's walk along
 // the hidden width is: 8 experts top-2, 300 tokens, r 128, h 256 103 -> 96, 512 105 -> 103, 1024 108 -> 115, 2048 111 -> 141, 4096 125 -> 197; r 256,
 // h 1024 123 -> 130, 2048 134 -> 158; 8192 tokens, 0.9 of the round: r 128, h 2048 235 -> 223, r 256, h 2048 330 -> 311.
@@ -126,8 +128,9 @@ inline bool ffn_pair_pays(const ExpertCall& m) {
     }
     for (int even = 0; even < 2; ++even) {
         const double rounds = item_rounds(m, 2 * kPad, m.units / 2, even != 0), whole = std::ceil(1.03 * rounds);        // an estimate
-        if (whole > 1 ? rounds < least * whole : rounds < least_of_one) return false;
-        if (m.training && (whole > 1 ? rows < 176 : chunks > 2 && rows < (wide ? 100 : 176))) return false;
+        const bool one_tile = m.training && !wide && chunks <= 4 && rounds < 0.6 && rows >= 60 && rows <= 112;
+        if (!one_tile && (whole > 1 ? rounds < least * whole : rounds < least_of_one)) return false;
+        if (m.training && !one_tile && (whole > 1 ? rows < 176 : chunks > 2 && rows < (wide ? 60 : 176))) return false;
         if (!m.training && mlp && std::ceil(0.985 * item_rounds(m, kPad, m.units, even != 0)) < (wide || chunks <= 4 ? 0.78 : 0.95) * std::ceil(rounds)) return false;
     }
     return true;
