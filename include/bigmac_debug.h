@@ -78,8 +78,8 @@ const char *bigmac_profile_slot_name(int slot);
  *   "overlap" 0/1        backward pass on one stream / independent launches on the handle's second stream (default 1)
  *   "tc_pair" 0/1        never / where faster: the CTA-pair tcgen05 kernel (default 1)
  *   "groupk" 0/1         never / where it pays: the dynamically scheduled per-expert weight-gradient kernel (default 1)
- *   "ffn" 0/1/2          both contractions of an expert in one kernel never / where it pays / wherever it can (default 1); a training
- *                        forward and its backward must see the same value
+ *   "ffn" 0/1/2          both contractions of an expert in one kernel never / where it pays / wherever it can (default 1); read when a
+ *                        handle is created
  *   "fused_mlp" 0/1/2    inference expert GEMM1 + sigma + GEMM2 in one kernel never / on short tile lists / always (default 1)
  *   "epi_parts" 0/1/2/4  working epilogue warps per lane quadrant of plain epilogues (0 = default choice, 2)
  *   "chain" 0/1          kernels launched with programmatic stream serialisation (set-up overlaps the predecessor) (default 1)

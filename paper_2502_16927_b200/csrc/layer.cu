@@ -480,10 +480,10 @@ bool uses_fused_mlp(const bigmac_layer* L, const Dims& m) {
     return m.r <= 256 || m.N <= 48 * (int64_t)m.E;
 }
 
-// Do both contractions of the experts run in one kernel on CTA pairs?  A function of the handle, T and the debug switches: a
-// training forward and its backward must see the same (sigma' lies in memory as that kernel wants it).  ffn_pair_pays has the rule.
+// Do both contractions of the experts run in one kernel on CTA pairs?  In training a function of the handle and T: a forward and its
+// backward must agree (sigma' lies in memory as that kernel wants it).  ffn_pair_pays has the rule.
 bool uses_ffn(const bigmac_layer* L, const Dims& m, bool training) {
-    const int mode = switches().ffn;
+    const int mode = L->ffn;
     if (mode == 0 || m.bias || !sigma_as_bytes(L) || !ffn_pair_supported(m.r, m.h, m.E, m.dtype)) return false;
     if (mode == 2) return true;
     if (!training && switches().fused_mlp != 1) return false;
@@ -494,7 +494,7 @@ bool uses_ffn(const bigmac_layer* L, const Dims& m, bool training) {
 // launches for either direction and dW2, dW1 apart from the last contractions, and so: d 128, r 32, h 128, 8 experts top-2, 32 tokens
 // 52 -> 47 / 23 -> 21, 256 58 -> 52 / 24 -> 22, 2048 105 -> 83 / 39 -> 32; h 256, 32 experts top-4, 100 tokens 126 -> 77 / 45 -> 31; h 64, 4
 // experts top-1, 1024 tokens 72 -> 62 / 26.5 -> 25.4.  With r 64 it is not always the faster one (h 256, 16 experts, 256 tokens 96 -> 99).
-bool uses_ffn_simt(const Dims& m) { return switches().ffn != 0 && !m.bias && ffn_simt_supported(m.r, m.h, m.dtype); }
+bool uses_ffn_simt(const bigmac_layer* L, const Dims& m) { return L->ffn != 0 && !m.bias && ffn_simt_supported(m.r, m.h, m.dtype); }
 
 // Is the dispatch fused into its consumers' operand loads (F5 of the forward disappears as a launch, the grouped
 // copy xg of x' is never written)?  Inference: expert GEMM1 gathers the rows of x' itself.  Training: so does the
@@ -556,6 +556,7 @@ int bigmac_layer_create(const bigmac_config_t* cfg, bigmac_layer_t** out) {
     L->cfg = *cfg;
     L->use_tc = cfg->dtype == BIGMAC_BF16 && !(cfg->flags & BIGMAC_FLAG_SIMT_GEMM);
     L->tc_mask = switches().tc_mask;
+    L->ffn = switches().ffn;
     // memory of the small-batch kernel where the configuration can reach it
     const bool plain = L->use_tc && !(cfg->flags & (BIGMAC_FLAG_CDAC | BIGMAC_FLAG_GATE_LOW | BIGMAC_FLAG_EXPERT_BIAS)) &&
                        cfg->capacity_factor == 0 && cfg->aux_loss_coef == 0;
@@ -735,7 +736,7 @@ int bigmac_forward(bigmac_layer_t* L, const void* x, int32_t T, const bigmac_wei
     if (mlp_fused) {
         Stage s(L, S_FUSED_MLP, st);
         BIGMAC_CUDA(launch_fused_mlp(b.xg, W->w1, W->w2, b.a, m.P, m.N, slicing, m.r, m.h, m.E, c.act, b.tb, L->status, st));
-    } else if (uses_ffn_simt(m)) {
+    } else if (uses_ffn_simt(L, m)) {
         Stage s(L, S_FUSED_MLP, st);
         BIGMAC_CUDA(launch_ffn_simt_forward(b.xg, W->w1, W->w2, b.a, training ? b.z : nullptr, b.u, m.P, m.r, m.h, c.act, b.tb, st));
     } else if (in_pairs) {
@@ -887,7 +888,7 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         g.group = GROUP_K; g.num_experts = m.E; g.poffsets = b.tb.poffsets; g.accumulate = acc;
         BIGMAC_TRY(batch ? together.add(G_DW2, g, st) : expert_weight_grad(L, G_DW2, g, b.expert_ws, st));
     }
-    const bool narrow = uses_ffn_simt(m);        // (dz over sigma', which nothing else reads)
+    const bool narrow = uses_ffn_simt(L, m);        // (dz over sigma', which nothing else reads)
     const bool in_pairs = b.dz && !dispatch_is_fused(L, m, true) && uses_ffn(L, m, true);
     if (narrow) {
         Stage s(L, S_FUSED_MLP_BWD, st);

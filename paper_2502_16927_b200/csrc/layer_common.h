@@ -21,6 +21,7 @@ struct bigmac_layer {
     int decode_place = -1;
     bool use_tc;        // bf16 contractions on tcgen05
     unsigned tc_mask;   // debug: bit i set = contraction i runs on tcgen05 (the tc_mask switch at creation)
+    int ffn;            // debug: the ffn switch at creation (it decides how sigma' lies in `saved`)
     // second stream of the backward pass (created on first use): launches that do not depend on each other and lean
     // on different units (a tensor-bound weight gradient beside an HBM-bound row move) run side by side
     cudaStream_t side = nullptr;

@@ -9,8 +9,8 @@ struct Switches {
     int tc_pair = 1;        // CTA-pair tcgen05 kernel where it is the faster one (0: one-CTA kernel everywhere)
     int groupk = 1;         // dynamically scheduled per-expert weight-gradient kernel where it pays (0: never)
     int fused_mlp = 1;      // inference: expert GEMM1 + sigma + GEMM2 in one kernel on short tile lists (0: never, 2: always)
-    int ffn = 1;            // both contractions of an expert in one kernel on CTA pairs where it pays (0: never, 2: wherever it can);
-                            // a training forward and its backward must see the same value
+    int ffn = 1;            // both contractions of an expert in one kernel where it pays (0: never, 2: wherever it can); read when a
+                            // handle is created
     int epi_parts = 0;      // working epilogue warps per lane quadrant of plain epilogues (1, 2, 4; 0: the default, 2)
     int staged_stores = 1;  // wide bf16 outputs leave through shared-memory boxes and TMA stores (0: always 32-byte direct stores)
     int fuse_dispatch = 0;  // 1: expert GEMM1 (and dW1) gather the rows of x' themselves, no dispatch launch, no grouped copy.

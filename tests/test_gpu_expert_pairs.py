@@ -30,9 +30,9 @@ def test_equals_the_separate_contractions(r, h, E, k, T, skew, act):
     dev = to_device(w, inp)
     out = {}
     for mode in (0, 2):
-        layer = make_layer(w)
         try:
-            binding.bigmac_debug_set("ffn", mode)
+            binding.bigmac_debug_set("ffn", mode)           # read at creation
+            layer = make_layer(w)
             binding.bigmac_debug_set("fused_mlp", 0)
             infer = layer.forward(dev["x"], dev)
             y = layer.forward(dev["x"], dev, training=True)
@@ -59,9 +59,9 @@ def test_fp32_in_one_launch(d, r, h, E, k, T, capacity):
     dev = to_device(w, wl.make_inputs(w))
     out = {}
     for mode in (0, 1):
-        layer = make_layer(w, capacity_factor=capacity)
         try:
             binding.bigmac_debug_set("ffn", mode)
+            layer = make_layer(w, capacity_factor=capacity)
             infer = layer.forward(dev["x"], dev)
             y = layer.forward(dev["x"], dev, training=True)
             grads = empty_grads(w, dev)
@@ -101,3 +101,30 @@ def test_inference_under_a_capacity_limit_keeps_u_in_fp32():
         assert layer.status() == 0
         layer.close()
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("dtype,r,h,T", [(wl.DTYPE_BF16, 256, 256, 300), (wl.DTYPE_F32, 32, 128, 90)])
+@pytest.mark.parametrize("before,after", [(2, 0), (0, 2)])
+def test_switch_between_a_forward_and_its_backward(dtype, r, h, T, before, after):
+    """The kernels of the two directions agree on where sigma' lies: what the switch says when the handle is created holds for both."""
+    import torch
+    from paper_2502_16927_b200 import binding
+
+    w = wl.Workload("switch", T=T, d=128, r=r, h=h, E=5, k=2, dtype=dtype, act=wl.ACT_GELU_ERF, seed=5)
+    dev = to_device(w, wl.make_inputs(w))
+    out = []
+    for later in (before, after):
+        try:
+            binding.bigmac_debug_set("ffn", before)
+            layer = make_layer(w)
+            layer.forward(dev["x"], dev, training=True)
+            binding.bigmac_debug_set("ffn", later)
+            grads = empty_grads(w, dev)
+            dx = layer.backward(dev["x"], dev["dy"], dev, grads)
+            torch.cuda.synchronize()
+        finally:
+            binding.bigmac_debug_set("defaults")
+        out.append(dict(grads, dx=dx))
+        layer.close()
+    for name, ref in out[0].items():
+        assert torch.equal(ref, out[1][name]), name
