@@ -49,6 +49,49 @@ def test_equals_the_separate_contractions(r, h, E, k, T, skew, act):
         assert torch.isfinite(ref.float()).all(), name
 
 
+@pytest.mark.parametrize("variant,r,h,E,k,T", [("capacity", 256, 256, 6, 3, 500), ("capacity", 128, 128, 8, 2, 900), ("cdac", 128, 256, 5, 2, 300),
+                                               ("cdac", 256, 128, 3, 1, 700), ("gate_low", 256, 384, 6, 2, 333), ("accumulate", 128, 256, 7, 3, 400),
+                                               ("accumulate", 256, 128, 4, 2, 129), ("nan", 256, 256, 9, 2, 300), ("nan", 128, 384, 5, 1, 650)])
+def test_variants_equal_the_separate_contractions(variant, r, h, E, k, T):
+    """A capacity limit, the layer without projections, the gate on x', gradients added to others; tokens of NaN, whose rows lie beside the
+    unused half of another expert's last pair and leave no trace there."""
+    import torch
+    from paper_2502_16927_b200 import binding
+
+    w = wl.Workload("variant", T=T, d=r if variant == "cdac" else 192, r=r, h=h, E=E, k=k, dtype=wl.DTYPE_BF16, act=wl.ACT_GELU_ERF, seed=50 + T,
+                    cdac=variant == "cdac", gate_low=variant == "gate_low")
+    inp = wl.make_inputs(w)
+    inp["b_gate"] = np.linspace(1.0, -1.0, w.E).astype(np.float32)
+    if variant == "nan":
+        inp["x"][[0, T // 2, T - 1]] = np.nan
+    dev = to_device(w, inp)
+    out = {}
+    for mode in (0, 2):
+        try:
+            binding.bigmac_debug_set("ffn", mode)
+            layer = make_layer(w, capacity_factor=0.6 if variant == "capacity" else 0.0)
+            binding.bigmac_debug_set("fused_mlp", 0)
+            infer = layer.forward(dev["x"], dev)
+            y = layer.forward(dev["x"], dev, training=True)
+            grads = empty_grads(w, dev, fill=0.25)
+            dx = layer.backward(dev["x"], dev["dy"], dev, grads, accumulate=variant == "accumulate")
+            torch.cuda.synchronize()
+        finally:
+            binding.bigmac_debug_set("defaults")
+        assert layer.status() == 0
+        out[mode] = dict(grads, infer=infer, y=y, dx=dx)
+        layer.close()
+    for name, ref in out[0].items():
+        got = out[2][name]
+        assert torch.equal(ref.isnan(), got.isnan()) and torch.equal(ref.nan_to_num(), got.nan_to_num()), name
+    rest = torch.ones(T, dtype=torch.bool, device="cuda")
+    if variant == "nan":
+        rest[[0, T // 2, T - 1]] = False
+        assert out[2]["y"][~rest].isnan().all()
+    for name in ("infer", "y", "dx"):
+        assert torch.isfinite(out[2][name][rest].float()).all(), name
+
+
 @pytest.mark.parametrize("d,r,h,E,k,T,capacity", [(128, 32, 128, 8, 2, 33, 0.0), (64, 4, 4, 3, 1, 7, 0.0), (64, 12, 132, 5, 2, 130, 0.0),
                                                  (128, 32, 256, 6, 3, 200, 0.7), (64, 20, 60, 4, 2, 5000, 0.0), (64, 28, 252, 40, 2, 300, 0.0)])
 def test_fp32_in_one_launch(d, r, h, E, k, T, capacity):

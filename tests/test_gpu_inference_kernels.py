@@ -19,6 +19,15 @@ def _inputs(w, skew):
     return inp
 
 
+def _launches(layer, start=False):
+    """Counts the layer's launches from `start` on."""
+    from paper_2502_16927_b200 import binding
+
+    if start:
+        return binding.bigmac_profile_enable(layer.handle, True)
+    return binding.bigmac_profile_read(layer.handle)["launches"]
+
+
 def _check_tables(R, rt):
     for name in ("topk_idx", "counts", "counts_chosen", "offsets", "row_of_slot", "slot_of_row"):
         np.testing.assert_array_equal(to_numpy(R[name]), getattr(rt, name).reshape(-1), err_msg=name)
@@ -80,18 +89,25 @@ def test_experts_in_one_kernel_many_units(r, h, E):
 @pytest.mark.parametrize("E,k", [(4, 1), (8, 8), (36, 3), (64, 8), (100, 5), (256, 8)])
 @pytest.mark.parametrize("T", [1, 4, 31, 33, 128, 4737, 20003])
 def test_routing_in_two_launches(E, k, T):
+    """With a load-balancing loss every size goes through two launches (the top-k with the blocks' counts, the placement); without one, up to
+    512 tokens of at most 128 experts go through one."""
     import torch
 
     w = wl.Workload("route", T=T, d=32, r=8, h=8, E=E, k=k, dtype=wl.DTYPE_F32, act=wl.ACT_RELU, seed=33)
     inp = _inputs(w, 1.0)
     dev = to_device(w, inp)
     for f in (0.0, 0.6):
-        layer = make_layer(w, capacity_factor=f)
-        R = layer.route(dev["x"], dev)
-        torch.cuda.synchronize()
-        assert layer.status() == 0
-        _check_tables(R, oracle.route(inp, w.k, capacity_factor=f))
-        layer.close()
+        rt = oracle.route(inp, w.k, capacity_factor=f)
+        for aux in (0.0, 0.01):
+            layer = make_layer(w, capacity_factor=f, aux_loss_coef=aux)
+            _launches(layer, True)
+            R = layer.route(dev["x"], dev)
+            torch.cuda.synchronize()
+            # the logits' launch, then one or two
+            assert _launches(layer) == (2 if aux == 0 and T <= 512 and E <= 128 else 3)
+            assert layer.status() == 0
+            _check_tables(R, rt)
+            layer.close()
 
 
 @pytest.mark.parametrize("E,k,T", [(4, 1, 1), (64, 8, 5), (128, 8, 127), (132, 3, 129), (256, 8, 300), (36, 3, 512), (64, 8, 513), (128, 8, 1500), (32, 4, 3000)])
