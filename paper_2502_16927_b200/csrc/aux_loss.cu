@@ -114,8 +114,7 @@ __global__ void __launch_bounds__(256) gate_bwd_aux_kernel(float* __restrict__ d
                                                                       const float* __restrict__ logits,
                                                                       const float* __restrict__ b_gate, float coef,
                                                                       T* __restrict__ dlogits, float* __restrict__ aux_partial,
-                                                                      int n_tokens, int E, int width, int ld, int k,
-                                                                      const int32_t* __restrict__ prow_of_slot /* nullable */) {
+                                                                      int n_tokens, int E, int width, int ld, int k) {
     grid_dependency_wait();
     grid_dependency_launch();
     extern __shared__ float smem[];                  // [warps][E] column sums, [warps][E] the row being built, [E] f
@@ -152,10 +151,7 @@ __global__ void __launch_bounds__(256) gate_bwd_aux_kernel(float* __restrict__ d
         const float* pw = topk_w + (int64_t)t * k;
         float* gp = dp + (int64_t)t * k;
         float part = 0.0f;
-        for (int j = lane; j < k; j += 32) {
-            if (prow_of_slot && prow_of_slot[(int64_t)t * k + j] < 0) gp[j] = 0.0f;   // dropped under a capacity limit
-            part = fmaf(pw[j], gp[j], part);
-        }
+        for (int j = lane; j < k; j += 32) part = fmaf(pw[j], gp[j], part);
         part = warp_sum(part);
         __syncwarp();
         for (int j = lane; j < k; j += 32) {
@@ -190,18 +186,17 @@ cudaError_t launch_aux_loss(const float* logits, const float* b_gate, const int3
 
 cudaError_t launch_gate_bwd_aux(float* dp, const Tables& tb, void* dlogits, const float* logits, const float* b_gate,
                                 float coef, float* aux_partial, int T, int E, int width, int ld, int k, int dtype,
-                                cudaStream_t stream, bool may_drop) {
+                                cudaStream_t stream) {
     if (T == 0) return cudaSuccess;
-    const int32_t* prow = may_drop ? tb.prow_of_slot : nullptr;
     const int warps = aux_warps(E);
     const size_t smem = sizeof(float) * (2 * warps + 1) * E;          // at most 36 KB (E <= 1024)
     if (dtype == BIGMAC_BF16)
         (void)launch_chained(gate_bwd_aux_kernel<__nv_bfloat16>, kAuxChunks, warps * 32, smem, stream, 
             dp, tb.topk_w, tb.topk_idx, tb.counts_chosen, logits, b_gate, coef, (__nv_bfloat16*)dlogits, aux_partial, T, E,
-            width, ld, k, prow);
+            width, ld, k);
     else
         (void)launch_chained(gate_bwd_aux_kernel<float>, kAuxChunks, warps * 32, smem, stream, 
-            dp, tb.topk_w, tb.topk_idx, tb.counts_chosen, logits, b_gate, coef, (float*)dlogits, aux_partial, T, E, width, ld, k, prow);
+            dp, tb.topk_w, tb.topk_idx, tb.counts_chosen, logits, b_gate, coef, (float*)dlogits, aux_partial, T, E, width, ld, k);
     return cudaGetLastError();
 }
 

@@ -266,10 +266,9 @@ constexpr int kAuxChunks = 1184;
 cudaError_t launch_aux_loss(const float* logits, const float* b_gate, const int32_t* counts_chosen, int T, int E, int k,
                             float coef, float* partial, float* loss, cudaStream_t stream);
 // launch_gate_bwd plus dL_aux/dl: dlogits[t,e] = (top-k part) + (coef E / T) p[t,e] (f_e - sum_j f_j p[t,j]); the
-// column sums of the second term go to aux_partial [kAuxChunks, E] for launch_gate_colsum.
+// column sums of the second term go to aux_partial [kAuxChunks, E] for launch_gate_colsum.  (dp of a slot without a row is 0 already.)
 cudaError_t launch_gate_bwd_aux(float* dp, const Tables& tb, void* dlogits, const float* logits, const float* b_gate,
-                                float coef, float* aux_partial, int T, int E, int width, int ld, int k, int dtype,
-                                cudaStream_t stream, bool may_drop = false);
+                                float coef, float* aux_partial, int T, int E, int width, int ld, int k, int dtype, cudaStream_t stream);
 // db[e] (+)= sum over the slots routed to e of dl_slot[slot] (the fp32 per-slot gate gradients launch_gate_bwd
 // leaves in dp); `partial` holds kColsumChunks * E floats of scratch.  Deterministic summation order.
 constexpr int kColsumChunks = 296;

@@ -871,7 +871,7 @@ static int backward_launches(bigmac_layer_t* L, const void* x, const void* dy, i
         aux_part = b.colsum_part + (size_t)kColsumChunks * m.E;
         Stage s(L, S_GATE_BWD, st);
         BIGMAC_CUDA(launch_gate_bwd_aux(b.dp, b.tb, b.dlogits, b.logits_saved, W->b_gate, m.aux, aux_part, m.T, m.E, m.E64,
-                                        ldcat, m.k, m.dtype, st, m.cap != kNoCapacity));
+                                        ldcat, m.k, m.dtype, st));
     }
     bool colsum_done = false;
     if (overlap && G->db_gate) {
