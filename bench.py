@@ -84,10 +84,40 @@ GEMM_BYTES = {
     "gemm_dx_gate": lambda w, b: (w.T * _e64(w) + w.E * w.d) * b,
     "gemm_dw_down": lambda w, b: (w.T * w.r + w.T * w.d + w.r * w.d) * b,
     "gemm_dw_gate": lambda w, b: (w.T * _e64(w) + w.E * w.d) * b,
-    # both contractions of an expert in one launch; a training step also writes (reads) a or dz and sigma' (BF16 path only)
-    "fused_expert_mlp": lambda w, b: (2.0 * w.N * w.r + 2.0 * w.E * w.h * w.r + w.N * w.h) * b + w.N * w.h,
-    "fused_expert_mlp_bwd": lambda w, b: (2.0 * w.N * w.r + 2.0 * w.E * w.h * w.r + w.N * w.h) * b + w.N * w.h,
+    # both contractions of an expert in one launch; a training step also writes (reads) a or dz and sigma'
+    "fused_expert_mlp": lambda w, b: (2.0 * w.N * w.r + 2.0 * w.E * w.h * w.r + w.N * w.h) * b + w.N * w.h * (1 if b == 2 else b),
+    "fused_expert_mlp_bwd": lambda w, b: (2.0 * w.N * w.r + 2.0 * w.E * w.h * w.r + w.N * w.h) * b + w.N * w.h * (1 if b == 2 else b),
 }
+
+
+def stage_work(w, b, calls, steps, training):
+    """FLOPs and bytes per launch of every contraction stage, given the launches recorded of each in `steps` steps: what a
+    launch does for a stage that has none of its own is counted with it."""
+    flops = {name: fn(w) for name, fn in GEMM_FLOPS.items()}
+    size = {name: fn(w, b) for name, fn in GEMM_BYTES.items()}
+    if not training:                                # the hidden activations stay on the chip
+        size["fused_expert_mlp"] = (2.0 * w.N * w.r + 2.0 * w.E * w.h * w.r) * b
+    if "gemm_batch" in calls:                       # fp32 path: independent contractions in one launch
+        inside = {"fused_expert_mlp": ("gemm_expert1", "gemm_expert2"), "fused_expert_mlp_bwd": ("gemm_dz", "gemm_dxg")}
+        taken = {n for stage, parts in inside.items() if stage in calls for n in parts} | set(inside) | set(calls)
+        if not training:
+            taken |= set(GEMM_FLOPS) - {"gemm_logits", "gemm_descend"}
+        batched = [n for n in GEMM_FLOPS if n not in taken]
+        launches = calls["gemm_batch"] / steps
+        flops["gemm_batch"] = sum(flops[n] for n in batched) / launches
+        size["gemm_batch"] = sum(size[n] for n in batched) / launches
+        return flops, size
+    if "gemm_logits" not in calls:                  # gate logits computed by the descend launch
+        flops["gemm_descend"] += flops["gemm_logits"]
+        size["gemm_descend"] += b * w.E * w.d + 4.0 * w.T * w.E
+    if "gemm_dx_gate" not in calls:                 # gate part fused into the dx contraction
+        flops["gemm_dx"] += flops["gemm_dx_gate"]
+        size["gemm_dx"] += size["gemm_dx_gate"]
+    if "gemm_dw_gate" not in calls:                 # dW_gate computed together with dW_down
+        flops["gemm_dw_down"] += flops["gemm_dw_gate"]
+        size["gemm_dw_down"] += size["gemm_dw_gate"]
+    return flops, size
+
 
 # DRAM bytes per launch of the two output-heavy contractions as ncu counted them (dram__bytes_read.sum +
 # dram__bytes_write.sum) on a SMALL case of the large workload's widths (T = 8192, N = 65536 routed rows, one launch
@@ -997,25 +1027,12 @@ def run_ours(args, w):
                                                  and not forward_only_workload) else None
     stages = {}
     gemm_ms = gemm_flops = 0.0
-    flops_of = {name: fn(w) for name, fn in GEMM_FLOPS.items()}
-    if "gemm_logits" not in prof["stages"]:         # gate logits computed by the descend launch
-        flops_of["gemm_descend"] += flops_of["gemm_logits"]
-    if "gemm_dx_gate" not in prof["stages"]:        # gate part fused into the dx contraction
-        flops_of["gemm_dx"] += flops_of["gemm_dx_gate"]
-    if "gemm_dw_gate" not in prof["stages"]:        # dW_gate computed together with dW_down
-        flops_of["gemm_dw_down"] += flops_of["gemm_dw_gate"]
-    bytes_of = {name: fn(w, esz) for name, fn in GEMM_BYTES.items()}
-    if "gemm_logits" not in prof["stages"]:
-        bytes_of["gemm_descend"] += esz * w.E * w.d + 4.0 * w.T * w.E
-    if "gemm_dx_gate" not in prof["stages"]:
-        bytes_of["gemm_dx"] += bytes_of["gemm_dx_gate"]
-    if "gemm_dw_gate" not in prof["stages"]:
-        bytes_of["gemm_dw_down"] += bytes_of["gemm_dw_gate"]
+    flops_of, bytes_of = stage_work(w, esz, {name: calls for name, (_, calls) in prof["stages"].items()}, args.steps, not forward_only_workload)
     gemm_bytes = 0.0
     for name, (ms, calls) in prof["stages"].items():
         per = ms / calls
         entry = {"ms": round(per, 4), "launches_per_step": calls // args.steps}
-        if name in GEMM_FLOPS:
+        if name in flops_of:
             fl = flops_of[name]
             entry["tflops"] = round(fl / (per * 1e-3) / 1e12, 1)
             entry["frac_of_measured_sustained"] = round(entry["tflops"] / peaks["tflops_sustained"], 3)
@@ -1045,11 +1062,11 @@ def run_ours(args, w):
                                                       "frac_of_measured_hbm": round(m_gbs / peaks["hbm_gbs"], 3)}}
     achieved = gemm_flops / (gemm_ms * 1e-3) / 1e12 if gemm_ms > 0 else 0.0
     fwd_fl = forward_flops(w)
-    all_gemms = {"kernels": "every tcgen05 contraction launch of a step", "launches_per_step": sum(stages[n]["launches_per_step"] for n in stages if n in GEMM_FLOPS),
+    all_gemms = {"kernels": "every tcgen05 contraction launch of a step", "launches_per_step": sum(stages[n]["launches_per_step"] for n in stages if n in flops_of),
                  "achieved": round(achieved, 1), "unit": "TFLOP/s", "frac": round(achieved / peaks["tflops_sustained"], 4),
                  "frac_of_burst_peak": round(achieved / peaks["tflops_burst"], 4), "ms_per_step": round(gemm_ms / args.steps, 4),
                  "algorithmic_bytes_per_step": gemm_bytes / args.steps}
-    gemm_stages = [n for n in stages if n in GEMM_FLOPS]
+    gemm_stages = [n for n in stages if n in flops_of]
     if forward_only_workload:
         # decode-shaped batches stream the touched weights once: the bound is HBM, not the tensor pipe
         roofline = {"bound": "hbm", "kernel": "inference forward (every launch of a call)",

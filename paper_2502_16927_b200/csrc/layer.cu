@@ -268,7 +268,7 @@ struct Together {
     }
     int flush() {
         if (n == 0) return BIGMAC_OK;
-        Stage stage(L, first_id, st);
+        Stage stage(L, n == 1 ? first_id : (int)S_GEMM_BATCH, st);
         const cudaError_t err = gemm_simt_batch(g, n, L->cfg.dtype, st);
         n = 0;
         return err == cudaSuccess ? BIGMAC_OK : BIGMAC_ERR_CUDA;

@@ -44,12 +44,12 @@ namespace detail {
 enum { G_LOGITS = 0, G_DESCEND, G_EXPERT1, G_EXPERT2, G_ASCEND, G_DY_LO, G_DW_UP, G_DZ, G_DW2, G_DXG, G_DW1,
        G_DX, G_DX_GATE, G_DW_DOWN, G_DW_GATE,
        S_TOPK, S_TABLES, S_DISPATCH, S_COMBINE, S_COMBINE_BWD, S_GATE_BWD, S_DXLO_GATHER, S_COLSUM, S_SPLITK_REDUCE,
-       S_DECODE, S_FUSED_MLP, S_AUX_LOSS, S_FUSED_MLP_BWD, S_COUNT };
+       S_DECODE, S_FUSED_MLP, S_AUX_LOSS, S_FUSED_MLP_BWD, S_GEMM_BATCH, S_COUNT };
 const char* const kSlotNames[S_COUNT] = {
     "gemm_logits", "gemm_descend", "gemm_expert1", "gemm_expert2", "gemm_ascend", "gemm_dy_lo", "gemm_dw_up",
     "gemm_dz", "gemm_dw2", "gemm_dxg", "gemm_dw1", "gemm_dx", "gemm_dx_gate", "gemm_dw_down", "gemm_dw_gate",
     "topk", "tables", "dispatch", "combine", "combine_bwd", "gate_bwd", "dxlo_gather", "colsum",
-    "splitk_reduce", "decode_forward", "fused_expert_mlp", "aux_loss", "fused_expert_mlp_bwd"};
+    "splitk_reduce", "decode_forward", "fused_expert_mlp", "aux_loss", "fused_expert_mlp_bwd", "gemm_batch"};
 constexpr size_t kEventPairs = 8192;
 constexpr int kMaxSplitK = 8;
 
