@@ -189,12 +189,12 @@ void carve_backward_scratch(Carver& cv, const Dims& m, Buffers& b) {
 // shapes 4.5 %, small layers of d 512 up to 6 %); from 700 to 1500 tokens of d 1024, and 700 to 1000 of d 2048, one part would be the
 // better choice (39.3 against 35.1 us, 57.3 against 52.1).  A function of the shape only: every call of a handle with the same T takes the same path.
 int split_parts(const Dims& m, int n) {
-    const int num_kb = m.d / 64;
+    const int num_kb = m.d / 64, sms = gemm_tc_sm_count();
     int best = 1;
     double best_cost = 0;
     for (int s = 1; s <= kMaxSplitK && s <= num_kb; ++s) {
         const bool pairs = n >= 256 && !(m.r % 128 == 0 && gemm_tc_one_round(m.T, n, s));
-        const int b = pairs ? 256 : 128, units = gemm_tc_sm_count() / (pairs ? 2 : 1);
+        const int b = pairs ? 256 : 128, units = sms / (pairs ? 2 : 1);
         const int64_t tiles = (int64_t)((m.T + b - 1) / b) * ((n + b - 1) / b);
         double cost = (double)((tiles * s + units - 1) / units) * ((num_kb + s - 1) / s) * (pairs ? 0.35 : 0.2);
         if (s > 1) cost += (double)s * m.T * n * 4.0 * 0.8e-6;
