@@ -6,7 +6,9 @@
 //
 // A block has ROWS rows of one expert and walks the hidden width in chunks of 128 columns: both weight chunks and the rows are
 // staged at once; a thread sums ROWS / 8 x 4 of the chunk's ROWS x 128 middle (its warp shares the rows: broadcasts; the columns are 32
-// apart: no conflicts), then ROWS / 16 x r / 16 of the ROWS x r output, whose sums stay in registers over the chunks.
+// apart: no conflicts), then ROWS / 16 x r / 16 of the ROWS x r output, whose sums stay in registers over the chunks.  Four terms of the
+// middle and sixteen of the output are added up before they join the others: the separate contractions, whose warps each have a
+// part of the sum, are as exact; one running sum was 1.15 to 1.6 times as far from 64 bits (256 tokens 50.3 -> 50.6 us a training step).
 // Bound by latency.  Blocks of 16 rows while four of them for an SM are enough, else of 32 (256 tokens, training: 59.5 us with 32
 // rows, 58.4 with separate contractions, 55 with 16); blocks with nothing but padding rows only write the zeros that the weight
 // gradients want there (55 -> 52).  Figures at uses_ffn_simt.
@@ -99,11 +101,10 @@ __global__ void __launch_bounds__(kThreads, 3) ffn_simt_kernel(const FfnSimtArgs
                     for (int q = 0; q < 4; ++q) b[j][q] = s_w2[(k + q) * LDC + tn + 32 * j];
             }
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
+            for (int i = 0; i < RI; ++i)
 #pragma unroll
-                for (int i = 0; i < RI; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i][q], b[j][q], acc[i][j]);
+                for (int j = 0; j < 4; ++j)              // four terms, then to the others
+                    acc[i][j] += fmaf(a[i][3], b[j][3], fmaf(a[i][2], b[j][2], fmaf(a[i][1], b[j][1], a[i][0] * b[j][0])));
         }
 #pragma unroll
         for (int i = 0; i < RI; ++i)
@@ -125,24 +126,33 @@ __global__ void __launch_bounds__(kThreads, 3) ffn_simt_kernel(const FfnSimtArgs
             }
         }
         __syncthreads();
-#pragma unroll 4
-        for (int k = 0; k < width; k += 4) {
-            float a[RO][4];
+        for (int k0 = 0; k0 < width; k0 += 16) {         // sixteen terms, then to the others
+            float part[RO][kMaxR / 16] = {};
 #pragma unroll
-            for (int i = 0; i < RO; ++i) *reinterpret_cast<float4*>(a[i]) = *reinterpret_cast<const float4*>(s_mid + (om + i) * LDC + k);
+            for (int kk = 0; kk < 16; kk += 4) {
+                const int k = k0 + kk;
+                if (k >= width) break;
+                float a[RO][4];
 #pragma unroll
-            for (int j = 0; j < kMaxR / 16; ++j) {
-                if (on + 16 * j >= r) continue;
-                float b[4];
-                if (!BWD) *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(s_w2 + (on + 16 * j) * LDC + k);
-                else
+                for (int i = 0; i < RO; ++i) *reinterpret_cast<float4*>(a[i]) = *reinterpret_cast<const float4*>(s_mid + (om + i) * LDC + k);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) b[q] = s_w1[(k + q) * ldr + on + 16 * j];
+                for (int j = 0; j < kMaxR / 16; ++j) {
+                    if (on + 16 * j >= r) continue;
+                    float b[4];
+                    if (!BWD) *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(s_w2 + (on + 16 * j) * LDC + k);
+                    else
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
+                        for (int q = 0; q < 4; ++q) b[q] = s_w1[(k + q) * ldr + on + 16 * j];
 #pragma unroll
-                    for (int i = 0; i < RO; ++i) out[i][j] = fmaf(a[i][q], b[q], out[i][j]);
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int i = 0; i < RO; ++i) part[i][j] = fmaf(a[i][q], b[q], part[i][j]);
+                }
             }
+#pragma unroll
+            for (int i = 0; i < RO; ++i)
+#pragma unroll
+                for (int j = 0; j < kMaxR / 16; ++j) out[i][j] += part[i][j];
         }
     }
 #pragma unroll

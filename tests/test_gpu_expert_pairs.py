@@ -171,3 +171,48 @@ def test_switch_between_a_forward_and_its_backward(dtype, r, h, T, before, after
         layer.close()
     for name, ref in out[0].items():
         assert torch.equal(ref, out[1][name]), name
+
+
+def _step_in_64_bits(w, dev, idx):
+    """y and the gradients of a layer without biases or limit, for the given routing, by torch in 64 bits."""
+    import torch
+
+    P = {n: dev[n].double().requires_grad_() for n in ("w_gate", "w_down", "w1", "w2", "w_up")}
+    x = dev["x"].double().requires_grad_()
+    weight = torch.softmax((x @ P["w_gate"].t()).gather(1, idx), 1)
+    low = x @ P["w_down"].t()
+    mixed = torch.zeros_like(low)
+    for e in range(w.E):
+        t, j = (idx == e).nonzero(as_tuple=True)
+        u = torch.nn.functional.gelu(low[t] @ P["w1"][e].t()) @ P["w2"][e].t()
+        mixed = mixed.index_add(0, t, weight[t, j, None] * u)
+    y = mixed @ P["w_up"].t()
+    y.backward(dev["dy"].double())
+    return dict({"d" + n: p.grad for n, p in P.items()}, y=y.detach(), dx=x.grad)
+
+
+@pytest.mark.parametrize("d,r,h,E,k,T", [(128, 32, 128, 8, 2, 2048), (128, 32, 256, 16, 4, 700), (256, 16, 252, 12, 3, 700), (64, 32, 128, 4, 2, 6000)])
+def test_fp32_in_one_launch_is_as_exact(d, r, h, E, k, T):
+    """Distance from 64 bits: no larger than that of the separate contractions, whose sums are of short parts.  (Distances of these
+    sizes repeat within 4 % from seed to seed; one running sum of h terms was 1.15 to 1.6 times as far off.)"""
+    import torch
+    from paper_2502_16927_b200 import binding
+
+    w = wl.Workload("exact", T=T, d=d, r=r, h=h, E=E, k=k, dtype=wl.DTYPE_F32, act=wl.ACT_GELU_ERF, seed=12 + T)
+    dev = to_device(w, wl.make_inputs(w))
+    far = {}
+    for mode in (0, 1):
+        try:
+            binding.bigmac_debug_set("ffn", mode)
+            layer = make_layer(w)
+            y, R = layer.forward(dev["x"], dev, training=True, want_routing=True)
+            grads = empty_grads(w, dev)
+            dx = layer.backward(dev["x"], dev["dy"], dev, grads)
+            torch.cuda.synchronize()
+        finally:
+            binding.bigmac_debug_set("defaults")
+        ref = _step_in_64_bits(w, dev, R["topk_idx"].view(T, k).long())
+        far[mode] = {n: float((g.double() - ref[n]).norm() / ref[n].norm()) for n, g in dict(grads, y=y, dx=dx).items() if n in ref}
+        layer.close()
+    for name, before in far[0].items():
+        assert far[1][name] <= 1.08 * before, (name, far[1][name], before)
