@@ -80,7 +80,7 @@ inline double item_rounds(const ExpertCall& m, int size, int units, bool even) {
 // Where the kernel on CTA pairs pays, among the widths it takes.  How full its last round of pairs is depends on the loads, which only
 // the device knows, so both estimates have to allow it.  The lines were set on steps and forwards of r 128 (d 1024) and r 256 (d 2048) with
 // h 128 to 4096, 8 to 256 experts, 8 to 3000 rows an expert, even and Zipf loads: of 1684 shapes a training step goes to the pairs
-// with 624, 553 of them faster by more than 1.5 % and two slower (2.2 %), a forward with 452, 428 faster and seven slower (3.5 % at most; up
+// with 630, 555 of them faster by more than 1.5 % and two slower (2.2 %), a forward with 452, 428 faster and seven slower (3.5 % at most; up
 // to 10 % where loads just miss the estimated number of rounds).
 // Figures: us, the other kernels -> this one; loads even unless said.
 //
@@ -94,7 +94,8 @@ inline double item_rounds(const ExpertCall& m, int size, int units, bool even) {
 // the hidden width is: 8 experts top-2, 300 tokens, r 128, h 256 103 -> 96, 512 105 -> 103, 1024 108 -> 115, 2048 111 -> 141, 4096 125 -> 197; r 256,
 // h 1024 123 -> 130, 2048 134 -> 158; 8192 tokens, 0.9 of the round: r 128, h 2048 235 -> 223, r 256, h 2048 330 -> 311.
 // With more rounds an expert needs the rows, a pair that is half empty costs a whole one: 256 experts top-8, 1280 tokens (40 rows), r 256, h 256
-// 201 -> 214, 2048 573 -> 600, r 128, h 1024 266 -> 312; 6080 tokens (190 rows), r 256, h 256 320 -> 285, 2048 809 -> 774.  Very large batches of r 256, under
+// 201 -> 214, 2048 573 -> 600, r 128, h 1024 266 -> 312; 6080 tokens (190 rows), r 256, h 256 320 -> 285, 2048 809 -> 774; r 128, h 512, 128
+// experts, Zipf, 190 to 256 rows 195 -> 207 and 219 -> 239, 375 and 512 rows 267 -> 271 and 325 -> 317.  Very large batches of r 256, under
 // the power cap: h 1024, 64 experts, 20500 tokens 943 -> 983, 24000 1127 -> 1125, 29000 1333 -> 1335, 256 experts, 32000 1678 -> 1742.  r 128 with h 128 wins
 // little (64 experts, 3000 tokens 117 -> 115; 256 experts, 12000 254 -> 259).
 //
@@ -130,7 +131,7 @@ inline bool ffn_pair_pays(const ExpertCall& m) {
         const double rounds = item_rounds(m, 2 * kPad, m.units / 2, even != 0), whole = std::ceil(1.03 * rounds);        // an estimate
         const bool one_tile = m.training && !wide && chunks <= 4 && rounds < 0.6 && rows >= 60 && rows <= 112;
         if (!one_tile && (whole > 1 ? rounds < least * whole : rounds < least_of_one)) return false;
-        if (m.training && !one_tile && (whole > 1 ? rows < 176 : chunks > 2 && rows < (wide ? 60 : 176))) return false;
+        if (m.training && !one_tile && (whole > 1 ? rows < (wide || chunks <= 2 ? 176 : 300) : chunks > 2 && rows < (wide ? 60 : 176))) return false;
         if (!m.training && mlp && std::ceil(0.985 * item_rounds(m, kPad, m.units, even != 0)) < (wide || chunks <= 4 ? 0.78 : 0.95) * std::ceil(rounds)) return false;
     }
     return true;
