@@ -19,9 +19,10 @@
 // memory and back in an order of its own, which only this kernel knows: the bytes of (row tile, chunk, warp) in the order of
 // the warp's 16-byte accesses.
 //
-// What bounds it: the epilogue warps beside the writing of the middle.  Clock stamps, d 2048 r 256 h 1024, cycles a chunk of 128
-// columns: 4600 forward, 4100 backward, of which the MMAs need 2050; 3200 without the stores, 2750 without arithmetic either.
-// 131072 rows forward write 0.40 GB (103 us at the 3.9 TB/s this part writes at) in 155 us at 1.9 GHz; as two launches 126 + 82 us.
+// What bounds it: the epilogue warps beside the writing of the middle.  d 2048 r 256 h 1024, 3001 tokens, cycles a chunk of 128 columns (ncu, active
+// cycles over the chunks of a pair): 4900 training forward, 4300 backward, 3650 inference, of which the MMAs need 2050; clock stamps of an
+// earlier build had 3200 forward without the stores, 2750 without arithmetic either.  131072 rows forward write 0.40 GB (103 us at the
+// 3.9 TB/s this part writes at) in 190 us under the power cap (as two launches 133 + 78), backward 168 (99 + 78).
 // Measured on the way there (3001 tokens' experts, inference / training forward, us): all sixteen warps on every chunk, A one
 // ahead 54 / 64; two groups 48 / 59; A two ahead 44 / 59; sigma' past shared memory, whose place the ring takes 43 / 53.
 #include "tc_pair.cuh"
