@@ -80,7 +80,7 @@ inline double item_rounds(const ExpertCall& m, int size, int units, bool even) {
 // Where the kernel on CTA pairs pays, among the widths it takes.  How full its last round of pairs is depends on the loads, which only
 // the device knows, so both estimates have to allow it.  The lines were set on steps and forwards of r 128 (d 1024) and r 256 (d 2048) with
 // h 128 to 4096, 8 to 256 experts, 8 to 3000 rows an expert, even and Zipf loads: of 1684 shapes a training step goes to the pairs
-// with 630, 555 of them faster by more than 1.5 % and two slower (2.2 %), a forward with 452, 428 faster and seven slower (3.5 % at most; up
+// with 626, 553 of them faster by more than 1.5 % and two slower (2.2 %), a forward with 452, 428 faster and seven slower (3.5 % at most; up
 // to 10 % where loads just miss the estimated number of rounds).
 // Figures: us, the other kernels -> this one; loads even unless said.
 //
@@ -120,7 +120,7 @@ inline bool ffn_pair_pays(const ExpertCall& m) {
     if (m.training) {
         if (wide ? chunks > 2 && m.N() > 160000 : chunks == 1) return false;
         if (wide && chunks >= 16) least = 0.8;
-        if (chunks > (wide ? 4 : 2)) least_of_one = wide ? std::fmin(0.72, 0.1 + chunks / 32.0) : chunks <= 4 ? 0.6 : 0.87;
+        if (chunks > (wide ? 4 : 2)) least_of_one = wide ? std::fmin(0.72, 0.08 + chunks / 27.0) : chunks <= 4 ? 0.6 : 0.87;
     } else {
         const double fewest = (double)m.k * std::fmin((double)m.T, (double)m.cap);
         const double cut_up_to = 128.0 * m.units * (chunks <= 10 ? 0.5 : chunks / 8.0);    // rows

@@ -67,7 +67,7 @@ def test_pairs_only_where_they_were_the_faster_ones(tmp_path):
     the kernel on CTA pairs made slower by 3 to 45 % keep their kernels, the ones that it made faster have it."""
     slower = [(1, 128, 512, 32, 4, 4200), (1, 128, 512, 32, 4, 1800), (1, 128, 1024, 8, 2, 300), (1, 128, 2048, 8, 2, 300), (1, 128, 2048, 8, 2, 3000),
               (1, 128, 4096, 8, 2, 32), (1, 128, 2048, 64, 2, 1678), (1, 128, 1024, 256, 8, 1280), (1, 128, 128, 256, 8, 9000), (1, 128, 512, 128, 2, 13177), (1, 256, 2048, 8, 2, 300),
-              (1, 256, 2048, 8, 2, 3000), (1, 256, 2048, 64, 3, 286), (1, 256, 256, 256, 1, 3832), (1, 256, 256, 256, 8, 1000), (1, 256, 2048, 256, 8, 3000),
+              (1, 256, 2048, 8, 2, 3000), (1, 256, 2048, 64, 3, 286), (1, 256, 2048, 16, 1, 9386), (1, 256, 256, 256, 1, 3832), (1, 256, 256, 256, 8, 1000), (1, 256, 2048, 256, 8, 3000),
               (1, 256, 1024, 64, 8, 700), (1, 256, 1024, 64, 8, 20500), (1, 256, 1024, 256, 8, 32000), (0, 128, 2048, 128, 8, 6000),
               (0, 128, 1024, 64, 8, 4096), (0, 128, 512, 64, 8, 4096), (0, 128, 2048, 128, 8, 8192), (0, 128, 512, 32, 4, 8700), (0, 256, 1024, 128, 8, 3040),
               (0, 256, 2048, 128, 8, 6000), (0, 256, 1024, 64, 8, 1150), (0, 128, 128, 256, 8, 16384)]
